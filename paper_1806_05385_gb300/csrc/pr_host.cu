@@ -359,16 +359,6 @@ pr_status derive_view(const pr_view &in, int tile, int bound, int fp64, ViewDev 
     v.H = in.H;
     v.mode = in.mode;
     v.S = tile;
-    {
-        // division by the blocks per row as a multiply (the round-up
-        // reciprocal of Granlund and Montgomery, 1994): lb bw_mul / 2^40
-        // exceeds lb / bw by lb e / (bw 2^40), e = bw_mul bw - 2^40 < bw; for
-        // lb < 2^23 and bw <= 2^11 that is below 2^-6 / bw, less than the
-        // 1 / bw from any fraction of lb / bw to the next integer, so the
-        // floor is exact
-        const unsigned long long bw = (unsigned long long)((in.W + kBlkW - 1) / kBlkW);
-        v.bw_mul = ((1ull << 40) + bw - 1) / bw;
-    }
     v.tiles_x = (in.W + tile - 1) / tile;
     v.tiles_y = (in.H + tile - 1) / tile;
     v.bound = bound;
@@ -395,6 +385,31 @@ pr_status make_viewdev(const pr_view &in, const pr_scene *sc, int tile, int boun
     return PR_OK;
 }
 
+// Lays out the views' strips of pixel blocks: blk_off and bw_mul of each
+// view, blk[0..n] their offsets.  Returns the blocks per strip.
+int set_strips(ViewDev *vd, int n, long long *blk)
+{
+    long long blocks = 0;
+    for (int k = 0; k < n; ++k)
+        blocks += pixel_blocks(vd[k].W, vd[k].H);
+    const int nsub = strip_blocks(blocks);
+    blk[0] = 0;
+    for (int k = 0; k < n; ++k) {
+        ViewDev &v = vd[k];
+        // division by the strips per row as a multiply (the round-up
+        // reciprocal of Granlund and Montgomery, 1994): lb bw_mul / 2^40
+        // exceeds lb / bw by lb e / (bw 2^40), e = bw_mul bw - 2^40 < bw; for
+        // lb < 2^23 and bw <= 2^11 that is below 2^-6 / bw, less than the
+        // 1 / bw from any fraction of lb / bw to the next integer, so the
+        // floor is exact
+        const unsigned long long bw = (unsigned long long)((v.W + nsub * kBlkW - 1) / (nsub * kBlkW));
+        v.bw_mul = ((1ull << 40) + bw - 1) / bw;
+        v.blk_off = blk[k];
+        blk[k + 1] = blk[k] + pixel_blocks(v.W, v.H, nsub);
+    }
+    return nsub;
+}
+
 pr_params default_params(const pr_params *p)
 {
     pr_params d{PR_BOUND_ZENON, kDefaultTile, 0, kDefaultSeg, PR_FOV_SECTOR, 0};
@@ -414,6 +429,7 @@ struct BatchPlan {
     std::vector<ViewDev> vd;          // in `order`
     std::vector<long long> tri_off, tile_off, pix_off, blk_off;
     long long ttot = 0, ntiles = 0, npix = 0, nblk = 0;
+    int nsub = 1;                     // pixel blocks per strip (nblk strips)
     struct Cls {
         int S;
         bool fp64;
@@ -476,8 +492,6 @@ pr_status plan_batch(const pr_batch_view *views, int n, const pr_params &prm, Ba
         v.tri_off = P.tri_off[q];
         v.tile_off = P.tile_off[q];
         v.pix_off = P.pix_off[q];
-        v.blk_off = P.blk_off[q];
-        P.blk_off[q + 1] = P.blk_off[q] + pixel_blocks(v.W, v.H);
         P.tri_off[q + 1] = P.tri_off[q] + bv.scene->T;
         P.tile_off[q + 1] = P.tile_off[q] + (long long)v.tiles_x * v.tiles_y;
         P.pix_off[q + 1] = P.pix_off[q] + (long long)v.W * v.H;
@@ -516,6 +530,7 @@ pr_status plan_batch(const pr_batch_view *views, int n, const pr_params &prm, Ba
     P.ttot = P.tri_off[n];
     P.ntiles = P.tile_off[n];
     P.npix = P.pix_off[n];
+    P.nsub = set_strips(P.vd.data(), n, P.blk_off.data());
     P.nblk = P.blk_off[n];
     P.stage_bytes = stage;
     if (P.ttot >= (1ll << 32) - 1)
@@ -716,7 +731,7 @@ pr_status enqueue_batch(pr_workspace *ws, BatchPlan &P, int seg, bool shade, cud
         PR_TRY(launch_resolve(dv, n, pix_offs, P.npix, ws->keys.as<unsigned long long>(), reader_resets, st));
     PR_TRY(mark(5));
     if (shade)  // resolves the keys too, and in a training frame runs the adjoint
-        PR_TRY(launch_shade(dv, n, blk_offs, P.nblk, ws->keys.as<unsigned long long>(), reader_resets,
+        PR_TRY(launch_shade(dv, n, blk_offs, P.nblk, P.nsub, ws->keys.as<unsigned long long>(), reader_resets,
                             !P.grads.empty(), cnt, shade_features(P.vd.data(), n), st, P.vd.data()));
     if (shade && P.any_loss)  // the views' loss partial sums into the callers' losses
         PR_TRY(launch_loss_finalize(dv, n, cnt, st));
@@ -821,17 +836,17 @@ pr_status single_view(pr_scene *sc, const pr_view *view, const pr_params *params
 }
 
 // One-view table for stages (d)/(e) called on their own.
-pr_status upload_single(pr_scene *sc, const ViewDev &v, cudaStream_t st)
+pr_status upload_single(pr_scene *sc, ViewDev &v, int &nsub, long long &nblk, cudaStream_t st)
 {
     pr_workspace *ws = &sc->ws;
     PR_TRY(ensure(ws->views, sizeof(ViewDev)));
     PR_TRY(ensure(ws->offs, sizeof(long long) * 6));
     PR_TRY(ws->h_views.ensure(1));
     PR_TRY(ws->h_offs.ensure(6));
-    ws->h_views.p[0] = v;
     long long *o = ws->h_offs.p;
-    o[0] = 0;
-    o[1] = pixel_blocks(v.W, v.H);  // warp pixel blocks
+    nsub = set_strips(&v, 1, o);
+    nblk = o[1];
+    ws->h_views.p[0] = v;
     o[2] = o[3] = o[4] = o[5] = 0;
     PR_TRY(cudaMemcpyAsync(ws->views.p, ws->h_views.p, sizeof(ViewDev), cudaMemcpyHostToDevice, st));
     PR_TRY(cudaMemcpyAsync(ws->offs.p, o, sizeof(long long) * 2, cudaMemcpyHostToDevice, st));
@@ -1047,12 +1062,13 @@ pr_status pr_shade(pr_scene *sc, const pr_view *view, const uint32_t *id, float 
         PR_TRY(ensure(*ob, sizeof(float) * 3 * np));
     v.id_in = did;
     v.rgb_out = host_out ? ob->as<float>() : rgb_out;
-    s = upload_single(sc, v, st);
+    int nsub = 1;
+    long long nblk = 0;
+    s = upload_single(sc, v, nsub, nblk, st);
     if (s != PR_OK)
         return s;
-    PR_TRY(launch_shade(sc->ws.views.as<ViewDev>(), 1, sc->ws.offs.as<long long>(),
-                        pixel_blocks(v.W, v.H), nullptr, false, false, nullptr,
-                        shade_features(&v, 1), st, &v));
+    PR_TRY(launch_shade(sc->ws.views.as<ViewDev>(), 1, sc->ws.offs.as<long long>(), nblk, nsub, nullptr, false, false,
+                        nullptr, shade_features(&v, 1), st, &v));
     if (host_out)
         PR_TRY(cudaMemcpyAsync(rgb_out, ob->p, sizeof(float) * 3 * np, cudaMemcpyDeviceToHost, st));
     PR_TRY(cudaStreamSynchronize(st));
@@ -1100,11 +1116,13 @@ pr_status pr_backward(pr_scene *sc, const pr_view *view, const uint32_t *id, con
     v.dcol = douts[0];
     v.dpos = douts[1];
     v.dvel = douts[2];
-    s = upload_single(sc, v, st);
+    int nsub = 1;
+    long long nblk = 0;
+    s = upload_single(sc, v, nsub, nblk, st);
     if (s != PR_OK)
         return s;
-    PR_TRY(launch_backward(sc->ws.views.as<ViewDev>(), 1, sc->ws.offs.as<long long>(),
-                           pixel_blocks(v.W, v.H), nullptr, shade_features(&v, 1), st, &v));
+    PR_TRY(launch_backward(sc->ws.views.as<ViewDev>(), 1, sc->ws.offs.as<long long>(), nblk, nsub, shade_features(&v, 1),
+                           st, &v));
     for (int a = 0; a < 3; ++a)
         if (host[a])
             PR_TRY(cudaMemcpyAsync(outs[a], douts[a], sizeof(float) * 3 * V, cudaMemcpyDeviceToHost, st));
@@ -1122,7 +1140,6 @@ pr_status pr_backward_batch(pr_workspace *ws, const pr_backward_view *views, int
     PR_TRY(ensure(ws->views, sizeof(ViewDev) * n));
     PR_TRY(ensure(ws->offs, sizeof(long long) * (n + 1)));
     long long *blk = ws->h_offs.p;
-    blk[0] = 0;
     for (int k = 0; k < n; ++k) {
         const pr_backward_view &b = views[k];
         if (!b.scene || !b.id || !b.grad_rgb || !is_device_ptr(b.id) || !is_device_ptr(b.grad_rgb) ||
@@ -1138,13 +1155,12 @@ pr_status pr_backward_batch(pr_workspace *ws, const pr_backward_view *views, int
         v.dcol = b.dcol;
         v.dpos = b.dpos;
         v.dvel = b.dvel;
-        v.blk_off = blk[k];
-        blk[k + 1] = blk[k] + pixel_blocks(v.W, v.H);
         ws->h_views.p[k] = v;
     }
+    const int nsub = set_strips(ws->h_views.p, n, blk);
     PR_TRY(cudaMemcpyAsync(ws->views.p, ws->h_views.p, sizeof(ViewDev) * n, cudaMemcpyHostToDevice, st));
     PR_TRY(cudaMemcpyAsync(ws->offs.p, blk, sizeof(long long) * (n + 1), cudaMemcpyHostToDevice, st));
-    PR_TRY(launch_backward(ws->views.as<ViewDev>(), n, ws->offs.as<long long>(), blk[n], nullptr,
+    PR_TRY(launch_backward(ws->views.as<ViewDev>(), n, ws->offs.as<long long>(), blk[n], nsub,
                            shade_features(ws->h_views.p, n), st, ws->h_views.p));
     PR_TRY(cudaStreamSynchronize(st));
     return PR_OK;

@@ -15,13 +15,22 @@ constexpr float kEpsDisp = 1e-5f;                  // display-space safety margi
 constexpr float kEpsT = 1e-4f;                     // time margin of every catch-up interval
 constexpr int kMaxHp = 8;                          // half-planes per bound: <= 6 hull edges + 2 time-strip edges
 constexpr int kRecF4 = 6;                          // float4 per fragment record
-// the pixel block of one warp in shading and the adjoint (32 pixels)
+// the pixel block that a warp shades at a time, one pixel per lane; a warp
+// takes a strip of nsub (1 or 4) blocks side by side
 constexpr int kBlkW = 8, kBlkH = 4;
 static_assert(kBlkW * kBlkH == 32, "one pixel per lane");
-__host__ __device__ inline long long pixel_blocks(int W, int H)
+__host__ __device__ inline long long pixel_blocks(int W, int H, int nsub = 1)
 {
-    return (long long)((W + kBlkW - 1) / kBlkW) * ((H + kBlkH - 1) / kBlkH);
+    return (long long)((W + nsub * kBlkW - 1) / (nsub * kBlkW)) * ((H + kBlkH - 1) / kBlkH);
 }
+// Blocks per strip for a launch over this many blocks: strips of four keep
+// four blocks' loads in flight per warp and share the warp's set-up (64
+// views, 2.74 M blocks: 1.33 against 2.04 ms for the training frame's
+// shading; stereo HMD frame, 144,000 blocks: 0.126 against 0.162 ms), but a
+// launch with fewer blocks than about twice the 152 x 40 resident warps
+// times four leaves SMs idle with them.
+constexpr long long kStripMinBlocks = 40000;
+inline int strip_blocks(long long nblocks) { return nblocks >= kStripMinBlocks ? 4 : 1; }
 constexpr int kMaxSeg = 1024;                      // longest bin run of one work item (pr_params.seg)
 constexpr int kLossSlots = 256;                    // partial sums per view of a training frame's loss
 
@@ -51,7 +60,7 @@ struct ViewDev {
     int tiles_x, tiles_y, bound, fp64;
     int fov_bound;                     // pr_fov_bound
     long long tri_off, tile_off, pix_off;  // offsets of this view in the batch-wide arrays
-    long long blk_off;                 // offset of its warp pixel blocks (stages d, e)
+    long long blk_off;                 // offset of its strips of pixel blocks (stages d, e)
     int T, V;
     const float4 *vtx;                 // scene vertices, two float4 each: (px, py, pz, vx), (vy, vz, 0, 0)
     const float4 *col4;                // per-vertex colour (r, g, b, 0)
@@ -68,7 +77,7 @@ struct ViewDev {
     const unsigned *scene_status;      // the scene's status word (ST_NONFINITE after an update), or null
     float *dcol, *dpos, *dvel;         // adjoint outputs [V][3]
     const float4 *rec;                 // this frame's stage (a) records (batch-wide index), or null
-    unsigned long long bw_mul;         // ceil(2^40 / bw), bw = 8-pixel blocks per row: lb / bw = (lb * bw_mul) >> 40
+    unsigned long long bw_mul;         // ceil(2^40 / bw), bw = strips per row: lb / bw = (lb * bw_mul) >> 40 (set_strips)
 };
 
 // The views of a launch passed by value in the kernel's parameter space, for

@@ -73,7 +73,15 @@ constexpr float kRelCoordShade = 6e-8f;
 // interpolation of M_s v_s and M_e v_e at the pixel time, the ray-plane
 // barycentrics b_k = w_k / sum w with w_0 = dir.(B x C) (cyclically) and the
 // face normal turned to face the viewer.
-__device__ __noinline__ void pixel_hit64(const ViewDev &v, int i, int j, struct PixelHit &h);
+// Out of line, with a result struct of its own, so that the PixelHit of the
+// callers stays in registers.
+struct Hit64Out {
+    float b0, b1, b2, det, inv_det;
+    float3 n, A, B, C;
+    float inl;
+    int has_b, has_n;  // barycentrics / normal are defined
+};
+__device__ __noinline__ void pixel_hit64(const ViewDev &v, int i, int j, int ia, int ib, int ic, Hit64Out &o);
 
 template <int kFeat>
 __device__ __forceinline__ void pixel_hit(const ViewDev &v, int i, int j, unsigned id, PixelHit &h)
@@ -127,7 +135,24 @@ __device__ __forceinline__ void pixel_hit(const ViewDev &v, int i, int j, unsign
         const float zm = fmaxf(fabsf(h.A.z), fmaxf(fabsf(h.B.z), fabsf(h.C.z)));
         const float mag = zm * (1.f + fabsf(dx) + fabsf(dy)) + sm;
         if (2.f * kRelCoordShade * mag * sm > kBaryRel * fabsf(h.det))
-            pixel_hit64(v, i, j, h);
+        {
+            Hit64Out o;
+            pixel_hit64(v, i, j, h.ia, h.ib, h.ic, o);
+            if (o.has_b) {
+                h.b0 = o.b0;
+                h.b1 = o.b1;
+                h.b2 = o.b2;
+                h.det = o.det;
+                h.inv_det = o.inv_det;
+            }
+            if (o.has_n) {
+                h.n = o.n;
+                h.inl = o.inl;
+            }
+            h.A = o.A;
+            h.B = o.B;
+            h.C = o.C;
+        }
     }
     float3 l = make_float3(fmaf(t, v.l1[0] - v.l0[0], v.l0[0]), fmaf(t, v.l1[1] - v.l0[1], v.l0[1]),
                            fmaf(t, v.l1[2] - v.l0[2], v.l0[2]));
@@ -146,11 +171,11 @@ __device__ __forceinline__ void pixel_hit(const ViewDev &v, int i, int j, unsign
     }
 }
 
-__device__ __noinline__ void pixel_hit64(const ViewDev &v, int i, int j, PixelHit &h)
+__device__ __noinline__ void pixel_hit64(const ViewDev &v, int i, int j, int ia, int ib, int ic, Hit64Out &h)
 {
     const Ray64 ry = pixel_ray64(v, i, j);
     const double d[3] = {ry.dx, ry.dy, 1.0};
-    const int vid[3] = {h.ia, h.ib, h.ic};
+    const int vid[3] = {ia, ib, ic};
     double P[3][3];
     for (int k = 0; k < 3; ++k) {
         const float4 va = v.vtx[2 * vid[k]], vb = v.vtx[2 * vid[k] + 1];
@@ -169,6 +194,7 @@ __device__ __noinline__ void pixel_hit64(const ViewDev &v, int i, int j, PixelHi
         w[k] = d[0] * (b[1] * c[2] - b[2] * c[1]) + d[1] * (b[2] * c[0] - b[0] * c[2]) + d[2] * (b[0] * c[1] - b[1] * c[0]);
     }
     const double sw = w[0] + w[1] + w[2];
+    h.has_b = sw != 0.0;
     if (sw != 0.0) {
         const double isw = 1.0 / sw;
         h.b0 = (float)(w[0] * isw);
@@ -181,6 +207,7 @@ __device__ __noinline__ void pixel_hit64(const ViewDev &v, int i, int j, PixelHi
     const double e2[3] = {P[2][0] - P[0][0], P[2][1] - P[0][1], P[2][2] - P[0][2]};
     const double n[3] = {e1[1] * e2[2] - e1[2] * e2[1], e1[2] * e2[0] - e1[0] * e2[2], e1[0] * e2[1] - e1[1] * e2[0]};
     const double nn = n[0] * n[0] + n[1] * n[1] + n[2] * n[2];
+    h.has_n = nn > 0.0;
     if (nn > 0.0) {
         const double il = rsqrt(nn);
         const double s = n[0] * d[0] + n[1] * d[1] + n[2] * d[2] > 0.0 ? -il : il;
@@ -192,38 +219,62 @@ __device__ __noinline__ void pixel_hit64(const ViewDev &v, int i, int j, PixelHi
     h.C = make_float3((float)P[2][0], (float)P[2][1], (float)P[2][2]);
 }
 
-// Stages (d) and (e) run each warp over kShadeBlocks consecutive pixel
-// blocks of kBlkW x kBlkH (8 x 4; lane -> column lane % kBlkW, row
-// lane / kBlkW of each), so the lanes of a
-// warp mostly see the same triangles: gathers of vertex data coalesce, and
-// the adjoint sums a triangle's contributions over a lane's pixels and then
-// over the warp before touching memory.  blk_offs[q] = first pixel block of
-// view q in the batch.  One block per warp measured fastest on the stereo
-// HMD frame (0.170 ms against 0.229 ms for two and 0.242 ms for four): the
-// running sums held across pixels push the kernel into register spills
-// that cost more than the warp reductions they save.
-constexpr int kShadeBlocks = 1;
+// Stages (d) and (e) run each warp over one strip of nsub pixel blocks of
+// kBlkW x kBlkH (8 x 4) side by side: 32 x 4 pixels for nsub = 4, one block
+// for nsub = 1 (strip_blocks: frames too small to fill the chip with
+// strips).  First the whole strip is resolved row by row (every load of the
+// strip in flight at once, rows coalesced): ids, depths, the background's
+// colour and loss, the keys' reset.  Then its blocks that show a triangle
+// are shaded one after the other, one pixel per lane (lane -> column
+// lane % kBlkW, row lane / kBlkW), so that the lanes mostly share a
+// triangle.  blk_offs[q] = first strip of view q in the batch.
+// CTAs of the shading kernels: 64 threads (two warps), 20 resident per SM
+// (48 registers; the precision form and the stand-alone adjoint 18, 56
+// registers).  A CTA's slot frees only when its slowest warp finishes, and
+// the warps of a CTA see different strips (background, one triangle,
+// several), so small CTAs keep the SM fuller.  Training frame's shading,
+// 64 views / HMD frame / 1M-triangle precision form: 1.29 / 0.126 / 0.493 ms
+// with 20, 1.34 / 0.128 / 0.475 with 18, 1.37 / 0.127 / 0.464 with 16; the
+// stand-alone adjoint of four views 0.0466 ms with 20, 0.0459 with 18.
+constexpr int kShadeThreads = 64;
+constexpr int kShadeWarps = kShadeThreads / 32;
+constexpr int shade_ctas(int feat) { return feat & kFeatF64 ? 18 : 20; }
+constexpr int kBackwardCtas = 18;
 
-// CTAs of the shading kernels: 64 threads (two warps), 18 resident per SM,
-// which caps them at 56 registers (36 warps per SM).  A CTA's slot frees
-// only when its slowest warp finishes, and the warps of a CTA see different
-// pixel blocks (background, one triangle, several), so small CTAs keep the
-// SM fuller: 64 x 18 measured fastest against 256 x 4, 128 x 8, 128 x 9,
-// 128 x 10, 64 x 16 and 32 x 32.
-constexpr int kShadeThreads = 64, kShadeCtasPerSm = 18;
+// The strip's visible ids in shared memory, rows apart by an odd multiple of
+// eight words (a block's four rows of eight columns meet all banks).
+constexpr int kIdPitch = 40;
 
-__device__ __forceinline__ bool block_pixel(const ViewDev *views, int nviews, const long long *blk_offs, long long b,
-                                            int lane, int &q, long long &lin, int &i, int &j)
+// Position of a warp's strip.
+struct Strip {
+    int q;       // view
+    int i0, j0;  // first pixel
+    int sh;      // log2 of the strip's width
+};
+
+__device__ __forceinline__ Strip strip_of(const ViewDev *views, int nviews, const long long *blk_offs, long long b,
+                                          int nsub)
 {
-    q = find_view_warp(blk_offs, nviews, b);  // b is the warp's
-    const ViewDev &v = views[q];
-    const int lb = (int)(b - v.blk_off);  // < 2^23 blocks per view
-    const int bw = (v.W + kBlkW - 1) / kBlkW;
+    Strip s;
+    s.q = find_view_warp(blk_offs, nviews, b);  // b is the warp's
+    const ViewDev &v = views[s.q];
+    s.sh = nsub == 1 ? 3 : 5;
+    const int lb = (int)(b - v.blk_off);  // < 2^23 strips per view
+    const int bw = (v.W + (1 << s.sh) - 1) >> s.sh;
     const int by = (int)(((unsigned long long)(unsigned)lb * v.bw_mul) >> 40);  // lb / bw
-    i = (lb - by * bw) * kBlkW + lane % kBlkW;
-    j = by * kBlkH + lane / kBlkW;
-    lin = (long long)j * v.W + i;
-    return i < v.W && j < v.H;
+    s.i0 = (lb - by * bw) << s.sh;
+    s.j0 = by * kBlkH;
+    return s;
+}
+
+// Which of the strip's blocks the set lanes of a row's ballot belong to, as
+// bits 0..3.
+__device__ __forceinline__ unsigned blocks_of(unsigned lanes, int nsub)
+{
+    if (nsub == 1)
+        return lanes ? 1u : 0u;
+    return (lanes & 0xFFu ? 1u : 0u) | (lanes & 0xFF00u ? 2u : 0u) | (lanes & 0xFF0000u ? 4u : 0u) |
+           (lanes & 0xFF000000u ? 8u : 0u);
 }
 
 // Vertex colours of the visible triangle and the interpolated albedo
@@ -248,41 +299,66 @@ __device__ __forceinline__ void pixel_albedo(const ViewDev &v, const PixelHit &h
         pa.a[c] = fmaf(h.b0, pa.col[0][c], fmaf(h.b1, pa.col[1][c], h.b2 * pa.col[2][c]));
 }
 
-// Sums value l of every lane of `mask` over the warp and adds it to
-// gradient l of the warp's triangle with vertices (v0, v1, v2): value 9k + c
-// is d/dcol_k[c], 9k + 3 + c the sum of (1 - t) dL/dc_k[c] and 9k + 6 + c
-// the sum of t dL/dc_k[c], with c_k the moved camera-space vertex k.  The
-// position and velocity gradients follow once per triangle from the last
-// two: dc/dp = (1-t) R0 + t R1 and dc/dv = t R1, so dL/dp = R0^T sum (1-t)
-// dL/dc + R1^T sum t dL/dc and dL/dv = R1^T sum t dL/dc.  Lanes outside the
-// group pass zeros.  Reduce-scatter: at each of five steps a lane keeps the
-// half of its values selected by its lane bit and adds its partner's copy
-// of that half, so lane l ends with the warp sum of value l (31 shuffles
-// instead of 27 full butterflies).
-__device__ __forceinline__ void reduce_add_triangle(const ViewDev &v, float (&s)[32], int v0, int v1, int v2)
+// The adjoint's sums over pixels.  A triangle has 27 gradient values: value
+// 9k + c is d/dcol_k[c], 9k + 3 + c the sum of (1 - t) dL/dc_k[c] and
+// 9k + 6 + c the sum of t dL/dc_k[c], with c_k the moved camera-space vertex
+// k; the position and velocity gradients follow once per triangle from the
+// last two: dc/dp = (1-t) R0 + t R1 and dc/dv = t R1, so dL/dp = R0^T sum
+// (1-t) dL/dc + R1^T sum t dL/dc and dL/dv = R1^T sum t dL/dc.  Every value
+// is a sum over pixels of a product x y of two of 17 per-pixel numbers:
+// x = (g sigma)_c with y = b_k, or x = dL/dc_k[c] with y = 1 - t or t.
+//
+// So a block's pixels write those 17 numbers to the warp's rows in shared
+// memory (as soon as each is known, which frees its register), and lane l
+// then sums value l over the pixels with 16-byte loads of its two rows: 17
+// stores, 16 loads and 32 multiply-adds per block, against 31 shuffles, 62
+// selects and 31 adds for a shuffle reduce-scatter of the 27 products,
+// which also had to live in registers at once (and spilled).  A value's sum
+// is one register of one lane, kept while the warp's pixels stay on one
+// triangle and written out when the triangle changes.
+//
+// Row numbers: the rows that eight neighbouring lanes read differ modulo 8
+// (but for one pair), so the 16-byte loads meet different banks.
+constexpr int kRowPitch = 36, kRows = 17;
+__device__ __forceinline__ constexpr int row_gs(int c) { return c; }
+__device__ __forceinline__ constexpr int row_b(int k) { return 8 + k; }
+__device__ __forceinline__ constexpr int row_g(int k, int c)
+{
+    return k == 0 ? 3 + c : (k == 1 ? (c == 0 ? 11 : 5 + c) : (c == 0 ? 16 : 11 + c));
+}
+constexpr int kRowOmt = 14, kRowT = 15;
+
+// What a lane sums: its two rows, and where the value goes.
+struct ValueLane {
+    int x, y;
+};
+
+__device__ __forceinline__ ValueLane value_lane()
 {
     const int lane = threadIdx.x & 31;
-#pragma unroll
-    for (int step = 0; step < 5; ++step) {
-        const int half = 16 >> step;
-        const bool upper = (lane & half) != 0;
-#pragma unroll
-        for (int k = 0; k < half; ++k) {
-            const float send = upper ? s[k] : s[k + half];
-            const float keep = upper ? s[k + half] : s[k];
-            s[k] = keep + __shfl_xor_sync(0xffffffffu, send, half);
-        }
-    }
+    const int k = min(lane / 9, 2), r = min(lane - 9 * k, 8);
+    ValueLane vl;
+    const int c = r < 3 ? r : (r < 6 ? r - 3 : r - 6);
+    vl.x = (r < 3 ? row_gs(c) : row_g(k, c)) * kRowPitch;
+    vl.y = (r < 3 ? row_b(k) : (r < 6 ? kRowOmt : kRowT)) * kRowPitch;
+    return vl;
+}
+
+// Adds a triangle's 27 sums (lane l: value l) to the gradients.
+__device__ __forceinline__ void add_triangle(const ViewDev &v, unsigned id, float sum)
+{
+    const int lane = threadIdx.x & 31;
     const int k = min(lane / 9, 2), r = lane - 9 * k;
     const int base = 9 * k;
-    const float o0 = __shfl_sync(0xffffffffu, s[0], base + 3), o1 = __shfl_sync(0xffffffffu, s[0], base + 4),
-                o2 = __shfl_sync(0xffffffffu, s[0], base + 5);
-    const float t0 = __shfl_sync(0xffffffffu, s[0], base + 6), t1 = __shfl_sync(0xffffffffu, s[0], base + 7),
-                t2 = __shfl_sync(0xffffffffu, s[0], base + 8);
+    const float o0 = __shfl_sync(0xffffffffu, sum, base + 3), o1 = __shfl_sync(0xffffffffu, sum, base + 4),
+                o2 = __shfl_sync(0xffffffffu, sum, base + 5);
+    const float t0 = __shfl_sync(0xffffffffu, sum, base + 6), t1 = __shfl_sync(0xffffffffu, sum, base + 7),
+                t2 = __shfl_sync(0xffffffffu, sum, base + 8);
     if (lane < 27) {
+        const int4 tv = v.tri4[id];
         const int c = r < 3 ? r : (r < 6 ? r - 3 : r - 6);
-        const int vk = k == 0 ? v0 : (k == 1 ? v1 : v2);
-        float val = s[0];
+        const int vk = k == 0 ? tv.x : (k == 1 ? tv.y : tv.z);
+        float val = sum;
         if (r >= 3) {
             val = fmaf(v.R1[c], t0, fmaf(v.R1[3 + c], t1, v.R1[6 + c] * t2));
             if (r < 6)
@@ -304,141 +380,113 @@ __device__ __forceinline__ void reduce_add_triangle(const ViewDev &v, float (&s)
 //    cross products with dir;
 //  - the unit normal n = flip (B-A)x(C-A) / |.|: dn gets (I - n n^T)/|.|;
 //  - moved vertex c(t) = (1-t) S + t E with S = R0 p + T0, E = R1 (p + v) + T1
-//    (applied per triangle after the warp sum, reduce_add_triangle).
-// The pixel's 27 values (layout of reduce_add_triangle) are ADDED to acc.
+//    (applied per triangle after the sum, add_triangle).
+// Writes the pixel's 17 numbers to column `lane` of the warp's rows.
 template <int kFeat>
-__device__ __forceinline__ void adjoint_add(const ViewDev &v, const PixelHit &h, const PixelAlbedo &pa, float g0,
-                                            float g1, float g2, float (&acc)[27])
+__device__ __forceinline__ void adjoint_rows(const ViewDev &v, const PixelHit &h, const PixelAlbedo &pa, float g0,
+                                             float g1, float g2, float *col)
 {
-    {
-        const float b[3] = {h.b0, h.b1, h.b2};
-        const float gs[3] = {g0 * h.sigma, g1 * h.sigma, g2 * h.sigma};
-        float gb[3];
+    const float b[3] = {h.b0, h.b1, h.b2};
+    const float gs[3] = {g0 * h.sigma, g1 * h.sigma, g2 * h.sigma};
+    float gb[3];
 #pragma unroll
-        for (int k = 0; k < 3; ++k) {
-#pragma unroll
-            for (int c = 0; c < 3; ++c)
-                acc[9 * k + c] = fmaf(gs[c], b[k], acc[9 * k + c]);
-            gb[k] = fmaf(gs[0], pa.col[k][0], fmaf(gs[1], pa.col[k][1], gs[2] * pa.col[k][2]));
-        }
-        const float gsig = fmaf(g0, pa.a[0], fmaf(g1, pa.a[1], g2 * pa.a[2]));
-        // barycentrics -> moved vertices: with w_0 = D.(B x C) etc.,
-        // dL/dA = gw1 (D x C) + gw2 (B x D) = D x (gw1 C - gw2 B), cyclically
-        const float gdotb = fmaf(gb[0], b[0], fmaf(gb[1], b[1], gb[2] * b[2]));
-        const float isw = -h.inv_det;  // 1 / sum w, sum w = -det (exactly the negated reciprocal)
-        const float gw0 = (gb[0] - gdotb) * isw, gw1 = (gb[1] - gdotb) * isw, gw2 = (gb[2] - gdotb) * isw;
-        const float3 D = h.dir;
-        float3 gA = cross3(D, sub3(scale3(h.C, gw1), scale3(h.B, gw2)));
-        float3 gB = cross3(D, sub3(scale3(h.A, gw2), scale3(h.C, gw0)));
-        float3 gC = cross3(D, sub3(scale3(h.B, gw0), scale3(h.A, gw1)));
-        // normal -> moved vertices: the diffuse term through n.l, the
-        // specular term k_s (n.h)^m (white) through n.h; the three
-        // contributions (B-C) x gn, (C-A) x gn, (A-B) x gn sum to zero
-        const bool dif = h.ndl > 0.f, spc = (kFeat & kFeatSpec) && h.spec > 0.f;
-        if ((dif || spc) && h.inl != 0.f) {
-            float3 gnh = scale3(h.l, dif ? gsig * v.k_d : 0.f);
-            if (spc)
-                gnh = add3(gnh, scale3(h.hv, (g0 + g1 + g2) * v.shininess * h.spec / h.ndh));
-            const float pr = dot3(h.n, gnh);
-            const float3 gnn = scale3(sub3(gnh, scale3(h.n, pr)), h.inl);
-            const float3 na = cross3(sub3(h.B, h.C), gnn), nb = cross3(sub3(h.C, h.A), gnn);
-            gA = add3(gA, na);
-            gB = add3(gB, nb);
-            gC = sub3(gC, add3(na, nb));
-        }
-        // the moved vertices' gradients, split by the weights (1 - t) of S
-        // and t of E
-        const float3 gk[3] = {gA, gB, gC};
-        const float t = h.t, omt = 1.f - t;
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            acc[9 * k + 3] = fmaf(omt, gk[k].x, acc[9 * k + 3]);
-            acc[9 * k + 4] = fmaf(omt, gk[k].y, acc[9 * k + 4]);
-            acc[9 * k + 5] = fmaf(omt, gk[k].z, acc[9 * k + 5]);
-            acc[9 * k + 6] = fmaf(t, gk[k].x, acc[9 * k + 6]);
-            acc[9 * k + 7] = fmaf(t, gk[k].y, acc[9 * k + 7]);
-            acc[9 * k + 8] = fmaf(t, gk[k].z, acc[9 * k + 8]);
-        }
+    for (int k = 0; k < 3; ++k) {
+        col[row_gs(k) * kRowPitch] = gs[k];
+        col[row_b(k) * kRowPitch] = b[k];
+        gb[k] = fmaf(gs[0], pa.col[k][0], fmaf(gs[1], pa.col[k][1], gs[2] * pa.col[k][2]));
     }
+    const float gsig = fmaf(g0, pa.a[0], fmaf(g1, pa.a[1], g2 * pa.a[2]));
+    // barycentrics -> moved vertices: with w_0 = D.(B x C) etc.,
+    // dL/dA = gw1 (D x C) + gw2 (B x D) = D x (gw1 C - gw2 B), cyclically
+    const float gdotb = fmaf(gb[0], b[0], fmaf(gb[1], b[1], gb[2] * b[2]));
+    const float isw = -h.inv_det;  // 1 / sum w, sum w = -det (exactly the negated reciprocal)
+    const float gw0 = (gb[0] - gdotb) * isw, gw1 = (gb[1] - gdotb) * isw, gw2 = (gb[2] - gdotb) * isw;
+    const float3 D = h.dir;
+    float3 gA = cross3(D, sub3(scale3(h.C, gw1), scale3(h.B, gw2)));
+    float3 gB = cross3(D, sub3(scale3(h.A, gw2), scale3(h.C, gw0)));
+    float3 gC = cross3(D, sub3(scale3(h.B, gw0), scale3(h.A, gw1)));
+    // normal -> moved vertices: the diffuse term through n.l, the
+    // specular term k_s (n.h)^m (white) through n.h; the three
+    // contributions (B-C) x gn, (C-A) x gn, (A-B) x gn sum to zero
+    const bool dif = h.ndl > 0.f, spc = (kFeat & kFeatSpec) && h.spec > 0.f;
+    if ((dif || spc) && h.inl != 0.f) {
+        float3 gnh = scale3(h.l, dif ? gsig * v.k_d : 0.f);
+        if (spc)
+            gnh = add3(gnh, scale3(h.hv, (g0 + g1 + g2) * v.shininess * h.spec / h.ndh));
+        const float pr = dot3(h.n, gnh);
+        const float3 gnn = scale3(sub3(gnh, scale3(h.n, pr)), h.inl);
+        const float3 na = cross3(sub3(h.B, h.C), gnn), nb = cross3(sub3(h.C, h.A), gnn);
+        gA = add3(gA, na);
+        gB = add3(gB, nb);
+        gC = sub3(gC, add3(na, nb));
+    }
+    const float3 gk[3] = {gA, gB, gC};
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        col[row_g(k, 0) * kRowPitch] = gk[k].x;
+        col[row_g(k, 1) * kRowPitch] = gk[k].y;
+        col[row_g(k, 2) * kRowPitch] = gk[k].z;
+    }
+    col[kRowOmt * kRowPitch] = 1.f - h.t;
+    col[kRowT * kRowPitch] = h.t;
 }
 
-// A lane's running sums of the adjoint values of the pixels it has seen
-// since the last flush, all of one triangle of one view.
-struct AdjointSum {
-    float s[27];
-    int q;  // view of the triangle (-1: nothing summed)
-    unsigned id;
-    int ia, ib, ic;
+// A warp's running sums of one triangle of its view.
+struct TriangleSum {
+    float s;      // lane l: value l
+    unsigned id;  // the triangle (0xFFFFFFFF: none)
 };
 
-__device__ __forceinline__ void adjoint_reset(AdjointSum &a)
+// Adds the block's pixels (valid lanes, triangle id; their numbers in the
+// warp's rows, columns of the other lanes zero) to the running sum,
+// triangle by triangle.  Called by the whole warp.
+__device__ __forceinline__ void sum_block(const ViewDev &v, const float *rows, const ValueLane &vl, bool valid,
+                                          unsigned id, TriangleSum &ts)
 {
+    const unsigned all = __ballot_sync(0xffffffffu, valid);
+    unsigned rem = all;
+    const float4 *x4 = reinterpret_cast<const float4 *>(rows + vl.x);
+    const float4 *y4 = reinterpret_cast<const float4 *>(rows + vl.y);
+    unsigned m = __ballot_sync(0xffffffffu, valid && id == ts.id);  // the running triangle first
+    while (rem) {
+        if (!m) {
+            const unsigned tid = __shfl_sync(0xffffffffu, id, __ffs(rem) - 1);
+            if (ts.id != 0xFFFFFFFFu)
+                add_triangle(v, ts.id, ts.s);
+            ts.id = tid;
+            ts.s = 0.f;
+            m = __ballot_sync(0xffffffffu, valid && id == tid);
+        }
+        float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
+        if (m == all) {  // one triangle (the common case): the other lanes' columns are zero
 #pragma unroll
-    for (int e = 0; e < 27; ++e)
-        a.s[e] = 0.f;
-    a.q = -1;
-}
-
-// Sums the lanes' running sums over the warp per distinct (view, triangle),
-// adds them to the gradients and resets them.  Called by every lane.
-__device__ __forceinline__ void adjoint_flush(const ViewDev *views, AdjointSum &a)
-{
-    unsigned rem = __ballot_sync(0xffffffffu, a.q >= 0);
-    if (rem) {
-        int leader = __ffs(rem) - 1;
-        int tq = __shfl_sync(0xffffffffu, a.q, leader);
-        unsigned tid = __shfl_sync(0xffffffffu, a.id, leader);
-        float s[32];
-        if (__all_sync(0xffffffffu, a.q < 0 || (a.q == tq && a.id == tid))) {
-            // one triangle over the warp (the common case): lanes without
-            // a sum hold zeros already
-#pragma unroll
-            for (int e = 0; e < 27; ++e)
-                s[e] = a.s[e];
-#pragma unroll
-            for (int e = 27; e < 32; ++e)
-                s[e] = 0.f;
-            reduce_add_triangle(views[tq], s, __shfl_sync(0xffffffffu, a.ia, leader),
-                                __shfl_sync(0xffffffffu, a.ib, leader), __shfl_sync(0xffffffffu, a.ic, leader));
+            for (int q = 0; q < 8; ++q) {
+                const float4 x = x4[q], y = y4[q];
+                s0 = fmaf(x.x, y.x, s0);
+                s1 = fmaf(x.y, y.y, s1);
+                s2 = fmaf(x.z, y.z, s2);
+                s3 = fmaf(x.w, y.w, s3);
+            }
         } else {
-            while (true) {
-                const bool mine = a.q == tq && a.id == tid;
-                rem &= ~__ballot_sync(0xffffffffu, mine);
-#pragma unroll
-                for (int e = 0; e < 27; ++e)
-                    s[e] = mine ? a.s[e] : 0.f;
-#pragma unroll
-                for (int e = 27; e < 32; ++e)
-                    s[e] = 0.f;
-                reduce_add_triangle(views[tq], s, __shfl_sync(0xffffffffu, a.ia, leader),
-                                    __shfl_sync(0xffffffffu, a.ib, leader), __shfl_sync(0xffffffffu, a.ic, leader));
-                if (!rem)
-                    break;
-                leader = __ffs(rem) - 1;
-                tq = __shfl_sync(0xffffffffu, a.q, leader);
-                tid = __shfl_sync(0xffffffffu, a.id, leader);
+#pragma unroll 2
+            for (int q = 0; q < 8; ++q) {
+                const unsigned nib = (m >> (4 * q)) & 15u;
+                if (!nib)
+                    continue;  // warp-uniform
+                const float4 x = x4[q], y = y4[q];
+                if (nib & 1u)
+                    s0 = fmaf(x.x, y.x, s0);
+                if (nib & 2u)
+                    s1 = fmaf(x.y, y.y, s1);
+                if (nib & 4u)
+                    s2 = fmaf(x.z, y.z, s2);
+                if (nib & 8u)
+                    s3 = fmaf(x.w, y.w, s3);
             }
         }
-    }
-    adjoint_reset(a);
-}
-
-// Adds a valid lane's pixel (triangle id of view q) to its running sum;
-// first, if any lane's sum is of another triangle or view, the warp
-// flushes.  Called by every lane.
-template <int kFeat>
-__device__ __forceinline__ void adjoint_step(const ViewDev *views, AdjointSum &a, bool valid, int q, unsigned id,
-                                             const PixelHit &h, const PixelAlbedo &pa, float g0, float g1, float g2)
-{
-    if (__any_sync(0xffffffffu, valid && a.q >= 0 && (a.q != q || a.id != id)))
-        adjoint_flush(views, a);
-    if (valid) {
-        adjoint_add<kFeat>(views[q], h, pa, g0, g1, g2, a.s);
-        a.q = q;
-        a.id = id;
-        a.ia = h.ia;
-        a.ib = h.ib;
-        a.ic = h.ic;
+        ts.s += (s0 + s1) + (s2 + s3);
+        rem &= ~m;
+        m = 0u;
     }
 }
 
@@ -452,122 +500,188 @@ __device__ __forceinline__ bool frame_overflowed(const Counters *frame_cnt)
 // pass.  kAdjoint (a training frame): for views with a gradient input, the
 // stage (e) adjoint of the pixel follows from the same PixelHit -- with an
 // L2 target, from the colour just computed -- so the frame needs no
-// separate adjoint pass.  Whole warps run (the adjoint's reductions).
+// separate adjoint pass.  Whole warps run (the adjoint's sums).
 // views: the device table, or the kernel's parameter table (k_shade_pv).
+//
+// Bound: instruction issue (73 % of peak on 64 views, DRAM 27 %, about 850
+// warp instructions per block that shows a triangle) and, on the background,
+// DRAM writes.
 template <bool kAdjoint, int kFeat>
 __device__ __forceinline__ void shade_body(const ViewDev *__restrict__ views, int nviews,
-                                           const long long *__restrict__ blk_offs, long long nblocks,
+                                           const long long *__restrict__ blk_offs, long long nblocks, int nsub,
                                            unsigned long long *__restrict__ keys, int reset_keys,
                                            const Counters *__restrict__ frame_cnt)
 {
-    const long long b0 = (((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * kShadeBlocks;
+    __shared__ unsigned s_id[kShadeWarps][kBlkH * kIdPitch];
+    __shared__ __align__(16) float s_rows[kAdjoint ? kShadeWarps : 1][kAdjoint ? kRows * kRowPitch : 4];
+    const long long b0 = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (b0 >= nblocks)
         return;  // whole warps
-    const int lane = threadIdx.x & 31;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     // a training frame whose forward overflowed is rerun by the host: its
     // adjoint must not accumulate
     const bool adjoint = kAdjoint && !frame_overflowed(frame_cnt);
-    AdjointSum acc;
-    adjoint_reset(acc);
-    for (int p = 0; p < kShadeBlocks && b0 + p < nblocks; ++p) {
-        int q, pi, pj;
-        long long lin;
-        const bool inside = block_pixel(views, nviews, blk_offs, b0 + p, lane, q, lin, pi, pj);
-        const ViewDev &v = views[q];
-        const long long plane = (long long)v.W * v.H;
-        const bool grad = adjoint && (v.grad_in || v.target || v.target_u8);
-        // the upstream gradient (or L2 target) does not depend on the hit:
-        // its loads go out first, before the key and the stores below
-        float gin[3] = {0.f, 0.f, 0.f};
-        if (grad && inside) {
-            if (v.target_u8) {
-                gin[0] = u8_unit(v.target_u8[lin]);
-                gin[1] = u8_unit(v.target_u8[plane + lin]);
-                gin[2] = u8_unit(v.target_u8[2 * plane + lin]);
-            } else {
-                const float *gsrc = v.grad_in ? v.grad_in : v.target;
-                gin[0] = gsrc[lin];
-                gin[1] = gsrc[plane + lin];
-                gin[2] = gsrc[2 * plane + lin];
-            }
-        }
-        unsigned id = 0xFFFFFFFFu;
-        if (inside) {
-            if (keys) {
-                const unsigned long long key = keys[v.pix_off + lin];
-                const bool bg = key == ~0ull;
-                if (!bg && reset_keys)
-                    keys[v.pix_off + lin] = ~0ull;  // left as the next frame wants it
-                id = bg ? 0xFFFFFFFFu : (unsigned)(key & 0xFFFFFFFFull);
-                if (v.id_out)
-                    v.id_out[lin] = id;
-                if (v.depth_out)
-                    v.depth_out[lin] = bg ? INFINITY : __uint_as_float((unsigned)(key >> 32));
-            } else {
-                id = v.id_in[lin];
-            }
-        }
-        // a view with neither an image nor a gradient only needs the resolve
-        const bool hit = inside && id < (unsigned)v.T && (v.rgb_out || grad);
-        PixelHit h;
-        PixelAlbedo pa;
-        float rgb[3] = {0.f, 0.f, 0.f};
-        if (hit) {
-            pixel_hit<kFeat>(v, pi, pj, id, h);
-            pixel_albedo(v, h, pa);
-            rgb[0] = fmaf(pa.a[0], h.sigma, h.spec);
-            rgb[1] = fmaf(pa.a[1], h.sigma, h.spec);
-            rgb[2] = fmaf(pa.a[2], h.sigma, h.spec);
-        }
-        if (inside && v.rgb_out) {
-            v.rgb_out[lin] = rgb[0];
-            v.rgb_out[plane + lin] = rgb[1];
-            v.rgb_out[2 * plane + lin] = rgb[2];
-        }
-        if (kAdjoint) {
-            const bool valid = hit && grad;
-            float g0 = gin[0], g1 = gin[1], g2 = gin[2];
-            float lsum = 0.f;  // this pixel's share of the L2 loss (background: rgb = 0)
-            if (grad && inside && !v.grad_in) {
-                // L2 loss sum (rgb - target)^2: its gradient from this frame's image
-                const float e0 = rgb[0] - gin[0], e1 = rgb[1] - gin[1], e2 = rgb[2] - gin[2];
-                lsum = fmaf(e0, e0, fmaf(e1, e1, e2 * e2));
-                g0 = 2.f * e0;
-                g1 = 2.f * e1;
-                g2 = 2.f * e2;
-            }
-            adjoint_step<kFeat>(views, acc, valid, q, id, h, pa, g0, g1, g2);
-            if (adjoint && v.loss) {
-                // one view per warp: a warp sum, then one atomic into one of
-                // the view's partial sums (one address for every warp of a
-                // view would serialise them)
+    const Strip sp = strip_of(views, nviews, blk_offs, b0, nsub);
+    const ViewDev &v = views[sp.q];
+    const int W = v.W, H = v.H;
+    const int plane = W * H;  // <= 2^28
+    const bool grad = adjoint && (v.grad_in || v.target || v.target_u8);
+    // a view with neither an image nor a gradient only needs the resolve
+    const bool shaded = v.rgb_out || grad;
+    float lsum = 0.f;  // the lane's share of the L2 loss (background: rgb = 0)
+    unsigned live = 0u;  // blocks of the strip that show a triangle
+
+    // the strip row by row: keys first, all in flight at once
+    {
+        const int col = sp.i0 + (lane & ((1 << sp.sh) - 1)), row0 = sp.j0 + (lane >> sp.sh), rstep = 32 >> sp.sh;
+        unsigned long long key[kBlkH];
 #pragma unroll
-                for (int o = 16; o > 0; o >>= 1)
-                    lsum += __shfl_xor_sync(0xffffffffu, lsum, o);
-                if (lane == 0)
-                    atomicAdd(&v.loss_part[(unsigned)b0 & (kLossSlots - 1)], lsum);
+        for (int k = 0; k < kBlkH; ++k) {
+            key[k] = ~0ull;
+            const int j = row0 + k * rstep;
+            if (k < nsub && col < W && j < H) {
+                if (keys)
+                    key[k] = keys[v.pix_off + j * W + col];
+                else
+                    key[k] = v.id_in[j * W + col] | 0xFFFFFFFF00000000ull;
             }
+        }
+#pragma unroll
+        for (int k = 0; k < kBlkH; ++k) {
+            if (k >= nsub)
+                break;
+            const int j = row0 + k * rstep, lin = j * W + col;
+            const bool inside = col < W && j < H;
+            const unsigned id = (unsigned)key[k];
+            const bool hit = inside && id < (unsigned)v.T && shaded;
+            if (inside) {
+                if (keys) {
+                    const bool bg = key[k] == ~0ull;
+                    if (!bg && reset_keys)
+                        keys[v.pix_off + lin] = ~0ull;  // left as the next frame wants it
+                    if (v.id_out)
+                        v.id_out[lin] = id;
+                    if (v.depth_out)
+                        v.depth_out[lin] = bg ? INFINITY : __uint_as_float((unsigned)(key[k] >> 32));
+                }
+                if (!hit) {
+                    if (v.rgb_out) {
+                        v.rgb_out[lin] = 0.f;
+                        v.rgb_out[plane + lin] = 0.f;
+                        v.rgb_out[2 * plane + lin] = 0.f;
+                    }
+                    if (kAdjoint && grad && v.loss) {
+                        float e0, e1, e2;
+                        if (v.target_u8) {
+                            e0 = u8_unit(v.target_u8[lin]);
+                            e1 = u8_unit(v.target_u8[plane + lin]);
+                            e2 = u8_unit(v.target_u8[2 * plane + lin]);
+                        } else {
+                            e0 = v.target[lin];
+                            e1 = v.target[plane + lin];
+                            e2 = v.target[2 * plane + lin];
+                        }
+                        lsum += fmaf(e0, e0, fmaf(e1, e1, e2 * e2));
+                    }
+                }
+            }
+            s_id[warp][(k * rstep + (lane >> sp.sh)) * kIdPitch + (lane & ((1 << sp.sh) - 1))] =
+                hit ? id : 0xFFFFFFFFu;
+            live |= blocks_of(__ballot_sync(0xffffffffu, hit), nsub);
         }
     }
-    if (kAdjoint)
-        adjoint_flush(views, acc);
+    __syncwarp();
+
+    // the blocks that show a triangle, one pixel per lane
+    TriangleSum ts;
+    ts.s = 0.f;
+    ts.id = 0xFFFFFFFFu;
+    const ValueLane vl = value_lane();
+    float *rows = s_rows[kAdjoint ? warp : 0];
+    for (; live; live &= live - 1u) {
+        const int x = (__ffs(live) - 1) * kBlkW + lane % kBlkW, y = lane / kBlkW;
+        const unsigned id = s_id[warp][y * kIdPitch + x];
+        const int pi = sp.i0 + x, pj = sp.j0 + y, lin = pj * W + pi;
+        const bool hit = id != 0xFFFFFFFFu;
+        if (kAdjoint && grad && !hit) {
+#pragma unroll
+            for (int r = 0; r < kRows; ++r)
+                rows[r * kRowPitch + lane] = 0.f;
+        }
+        if (hit) {
+            // the upstream gradient (or L2 target) does not depend on the
+            // hit: its loads go out first
+            float gin[3] = {0.f, 0.f, 0.f};
+            if (kAdjoint && grad) {
+                if (v.target_u8) {
+                    gin[0] = u8_unit(v.target_u8[lin]);
+                    gin[1] = u8_unit(v.target_u8[plane + lin]);
+                    gin[2] = u8_unit(v.target_u8[2 * plane + lin]);
+                } else {
+                    const float *gsrc = v.grad_in ? v.grad_in : v.target;
+                    gin[0] = gsrc[lin];
+                    gin[1] = gsrc[plane + lin];
+                    gin[2] = gsrc[2 * plane + lin];
+                }
+            }
+            PixelHit h;
+            PixelAlbedo pa;
+            pixel_hit<kFeat>(v, pi, pj, id, h);
+            pixel_albedo(v, h, pa);
+            const float rgb[3] = {fmaf(pa.a[0], h.sigma, h.spec), fmaf(pa.a[1], h.sigma, h.spec),
+                                  fmaf(pa.a[2], h.sigma, h.spec)};
+            if (v.rgb_out) {
+                v.rgb_out[lin] = rgb[0];
+                v.rgb_out[plane + lin] = rgb[1];
+                v.rgb_out[2 * plane + lin] = rgb[2];
+            }
+            if (kAdjoint && grad) {
+                if (!v.grad_in) {
+                    // L2 loss sum (rgb - target)^2: its gradient from this frame's image
+                    const float e0 = rgb[0] - gin[0], e1 = rgb[1] - gin[1], e2 = rgb[2] - gin[2];
+                    lsum += fmaf(e0, e0, fmaf(e1, e1, e2 * e2));
+                    gin[0] = 2.f * e0;
+                    gin[1] = 2.f * e1;
+                    gin[2] = 2.f * e2;
+                }
+                adjoint_rows<kFeat>(v, h, pa, gin[0], gin[1], gin[2], rows + lane);
+            }
+        }
+        if (kAdjoint && grad) {
+            __syncwarp();
+            sum_block(v, rows, vl, hit, id, ts);
+            __syncwarp();  // the rows are written again by the next block
+        }
+    }
+    if (kAdjoint && ts.id != 0xFFFFFFFFu)
+        add_triangle(v, ts.id, ts.s);
+    if (kAdjoint && adjoint && v.loss) {
+        // one view per warp: a warp sum, then one atomic into one of the
+        // view's partial sums (one address for every warp of a view would
+        // serialise them)
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+            lsum += __shfl_xor_sync(0xffffffffu, lsum, o);
+        if (lane == 0)
+            atomicAdd(&v.loss_part[(unsigned)b0 & (kLossSlots - 1)], lsum);
+    }
 }
 
 template <bool kAdjoint, int kFeat>
-__global__ void __launch_bounds__(kShadeThreads, kShadeCtasPerSm)
-    k_shade(const ViewDev *__restrict__ views, int nviews, const long long *__restrict__ blk_offs, long long nblocks,
+__global__ void __launch_bounds__(kShadeThreads, shade_ctas(kFeat))
+    k_shade(const ViewDev *__restrict__ views, int nviews, const long long *__restrict__ blk_offs, long long nblocks, int nsub,
             unsigned long long *__restrict__ keys, int reset_keys, const Counters *__restrict__ frame_cnt)
 {
-    shade_body<kAdjoint, kFeat>(views, nviews, blk_offs, nblocks, keys, reset_keys, frame_cnt);
+    shade_body<kAdjoint, kFeat>(views, nviews, blk_offs, nblocks, nsub, keys, reset_keys, frame_cnt);
 }
 
 template <bool kAdjoint, int kFeat>
-__global__ void __launch_bounds__(kShadeThreads, kShadeCtasPerSm)
+__global__ void __launch_bounds__(kShadeThreads, shade_ctas(kFeat))
     k_shade_pv(const __grid_constant__ ParamViews pv, int nviews, const long long *__restrict__ blk_offs,
-               long long nblocks, unsigned long long *__restrict__ keys, int reset_keys,
+               long long nblocks, int nsub, unsigned long long *__restrict__ keys, int reset_keys,
                const Counters *__restrict__ frame_cnt)
 {
-    shade_body<kAdjoint, kFeat>(pv.v, nviews, blk_offs, nblocks, keys, reset_keys, frame_cnt);
+    shade_body<kAdjoint, kFeat>(pv.v, nviews, blk_offs, nblocks, nsub, keys, reset_keys, frame_cnt);
 }
 
 // A training frame's losses: one block per view sums the view's partial
@@ -601,11 +715,10 @@ cudaError_t launch_loss_finalize(const ViewDev *views, int nviews, const Counter
     return cudaGetLastError();
 }
 
-// Warps of kShadeBlocks blocks, kShadeThreads threads per CTA.
+// One warp per strip, kShadeThreads threads per CTA.
 static unsigned shade_grid(long long nblocks)
 {
-    const long long warps = (nblocks + kShadeBlocks - 1) / kShadeBlocks;
-    return (unsigned)((warps * 32 + kShadeThreads - 1) / kShadeThreads);
+    return (unsigned)((nblocks * 32 + kShadeThreads - 1) / kShadeThreads);
 }
 
 // The parameter table of a launch's views (null: the batch is too large, or
@@ -621,43 +734,43 @@ static const ParamViews *param_views(const ViewDev *host_views, int nviews)
 
 template <bool kAdjoint, int kFeat>
 static void launch_shade_one(unsigned g, const ViewDev *views, const ParamViews *pv, int nviews,
-                             const long long *blk_offs, long long nblocks, unsigned long long *keys, int reset_keys,
-                             const Counters *frame_cnt, cudaStream_t st)
+                             const long long *blk_offs, long long nblocks, int nsub, unsigned long long *keys,
+                             int reset_keys, const Counters *frame_cnt, cudaStream_t st)
 {
     if (pv)
-        k_shade_pv<kAdjoint, kFeat><<<g, kShadeThreads, 0, st>>>(*pv, nviews, blk_offs, nblocks, keys, reset_keys,
+        k_shade_pv<kAdjoint, kFeat><<<g, kShadeThreads, 0, st>>>(*pv, nviews, blk_offs, nblocks, nsub, keys, reset_keys,
                                                                  frame_cnt);
     else
-        k_shade<kAdjoint, kFeat><<<g, kShadeThreads, 0, st>>>(views, nviews, blk_offs, nblocks, keys, reset_keys,
+        k_shade<kAdjoint, kFeat><<<g, kShadeThreads, 0, st>>>(views, nviews, blk_offs, nblocks, nsub, keys, reset_keys,
                                                               frame_cnt);
 }
 
 template <bool kAdjoint>
 static void launch_shade_t(int feat, unsigned g, const ViewDev *views, const ParamViews *pv, int nviews,
-                           const long long *blk_offs, long long nblocks, unsigned long long *keys, int reset_keys,
+                           const long long *blk_offs, long long nblocks, int nsub, unsigned long long *keys, int reset_keys,
                            const Counters *frame_cnt, cudaStream_t st)
 {
     if (feat == kFeatF64) {  // the precision form without the specular and sampled-foveation paths
-        launch_shade_one<kAdjoint, kFeatF64>(g, views, pv, nviews, blk_offs, nblocks, keys, reset_keys, frame_cnt, st);
+        launch_shade_one<kAdjoint, kFeatF64>(g, views, pv, nviews, blk_offs, nblocks, nsub, keys, reset_keys, frame_cnt, st);
         return;
     }
     if (feat & kFeatF64) {  // the precision form with either: one variant with every path (same bits)
-        launch_shade_one<kAdjoint, kFeatSpec | kFeatLut | kFeatF64>(g, views, pv, nviews, blk_offs, nblocks, keys,
+        launch_shade_one<kAdjoint, kFeatSpec | kFeatLut | kFeatF64>(g, views, pv, nviews, blk_offs, nblocks, nsub, keys,
                                                                     reset_keys, frame_cnt, st);
         return;
     }
     switch (feat) {
     case 0:
-        launch_shade_one<kAdjoint, 0>(g, views, pv, nviews, blk_offs, nblocks, keys, reset_keys, frame_cnt, st);
+        launch_shade_one<kAdjoint, 0>(g, views, pv, nviews, blk_offs, nblocks, nsub, keys, reset_keys, frame_cnt, st);
         break;
     case kFeatSpec:
-        launch_shade_one<kAdjoint, kFeatSpec>(g, views, pv, nviews, blk_offs, nblocks, keys, reset_keys, frame_cnt, st);
+        launch_shade_one<kAdjoint, kFeatSpec>(g, views, pv, nviews, blk_offs, nblocks, nsub, keys, reset_keys, frame_cnt, st);
         break;
     case kFeatLut:
-        launch_shade_one<kAdjoint, kFeatLut>(g, views, pv, nviews, blk_offs, nblocks, keys, reset_keys, frame_cnt, st);
+        launch_shade_one<kAdjoint, kFeatLut>(g, views, pv, nviews, blk_offs, nblocks, nsub, keys, reset_keys, frame_cnt, st);
         break;
     default:
-        launch_shade_one<kAdjoint, kFeatSpec | kFeatLut>(g, views, pv, nviews, blk_offs, nblocks, keys, reset_keys,
+        launch_shade_one<kAdjoint, kFeatSpec | kFeatLut>(g, views, pv, nviews, blk_offs, nblocks, nsub, keys, reset_keys,
                                                          frame_cnt, st);
     }
 }
@@ -676,7 +789,7 @@ int shade_features(const ViewDev *vd, int n)
     return f;
 }
 
-cudaError_t launch_shade(const ViewDev *views, int nviews, const long long *blk_offs, long long nblocks,
+cudaError_t launch_shade(const ViewDev *views, int nviews, const long long *blk_offs, long long nblocks, int nsub,
                          unsigned long long *keys, bool reset_keys, bool adjoint, const Counters *frame_cnt, int feat,
                          cudaStream_t st, const ViewDev *host_views)
 {
@@ -684,111 +797,129 @@ cudaError_t launch_shade(const ViewDev *views, int nviews, const long long *blk_
         const unsigned g = shade_grid(nblocks);
         const ParamViews *pv = param_views(host_views, nviews);
         if (adjoint)
-            launch_shade_t<true>(feat, g, views, pv, nviews, blk_offs, nblocks, keys, reset_keys, frame_cnt, st);
+            launch_shade_t<true>(feat, g, views, pv, nviews, blk_offs, nblocks, nsub, keys, reset_keys, frame_cnt, st);
         else
-            launch_shade_t<false>(feat, g, views, pv, nviews, blk_offs, nblocks, keys, reset_keys, frame_cnt, st);
+            launch_shade_t<false>(feat, g, views, pv, nviews, blk_offs, nblocks, nsub, keys, reset_keys, frame_cnt, st);
     }
     return cudaGetLastError();
 }
 
 // Stage (e) on its own: the adjoint of a shaded frame from its id buffer
-// and an upstream gradient.
+// and an upstream gradient (grad_in of every view).
 template <int kFeat>
 __device__ __forceinline__ void backward_body(const ViewDev *__restrict__ views, int nviews,
-                                              const long long *__restrict__ blk_offs, long long nblocks,
-                                              const Counters *__restrict__ frame_cnt)
+                                              const long long *__restrict__ blk_offs, long long nblocks, int nsub)
 {
-    const long long b0 = (((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * kShadeBlocks;
+    __shared__ unsigned s_id[kShadeWarps][kBlkH * kIdPitch];
+    __shared__ __align__(16) float s_rows[kShadeWarps][kRows * kRowPitch];
+    const long long b0 = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (b0 >= nblocks)
         return;  // whole warps
-    // in a training frame: a forward that overflowed is rerun by the host,
-    // so its adjoint must not accumulate
-    if (frame_overflowed(frame_cnt))
-        return;
-    const int lane = threadIdx.x & 31;
-    AdjointSum acc;
-    adjoint_reset(acc);
-    for (int p = 0; p < kShadeBlocks && b0 + p < nblocks; ++p) {
-        int q, pi, pj;
-        long long lin;
-        const bool inside = block_pixel(views, nviews, blk_offs, b0 + p, lane, q, lin, pi, pj);
-        const ViewDev &v = views[q];
-        unsigned id = 0xFFFFFFFFu;
-        if (inside && (v.grad_in || v.target))  // views of a batch without a gradient are skipped
-            id = v.id_in[lin];
-        const bool valid = id < (unsigned)v.T;
-        PixelHit h;
-        PixelAlbedo pa;
-        float g0 = 0.f, g1 = 0.f, g2 = 0.f;
-        if (valid) {
-            const long long plane = (long long)v.W * v.H;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const Strip sp = strip_of(views, nviews, blk_offs, b0, nsub);
+    const ViewDev &v = views[sp.q];
+    const int W = v.W, H = v.H;
+    const int plane = W * H;  // <= 2^28
+    unsigned live = 0u;
+    {
+        const int col = sp.i0 + (lane & ((1 << sp.sh) - 1)), row0 = sp.j0 + (lane >> sp.sh), rstep = 32 >> sp.sh;
+        unsigned id[kBlkH];
+#pragma unroll
+        for (int k = 0; k < kBlkH; ++k) {
+            id[k] = 0xFFFFFFFFu;
+            const int j = row0 + k * rstep;
+            if (k < nsub && col < W && j < H)
+                id[k] = v.id_in[j * W + col];
+        }
+#pragma unroll
+        for (int k = 0; k < kBlkH; ++k) {
+            if (k >= nsub)
+                break;
+            const bool hit = id[k] < (unsigned)v.T;
+            s_id[warp][(k * rstep + (lane >> sp.sh)) * kIdPitch + (lane & ((1 << sp.sh) - 1))] =
+                hit ? id[k] : 0xFFFFFFFFu;
+            live |= blocks_of(__ballot_sync(0xffffffffu, hit), nsub);
+        }
+    }
+    __syncwarp();
+    TriangleSum ts;
+    ts.s = 0.f;
+    ts.id = 0xFFFFFFFFu;
+    const ValueLane vl = value_lane();
+    float *rows = s_rows[warp];
+    for (; live; live &= live - 1u) {
+        const int x = (__ffs(live) - 1) * kBlkW + lane % kBlkW, y = lane / kBlkW;
+        const unsigned id = s_id[warp][y * kIdPitch + x];
+        const int pi = sp.i0 + x, pj = sp.j0 + y, lin = pj * W + pi;
+        const bool hit = id != 0xFFFFFFFFu;
+        if (hit) {
+            const float g0 = v.grad_in[lin], g1 = v.grad_in[plane + lin], g2 = v.grad_in[2 * plane + lin];
+            PixelHit h;
+            PixelAlbedo pa;
             pixel_hit<kFeat>(v, pi, pj, id, h);
             pixel_albedo(v, h, pa);
-            if (v.target) {
-                // L2 loss sum (rgb - target)^2: its gradient from this frame's image
-                g0 = 2.f * (v.rgb_out[lin] - v.target[lin]);
-                g1 = 2.f * (v.rgb_out[plane + lin] - v.target[plane + lin]);
-                g2 = 2.f * (v.rgb_out[2 * plane + lin] - v.target[2 * plane + lin]);
-            } else {
-                g0 = v.grad_in[lin];
-                g1 = v.grad_in[plane + lin];
-                g2 = v.grad_in[2 * plane + lin];
-            }
+            adjoint_rows<kFeat>(v, h, pa, g0, g1, g2, rows + lane);
+        } else {
+#pragma unroll
+            for (int r = 0; r < kRows; ++r)
+                rows[r * kRowPitch + lane] = 0.f;
         }
-        adjoint_step<kFeat>(views, acc, valid, q, id, h, pa, g0, g1, g2);
+        __syncwarp();
+        sum_block(v, rows, vl, hit, id, ts);
+        __syncwarp();  // the rows are written again by the next block
     }
-    adjoint_flush(views, acc);
+    if (ts.id != 0xFFFFFFFFu)
+        add_triangle(v, ts.id, ts.s);
 }
 
 template <int kFeat>
-__global__ void __launch_bounds__(kShadeThreads, kShadeCtasPerSm)
+__global__ void __launch_bounds__(kShadeThreads, kBackwardCtas)
     k_backward(const ViewDev *__restrict__ views, int nviews, const long long *__restrict__ blk_offs, long long nblocks,
-               const Counters *__restrict__ frame_cnt)
+               int nsub)
 {
-    backward_body<kFeat>(views, nviews, blk_offs, nblocks, frame_cnt);
+    backward_body<kFeat>(views, nviews, blk_offs, nblocks, nsub);
 }
 
 template <int kFeat>
-__global__ void __launch_bounds__(kShadeThreads, kShadeCtasPerSm)
+__global__ void __launch_bounds__(kShadeThreads, kBackwardCtas)
     k_backward_pv(const __grid_constant__ ParamViews pv, int nviews, const long long *__restrict__ blk_offs,
-                  long long nblocks, const Counters *__restrict__ frame_cnt)
+                  long long nblocks, int nsub)
 {
-    backward_body<kFeat>(pv.v, nviews, blk_offs, nblocks, frame_cnt);
+    backward_body<kFeat>(pv.v, nviews, blk_offs, nblocks, nsub);
 }
 
 template <int kFeat>
 static void launch_backward_one(unsigned g, const ViewDev *views, const ParamViews *pv, int nviews,
-                                const long long *blk_offs, long long nblocks, const Counters *frame_cnt,
-                                cudaStream_t st)
+                                const long long *blk_offs, long long nblocks, int nsub, cudaStream_t st)
 {
     if (pv)
-        k_backward_pv<kFeat><<<g, kShadeThreads, 0, st>>>(*pv, nviews, blk_offs, nblocks, frame_cnt);
+        k_backward_pv<kFeat><<<g, kShadeThreads, 0, st>>>(*pv, nviews, blk_offs, nblocks, nsub);
     else
-        k_backward<kFeat><<<g, kShadeThreads, 0, st>>>(views, nviews, blk_offs, nblocks, frame_cnt);
+        k_backward<kFeat><<<g, kShadeThreads, 0, st>>>(views, nviews, blk_offs, nblocks, nsub);
 }
 
-cudaError_t launch_backward(const ViewDev *views, int nviews, const long long *blk_offs, long long nblocks,
-                            const Counters *frame_cnt, int feat, cudaStream_t st, const ViewDev *host_views)
+cudaError_t launch_backward(const ViewDev *views, int nviews, const long long *blk_offs, long long nblocks, int nsub,
+                            int feat, cudaStream_t st, const ViewDev *host_views)
 {
     if (nblocks > 0) {
         const unsigned g = shade_grid(nblocks);
         const ParamViews *pv = param_views(host_views, nviews);
         if (feat & kFeatF64) {
-            launch_backward_one<kFeatSpec | kFeatLut | kFeatF64>(g, views, pv, nviews, blk_offs, nblocks, frame_cnt, st);
+            launch_backward_one<kFeatSpec | kFeatLut | kFeatF64>(g, views, pv, nviews, blk_offs, nblocks, nsub, st);
             return cudaGetLastError();
         }
         switch (feat) {
         case 0:
-            launch_backward_one<0>(g, views, pv, nviews, blk_offs, nblocks, frame_cnt, st);
+            launch_backward_one<0>(g, views, pv, nviews, blk_offs, nblocks, nsub, st);
             break;
         case kFeatSpec:
-            launch_backward_one<kFeatSpec>(g, views, pv, nviews, blk_offs, nblocks, frame_cnt, st);
+            launch_backward_one<kFeatSpec>(g, views, pv, nviews, blk_offs, nblocks, nsub, st);
             break;
         case kFeatLut:
-            launch_backward_one<kFeatLut>(g, views, pv, nviews, blk_offs, nblocks, frame_cnt, st);
+            launch_backward_one<kFeatLut>(g, views, pv, nviews, blk_offs, nblocks, nsub, st);
             break;
         default:
-            launch_backward_one<kFeatSpec | kFeatLut>(g, views, pv, nviews, blk_offs, nblocks, frame_cnt, st);
+            launch_backward_one<kFeatSpec | kFeatLut>(g, views, pv, nviews, blk_offs, nblocks, nsub, st);
         }
     }
     return cudaGetLastError();
