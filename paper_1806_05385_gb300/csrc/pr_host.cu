@@ -151,7 +151,8 @@ struct pr_workspace {
     DevBuf flag_bits, flag_list;   // pixels flagged for the FP64 re-test (bitmap + list)
     DevBuf loss_part;              // training frames: kLossSlots partial sums of each view's loss
     DevBuf stage;                  // device copies of host-side outputs
-    long long cap_pairs = 0, cap_items = 0;
+    long long cap_pairs = 0, cap_items = 0;  // cap_items: of each tile-size class
+    long long want_items = 0;                // items a class needed when it overflowed
     // leading keys known to hold ~0: every frame's reader (the resolve or the
     // shading) sets the keys it reads back to ~0, so a frame clears only
     // beyond this count (and after a new allocation)
@@ -438,6 +439,7 @@ struct BatchPlan {
     bool any_fp64 = false;
     bool any_paper_fov = false;  // some foveated view asks for the paper's edge bound
     bool any_loss = false;       // some view of a training frame accumulates its loss
+    double max_cand = 0;         // no frame has more candidate (triangle, tile) pairs: sum of T x tiles
     std::vector<Cls> classes;
     // output staging: per view (in order) device pointers used by kernels
     std::vector<pr_frame_grad> grads;  // per view (in order); empty: no adjoint
@@ -494,6 +496,7 @@ pr_status plan_batch(const pr_batch_view *views, int n, const pr_params &prm, Ba
         v.pix_off = P.pix_off[q];
         P.tri_off[q + 1] = P.tri_off[q] + bv.scene->T;
         P.tile_off[q + 1] = P.tile_off[q] + (long long)v.tiles_x * v.tiles_y;
+        P.max_cand += (double)bv.scene->T * ((double)v.tiles_x * v.tiles_y);
         P.pix_off[q + 1] = P.pix_off[q] + (long long)v.W * v.H;
         const long long np = (long long)v.W * v.H;
         BatchPlan::Out &o = P.out[q];
@@ -560,9 +563,8 @@ pr_status size_workspace(pr_workspace *ws, const BatchPlan &P, int seg)
     PR_TRY(ensure(ws->tile_cnt, sizeof(unsigned long long) * std::max(P.ntiles, 1ll)));
     PR_TRY(ensure(ws->scan, sizeof(unsigned long long) * (P.ntiles + 1)));
     PR_TRY(ensure(ws->fill, sizeof(unsigned) * std::max(P.ntiles, 1ll)));
-    // two scans' look-back states: the candidate-tile scan, then the tile scan
-    PR_TRY(ensure(ws->sums,
-                  sizeof(unsigned long long) * (scan_block_sums_needed(P.ttot) + scan_block_sums_needed(P.ntiles))));
+    // the candidate scan's look-back state
+    PR_TRY(ensure(ws->sums, sizeof(unsigned long long) * scan_block_sums_needed(P.ttot)));
     PR_TRY(ensure(ws->cand, sizeof(unsigned long long) * std::max(P.ttot, 1ll)));
     PR_TRY(ensure(ws->cand_off, sizeof(unsigned long long) * (P.ttot + 1)));
     PR_TRY(ensure(ws->binned, sizeof(int) * std::max(P.ttot, 1ll)));
@@ -586,11 +588,13 @@ pr_status size_workspace(pr_workspace *ws, const BatchPlan &P, int seg)
     ws->cap_pairs = std::min((long long)(ws->pairs.cap / sizeof(unsigned long long)), kMaxPairs);
     PR_TRY(ensure(ws->hit_entry, sizeof(unsigned long long) * ws->cap_pairs));
     PR_TRY(ensure(ws->hit_tile, sizeof(unsigned) * ws->cap_pairs));
-    const long long want_items = std::max(ws->cap_items, ws->cap_pairs / seg + P.ntiles + 1024);
+    // the classes' items side by side, room for every class in any frame (so
+    // that a frame with more classes does not regrow the buffer)
+    const long long want_items = kMaxClasses * std::max(ws->want_items, ws->cap_pairs / seg + P.ntiles + 1024);
     if ((size_t)want_items * sizeof(int4) > ws->items.cap || !ws->items.p) {
         PR_TRY(ensure(ws->items, sizeof(int4) * want_items));
     }
-    ws->cap_items = std::min((long long)(ws->items.cap / sizeof(int4)), kMaxPairs);
+    ws->cap_items = std::min((long long)(ws->items.cap / sizeof(int4)) / kMaxClasses, kMaxPairs);
     PR_TRY(ws->h_views.ensure(n));
     PR_TRY(ws->h_offs.ensure(4 * (n + 1)));
     PR_TRY(ws->h_cnt.ensure(1));
@@ -656,8 +660,7 @@ pr_status enqueue_batch(pr_workspace *ws, BatchPlan &P, int seg, bool shade, cud
     const long long *tri_offs = tab_offs, *tile_offs = tri_offs + n + 1, *pix_offs = tile_offs + n + 1;
     const long long *blk_offs = pix_offs + n + 1;
     Counters *cnt = ws->counters.as<Counters>();
-    unsigned long long *state_a = ws->sums.as<unsigned long long>();
-    unsigned long long *state_b = state_a + scan_block_sums_needed(P.ttot);
+    unsigned long long *state = ws->sums.as<unsigned long long>();
     float4 *rec = ws->rec.as<float4>(), *hp = ws->hp.as<float4>(), *tile_box = ws->tile_box.as<float4>();
     int4 *tbox = ws->tbox.as<int4>();
     unsigned long long *tile_cnt = ws->tile_cnt.as<unsigned long long>(), *scan = ws->scan.as<unsigned long long>();
@@ -671,10 +674,14 @@ pr_status enqueue_batch(pr_workspace *ws, BatchPlan &P, int seg, bool shade, cud
     auto mark = [&](int k) {
         return marks || !capturing ? cudaEventRecordWithFlags(ev[k], st, ev_flags) : cudaSuccess;
     };
-    unsigned long long *cand = ws->cand.as<unsigned long long>(), *cand_off = ws->cand_off.as<unsigned long long>();
+    CandList list;
+    list.binned = ws->binned.as<int>();
+    list.off = ws->cand_off.as<unsigned long long>();
+    list.cand = ws->cand.as<unsigned long long>();
+    list.shift = P.any_paper_fov ? 0 : cand_shift(P.ttot, P.max_cand);
     PR_TRY(mark(0));
-    // one launch clears the counters, queue heads, tile counts and cursors,
-    // both scans' tickets and flags, the FP64 flags, and computes the tiles'
+    // one launch clears the counters, queue heads, tile counts, the candidate
+    // scan's ticket and flags, the FP64 flags, and computes the tiles'
     // display boxes.  The keys: a frame whose keys fit in L2 clears them
     // here, where the fragment stage then finds them in L2; a larger frame
     // has its reader (resolve or shading, which reads every key anyway) set
@@ -684,22 +691,20 @@ pr_status enqueue_batch(pr_workspace *ws, BatchPlan &P, int seg, bool shade, cud
     const bool reader_resets = keys_reset_by_reader(P.npix);
     const long long clean_before = reader_resets ? ws->keys_clean_n : 0;
     ws->keys_clean_n = 0;
-    PR_TRY(launch_frame_init(dv, n, tile_offs, tile_box, cnt, ws->heads.as<int>(), tile_cnt, ws->fill.as<unsigned>(),
-                             P.ntiles, state_a, scan_state_words(P.ttot), state_b, scan_state_words(P.ntiles),
-                             ws->flag_bits.as<unsigned>(), P.any_fp64 ? (P.npix + 31) / 32 + 1 : 0,
-                             ws->keys.as<unsigned long long>(), P.npix > clean_before ? P.npix : 0,
-                             ws->loss_part.as<float>(), P.any_loss ? (long long)kLossSlots * n : 0, st));
-    int *binned = ws->binned.as<int>();
-    PR_TRY(launch_bound(dv, n, tri_offs, P.ttot, rec, hp, tbox, cand, binned, cnt, st));
+    PR_TRY(launch_frame_init(dv, n, tile_offs, tile_box, cnt, ws->heads.as<int>(), tile_cnt, P.ntiles, state,
+                             list.shift ? 0 : scan_state_words(P.ttot), ws->flag_bits.as<unsigned>(),
+                             P.any_fp64 ? (P.npix + 31) / 32 + 1 : 0, ws->keys.as<unsigned long long>(),
+                             P.npix > clean_before ? P.npix : 0, ws->loss_part.as<float>(),
+                             P.any_loss ? (long long)kLossSlots * n : 0, st));
+    PR_TRY(launch_bound(dv, n, tri_offs, P.ttot, rec, hp, tbox, list, cnt, st));
     if (P.any_paper_fov)
-        PR_TRY(launch_paper_fov(dv, n, tri_offs, P.ttot, rec, hp, tbox, cand, st));
+        PR_TRY(launch_paper_fov(dv, n, tri_offs, P.ttot, rec, hp, tbox, list.cand, st));
     PR_TRY(mark(1));
-    // candidate tiles of the binned triangles (count known on the device)
-    PR_TRY(launch_scan(cand, cand_off, state_a, P.ttot, 0, cnt, st, true, binned, &cnt->binned));
-    PR_TRY(launch_bin_count(dv, n, tri_offs, P.ttot, binned, cand_off, rec, hp, tbox, tile_box, tile_cnt,
+    if (!list.shift)  // candidate tiles of the listed triangles (count known on the device)
+        PR_TRY(launch_cand_scan(list, state, P.ttot, cnt, st));
+    PR_TRY(launch_bin_count(dv, n, tri_offs, P.ttot, list, rec, hp, tbox, tile_box, tile_cnt,
                             ws->hit_entry.as<unsigned long long>(), ws->hit_tile.as<unsigned>(), ws->cap_pairs, cnt,
                             st));
-    // the scan of the tile counts also emits the work items
     ItemsOut io;
     io.views = dv;
     io.nviews = n;
@@ -707,20 +712,22 @@ pr_status enqueue_batch(pr_workspace *ws, BatchPlan &P, int seg, bool shade, cud
     io.items = ws->items.as<int4>();
     io.cap_items = ws->cap_items;
     io.cap_pairs = ws->cap_pairs;
-    PR_TRY(launch_scan(tile_cnt, scan, state_b, P.ntiles, seg, cnt, st, true, nullptr, nullptr, &io));
-    PR_TRY(launch_bin_scatter(ws->hit_entry.as<unsigned long long>(), ws->hit_tile.as<unsigned>(), scan,
+    io.ncls = (int)P.classes.size();
+    for (int c = 0; c < io.ncls; ++c)
+        io.cls_end[c] = P.classes[c].tile_hi;
+    PR_TRY(launch_tile_alloc(tile_cnt, scan, ws->fill.as<unsigned>(), P.ntiles, seg, cnt, io, st));
+    PR_TRY(launch_bin_scatter(ws->hit_entry.as<unsigned long long>(), ws->hit_tile.as<unsigned>(),
                               ws->fill.as<unsigned>(), ws->pairs.as<unsigned long long>(), ws->cap_pairs, P.ntiles, cnt,
                               st));
-    PR_TRY(launch_sort_items(ws->items.as<int4>(), scan, P.ntiles, ws->cap_items, seg,
-                             ws->pairs.as<unsigned long long>(), cnt, st));
+    PR_TRY(launch_sort_items(io, P.ntiles, seg, ws->pairs.as<unsigned long long>(), cnt, st));
     PR_TRY(mark(2));
     int *heads = ws->heads.as<int>();
     for (size_t c = 0; c < P.classes.size(); ++c) {
         const auto &cl = P.classes[c];
-        PR_TRY(launch_fragment(cl.S, cl.fp64, dv, ws->items.as<int4>(), scan, cl.tile_lo, cl.tile_hi, ws->cap_items,
-                               heads + c, ws->pairs.as<unsigned long long>(), rec, ws->keys.as<unsigned long long>(),
-                               ws->flag_bits.as<unsigned>(), ws->flag_list.as<long long>(), cnt,
-                               fragment_grid(cl.S, cl.fp64), st));
+        PR_TRY(launch_fragment(cl.S, cl.fp64, dv, io, (int)c, heads + c, ws->pairs.as<unsigned long long>(), rec,
+                               ws->keys.as<unsigned long long>(), ws->flag_bits.as<unsigned>(),
+                               ws->flag_list.as<long long>(), cnt,
+                               fragment_grid(cl.S, cl.fp64, cl.tile_hi - cl.tile_lo, P.ttot, seg), st));
     }
     PR_TRY(mark(3));
     if (P.any_fp64)
@@ -763,7 +770,7 @@ pr_status finish_stats(pr_workspace *ws, const BatchPlan &P)
     ws->stats.tests = c.tests;
     ws->stats.hits = c.hits;
     ws->stats.pairs = c.pairs_total;
-    ws->stats.items = c.items_total;
+    ws->stats.items = c.items_total();
     ws->stats.culled = c.culled;
     ws->stats.flagged = c.flagged;
     ws->stats.changed = c.changed;
@@ -810,12 +817,14 @@ pr_status run_batch(pr_workspace *ws, const pr_batch_view *views, int n, const p
         const Counters &c = *ws->h_cnt.p;
         // work items address bin entries with 32-bit offsets: a frame with
         // more entries than that is refused, not regrown
-        if ((long long)c.pairs_total > kMaxPairs || (long long)c.items_total > kMaxPairs)
+        if ((long long)c.pairs_total > kMaxPairs || (long long)c.items_total() > kMaxPairs)
             return PR_ERR_OVERFLOW;
         ws->cap_pairs = std::max<long long>(ws->cap_pairs, (long long)c.pairs_total + 1024);
-        ws->cap_items = std::max<long long>(ws->cap_items, (long long)c.items_total + 1024);
-        ws->cap_pairs = std::min(ws->cap_pairs + ws->cap_pairs / 4, kMaxPairs);
-        ws->cap_items = std::min(ws->cap_items + ws->cap_items / 4, kMaxPairs);  // size_workspace grows both to these
+        ws->cap_pairs = std::min(ws->cap_pairs + ws->cap_pairs / 4, kMaxPairs);  // size_workspace grows both to these
+        const long long items =
+            (long long)std::max(c.items_n[0], std::max(c.items_n[1], c.items_n[2])) + 1024;
+        if (items > ws->cap_items)
+            ws->want_items = std::min(items + items / 4, kMaxPairs);
     }
     return PR_ERR_OVERFLOW;
 }
@@ -1414,7 +1423,7 @@ pr_status pr_graph_status(pr_graph *g)
     ws->stats.tests = c.tests;
     ws->stats.hits = c.hits;
     ws->stats.pairs = c.pairs_total;
-    ws->stats.items = c.items_total;
+    ws->stats.items = c.items_total();
     ws->stats.culled = c.culled;
     ws->stats.flagged = c.flagged;
     ws->stats.changed = c.changed;
@@ -1487,8 +1496,9 @@ pr_status pr_debug_bounds(const pr_scene *sc, int32_t *pix_box, float *t_range)
         pix_box[4 * k + 1] = b.y & 0xffff;
         pix_box[4 * k + 2] = (b.x >> 16) & 0xffff;
         pix_box[4 * k + 3] = (b.y >> 16) & 0xffff;  // a culled triangle has the empty box [1, 0]
-        t_range[2 * k + 0] = rec[k * kRecF4 + 5].x;
-        t_range[2 * k + 1] = rec[k * kRecF4 + 5].y;
+        const bool culled = b.x == 1 && b.y == 1 && b.w == 0;  // no record (0 is no finite depth's order key)
+        t_range[2 * k + 0] = culled ? INFINITY : rec[k * kRecF4 + 5].x;
+        t_range[2 * k + 1] = culled ? -INFINITY : rec[k * kRecF4 + 5].y;
     }
     return PR_OK;
 }

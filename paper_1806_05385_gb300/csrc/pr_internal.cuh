@@ -91,13 +91,36 @@ struct ParamViews {
 };
 static_assert(sizeof(ParamViews) <= 30 * 1024, "the view table must fit the kernel parameter space");
 
+constexpr int kMaxClasses = 3;  // tile sizes (8, 16, 32): a frame's fragment launches
+
 struct Counters {
     unsigned long long tests, hits, culled, flagged, changed;
-    unsigned long long pairs_total, items_total;  // copied from the scan for the host
+    unsigned long long pairs_total;               // bin entries handed out to the tiles
+    unsigned long long items_n[kMaxClasses];      // work items per tile-size class
     unsigned long long hits_listed;               // (triangle, tile) hits appended by the binning count pass
     unsigned long long binned;                    // triangles with candidate tiles, listed by the bound pass
+    unsigned long long binned_cand;               // or (CandList::shift > 0): that count and their candidate tiles, packed
     unsigned int status;
     unsigned int depth_err_bits;  // bits of the largest FP32-vs-FP64 relative depth error (re-test)
+    __host__ __device__ unsigned long long items_total() const { return items_n[0] + items_n[1] + items_n[2]; }
+};
+
+// The list of triangles with candidate tiles and the running sum of their
+// candidate counts (the index space of the binning pass).  shift > 0: the
+// bound pass hands out list places and candidate ranges together, with one
+// 64-bit atomic per warp on (candidates << shift) | triangles, so that the
+// list's offsets ascend; shift = 0: the counts go to `cand` and a scan makes
+// the offsets (when the sums might not fit 64 - shift bits, or a later pass
+// changes the counts).
+struct CandList {
+    int *binned;                     // batch-wide triangle index of every list entry
+    unsigned long long *off;         // candidates before every entry
+    unsigned long long *cand;        // shift = 0: candidates of every triangle
+    int shift;
+    __device__ unsigned long long length(const Counters *c) const
+    {
+        return shift ? c->binned_cand & ((1ull << shift) - 1ull) : c->binned;
+    }
 };
 
 __device__ __forceinline__ bool is_rolling(int mode) { return mode == PR_ROLLING || mode == PR_BOTH; }

@@ -26,62 +26,67 @@ constexpr int kSceneUpdateChunk = 64;  // scenes per launch (passed by value)
 cudaError_t launch_scene_update_batch(const SceneUpdate *u, int n, cudaStream_t st);
 
 // stage (a): per-triangle bounds (the tiles' display boxes come with the frame init)
-// binned: the triangles with candidate tiles are appended here (cnt->binned)
+// list: the triangles with candidate tiles are appended here.  A culled
+// triangle gets its empty pixel box in tbox and nothing else.
 cudaError_t launch_bound(const ViewDev *views, int nviews, const long long *tri_offs, long long ttot, float4 *rec,
-                         float4 *hp, int4 *tbox, unsigned long long *cand, int *binned, Counters *cnt,
-                         cudaStream_t st);
+                         float4 *hp, int4 *tbox, const CandList &list, Counters *cnt, cudaStream_t st);
+// the list's shift for ttot triangles that have at most max_cand candidate
+// tiles in all: 0 if the two do not fit a 64-bit word together
+int cand_shift(long long ttot, double max_cand);
 // the paper's foveation edge bounds for the views that select them (after launch_bound)
 cudaError_t launch_paper_fov(const ViewDev *views, int nviews, const long long *tri_offs, long long ttot,
                              const float4 *rec, float4 *hp, int4 *tbox, unsigned long long *cand, cudaStream_t st);
 
 // stage (b): tile binning -- count pass (tile counts, and every hit appended to the hit list)
-// over the binned triangles (cand_off: prefix of their candidate counts), then after the scan
-// the scatter of the list into the bins
+// over the listed triangles, then the bins' places (launch_tile_alloc) and
+// the scatter of the hit list into the bins
 cudaError_t launch_bin_count(const ViewDev *views, int nviews, const long long *tri_offs, long long ttot,
-                             const int *binned, const unsigned long long *cand_off, const float4 *rec,
-                             const float4 *hp, const int4 *tbox, const float4 *tile_box, unsigned long long *tile_cnt,
-                             unsigned long long *hit_entry, unsigned *hit_tile, long long cap_pairs, Counters *cnt,
-                             cudaStream_t st);
-cudaError_t launch_bin_scatter(const unsigned long long *hit_entry, const unsigned *hit_tile,
-                               const unsigned long long *scan, unsigned int *fill, unsigned long long *pairs,
-                               long long cap_pairs, long long ntiles, Counters *cnt, cudaStream_t st);
-// Where the scan of the tile counts writes the fragment stage's work items.
+                             const CandList &list, const float4 *rec, const float4 *hp, const int4 *tbox,
+                             const float4 *tile_box, unsigned long long *tile_cnt, unsigned long long *hit_entry,
+                             unsigned *hit_tile, long long cap_pairs, Counters *cnt, cudaStream_t st);
+// Where the fragment stage's work items go: class c (the tiles before
+// cls_end[c], after the previous class's) to items[c cap_items ..].
 struct ItemsOut {
     const ViewDev *views = nullptr;
     int nviews = 0;
     const long long *tile_offs = nullptr;
     int4 *items = nullptr;
     long long cap_items = 0, cap_pairs = 0;
+    int ncls = 0;
+    long long cls_end[kMaxClasses] = {};
 };
-// state_zeroed: the caller cleared the ticket and flags (state[0, 1 + nb)).
-// gather: scan in[gather[i]]; n_dev: the count is min(*n_dev, n) (device).
-// items (with seg > 0): also emit each tile's work items and the totals.
-cudaError_t launch_scan(const unsigned long long *in, unsigned long long *out, unsigned long long *state, long long n,
-                        int seg, Counters *cnt, cudaStream_t st, bool state_zeroed = false,
-                        const int *gather = nullptr, const unsigned long long *n_dev = nullptr,
-                        const ItemsOut *items = nullptr);
+// every tile's place in the bins (off, and cursor for the scatter) and its work items
+cudaError_t launch_tile_alloc(const unsigned long long *tile_cnt, unsigned long long *off, unsigned *cursor,
+                              long long ntiles, int seg, Counters *cnt, const ItemsOut &io, cudaStream_t st);
+cudaError_t launch_bin_scatter(const unsigned long long *hit_entry, const unsigned *hit_tile, unsigned *cursor,
+                               unsigned long long *pairs, long long cap_pairs, long long ntiles, Counters *cnt,
+                               cudaStream_t st);
+// the list's offsets from the counts (list.shift = 0); the caller cleared
+// the state's ticket and flags (state[0, scan_state_words))
+cudaError_t launch_cand_scan(const CandList &list, unsigned long long *state, long long ttot, Counters *cnt,
+                             cudaStream_t st);
 // the start of a frame: clears, the first npix keys to ~0 (0: none, where the
 // last frames' readers left them so), tile display boxes (one launch)
 cudaError_t launch_frame_init(const ViewDev *views, int nviews, const long long *tile_offs, float4 *tile_box,
-                              Counters *cnt, int *heads, unsigned long long *tile_cnt, unsigned *fill, long long ntiles,
-                              unsigned long long *state_a, long long nstate_a, unsigned long long *state_b,
-                              long long nstate_b, unsigned *flag_bits, long long nflag, unsigned long long *keys,
-                              long long npix, float *loss_part, long long nloss, cudaStream_t st);
+                              Counters *cnt, int *heads, unsigned long long *tile_cnt, long long ntiles,
+                              unsigned long long *state, long long nstate, unsigned *flag_bits, long long nflag,
+                              unsigned long long *keys, long long npix, float *loss_part, long long nloss,
+                              cudaStream_t st);
 size_t scan_block_sums_needed(long long n);
 // a scan whose look-back waits on a tile that never runs (status word out)
 cudaError_t scan_timeout_probe(cudaStream_t st, unsigned *status);
 // words of a scan's state that must start at zero (ticket and flags)
 long long scan_state_words(long long n);
 // sorts every item's run of bin entries (nearest first); runs <= kMaxSeg
-cudaError_t launch_sort_items(const int4 *items, const unsigned long long *scan, long long ntiles, long long cap_items,
-                              int seg, unsigned long long *pairs, const Counters *cnt, cudaStream_t st);
+cudaError_t launch_sort_items(const ItemsOut &io, long long ntiles, int seg, unsigned long long *pairs,
+                              const Counters *cnt, cudaStream_t st);
 
-// stage (c): per-fragment ray casting, FP64 re-test, resolve
-cudaError_t launch_fragment(int S, bool flag, const ViewDev *views, const int4 *items, const unsigned long long *scan,
-                            long long tile_lo, long long tile_hi, long long cap_items, int *head,
+// stage (c): per-fragment ray casting (the items of class cls), FP64 re-test, resolve
+cudaError_t launch_fragment(int S, bool flag, const ViewDev *views, const ItemsOut &io, int cls, int *head,
                             const unsigned long long *pairs, const float4 *rec, unsigned long long *keys,
                             unsigned *flag_bits, long long *flag_list, Counters *cnt, int grid, cudaStream_t st);
-int fragment_grid(int S, bool flag);
+// resident CTAs of the fragment kernel, or fewer for a frame of few items
+int fragment_grid(int S, bool flag, long long ntiles, long long ttot, int seg);
 cudaError_t launch_retest(const ViewDev *views, int nviews, const long long *pix_offs, const unsigned long long *scan,
                           const unsigned long long *tile_cnt, const unsigned long long *pairs, const float4 *rec,
                           const long long *flag_list, unsigned long long *keys, long long cap_pairs, Counters *cnt,

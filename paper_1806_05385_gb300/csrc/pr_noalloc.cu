@@ -203,8 +203,7 @@ extern "C" pr_status pr_rasterize_noalloc(const float *pos, const float *vel, co
     unsigned long long *hit_entry = (unsigned long long *)(arena + o_hit_e);
     unsigned *hit_tile = (unsigned *)(arena + o_hit_t);
     unsigned long long *keys = (unsigned long long *)(arena + o_keys);
-    // look-back states of the two scans: candidate tiles, then tile counts
-    unsigned long long *state_a = (unsigned long long *)(arena + o_sums), *state_b = state_a + scan_block_sums_needed(Tn);
+    unsigned long long *state = (unsigned long long *)(arena + o_sums);  // the candidate scan's look-back state
 
     // host-side constants go up by plain (pageable) copies; they complete
     // before the call returns, so the stack buffers may go out of scope
@@ -213,30 +212,38 @@ extern "C" pr_status pr_rasterize_noalloc(const float *pos, const float *vel, co
     const long long *tri_offs = doffs, *tile_offs = doffs + 2, *pix_offs = doffs + 4;
     // what must start at zero, the keys at ~0 (the arena keeps the previous
     // call's contents), and the tiles' display boxes
-    NA_TRY(launch_frame_init(dv, 1, tile_offs, tile_box, cnt, heads, tile_cnt, fill, nt, state_a, scan_state_words(T),
-                             state_b, scan_state_words(nt), nullptr, 0, keys, np, nullptr, 0, st));
+    CandList list;
+    list.binned = (int *)(arena + o_binned);
+    list.off = cand_off;
+    list.cand = cand;
+    const bool paper_fov = fov_bound != PR_FOV_SECTOR && (view->mode == PR_FOVEATED || view->mode == PR_BOTH);
+    list.shift = paper_fov ? 0 : cand_shift(T, (double)T * (double)nt);
+    NA_TRY(launch_frame_init(dv, 1, tile_offs, tile_box, cnt, heads, tile_cnt, nt, state,
+                             list.shift ? 0 : scan_state_words(T), nullptr, 0, keys, np, nullptr, 0, st));
     NA_TRY(launch_scene_pack(pos, vel, col, V, vtx, col4, st));
     NA_TRY(launch_scene_idx(tri, T, V, tri4, cnt, st));
     NA_TRY(launch_scene_check(vtx, col4, V, &cnt->status, st));
-    int *binned = (int *)(arena + o_binned);
-    NA_TRY(launch_bound(dv, 1, tri_offs, T, rec, hp, tbox, cand, binned, cnt, st));
-    if (fov_bound != PR_FOV_SECTOR && (view->mode == PR_FOVEATED || view->mode == PR_BOTH))
+    NA_TRY(launch_bound(dv, 1, tri_offs, T, rec, hp, tbox, list, cnt, st));
+    if (paper_fov)
         NA_TRY(launch_paper_fov(dv, 1, tri_offs, T, rec, hp, tbox, cand, st));
-    NA_TRY(launch_scan(cand, cand_off, state_a, T, 0, cnt, st, true, binned, &cnt->binned));
-    NA_TRY(launch_bin_count(dv, 1, tri_offs, T, binned, cand_off, rec, hp, tbox, tile_box, tile_cnt, hit_entry,
-                            hit_tile, cap_pairs, cnt, st));
-    ItemsOut io;  // the scan of the tile counts also emits the work items
+    if (!list.shift)
+        NA_TRY(launch_cand_scan(list, state, T, cnt, st));
+    NA_TRY(launch_bin_count(dv, 1, tri_offs, T, list, rec, hp, tbox, tile_box, tile_cnt, hit_entry, hit_tile, cap_pairs,
+                            cnt, st));
+    ItemsOut io;
     io.views = dv;
     io.nviews = 1;
     io.tile_offs = tile_offs;
     io.items = items;
     io.cap_items = cap_items;
     io.cap_pairs = cap_pairs;
-    NA_TRY(launch_scan(tile_cnt, scan, state_b, nt, seg, cnt, st, true, nullptr, nullptr, &io));
-    NA_TRY(launch_bin_scatter(hit_entry, hit_tile, scan, fill, pairs, cap_pairs, nt, cnt, st));
-    NA_TRY(launch_sort_items(items, scan, nt, cap_items, seg, pairs, cnt, st));
-    NA_TRY(launch_fragment(tile, false, dv, items, scan, 0, nt, cap_items, heads, pairs, rec, keys, nullptr,
-                           nullptr, cnt, fragment_grid(tile, false), st));
+    io.ncls = 1;
+    io.cls_end[0] = nt;
+    NA_TRY(launch_tile_alloc(tile_cnt, scan, fill, nt, seg, cnt, io, st));
+    NA_TRY(launch_bin_scatter(hit_entry, hit_tile, fill, pairs, cap_pairs, nt, cnt, st));
+    NA_TRY(launch_sort_items(io, nt, seg, pairs, cnt, st));
+    NA_TRY(launch_fragment(tile, false, dv, io, 0, heads, pairs, rec, keys, nullptr, nullptr, cnt,
+                           fragment_grid(tile, false, nt, T, seg), st));
     NA_TRY(launch_resolve(dv, 1, pix_offs, np, keys, false, st));
     Counters h;
     NA_TRY(cudaMemcpyAsync(&h, cnt, sizeof h, cudaMemcpyDeviceToHost, st));

@@ -762,25 +762,27 @@ __device__ __forceinline__ void compute_bound(const ViewDev &v, const float3 S[3
 //   [3] D1.x D1.y D1.z D2.x   [4] xmin xmax ymin ymax   [5] tmin tmax D2.y D2.z
 // S = camera-space vertex at t = 0, D = its motion over the frame, the box
 // and interval of stage (a).  tbox = (i0 | i1 << 16, j0 | j1 << 16, nhp, depth order
-// key of the nearest depth the triangle reaches).  cand = candidate tiles of
-// the framebuffer box; the triangles that have some are also appended to
-// `binned` (cnt->binned of them), the index space of the binning pass.
+// key of the nearest depth the triangle reaches).  A triangle with candidate
+// tiles (tiles of its framebuffer box) is also appended to the list.  A
+// culled triangle leaves only its empty tbox: nothing downstream reads the
+// rest (its record alone would be 96 of the pass's 204 bytes).
 __global__ void __launch_bounds__(128, 6) k_bound(const ViewDev *__restrict__ views, int nviews,
                                                const long long *__restrict__ tri_offs, long long ttot,
                                                float4 *__restrict__ rec, float4 *__restrict__ hp,
-                                               int4 *__restrict__ tbox, unsigned long long *__restrict__ cand,
-                                               int *__restrict__ binned, Counters *cnt)
+                                               int4 *__restrict__ tbox, const CandList list, Counters *cnt)
 {
     const long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     // the view of the warp's first triangle by the whole warp (no chain of
     // dependent loads), then each lane steps to its own: a warp's 32
     // triangles meet at most a few view boundaries
-    const long long g0 = g - (threadIdx.x & 31);
+    const int lane = threadIdx.x & 31;
+    const long long g0 = g - lane;
     if (g0 >= ttot)
         return;  // the whole warp
     int q = find_view_warp(tri_offs, nviews, g0);
     if (g >= ttot)
         return;
+    const unsigned valid = ttot - g0 >= 32 ? 0xffffffffu : (1u << (int)(ttot - g0)) - 1u;  // the lanes that go on
     while (q + 1 < nviews && g >= tri_offs[q + 1])
         ++q;
     const ViewDev &v = views[q];
@@ -800,57 +802,85 @@ __global__ void __launch_bounds__(128, 6) k_bound(const ViewDev *__restrict__ vi
     if (bad) {
         B.culled = true;
         const unsigned bm = __activemask();
-        if ((threadIdx.x & 31) == __ffs(bm) - 1)
+        if (lane == __ffs(bm) - 1)
             atomicOr(&cnt->status, ST_NONFINITE);
     } else {
         compute_bound(v, S, D, B);
     }
-    float4 *r = rec + g * kRecF4;
-    r[0] = make_float4(S[0].x, S[0].y, S[0].z, S[1].x);
-    r[1] = make_float4(S[1].y, S[1].z, S[2].x, S[2].y);
-    r[2] = make_float4(S[2].z, D[0].x, D[0].y, D[0].z);
-    r[3] = make_float4(D[1].x, D[1].y, D[1].z, D[2].x);
+    unsigned ncand = 0u;  // candidate tiles (at most 2^22)
     if (B.culled) {
-        r[4] = make_float4(INFINITY, -INFINITY, INFINITY, -INFINITY);
-        r[5] = make_float4(INFINITY, -INFINITY, D[2].y, D[2].z);
         tbox[g] = make_int4(1, 1, 0, 0);  // the empty box [1, 0] x [1, 0]
-        cand[g] = 0ull;
-        const unsigned cm = __activemask();  // one atomic per warp
-        if ((threadIdx.x & 31) == __ffs(cm) - 1)
-            atomicAdd(&cnt->culled, (unsigned long long)__popc(cm));
-        return;
-    }
-    r[4] = make_float4(B.xmin, B.xmax, B.ymin, B.ymax);
-    r[5] = make_float4(B.tmin - kEpsT, B.tmax + kEpsT, D[2].y, D[2].z);
-    int nhp = 0;
+        if (!list.shift)
+            list.cand[g] = 0ull;
+    } else {
+        float4 *r = rec + g * kRecF4;
+        r[0] = make_float4(S[0].x, S[0].y, S[0].z, S[1].x);
+        r[1] = make_float4(S[1].y, S[1].z, S[2].x, S[2].y);
+        r[2] = make_float4(S[2].z, D[0].x, D[0].y, D[0].z);
+        r[3] = make_float4(D[1].x, D[1].y, D[1].z, D[2].x);
+        r[4] = make_float4(B.xmin, B.xmax, B.ymin, B.ymax);
+        r[5] = make_float4(B.tmin - kEpsT, B.tmax + kEpsT, D[2].y, D[2].z);
+        int nhp = 0;
 #pragma unroll
-    for (int h = 0; h < kMaxHp; ++h)
-        if (B.hmask & (1u << h))
-            hp[g * kMaxHp + nhp++] = B.hp[h];
-    // nearest camera depth the moving triangle reaches (z is linear in t on
-    // every vertex): min_k S_k.z + min(0, D_k.z), the sort key of its pairs
-    const float near = fminf(fminf(S[0].z + fminf(0.f, D[0].z), S[1].z + fminf(0.f, D[1].z)),
-                             S[2].z + fminf(0.f, D[2].z));
-    tbox[g] = make_int4(B.i0 | (B.i1 << 16), B.j0 | (B.j1 << 16), nhp, (int)depth_order_key(near));
-    cand[g] = (unsigned long long)(B.i1 / v.S - B.i0 / v.S + 1) * (unsigned long long)(B.j1 / v.S - B.j0 / v.S + 1);
+        for (int h = 0; h < kMaxHp; ++h)
+            if (B.hmask & (1u << h))
+                hp[g * kMaxHp + nhp++] = B.hp[h];
+        // nearest camera depth the moving triangle reaches (z is linear in t on
+        // every vertex): min_k S_k.z + min(0, D_k.z), the sort key of its pairs
+        const float near = fminf(fminf(S[0].z + fminf(0.f, D[0].z), S[1].z + fminf(0.f, D[1].z)),
+                                 S[2].z + fminf(0.f, D[2].z));
+        tbox[g] = make_int4(B.i0 | (B.i1 << 16), B.j0 | (B.j1 << 16), nhp, (int)depth_order_key(near));
+        const int sh = __ffs(v.S) - 1;  // S is a power of two
+        ncand = (unsigned)((B.i1 >> sh) - (B.i0 >> sh) + 1) * (unsigned)((B.j1 >> sh) - (B.j0 >> sh) + 1);
+        if (!list.shift)
+            list.cand[g] = ncand;
+    }
     // list the triangle for binning (one atomic per warp; the list order
     // does not matter: every bin is sorted by depth later)
-    const unsigned m = __activemask();
-    const int lane = threadIdx.x & 31, leader = __ffs(m) - 1;
+    const unsigned m = __ballot_sync(valid, ncand != 0u);
+    if (!m)
+        return;
+    const int leader = __ffs(m) - 1;
+    unsigned inc = ncand;  // candidates up to this lane (32 x 2^22 at most)
+    if (list.shift) {
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned y = __shfl_up_sync(valid, inc, o);
+            if (lane >= o)
+                inc += y;
+        }
+    }
+    const unsigned total = __shfl_sync(valid, inc, 31 - __clz(valid));
     unsigned long long base = 0;
     if (lane == leader)
-        base = atomicAdd(&cnt->binned, (unsigned long long)__popc(m));
-    base = __shfl_sync(m, base, leader);
-    binned[base + __popc(m & ((1u << lane) - 1u))] = (int)g;
+        base = list.shift ? atomicAdd(&cnt->binned_cand,
+                                      ((unsigned long long)total << list.shift) | (unsigned long long)__popc(m))
+                          : atomicAdd(&cnt->binned, (unsigned long long)__popc(m));
+    base = __shfl_sync(valid, base, leader);
+    if (ncand) {
+        const unsigned long long place =
+            (list.shift ? base & ((1ull << list.shift) - 1ull) : base) + __popc(m & ((1u << lane) - 1u));
+        list.binned[place] = (int)g;
+        if (list.shift)
+            list.off[place] = (base >> list.shift) + (inc - ncand);
+    }
 }
 
 cudaError_t launch_bound(const ViewDev *views, int nviews, const long long *tri_offs, long long ttot, float4 *rec,
-                         float4 *hp, int4 *tbox, unsigned long long *cand, int *binned, Counters *cnt, cudaStream_t st)
+                         float4 *hp, int4 *tbox, const CandList &list, Counters *cnt, cudaStream_t st)
 {
     if (ttot > 0)
-        k_bound<<<(unsigned)((ttot + 127) / 128), 128, 0, st>>>(views, nviews, tri_offs, ttot, rec, hp, tbox, cand,
-                                                                binned, cnt);
+        k_bound<<<(unsigned)((ttot + 127) / 128), 128, 0, st>>>(views, nviews, tri_offs, ttot, rec, hp, tbox, list,
+                                                                cnt);
     return cudaGetLastError();
+}
+
+int cand_shift(long long ttot, double max_cand)
+{
+    int sh = 1;  // bits of the triangle count (ttot itself included)
+    while ((1ll << sh) <= ttot)
+        ++sh;
+    return max_cand < (double)(1ull << (63 - sh)) ? sh : 0;
 }
 
 // The paper's foveation edge bounds (pr_fov_bound SIMPLE / RECURSIVE), as
@@ -866,7 +896,7 @@ __global__ void __launch_bounds__(128) k_paper_fov(const ViewDev *__restrict__ v
 {
     const long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (g >= ttot || cand[g] == 0ull)
-        return;
+        return;  // culled: it has no record
     const ViewDev &v = views[find_view(tri_offs, nviews, g)];
     if (!is_foveated(v.mode) || v.fov_bound == PR_FOV_SECTOR)
         return;
@@ -931,7 +961,7 @@ __device__ __forceinline__ bool tile_meets(const float4 tb, const float4 bb, con
 
 // Bins.  Every triangle's framebuffer box spans a rectangle of candidate
 // tiles.  The triangles that have candidates are listed in `binned` (by the
-// bound pass, m of them) and cand_off is the prefix sum of their counts, so
+// bound pass, m of them) and cand_off is the running sum of their counts, so
 // candidate pair p belongs to list entry e with cand_off[e] <= p <
 // cand_off[e+1].  Warps take the pairs in tasks of consecutive pairs, which
 // keeps the work balanced when a few triangles -- near the fovea, where
@@ -990,28 +1020,38 @@ constexpr int kBinChunks = 8;
 // grid-stride, so CTAs that start late take the place of those whose tasks
 // ran short, which evens out the end of the pass.
 __global__ void __launch_bounds__(256, 4) k_bin(const ViewDev *__restrict__ views, int nviews,
-                                             const long long *__restrict__ tri_offs, const int *__restrict__ binned,
-                                             const unsigned long long *__restrict__ cand_off,
-                                             const float4 *__restrict__ rec, const float4 *__restrict__ hp,
-                                             const int4 *__restrict__ tbox, const float4 *__restrict__ tile_box,
+                                             const long long *__restrict__ tri_offs, long long ttot,
+                                             const CandList list, const float4 *__restrict__ rec,
+                                             const float4 *__restrict__ hp, const int4 *__restrict__ tbox,
+                                             const float4 *__restrict__ tile_box,
                                              unsigned long long *__restrict__ tile_cnt,
                                              unsigned long long *__restrict__ hit_entry,
-                                             unsigned *__restrict__ hit_tile, long long cap_pairs, Counters *cnt)
+                                             unsigned *__restrict__ hit_tile, long long cap_pairs, int resident,
+                                             Counters *cnt)
 {
-    const long long m = (long long)cnt->binned;
+    const long long m = (long long)list.length(cnt);
+    const unsigned long long *__restrict__ cand_off = list.off;
+    const int *__restrict__ binned = list.binned;
+    if (blockIdx.x == 0 && threadIdx.x == 0)
+        cnt->culled = (unsigned long long)(ttot - m);
     if (m == 0)
         return;
-    const long long total = (long long)cand_off[m];
+    const long long total = (long long)(list.shift ? cnt->binned_cand >> list.shift : cand_off[m]);
     const int lane = threadIdx.x & 31;
     const long long nwarps = (long long)gridDim.x * (blockDim.x >> 5);
-    // Each warp takes tasks of kBinChunks x 32 consecutive candidate pairs.
-    // The list entry of the task's first pair comes from a warp-wide 32-ary
-    // search; the entries of each chunk's pairs then follow from the offsets
-    // of the next 32 entries, loaded with one coalesced read and searched
-    // with shuffles (every entry owns at least one pair, so 32 pairs never
-    // reach past them).  All lanes run the same iterations (for the shuffles).
-    for (long long pt = ((long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * (32 * kBinChunks);
-         pt < total; pt += nwarps * (32 * kBinChunks)) {
+    // Each warp takes tasks of nch x 32 consecutive candidate pairs, up to
+    // kBinChunks x 32 where there are enough of them: a task's chunks run one
+    // after the other, each a chain of dependent loads, so a frame with few
+    // pairs spreads them over more of the resident warps (512^2, 10k
+    // triangles: 7 us, 20.7 us with eight chunks always).  The list entry of the task's first pair comes
+    // from a warp-wide 32-ary search; the entries of each chunk's pairs then
+    // follow from the offsets of the next 32 entries, loaded with one
+    // coalesced read and searched with shuffles (every entry owns at least
+    // one pair, so 32 pairs never reach past them).  All lanes run the same
+    // iterations (for the shuffles).
+    const int nch = (int)min((long long)kBinChunks, (total + 32ll * resident - 1) / (32ll * resident));
+    for (long long pt = ((long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * (32 * nch); pt < total;
+         pt += nwarps * (32 * nch)) {
         long long e0 = warp_owner(cand_off, m, pt);
         // the task's hits: per chunk the ballot, the lane's entry and tile
         unsigned want_c[kBinChunks];
@@ -1023,11 +1063,11 @@ __global__ void __launch_bounds__(256, 4) k_bin(const ViewDev *__restrict__ view
             ent_c[c] = 0ull;
             tile_c[c] = 0u;
             const long long pw = pt + 32 * c;
-            if (pw >= total)
+            if (c >= nch || pw >= total)
                 continue;  // warp-uniform
             const long long p = pw + lane;
             const long long el = e0 + 1 + lane;
-            const unsigned long long o = el <= m ? cand_off[el] : ~0ull;
+            const unsigned long long o = el < m ? cand_off[el] : (el == m ? (unsigned long long)total : ~0ull);
             // every lane takes part in every shuffle; the fallback search
             // (no warp operations) runs after them
             int k = 0;  // offsets of the window at or below p
@@ -1064,7 +1104,7 @@ __global__ void __launch_bounds__(256, 4) k_bin(const ViewDev *__restrict__ view
                 }
                 const float4 bb = rec[g * kRecF4 + 4];
                 const bool fbspace = (tb.z & 0x100) != 0;
-                const int nh = cand_off[e + 1] - off > 1 ? (tb.z & 0xff) : 0;
+                const int nh = w > 1 || (tb.y >> 16) >> sh != ty0 ? (tb.z & 0xff) : 0;  // more than one candidate
                 if (!ok_tile) {
                     hit = false;
                 } else if (!fbspace) {
@@ -1119,12 +1159,11 @@ __global__ void __launch_bounds__(256, 4) k_bin(const ViewDev *__restrict__ view
     }
 }
 
-// Moves the listed hits into their tile bins (after the scan of the tile
-// counts): entry k goes to scan[tile] + its rank among the tile's entries.
+// Moves the listed hits into their tile bins (after the tiles got their
+// places): the next free entry of the tile's bin, from its cursor.
 __global__ void __launch_bounds__(256) k_bin_scatter(const unsigned long long *__restrict__ hit_entry,
                                                      const unsigned *__restrict__ hit_tile,
-                                                     const unsigned long long *__restrict__ scan,
-                                                     unsigned int *__restrict__ fill,
+                                                     unsigned int *__restrict__ cursor,
                                                      unsigned long long *__restrict__ pairs, long long cap_pairs,
                                                      long long ntiles, Counters *cnt)
 {
@@ -1142,21 +1181,123 @@ __global__ void __launch_bounds__(256) k_bin_scatter(const unsigned long long *_
         const unsigned want = __ballot_sync(0xffffffffu, ok);
         if (!ok)
             continue;
-        // the bin start and the entry load while the cursor atomic runs
-        const unsigned long long first = scan[tile] & 0xFFFFFFFFFFull;
+        // the entry loads while the cursor atomic runs
         const unsigned long long ent = hit_entry[k];
         const unsigned peers = __match_any_sync(want, tile);
         const int leader = __ffs(peers) - 1;
         unsigned base = 0;
         if (lane == leader)
-            base = atomicAdd(&fill[tile], (unsigned)__popc(peers));
+            base = atomicAdd(&cursor[tile], (unsigned)__popc(peers));
         base = __shfl_sync(peers, base, leader);
-        const long long pos = (long long)first + base + __popc(peers & ((1u << lane) - 1u));
+        const long long pos = (long long)base + __popc(peers & ((1u << lane) - 1u));
         if (pos < cap_pairs)
             pairs[pos] = ent;
         else
             atomicOr(&cnt->status, ST_OVERFLOW_PAIRS);
     }
+}
+
+// Places in the bins.  Bins need no order among the tiles, so a CTA of 256
+// tiles takes its stretch of the bin buffer and of each class's work items
+// with one atomic each, instead of a scan over all tiles (stereo HMD frame,
+// 18,000 tiles: the scan's five CTAs with eight tiles per thread and a chain
+// of look-backs took 12-13 us).  Each tile's bin is cut into runs of at most
+// seg triangles, item = (view, tile in view, first entry, end entry).  Runs
+// past the bin buffer (its scatter overflowed) are clamped to it, so the
+// frame stays in bounds; the overflow status reruns it.
+constexpr int kAllocThreads = 256;
+__global__ void __launch_bounds__(kAllocThreads) k_tile_alloc(const unsigned long long *__restrict__ tile_cnt,
+                                                              unsigned long long *__restrict__ off_out,
+                                                              unsigned *__restrict__ cursor, long long ntiles,
+                                                              int seg, Counters *cnt, const ItemsOut io)
+{
+    __shared__ unsigned long long s_n[kAllocThreads / 32];
+    __shared__ unsigned s_it[kMaxClasses][kAllocThreads / 32];
+    __shared__ unsigned long long s_pairs;              // the CTA's first bin entry
+    __shared__ unsigned long long s_items[kMaxClasses];  // its first item of each class
+    const long long g = (long long)blockIdx.x * kAllocThreads + threadIdx.x;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const unsigned long long n = g < ntiles ? tile_cnt[g] : 0ull;
+    // a 32-bit division where the count allows it
+    const unsigned nit = n <= 0x7FFFFFFFull ? ((unsigned)n + (unsigned)seg - 1u) / (unsigned)seg
+                                            : (unsigned)((n + seg - 1) / seg);
+    const int cls = (io.ncls > 1 && g >= io.cls_end[0]) + (io.ncls > 2 && g >= io.cls_end[1]);
+    unsigned long long inc = n;  // entries and items (of its class) up to this lane
+    unsigned iit[kMaxClasses];
+#pragma unroll
+    for (int c = 0; c < kMaxClasses; ++c)
+        iit[c] = cls == c ? nit : 0u;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned long long y = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o)
+            inc += y;
+#pragma unroll
+        for (int c = 0; c < kMaxClasses; ++c) {
+            if (c >= io.ncls)
+                break;
+            const unsigned z = __shfl_up_sync(0xffffffffu, iit[c], o);
+            if (lane >= o)
+                iit[c] += z;
+        }
+    }
+    if (lane == 31) {
+        s_n[w] = inc;
+#pragma unroll
+        for (int c = 0; c < kMaxClasses; ++c)
+            s_it[c][w] = iit[c];
+    }
+    __syncthreads();
+    if (threadIdx.x <= kMaxClasses) {  // thread 0: the entries, thread 1 + c: the items of class c
+        unsigned long long sum = 0;
+#pragma unroll
+        for (int k = 0; k < kAllocThreads / 32; ++k)
+            sum += threadIdx.x == 0 ? s_n[k] : (unsigned long long)s_it[threadIdx.x - 1][k];
+        unsigned long long base = 0;
+        if (sum)
+            base = atomicAdd(threadIdx.x == 0 ? &cnt->pairs_total : &cnt->items_n[threadIdx.x - 1], sum);
+        if (threadIdx.x == 0)
+            s_pairs = base;
+        else
+            s_items[threadIdx.x - 1] = base;
+    }
+    __syncthreads();
+    if (g >= ntiles)
+        return;
+    long long off = (long long)(s_pairs + inc - n);
+    long long ioff = (long long)s_items[cls] - nit;
+#pragma unroll
+    for (int c = 0; c < kMaxClasses; ++c)
+        if (cls == c)
+            ioff += iit[c];
+    for (int k = 0; k < w; ++k) {
+        off += (long long)s_n[k];
+        ioff += s_it[cls][k];
+    }
+    off_out[g] = (unsigned long long)off;
+    cursor[g] = (unsigned)off;
+    if (n == 0)
+        return;
+    const int vi = find_view(io.tile_offs, io.nviews, g);
+    const int lt = (int)(g - io.views[vi].tile_off);
+    int4 *items = io.items + (long long)cls * io.cap_items;
+    for (unsigned q = 0; q < nit; ++q) {
+        const long long b0 = min(off + (long long)q * seg, io.cap_pairs),
+                        b1 = min(off + min((long long)n, ((long long)q + 1) * seg), io.cap_pairs);
+        if (ioff + q < io.cap_items)
+            items[ioff + q] = make_int4(vi, lt, (int)b0, (int)b1);
+        else
+            atomicOr(&cnt->status, ST_OVERFLOW_ITEMS);
+    }
+}
+
+cudaError_t launch_tile_alloc(const unsigned long long *tile_cnt, unsigned long long *off, unsigned *cursor,
+                              long long ntiles, int seg, Counters *cnt, const ItemsOut &io, cudaStream_t st)
+{
+    if (ntiles > 0)
+        k_tile_alloc<<<(unsigned)((ntiles + kAllocThreads - 1) / kAllocThreads), kAllocThreads, 0, st>>>(
+            tile_cnt, off, cursor, ntiles, seg, cnt, io);
+    return cudaGetLastError();
 }
 
 static int sm_count()
@@ -1176,42 +1317,46 @@ static int bin_grid() { return sm_count() * 8; }
 
 // k_bin: four waves of its four resident CTAs per SM (more waves measured
 // the same, fewer slower; the binning stage of the 64-view workload took
-// 0.43 ms with 2.7 waves of 3 CTAs per SM at 75 registers, 0.375 ms so)
-static int bin_count_grid() { return sm_count() * 16; }
+// 0.43 ms with 2.7 waves of 3 CTAs per SM at 75 registers, 0.375 ms so), or
+// one wave for a frame of few triangles
+static int bin_count_grid(long long ttot)
+{
+    return (int)std::min<long long>(sm_count() * 16, std::max<long long>(sm_count() * 4, ttot / 32));
+}
 
 cudaError_t launch_bin_count(const ViewDev *views, int nviews, const long long *tri_offs, long long ttot,
-                             const int *binned, const unsigned long long *cand_off, const float4 *rec,
-                             const float4 *hp, const int4 *tbox, const float4 *tile_box, unsigned long long *tile_cnt,
-                             unsigned long long *hit_entry, unsigned *hit_tile, long long cap_pairs, Counters *cnt,
-                             cudaStream_t st)
+                             const CandList &list, const float4 *rec, const float4 *hp, const int4 *tbox,
+                             const float4 *tile_box, unsigned long long *tile_cnt, unsigned long long *hit_entry,
+                             unsigned *hit_tile, long long cap_pairs, Counters *cnt, cudaStream_t st)
 {
     if (ttot > 0)
-        k_bin<<<bin_count_grid(), 256, 0, st>>>(views, nviews, tri_offs, binned, cand_off, rec, hp, tbox,
-                                                tile_box, tile_cnt, hit_entry, hit_tile, cap_pairs, cnt);
+        k_bin<<<bin_count_grid(ttot), 256, 0, st>>>(views, nviews, tri_offs, ttot, list, rec, hp, tbox, tile_box,
+                                                    tile_cnt, hit_entry, hit_tile, cap_pairs, sm_count() * 32, cnt);
     return cudaGetLastError();
 }
 
-cudaError_t launch_bin_scatter(const unsigned long long *hit_entry, const unsigned *hit_tile,
-                               const unsigned long long *scan, unsigned int *fill, unsigned long long *pairs,
-                               long long cap_pairs, long long ntiles, Counters *cnt, cudaStream_t st)
+cudaError_t launch_bin_scatter(const unsigned long long *hit_entry, const unsigned *hit_tile, unsigned *cursor,
+                               unsigned long long *pairs, long long cap_pairs, long long ntiles, Counters *cnt,
+                               cudaStream_t st)
 {
-    k_bin_scatter<<<bin_grid(), 256, 0, st>>>(hit_entry, hit_tile, scan, fill, pairs, cap_pairs, ntiles, cnt);
+    const int grid = (int)std::min<long long>(bin_grid(), (cap_pairs + 255) / 256);
+    k_bin_scatter<<<grid, 256, 0, st>>>(hit_entry, hit_tile, cursor, pairs, cap_pairs, ntiles, cnt);
     return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------- frame init
 
 // The start of a frame, in one launch: clears what the frame accumulates
-// into -- the counters, the work-queue heads, the per-tile counts and fill
-// cursors, the tickets and flags of two scans' look-back state
-// (scan_state_words of each), the FP64 flag bitmap (nflag words, may be 0)
-// -- sets every pixel's depth|id key to "no hit" (~0), and computes every
-// tile's display box (stage a: the image of its pixel centres under q).
+// into -- the counters, the work-queue heads, the per-tile counts, the
+// ticket and flags of the candidate scan's look-back state (nstate words,
+// may be 0), the FP64 flag bitmap (nflag words, may be 0) -- sets every
+// pixel's depth|id key to "no hit" (~0), and computes every tile's display
+// box (stage a: the image of its pixel centres under q).
 __global__ void k_frame_init(const ViewDev *__restrict__ views, int nviews, const long long *__restrict__ tile_offs,
                              float4 *__restrict__ tile_box, Counters *cnt, int *heads, unsigned long long *tile_cnt,
-                             unsigned *fill, long long ntiles, unsigned long long *state_a, long long nstate_a,
-                             unsigned long long *state_b, long long nstate_b, unsigned *flag_bits, long long nflag,
-                             unsigned long long *keys, long long npix, float *loss_part, long long nloss)
+                             long long ntiles, unsigned long long *state, long long nstate, unsigned *flag_bits,
+                             long long nflag, unsigned long long *keys, long long npix, float *loss_part,
+                             long long nloss)
 {
     const long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const long long stride = (long long)gridDim.x * blockDim.x;
@@ -1221,13 +1366,10 @@ __global__ void k_frame_init(const ViewDev *__restrict__ views, int nviews, cons
         heads[g] = 0;
     for (long long k = g; k < ntiles; k += stride) {
         tile_cnt[k] = 0ull;
-        fill[k] = 0u;
         tile_box[k] = tile_display_box(views, nviews, tile_offs, k);
     }
-    for (long long k = g; k < nstate_a; k += stride)
-        state_a[k] = 0ull;
-    for (long long k = g; k < nstate_b; k += stride)
-        state_b[k] = 0ull;
+    for (long long k = g; k < nstate; k += stride)
+        state[k] = 0ull;
     for (long long k = g; k < nflag; k += stride)
         flag_bits[k] = 0u;
     for (long long k = g; k < nloss; k += stride)
@@ -1241,20 +1383,16 @@ __global__ void k_frame_init(const ViewDev *__restrict__ views, int nviews, cons
 }
 
 cudaError_t launch_frame_init(const ViewDev *views, int nviews, const long long *tile_offs, float4 *tile_box,
-                              Counters *cnt, int *heads, unsigned long long *tile_cnt, unsigned *fill, long long ntiles,
-                              unsigned long long *state_a, long long nstate_a, unsigned long long *state_b,
-                              long long nstate_b, unsigned *flag_bits, long long nflag, unsigned long long *keys,
-                              long long npix, float *loss_part, long long nloss, cudaStream_t st)
+                              Counters *cnt, int *heads, unsigned long long *tile_cnt, long long ntiles,
+                              unsigned long long *state, long long nstate, unsigned *flag_bits, long long nflag,
+                              unsigned long long *keys, long long npix, float *loss_part, long long nloss,
+                              cudaStream_t st)
 {
-    static int grid = 0;
-    if (grid == 0) {
-        int dev = 0, sms = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        grid = sms * 8;
-    }
-    k_frame_init<<<grid, 256, 0, st>>>(views, nviews, tile_offs, tile_box, cnt, heads, tile_cnt, fill, ntiles, state_a,
-                                       nstate_a, state_b, nstate_b, flag_bits, nflag, keys, npix, loss_part, nloss);
+    // eight CTAs per SM, or as many as the longest of the loops has work for
+    const long long most = std::max(std::max(std::max(ntiles, nstate), std::max(nflag, nloss)), npix / 2);
+    const int grid = (int)std::min<long long>(sm_count() * 8, std::max<long long>(1, (most + 255) / 256));
+    k_frame_init<<<grid, 256, 0, st>>>(views, nviews, tile_offs, tile_box, cnt, heads, tile_cnt, ntiles, state, nstate,
+                                       flag_bits, nflag, keys, npix, loss_part, nloss);
     return cudaGetLastError();
 }
 
@@ -1266,23 +1404,11 @@ cudaError_t launch_frame_init(const ViewDev *views, int nviews, const long long 
 // 32 at a time, polling their flags -- until it meets a tile whose
 // inclusive prefix is published.  Tiles are numbered by an atomic ticket,
 // so every tile waited on belongs to a CTA that started earlier; each poll
-// is bounded (ST_TIMEOUT if it runs out).  With seg > 0 each input word is
-// first packed as low 40 bits = bin entries, high 24 bits = work items
-// (ceil(entries / seg)).  out[n] = the grand total.
+// is bounded (ST_TIMEOUT if it runs out).  out[n] = the grand total.  Used
+// for the candidate offsets when CandList::shift is 0.
 constexpr int kScanThreads = 512, kScanPer = 8, kScanBlock = kScanThreads * kScanPer;
 constexpr unsigned long long kFlagAgg = 1ull, kFlagPre = 2ull;
 constexpr int kScanSpinLimit = 1 << 22;
-
-__device__ __forceinline__ unsigned long long pack_items(unsigned long long c, int seg)
-{
-    const unsigned long long n = c & 0xFFFFFFFFFFull;
-    // a 32-bit division where the count allows it (a 64-bit one is a long
-    // instruction sequence)
-    const unsigned long long items = n <= 0x7FFFFFFFull
-                                         ? (unsigned long long)(((unsigned)n + (unsigned)seg - 1u) / (unsigned)seg)
-                                         : (n + seg - 1) / seg;
-    return n | (items << 40);
-}
 
 __device__ unsigned long long block_exclusive_scan(unsigned long long x, unsigned long long *total)
 {
@@ -1326,36 +1452,12 @@ __device__ __forceinline__ void store_volatile(unsigned long long *p, unsigned l
 // inclusive prefixes; the ticket and flags start at zero.  gather: element
 // i is in[gather[i]] (else in[i]).  n_dev: the element count is
 // min(*n_dev, n), known on the device only; tiles past it leave at once.
-// Emits the work items of tile g from its bin count n and its exclusive
-// prefix (bin entries, low 40 bits; work items, high 24): the bin cut into
-// runs of at most seg triangles, item = (view, tile in view, first entry,
-// end entry).  Runs past the bin buffer (its scatter overflowed) are clamped
-// to it, so the frame stays in bounds; the overflow status reruns it.
-__device__ __forceinline__ void emit_items(const ItemsOut &io, long long g, long long n, unsigned long long pre,
-                                           int seg, Counters *cnt)
-{
-    if (n == 0)
-        return;
-    const int vi = find_view(io.tile_offs, io.nviews, g);
-    const long long lt = g - io.views[vi].tile_off;
-    const long long off = (long long)(pre & 0xFFFFFFFFFFull), ioff = (long long)(pre >> 40);
-    const long long nit = (n + seg - 1) / seg;
-    for (long long q = 0; q < nit; ++q) {
-        const long long b0 = min(off + q * seg, io.cap_pairs), b1 = min(off + min(n, (q + 1) * seg), io.cap_pairs);
-        if (ioff + q < io.cap_items)
-            io.items[ioff + q] = make_int4(vi, (int)lt, (int)b0, (int)b1);
-        else
-            atomicOr(&cnt->status, ST_OVERFLOW_ITEMS);
-    }
-}
-
-template <bool kItems>
 __global__ void __launch_bounds__(kScanThreads) k_scan(const unsigned long long *__restrict__ in,
                                                       const int *__restrict__ gather,
                                                       const unsigned long long *__restrict__ n_dev,
-                                                      unsigned long long *__restrict__ out, long long n, int seg,
+                                                      unsigned long long *__restrict__ out, long long n,
                                                       unsigned long long *state, long long nb, Counters *cnt,
-                                                      ItemsOut io, int spin_limit)
+                                                      int spin_limit)
 {
     unsigned long long *flags = state + 1, *agg = state + 1 + nb, *inc = state + 1 + 2 * nb;
     __shared__ long long s_tile;
@@ -1378,8 +1480,8 @@ __global__ void __launch_bounds__(kScanThreads) k_scan(const unsigned long long 
         unsigned long long x = 0ull;
         if (base + k < n)
             x = in[gather ? (long long)gather[base + k] : base + k];
-        v[k] = seg > 0 ? pack_items(x, seg) : x;
-        sum += v[k];
+        v[k] = x;
+        sum += x;
     }
     unsigned long long total;
     unsigned long long run = block_exclusive_scan(sum, &total);
@@ -1444,20 +1546,13 @@ __global__ void __launch_bounds__(kScanThreads) k_scan(const unsigned long long 
     for (int k = 0; k < kScanPer; ++k) {
         if (base + k < n) {
             out[base + k] = excl + run;
-            if (kItems)
-                emit_items(io, base + k, (long long)(v[k] & 0xFFFFFFFFFFull), excl + run, seg, cnt);
         }
         run += v[k];
     }
     const bool holds_end =
         (n >= tile * kScanBlock && n < (tile + 1) * kScanBlock) || (tile == nb - 1 && n == nb * kScanBlock);
-    if (threadIdx.x == 0 && holds_end) {
+    if (threadIdx.x == 0 && holds_end)
         out[n] = excl + total;
-        if (kItems) {
-            cnt->pairs_total = (excl + total) & 0xFFFFFFFFFFull;
-            cnt->items_total = (excl + total) >> 40;
-        }
-    }
 }
 
 long long scan_state_words(long long n)
@@ -1471,26 +1566,14 @@ size_t scan_block_sums_needed(long long n)
     return (size_t)(3 * nb + 2);
 }
 
-cudaError_t launch_scan(const unsigned long long *in, unsigned long long *out, unsigned long long *state, long long n,
-                        int seg, Counters *cnt, cudaStream_t st, bool state_zeroed, const int *gather,
-                        const unsigned long long *n_dev, const ItemsOut *items)
+cudaError_t launch_cand_scan(const CandList &list, unsigned long long *state, long long ttot, Counters *cnt,
+                             cudaStream_t st)
 {
-    const long long nb = (n + kScanBlock - 1) / kScanBlock;
-    if (nb == 0) {
-        cudaMemsetAsync(out, 0, sizeof(unsigned long long), st);
-        return cudaGetLastError();
-    }
-    if (!state_zeroed) {
-        cudaError_t e = cudaMemsetAsync(state, 0, sizeof(unsigned long long) * (nb + 1), st);
-        if (e != cudaSuccess)
-            return e;
-    }
-    if (items && seg > 0)
-        k_scan<true><<<(unsigned)nb, kScanThreads, 0, st>>>(in, gather, n_dev, out, n, seg, state, nb, cnt, *items,
-                                                            kScanSpinLimit);
-    else
-        k_scan<false><<<(unsigned)nb, kScanThreads, 0, st>>>(in, gather, n_dev, out, n, seg, state, nb, cnt,
-                                                             ItemsOut{}, kScanSpinLimit);
+    const long long nb = (ttot + kScanBlock - 1) / kScanBlock;
+    if (nb == 0)
+        return cudaMemsetAsync(list.off, 0, sizeof(unsigned long long), st);
+    k_scan<<<(unsigned)nb, kScanThreads, 0, st>>>(list.cand, list.binned, &cnt->binned, list.off, ttot, state, nb, cnt,
+                                                  kScanSpinLimit);
     return cudaGetLastError();
 }
 
@@ -1523,8 +1606,7 @@ cudaError_t scan_timeout_probe(cudaStream_t st, unsigned *status)
         e = cudaMemcpyAsync(state, &one, sizeof one, cudaMemcpyHostToDevice, st);
     }
     if (e == cudaSuccess) {
-        k_scan<false><<<1, kScanThreads, 0, st>>>(in, nullptr, nullptr, out, n, 0, state, nb, cnt, ItemsOut{},
-                                                  1 << 12);
+        k_scan<<<1, kScanThreads, 0, st>>>(in, nullptr, nullptr, out, n, state, nb, cnt, 1 << 12);
         e = cudaGetLastError();
     }
     Counters h{};
@@ -1617,8 +1699,7 @@ __device__ __forceinline__ void sort_run_regs(unsigned long long *e, int n, int 
 
 template <bool kLong>
 __global__ void __launch_bounds__(kSortWarps * 32) k_sort_items(const int4 *__restrict__ items,
-                                                                const unsigned long long *__restrict__ scan,
-                                                                long long ntiles, long long cap_items,
+                                                                long long cap_items,
                                                                 unsigned long long *__restrict__ pairs,
                                                                 const Counters *__restrict__ cnt)
 {
@@ -1626,12 +1707,15 @@ __global__ void __launch_bounds__(kSortWarps * 32) k_sort_items(const int4 *__re
         return;  // an overflowed attempt (rerun) or a scan that gave up its wait (an error): bins incomplete
     __shared__ unsigned s_gid[kSortWarps][kSortRegMax];
     __shared__ unsigned long long s_run[kSortWarps][kLong ? kMaxSeg : 1];
-    const long long nitems = min((long long)(scan[ntiles] >> 40), cap_items);
+    // the classes' items one after the other
+    const long long n0 = min((long long)cnt->items_n[0], cap_items), n1 = min((long long)cnt->items_n[1], cap_items),
+                    n2 = min((long long)cnt->items_n[2], cap_items);
+    const long long nitems = n0 + n1 + n2;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     unsigned long long *run = s_run[w];
     const long long nwarps = (long long)gridDim.x * kSortWarps;
     for (long long it = (long long)blockIdx.x * kSortWarps + w; it < nitems; it += nwarps) {
-        const int4 item = items[it];
+        const int4 item = items[it < n0 ? it : (it < n0 + n1 ? it - n0 + cap_items : it - n0 - n1 + 2 * cap_items)];
         const int n = item.w - item.z;
         unsigned long long *e = pairs + item.z;
         if (n <= 1)
@@ -1678,18 +1762,19 @@ __global__ void __launch_bounds__(kSortWarps * 32) k_sort_items(const int4 *__re
     }
 }
 
-cudaError_t launch_sort_items(const int4 *items, const unsigned long long *scan, long long ntiles, long long cap_items,
-                              int seg, unsigned long long *pairs, const Counters *cnt, cudaStream_t st)
+cudaError_t launch_sort_items(const ItemsOut &io, long long ntiles, int seg, unsigned long long *pairs,
+                              const Counters *cnt, cudaStream_t st)
 {
     // 32 CTAs of four warps per SM, about three waves: the warps take the
     // items grid-stride, and runs of very different lengths even out when
     // late CTAs fill the slots of early ones (the 64-view workload's binning
-    // stage 0.371 -> 0.365 ms against 8 CTAs per SM)
-    const int grid = sm_count() * 32;
+    // stage 0.371 -> 0.365 ms against 8 CTAs per SM); fewer for a frame whose
+    // tiles (mostly one item each) would not fill them
+    const int grid = (int)std::min<long long>(sm_count() * 32, std::max<long long>(sm_count(), ntiles / kSortWarps));
     if (seg > kSortRegMax)
-        k_sort_items<true><<<grid, kSortWarps * 32, 0, st>>>(items, scan, ntiles, cap_items, pairs, cnt);
+        k_sort_items<true><<<grid, kSortWarps * 32, 0, st>>>(io.items, io.cap_items, pairs, cnt);
     else
-        k_sort_items<false><<<grid, kSortWarps * 32, 0, st>>>(items, scan, ntiles, cap_items, pairs, cnt);
+        k_sort_items<false><<<grid, kSortWarps * 32, 0, st>>>(io.items, io.cap_items, pairs, cnt);
     return cudaGetLastError();
 }
 

@@ -13,6 +13,8 @@
 // watertight test for the survivors, each lane for its two pixels.  Per
 // pixel the nearest key is kept in a register and merged into the frame
 // with one 64-bit atomicMin per item.
+#include <algorithm>
+
 #include "pr_launch.h"
 
 namespace pr {
@@ -174,8 +176,8 @@ constexpr int kStageF4 = 5;
 template <int S, bool kFlag>
 __global__ void __launch_bounds__(S *S / 2, PR_FRAG_MINB(S *S / 2))
     k_fragment(const ViewDev *__restrict__ views, const int4 *__restrict__ items,
-               const unsigned long long *__restrict__ scan, long long tile_lo, long long tile_hi, long long cap_items,
-               int *__restrict__ head, const unsigned long long *__restrict__ pairs, const float4 *__restrict__ rec,
+               const unsigned long long *__restrict__ nitems, long long cap_items, int *__restrict__ head,
+               const unsigned long long *__restrict__ pairs, const float4 *__restrict__ rec,
                unsigned long long *__restrict__ keys, unsigned *__restrict__ flag_bits,
                long long *__restrict__ flag_list, Counters *cnt)
 {
@@ -193,20 +195,19 @@ __global__ void __launch_bounds__(S *S / 2, PR_FRAG_MINB(S *S / 2))
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int ci = (warp % WPR) * 8 + (lane & 7);
     const int cj0 = (warp / WPR) * 8 + (lane >> 3), cj1 = cj0 + 4;
-    const long long it_lo = (long long)(scan[tile_lo] >> 40);
-    const long long it_hi = min((long long)(scan[tile_hi] >> 40), cap_items);
+    const long long it_hi = min((long long)*nitems, cap_items);
     float4 *wrec = s_rec[warp];
     unsigned long long n_tests = 0, n_hits = 0;
 
     if (threadIdx.x == 0)
-        s_item[0] = it_lo + atomicAdd(head, 1);
+        s_item[0] = atomicAdd(head, 1);
     __syncthreads();
     for (int par = 0;; par ^= 1) {
         const long long it = s_item[par];
         if (it >= it_hi)
             break;
         if (threadIdx.x == 0)  // the next item, fetched while this one runs
-            s_item[par ^ 1] = it_lo + atomicAdd(head, 1);
+            s_item[par ^ 1] = atomicAdd(head, 1);
         const int4 item = items[it];
         const ViewDev &v = views[item.x];
         const int tx = item.y % v.tiles_x, ty = item.y / v.tiles_x;
@@ -339,32 +340,35 @@ static int grid_for()
     return g;
 }
 
-int fragment_grid(int S, bool flag)
+int fragment_grid(int S, bool flag, long long ntiles, long long ttot, int seg)
 {
-    if (flag)
-        return S == 8 ? grid_for<8, true>() : (S == 16 ? grid_for<16, true>() : grid_for<32, true>());
-    return S == 8 ? grid_for<8, false>() : (S == 16 ? grid_for<16, false>() : grid_for<32, false>());
+    const int g = flag ? (S == 8 ? grid_for<8, true>() : (S == 16 ? grid_for<16, true>() : grid_for<32, true>()))
+                       : (S == 8 ? grid_for<8, false>() : (S == 16 ? grid_for<16, false>() : grid_for<32, false>()));
+    // a guess at the items of a small frame: one per tile, and the runs of bins
+    // that hold every triangle eight times
+    return (int)std::min<long long>(g, std::max<long long>(ntiles + 8 * ttot / seg, 1));
 }
 
 template <bool kFlag>
-static cudaError_t launch_fragment_t(int S, const ViewDev *views, const int4 *items, const unsigned long long *scan,
-                                     long long tile_lo, long long tile_hi, long long cap_items, int *head,
+static cudaError_t launch_fragment_t(int S, const ViewDev *views, const ItemsOut &io, int cls, int *head,
                                      const unsigned long long *pairs, const float4 *rec, unsigned long long *keys,
                                      unsigned *flag_bits, long long *flag_list, Counters *cnt, int grid,
                                      cudaStream_t st)
 {
+    const int4 *items = io.items + (long long)cls * io.cap_items;
+    const unsigned long long *n = &cnt->items_n[cls];
     switch (S) {
     case 8:
-        k_fragment<8, kFlag><<<grid, 32, 0, st>>>(views, items, scan, tile_lo, tile_hi, cap_items, head, pairs,
-                                                  rec, keys, flag_bits, flag_list, cnt);
+        k_fragment<8, kFlag><<<grid, 32, 0, st>>>(views, items, n, io.cap_items, head, pairs, rec, keys, flag_bits,
+                                                  flag_list, cnt);
         break;
     case 16:
-        k_fragment<16, kFlag><<<grid, 128, 0, st>>>(views, items, scan, tile_lo, tile_hi, cap_items, head,
-                                                    pairs, rec, keys, flag_bits, flag_list, cnt);
+        k_fragment<16, kFlag><<<grid, 128, 0, st>>>(views, items, n, io.cap_items, head, pairs, rec, keys, flag_bits,
+                                                    flag_list, cnt);
         break;
     case 32:
-        k_fragment<32, kFlag><<<grid, 512, 0, st>>>(views, items, scan, tile_lo, tile_hi, cap_items, head,
-                                                    pairs, rec, keys, flag_bits, flag_list, cnt);
+        k_fragment<32, kFlag><<<grid, 512, 0, st>>>(views, items, n, io.cap_items, head, pairs, rec, keys, flag_bits,
+                                                    flag_list, cnt);
         break;
     default:
         return cudaErrorInvalidValue;
@@ -372,16 +376,13 @@ static cudaError_t launch_fragment_t(int S, const ViewDev *views, const int4 *it
     return cudaGetLastError();
 }
 
-cudaError_t launch_fragment(int S, bool flag, const ViewDev *views, const int4 *items, const unsigned long long *scan,
-                            long long tile_lo, long long tile_hi, long long cap_items, int *head,
+cudaError_t launch_fragment(int S, bool flag, const ViewDev *views, const ItemsOut &io, int cls, int *head,
                             const unsigned long long *pairs, const float4 *rec, unsigned long long *keys,
                             unsigned *flag_bits, long long *flag_list, Counters *cnt, int grid, cudaStream_t st)
 {
     if (flag)
-        return launch_fragment_t<true>(S, views, items, scan, tile_lo, tile_hi, cap_items, head, pairs, rec,
-                                       keys, flag_bits, flag_list, cnt, grid, st);
-    return launch_fragment_t<false>(S, views, items, scan, tile_lo, tile_hi, cap_items, head, pairs, rec, keys,
-                                    flag_bits, flag_list, cnt, grid, st);
+        return launch_fragment_t<true>(S, views, io, cls, head, pairs, rec, keys, flag_bits, flag_list, cnt, grid, st);
+    return launch_fragment_t<false>(S, views, io, cls, head, pairs, rec, keys, flag_bits, flag_list, cnt, grid, st);
 }
 
 // ---------------------------------------------------------------- FP64 re-test
@@ -513,8 +514,8 @@ __device__ __forceinline__ RetestPixel retest_pixel(const ViewDev *views, int nv
     px.j = (int)lin / v.W;  // lin < 2^28
     px.i = (int)lin - px.j * v.W;
     const long long tile = v.tile_off + (long long)(px.j / v.S) * v.tiles_x + px.i / v.S;
-    px.off = (long long)(scan[tile] & 0xFFFFFFFFFFull);
-    px.n = min((long long)(tile_cnt[tile] & 0xFFFFFFFFFFull), max(cap_pairs - px.off, 0ll));
+    px.off = (long long)scan[tile];
+    px.n = min((long long)tile_cnt[tile], max(cap_pairs - px.off, 0ll));
     return px;
 }
 
