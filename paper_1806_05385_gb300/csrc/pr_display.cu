@@ -15,7 +15,8 @@
 //    filter into the foveated domain); weights are taken relative to the
 //    nearest sample, whose factor cancels, so they cannot all underflow.
 //
-// One thread per display pixel; planar rgb in and out, coalesced along x.
+// One thread per display pixel, CTAs of 32 x 8 pixels (neighbouring rows
+// share their texels in L1); planar rgb in and out, coalesced along x.
 #include <algorithm>
 #include <cstring>
 
@@ -26,10 +27,13 @@ namespace pr {
 constexpr int kMaxMipLevels = 16;  // 16384 x 16384 needs 15
 
 struct MipPyramid {
-    const float *lev[kMaxMipLevels];
-    int w[kMaxMipLevels], h[kMaxMipLevels];
+    const float *lev[kMaxMipLevels];  // level 0 = the framebuffer image, the others in the call's scratch
+    int w0, h0;                       // size of level 0; level k has ceil(w0 / 2^k) x ceil(h0 / 2^k) texels
     int L;
 };
+
+// Size of level k along one axis: halving with ceil k times.
+__host__ __device__ __forceinline__ int mip_size(int n, int k) { return (n + (1 << k) - 1) >> k; }
 
 // Display-step constants of a view (by value into the kernel).
 struct DisplayView {
@@ -39,112 +43,182 @@ struct DisplayView {
     float alpha, inv_alpha;
     const float *p_lut;  // or: the sampled p (then alpha is unused)
     int p_n;
+    float rWd, rHd;      // 1 / Wd, 1 / Hd, correctly rounded (pixel_centre)
     float scale;         // max(W / Wd, H / Hd)
     float sigma;         // projected filter width, display pixels
 };
 
-// Texel (x, y) of a level from the level below (w0 x h0): the 2x2 block's
-// mean, over the texels of the block that exist.
-__device__ __forceinline__ void mip_texel(const float *__restrict__ src, int w0, int h0, float *__restrict__ dst,
-                                          int w1, int h1, int x, int y)
+// The 2x2 block's mean of texels a, b (b beside a), c, d (below), over the
+// texels of the block that exist (xr: the right ones do, yr: the lower ones
+// do).  Scaling by 1, 1/2 or 1/4 is exact.
+__device__ __forceinline__ float mip_mean(float a, float b, float c, float d, bool xr, bool yr)
 {
-    const int x0 = 2 * x, y0 = 2 * y;
-    const bool xr = x0 + 1 < w0, yr = y0 + 1 < h0;
-    const float n = (float)((1 + xr) * (1 + yr));
-    for (int c = 0; c < 3; ++c) {
-        const float *s = src + (size_t)c * w0 * h0;
-        float a = s[(size_t)y0 * w0 + x0];
+    if (xr)
+        a += b;
+    if (yr) {
+        a += c;
         if (xr)
-            a += s[(size_t)y0 * w0 + x0 + 1];
-        if (yr) {
-            a += s[(size_t)(y0 + 1) * w0 + x0];
-            if (xr)
-                a += s[(size_t)(y0 + 1) * w0 + x0 + 1];
+            a += d;
+    }
+    return a * ((xr ? 0.5f : 1.f) * (yr ? 0.5f : 1.f));
+}
+
+// Levels 1 .. kTileLevels of a pyramid, a 64 x 64 tile of level 0 per CTA:
+// each level is formed from the one below in shared memory, so a frame's
+// pyramid takes two launches instead of one per level (stereo HMD frame: 54
+// us in eleven launches, most of them a few texels and a launch's latency).
+// Level 0 is read once; the bound is that read (DRAM).
+constexpr int kTileLevels = 6, kTileSide = 1 << kTileLevels, kTileThreads = 256;
+
+__device__ __forceinline__ void mip_tile(const MipPyramid &pyr, int tx, int ty)
+{
+    __shared__ float s_a[3][kTileSide / 2 * (kTileSide / 2)], s_b[3][kTileSide / 4 * (kTileSide / 4)];
+    const int W = pyr.w0, H = pyr.h0;
+    const int top = min(kTileLevels, pyr.L - 1);
+    if (top >= 1) {  // level 1 from the image: sixteen loads of a thread in flight
+        constexpr int side = kTileSide / 2, per = side * side / kTileThreads;
+        const int w = mip_size(W, 1), h = mip_size(H, 1);
+        const float *src = pyr.lev[0];
+        float *dst = const_cast<float *>(pyr.lev[1]);
+        for (int c = 0; c < 3; ++c, src += (size_t)W * H, dst += (size_t)w * h) {
+#pragma unroll
+            for (int i = 0; i < per; ++i) {
+                const int t = threadIdx.x + i * kTileThreads;
+                const int x = tx * side + t % side, y = ty * side + t / side;
+                if (x >= w || y >= h)
+                    continue;
+                const bool xr = 2 * x + 1 < W, yr = 2 * y + 1 < H;
+                const float *p = src + (unsigned)(2 * y * W + 2 * x);
+                const float *p1 = p + W;
+                const float v = mip_mean(__ldg(p), xr ? __ldg(p + 1) : 0.f, yr ? __ldg(p1) : 0.f,
+                                         xr && yr ? __ldg(p1 + 1) : 0.f, xr, yr);
+                dst[(unsigned)(y * w + x)] = v;
+                s_a[c][t] = v;
+            }
         }
-        dst[(size_t)c * w1 * h1 + (size_t)y * w1 + x] = a / n;
+        __syncthreads();
+    }
+    for (int k = 2; k <= top; ++k) {
+        const int side = kTileSide >> k, lg = kTileLevels - k;  // the tile's texels of this level
+        const int w = mip_size(W, k), h = mip_size(H, k), wb = mip_size(W, k - 1), hb = mip_size(H, k - 1);
+        float *dst = const_cast<float *>(pyr.lev[k]);
+        const unsigned plane = (unsigned)w * (unsigned)h;
+        for (int u = threadIdx.x; u < 3 * side * side; u += kTileThreads) {
+            const int c = u >> (2 * lg), t = u & (side * side - 1);
+            const int ly = t >> lg, lx = t & (side - 1);
+            const int x = (tx << lg) + lx, y = (ty << lg) + ly;
+            if (x >= w || y >= h)
+                continue;
+            const bool xr = 2 * x + 1 < wb, yr = 2 * y + 1 < hb;
+            const float *p = (k & 1 ? s_b[c] : s_a[c]) + 4 * side * ly + 2 * lx;  // odd levels sit in s_a, even in s_b
+            const float v = mip_mean(p[0], p[1], p[2 * side], p[2 * side + 1], xr, yr);
+            dst[plane * c + (unsigned)(y * w + x)] = v;
+            if (k & 1)
+                s_a[c][t] = v;
+            else
+                s_b[c][t] = v;
+        }
+        __syncthreads();
     }
 }
 
-__global__ void k_mip_down(const float *__restrict__ src, int w0, int h0, float *__restrict__ dst, int w1, int h1)
+// The levels above, one CTA per pyramid: a few texels each (level 6 of a
+// 2160^2 image is 34^2).
+__device__ __forceinline__ void mip_top(const MipPyramid &pyr)
 {
-    const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y * blockDim.y + threadIdx.y;
-    if (x >= w1 || y >= h1)
-        return;
-    mip_texel(src, w0, h0, dst, w1, h1, x, y);
+    for (int k = kTileLevels + 1; k < pyr.L; ++k) {
+        const int w = mip_size(pyr.w0, k), h = mip_size(pyr.h0, k);
+        const int wb = mip_size(pyr.w0, k - 1), hb = mip_size(pyr.h0, k - 1);
+        const float *src = pyr.lev[k - 1];
+        float *dst = const_cast<float *>(pyr.lev[k]);
+        for (int t = threadIdx.x; t < 3 * w * h; t += blockDim.x) {
+            const int c = t / (w * h), y = (t - c * w * h) / w, x = t - c * w * h - y * w;
+            const bool xr = 2 * x + 1 < wb, yr = 2 * y + 1 < hb;
+            const float *p = src + (size_t)c * wb * hb + (size_t)(2 * y) * wb + 2 * x;
+            dst[t] = mip_mean(p[0], xr ? p[1] : 0.f, yr ? p[wb] : 0.f, xr && yr ? p[wb + 1] : 0.f, xr, yr);
+        }
+        __syncthreads();  // this level is the next one's source
+    }
 }
+
+__global__ void __launch_bounds__(kTileThreads) k_mip_tile(const MipPyramid pyr)
+{
+    mip_tile(pyr, blockIdx.x, blockIdx.y);
+}
+
+__global__ void __launch_bounds__(512) k_mip_top(const MipPyramid pyr) { mip_top(pyr); }
+
+// x^e of q; the linear factor of alpha = 2 without the general power (some
+// eighty instructions; the same bits).
+__device__ __forceinline__ float radial_pow(float x, float e) { return e == 1.f ? x : powf(x, e); }
 
 // Display location q(c) of every framebuffer pixel centre c (the offset from
 // the fovea scaled by (|e|/D)^(alpha - 1)), for the projected filter.
-__device__ __forceinline__ float2 q_of(int W, int H, int fov, float fx, float fy, float alpha,
-                                       const float *__restrict__ p_lut, int p_n, int i, int j)
-{
-    float q0 = __fdiv_rn((float)i + 0.5f, (float)W), q1 = __fdiv_rn((float)j + 0.5f, (float)H);
-    if (fov) {
-        const float e0 = q0 - fx, e1 = q1 - fy, r = sqrtf(fmaf(e0, e0, e1 * e1));
-        const SampledP sp{p_lut, p_n};
-        const float s = r > 0.f ? (p_lut ? sp.p(r) / r : powf(r * (1.f / kSqrt2), alpha - 1.f)) : 0.f;
-        q0 = fmaf(e0, s, fx);
-        q1 = fmaf(e1, s, fy);
-    }
-    return make_float2(q0, q1);
-}
-
-__device__ __forceinline__ void q_entry(int W, int H, int fov, float fx, float fy, float alpha,
-                                        const float *__restrict__ p_lut, int p_n, float2 *__restrict__ table, int i,
-                                        int j)
-{
-    table[(size_t)j * W + i] = q_of(W, H, fov, fx, fy, alpha, p_lut, p_n, i, j);
-}
-
-__global__ void k_q_table(int W, int H, int fov, float fx, float fy, float alpha, const float *__restrict__ p_lut,
-                          int p_n, float2 *__restrict__ table)
+__global__ void k_q_table(const DisplayView dv, float rW, float rH, float2 *__restrict__ table)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y;
-    if (i >= W)
+    if (i >= dv.W)
         return;
-    q_entry(W, H, fov, fx, fy, alpha, p_lut, p_n, table, i, j);
-}
-
-__device__ __forceinline__ float bspline3(float x)
-{
-    x = fabsf(x);
-    if (x < 1.f)
-        return fmaf(0.5f * x, x * x, 2.f / 3.f - x * x);
-    if (x < 2.f) {
-        const float y = 2.f - x;
-        return y * y * y * (1.f / 6.f);
+    float q0 = pixel_centre(i, dv.W, rW), q1 = pixel_centre(j, dv.H, rH);
+    if (dv.fov) {
+        const float e0 = q0 - dv.fx, e1 = q1 - dv.fy, r = sqrtf(fmaf(e0, e0, e1 * e1));
+        const SampledP sp{dv.p_lut, dv.p_n};
+        const float s = r > 0.f ? (dv.p_lut ? sp.p(r) / r : radial_pow(r * (1.f / kSqrt2), dv.alpha - 1.f)) : 0.f;
+        q0 = fmaf(e0, s, dv.fx);
+        q1 = fmaf(e1, s, dv.fy);
     }
-    return 0.f;
+    table[(size_t)j * dv.W + i] = make_float2(q0, q1);
 }
 
-// 3-tap cubic sample of one level at texel coordinates (s, t).
+// Cubic B-spline weights of the taps at -1, 0, 1 for a sample at d in
+// [-1/2, 1/2] from the middle one: 2/3 - x^2 + x^3 / 2 within one texel,
+// (2 - x)^3 / 6 beyond.  With m = 1 - |d| the nearer side tap has x = m, the
+// farther one 2 - x = m.
+__device__ __forceinline__ void bspline_taps(float d, float (&w)[3])
+{
+    const float a = fabsf(d), m = 1.f - a;
+    const float m2 = m * m, m3 = m2 * m;
+    const float near = fmaf(0.5f, m3, 2.f / 3.f - m2), far = m3 * (1.f / 6.f);
+    w[0] = d < 0.f ? near : far;
+    w[1] = fmaf(fmaf(0.5f, a, -1.f), a * a, 2.f / 3.f);
+    w[2] = d < 0.f ? far : near;
+}
+
+// 3-tap cubic sample of one level at texel coordinates (s, t): the three
+// taps of each row first, then the rows.
 __device__ __forceinline__ void sample3(const float *__restrict__ lev, int w, int h, float s, float t, float out[3])
 {
     const float fs = floorf(s + 0.5f), ft = floorf(t + 0.5f);
-    float wx[3], wy[3], sx = 0.f, sy = 0.f;
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        wx[k] = bspline3(s - (fs + (float)(k - 1)));
-        wy[k] = bspline3(t - (ft + (float)(k - 1)));
-        sx += wx[k];
-        sy += wy[k];
-    }
-    const float inv = 1.f / (sx * sy);
-    out[0] = out[1] = out[2] = 0.f;
+    float wx[3], wy[3];
+    bspline_taps(s - fs, wx);
+    bspline_taps(t - ft, wy);
+    const float inv = 1.f / ((wx[0] + wx[1] + wx[2]) * (wy[0] + wy[1] + wy[2]));  // sums of about 1
     const int is = (int)fs, it = (int)ft;
-    const size_t plane = (size_t)w * h;
+    const unsigned plane = (unsigned)w * (unsigned)h;  // <= 2^28
+    out[0] = out[1] = out[2] = 0.f;
+    if (is >= 1 && is < w - 1 && it >= 1 && it < h - 1) {
+        // inside: the taps are neighbours, nine row addresses serve all
+        const float *p = lev + (unsigned)((it - 1) * w + is - 1);
 #pragma unroll
-    for (int ky = 0; ky < 3; ++ky) {
-        const int y = min(max(it + ky - 1, 0), h - 1);
-#pragma unroll
-        for (int kx = 0; kx < 3; ++kx) {
-            const int x = min(max(is + kx - 1, 0), w - 1);
-            const float wgt = wx[kx] * wy[ky] * inv;
-            const size_t o = (size_t)y * w + x;
-            out[0] = fmaf(wgt, __ldg(lev + o), out[0]);
-            out[1] = fmaf(wgt, __ldg(lev + plane + o), out[1]);
-            out[2] = fmaf(wgt, __ldg(lev + 2 * plane + o), out[2]);
+        for (int c = 0; c < 3; ++c, p += plane) {
+            const float *r1 = p + w, *r2 = r1 + w;
+            const float a = fmaf(wx[0], __ldg(p), fmaf(wx[1], __ldg(p + 1), wx[2] * __ldg(p + 2)));
+            const float b = fmaf(wx[0], __ldg(r1), fmaf(wx[1], __ldg(r1 + 1), wx[2] * __ldg(r1 + 2)));
+            const float d = fmaf(wx[0], __ldg(r2), fmaf(wx[1], __ldg(r2 + 1), wx[2] * __ldg(r2 + 2)));
+            out[c] = fmaf(wy[2], d, fmaf(wy[1], b, wy[0] * a)) * inv;
         }
+        return;
+    }
+    const int x0 = min(max(is - 1, 0), w - 1), x1 = min(max(is, 0), w - 1), x2 = min(max(is + 1, 0), w - 1);
+    const unsigned r0 = (unsigned)(min(max(it - 1, 0), h - 1) * w), r1 = (unsigned)(min(max(it, 0), h - 1) * w),
+                   r2 = (unsigned)(min(max(it + 1, 0), h - 1) * w);
+    const float *p = lev;
+#pragma unroll
+    for (int c = 0; c < 3; ++c, p += plane) {
+        const float a = fmaf(wx[0], __ldg(p + (r0 + x0)), fmaf(wx[1], __ldg(p + (r0 + x1)), wx[2] * __ldg(p + (r0 + x2))));
+        const float b = fmaf(wx[0], __ldg(p + (r1 + x0)), fmaf(wx[1], __ldg(p + (r1 + x1)), wx[2] * __ldg(p + (r1 + x2))));
+        const float d = fmaf(wx[0], __ldg(p + (r2 + x0)), fmaf(wx[1], __ldg(p + (r2 + x1)), wx[2] * __ldg(p + (r2 + x2))));
+        out[c] = fmaf(wy[2], d, fmaf(wy[1], b, wy[0] * a)) * inv;
     }
 }
 
@@ -154,7 +228,7 @@ __device__ __forceinline__ void unfoveate_pixel(const DisplayView &dv, const Mip
                                                 const float *__restrict__ rgb, const float2 *__restrict__ qtab,
                                                 float *__restrict__ out, int a, int b)
 {
-    const float x0 = __fdiv_rn((float)a + 0.5f, (float)dv.Wd), x1 = __fdiv_rn((float)b + 0.5f, (float)dv.Hd);
+    const float x0 = pixel_centre(a, dv.Wd, dv.rWd), x1 = pixel_centre(b, dv.Hd, dv.rHd);
     // u = q^-1(x): the offset from the fovea scaled by (|e|/D)^(1/alpha - 1)
     float u0 = x0, u1 = x1, tang = 1.f, stretch = 1.f;
     if (dv.fov) {
@@ -180,11 +254,11 @@ __device__ __forceinline__ void unfoveate_pixel(const DisplayView &dv, const Mip
         const int k0 = (int)floorf(lambda), k1 = min(k0 + 1, pyr.L - 1);
         const float f = lambda - (float)k0;
         float s0[3], s1[3];
-        sample3(pyr.lev[k0], pyr.w[k0], pyr.h[k0], fmaf(u0, (float)pyr.w[k0], -0.5f),
-                fmaf(u1, (float)pyr.h[k0], -0.5f), s0);
+        const int w0 = mip_size(dv.W, k0), h0 = mip_size(dv.H, k0);
+        sample3(pyr.lev[k0], w0, h0, fmaf(u0, (float)w0, -0.5f), fmaf(u1, (float)h0, -0.5f), s0);
         if (f > 0.f) {
-            sample3(pyr.lev[k1], pyr.w[k1], pyr.h[k1], fmaf(u0, (float)pyr.w[k1], -0.5f),
-                    fmaf(u1, (float)pyr.h[k1], -0.5f), s1);
+            const int w1 = mip_size(dv.W, k1), h1 = mip_size(dv.H, k1);
+            sample3(pyr.lev[k1], w1, h1, fmaf(u0, (float)w1, -0.5f), fmaf(u1, (float)h1, -0.5f), s1);
             for (int c = 0; c < 3; ++c)
                 res[c] = fmaf(f, s1[c] - s0[c], s0[c]);
         } else {
@@ -194,52 +268,58 @@ __device__ __forceinline__ void unfoveate_pixel(const DisplayView &dv, const Mip
     } else {
         const int i = min(max((int)floorf(u0 * (float)dv.W), 0), dv.W - 1);
         const int j = min(max((int)floorf(u1 * (float)dv.H), 0), dv.H - 1);
+        // The window's part inside the framebuffer.  Weights are taken
+        // relative to a reference sample m, whose factor cancels in the
+        // normalisation: exp(k2 (d^2 - d_m^2)) with d^2 - d_m^2 =
+        // (d - d_m)(d + d_m) per axis, where d - d_m comes from the difference
+        // of the two samples' display locations.  The reference must not be so
+        // much farther than the nearest sample that a weight overflows.  The
+        // window's centre is near enough by itself when k2 d^2 of it is above
+        // -60 (no weight can then exceed e^60); display pixels farther from
+        // their centre sample (beyond the framebuffer's disc, or a display of
+        // far more pixels) look for the nearest sample first.
+        const int dx0 = max(-2, -i), dx1 = min(2, dv.W - 1 - i), dy0 = max(-2, -j), dy1 = min(2, dv.H - 1 - j);
         const float k2 = -0.5f / (dv.sigma * dv.sigma);
-        const size_t plane = (size_t)dv.W * dv.H;
-        // display location q(c) of a window pixel's centre, from the table
-        auto qc = [&](int pi, int pj, float &q0, float &q1) {
-            const float2 q = __ldg(qtab + (size_t)pj * dv.W + pi);
-            q0 = q.x;
-            q1 = q.y;
-        };
-        // pass 1: the nearest sample in display space
-        float d2min = INFINITY, qm0 = 0.f, qm1 = 0.f;
-        for (int dy = -2; dy <= 2; ++dy)
-            for (int dx = -2; dx <= 2; ++dx) {
-                const int pi = i + dx, pj = j + dy;
-                if (pj < 0 || pj >= dv.H || pi < 0 || pi >= dv.W)
-                    continue;
-                float q0, q1;
-                qc(pi, pj, q0, q1);
-                const float d0 = (x0 - q0) * (float)dv.Wd, d1 = (x1 - q1) * (float)dv.Hd;
-                const float q2 = fmaf(d0, d0, d1 * d1);
-                if (q2 < d2min) {
-                    d2min = q2;
-                    qm0 = q0;
-                    qm1 = q1;
+        const float fWd = (float)dv.Wd, fHd = (float)dv.Hd;
+        const unsigned plane = (unsigned)dv.W * (unsigned)dv.H;  // <= 2^28
+        const float2 qm = __ldg(qtab + (unsigned)(j * dv.W + i));
+        float qm0 = qm.x, qm1 = qm.y;
+        {
+            const float d0 = (x0 - qm0) * fWd, d1 = (x1 - qm1) * fHd;
+            if (k2 * fmaf(d0, d0, d1 * d1) < -60.f) {
+                float d2min = INFINITY;
+                for (int dy = dy0; dy <= dy1; ++dy) {
+                    const float2 *qr = qtab + (unsigned)((j + dy) * dv.W + i + dx0);
+                    for (int dx = dx0; dx <= dx1; ++dx, ++qr) {
+                        const float2 q = __ldg(qr);
+                        const float e0 = (x0 - q.x) * fWd, e1 = (x1 - q.y) * fHd;
+                        const float q2 = fmaf(e0, e0, e1 * e1);
+                        if (q2 < d2min) {
+                            d2min = q2;
+                            qm0 = q.x;
+                            qm1 = q.y;
+                        }
+                    }
                 }
             }
-        // pass 2: weights relative to the nearest sample (its factor cancels
-        // in the normalisation, so they never all underflow), with
-        // d^2 - d_min^2 = (d - d_min)(d + d_min) per axis, where d - d_min
-        // comes from the difference of the two samples' display locations
+        }
+        const float s0 = 2.f * x0, s1 = 2.f * x1;
+        const float kw = k2 * 1.44269504f * fWd * fWd, kh = k2 * 1.44269504f * fHd * fHd;  // exp as a power of two
         float acc[3] = {0.f, 0.f, 0.f}, wsum = 0.f;
-        for (int dy = -2; dy <= 2; ++dy)
-            for (int dx = -2; dx <= 2; ++dx) {
-                const int pi = i + dx, pj = j + dy;
-                if (pj < 0 || pj >= dv.H || pi < 0 || pi >= dv.W)
-                    continue;
-                float q0, q1;
-                qc(pi, pj, q0, q1);
-                const float a0 = (qm0 - q0) * (float)dv.Wd, a1 = (qm1 - q1) * (float)dv.Hd;  // d - d_min
-                const float b0 = (2.f * x0 - q0 - qm0) * (float)dv.Wd, b1 = (2.f * x1 - q1 - qm1) * (float)dv.Hd;
-                const float w = expf(k2 * fmaf(a0, b0, a1 * b1));
-                const size_t o = (size_t)pj * dv.W + pi;
+        for (int dy = dy0; dy <= dy1; ++dy) {
+            const unsigned o = (unsigned)((j + dy) * dv.W + i + dx0);
+            const float2 *qr = qtab + o;
+            const float *p0 = rgb + o, *p1 = p0 + plane, *p2 = p1 + plane;
+            for (int dx = 0; dx <= dx1 - dx0; ++dx) {
+                const float2 q = __ldg(qr + dx);
+                const float t0 = (qm0 - q.x) * (s0 - q.x - qm0), t1 = (qm1 - q.y) * (s1 - q.y - qm1);
+                const float w = exp2f(fmaf(t0, kw, t1 * kh));
                 wsum += w;
-                acc[0] = fmaf(w, __ldg(rgb + o), acc[0]);
-                acc[1] = fmaf(w, __ldg(rgb + plane + o), acc[1]);
-                acc[2] = fmaf(w, __ldg(rgb + 2 * plane + o), acc[2]);
+                acc[0] = fmaf(w, __ldg(p0 + dx), acc[0]);
+                acc[1] = fmaf(w, __ldg(p1 + dx), acc[1]);
+                acc[2] = fmaf(w, __ldg(p2 + dx), acc[2]);
             }
+        }
         const float inv = 1.f / wsum;
         for (int c = 0; c < 3; ++c)
             res[c] = acc[c] * inv;
@@ -250,26 +330,35 @@ __device__ __forceinline__ void unfoveate_pixel(const DisplayView &dv, const Mip
     out[2 * dplane + o] = res[2];
 }
 
+// CTAs of the display kernels: 32 x 8 display pixels.
+constexpr int kDispW = 32, kDispH = 8;
+
 template <int kMethod>
-__global__ void __launch_bounds__(256) k_unfoveate(DisplayView dv, MipPyramid pyr, const float *__restrict__ rgb,
-                                                  const float2 *__restrict__ qtab, float *__restrict__ out)
+__global__ void __launch_bounds__(kDispW *kDispH) k_unfoveate(const DisplayView dv, const MipPyramid pyr,
+                                                             const float *__restrict__ rgb,
+                                                             const float2 *__restrict__ qtab, float *__restrict__ out)
 {
-    const int a = blockIdx.x * blockDim.x + threadIdx.x, b = blockIdx.y;
-    if (a >= dv.Wd)
+    const int a = blockIdx.x * kDispW + threadIdx.x % kDispW, b = blockIdx.y * kDispH + threadIdx.x / kDispW;
+    if (a >= dv.Wd || b >= dv.Hd)
         return;
     unfoveate_pixel<kMethod>(dv, pyr, rgb, qtab, out, a, b);
 }
 
-// ---- the batched display step (MIP): many views, one launch per pyramid
-// level and one for the display pixels of all views.  A launch's blocks are
-// numbered view after view (blk[q] = first block of view q, blk[n] = all);
-// a block finds its view by a binary search and runs the same per-texel and
-// per-pixel code as the single-view kernels, so the results are the same.
+// ---- the batched display step (MIP): many views, two launches for their
+// pyramids and one for the display pixels of all views.  A launch's blocks
+// are numbered view after view (blk[q] = first block of view q, blk[n] =
+// all); a block finds its view by a warp's ballot and runs the same
+// per-texel and per-pixel code as the single-view kernels, so the results
+// are the same.
 struct DisplayBatchView {
     DisplayView dv;
     MipPyramid pyr;  // level 0 = rgb
     const float *rgb;
     float *out;
+    // block / blocks per row as (block * mul) >> 40: the round-up reciprocals
+    // of Granlund and Montgomery (1994), exact for blocks < 2^23 and rows of
+    // at most 2^11
+    unsigned long long mul_disp, mul_tile;
 };
 
 // The view of block b (the same for every lane): the warp compares 32
@@ -279,36 +368,35 @@ __device__ __forceinline__ int block_view(const long long *__restrict__ blk, int
     return find_view_warp(blk, n, b);
 }
 
-// Level k of every view that has one (blocks of 256 texels, row-major).
-__global__ void __launch_bounds__(256) k_mip_down_batch(const DisplayBatchView *__restrict__ tab,
-                                                       const long long *__restrict__ blk, int n, int k)
+// Levels 1 .. kTileLevels of every view.
+__global__ void __launch_bounds__(kTileThreads) k_mip_tile_batch(const DisplayBatchView *__restrict__ tab,
+                                                                 const long long *__restrict__ blk, int n)
 {
     const int q = block_view(blk, n, blockIdx.x);
-    const MipPyramid &pyr = tab[q].pyr;
-    const int t = (int)(blockIdx.x - blk[q]) * (int)blockDim.x + (int)threadIdx.x;
-    const int w1 = pyr.w[k], h1 = pyr.h[k];
-    if (t >= w1 * h1)
-        return;
-    const int y = t / w1, x = t - y * w1;
-    // levels k >= 1 live in the call's scratch (only level 0, the caller's
-    // image, is read-only)
-    mip_texel(pyr.lev[k - 1], pyr.w[k - 1], pyr.h[k - 1], const_cast<float *>(pyr.lev[k]), w1, h1, x, y);
+    const DisplayBatchView &e = tab[q];
+    const unsigned b = (unsigned)(blockIdx.x - blk[q]);
+    const int ty = (int)((b * e.mul_tile) >> 40), tx = (int)b - ty * ((e.dv.W + kTileSide - 1) / kTileSide);
+    mip_tile(e.pyr, tx, ty);
 }
 
-// The display pixels of every view (blocks of 256, row-major; a view has
-// fewer than 2^28 pixels, so its pixel index is 32-bit).  The register cap
-// keeps the single-view kernel's occupancy (5 CTAs per SM): the view's
-// constants, parameters there, are registers here.
-__global__ void __launch_bounds__(256, 5) k_unfoveate_mip_batch(const DisplayBatchView *__restrict__ tab,
-                                                               const long long *__restrict__ blk, int n)
+// The levels above (blockIdx.x: view).
+__global__ void __launch_bounds__(512) k_mip_top_batch(const DisplayBatchView *__restrict__ tab)
+{
+    mip_top(tab[blockIdx.x].pyr);
+}
+
+// The display pixels of every view.
+__global__ void __launch_bounds__(kDispW *kDispH, 5) k_unfoveate_mip_batch(const DisplayBatchView *__restrict__ tab,
+                                                                          const long long *__restrict__ blk, int n)
 {
     const int q = block_view(blk, n, blockIdx.x);
     const DisplayBatchView &e = tab[q];
     const DisplayView dv = e.dv;
-    const int t = (int)(blockIdx.x - blk[q]) * (int)blockDim.x + (int)threadIdx.x;
-    if (t >= dv.Wd * dv.Hd)
+    const unsigned t = (unsigned)(blockIdx.x - blk[q]);
+    const int by = (int)((t * e.mul_disp) >> 40), bx = (int)t - by * ((dv.Wd + kDispW - 1) / kDispW);
+    const int a = bx * kDispW + threadIdx.x % kDispW, b = by * kDispH + threadIdx.x / kDispW;
+    if (a >= dv.Wd || b >= dv.Hd)
         return;
-    const int b = t / dv.Wd, a = t - b * dv.Wd;
     unfoveate_pixel<PR_UNFOVEATE_MIP_CUBIC>(dv, e.pyr, e.rgb, nullptr, e.out, a, b);
 }
 
@@ -337,6 +425,23 @@ size_t mip_pyramid_floats(int W, int H)
     }
 }
 
+// Level pointers of a pyramid with its levels 1 .. L - 1 at `p` one after the
+// other; false if it has more than kMaxMipLevels.
+static bool fill_pyramid(MipPyramid &pyr, int W, int H, const float *rgb, float *p)
+{
+    pyr.L = mip_level_count(W, H);
+    if (pyr.L > kMaxMipLevels)
+        return false;
+    pyr.w0 = W;
+    pyr.h0 = H;
+    pyr.lev[0] = rgb;
+    for (int k = 1; k < pyr.L; ++k) {
+        pyr.lev[k] = p;
+        p += (size_t)3 * mip_size(W, k) * mip_size(H, k);
+    }
+    return true;
+}
+
 cudaError_t launch_unfoveate(int method, int W, int H, int mode, float fx, float fy, float alpha, const float *p_lut,
                              int p_n, int Wd, int Hd, float sigma, const float *rgb, float *pyramid, float *out,
                              cudaStream_t st)
@@ -346,6 +451,8 @@ cudaError_t launch_unfoveate(int method, int W, int H, int mode, float fx, float
     dv.H = H;
     dv.Wd = Wd;
     dv.Hd = Hd;
+    dv.rWd = 1.f / (float)Wd;
+    dv.rHd = 1.f / (float)Hd;
     dv.fov = mode == PR_FOVEATED || mode == PR_BOTH;
     dv.fx = fx;
     dv.fy = fy;
@@ -357,30 +464,20 @@ cudaError_t launch_unfoveate(int method, int W, int H, int mode, float fx, float
     dv.sigma = sigma;
     MipPyramid pyr;
     std::memset(&pyr, 0, sizeof pyr);
-    const dim3 blk(256), grd((unsigned)((Wd + 255) / 256), (unsigned)Hd);
+    const dim3 blk(kDispW * kDispH), grd((unsigned)((Wd + kDispW - 1) / kDispW), (unsigned)((Hd + kDispH - 1) / kDispH));
     if (method == PR_UNFOVEATE_MIP_CUBIC) {
-        const int L = mip_level_count(W, H);
-        if (L > kMaxMipLevels)
+        if (!fill_pyramid(pyr, W, H, rgb, pyramid))
             return cudaErrorInvalidValue;
-        pyr.L = L;
-        pyr.lev[0] = rgb;
-        pyr.w[0] = W;
-        pyr.h[0] = H;
-        float *p = pyramid;
-        for (int k = 1; k < L; ++k) {
-            const int w1 = (pyr.w[k - 1] + 1) / 2, h1 = (pyr.h[k - 1] + 1) / 2;
-            const dim3 b2(32, 8), g2((unsigned)((w1 + 31) / 32), (unsigned)((h1 + 7) / 8));
-            k_mip_down<<<g2, b2, 0, st>>>(pyr.lev[k - 1], pyr.w[k - 1], pyr.h[k - 1], p, w1, h1);
-            pyr.lev[k] = p;
-            pyr.w[k] = w1;
-            pyr.h[k] = h1;
-            p += (size_t)3 * w1 * h1;
-        }
+        if (pyr.L > 1)
+            k_mip_tile<<<dim3((unsigned)((W + kTileSide - 1) / kTileSide), (unsigned)((H + kTileSide - 1) / kTileSide)),
+                         kTileThreads, 0, st>>>(pyr);
+        if (pyr.L > kTileLevels + 1)
+            k_mip_top<<<1, 512, 0, st>>>(pyr);
         k_unfoveate<PR_UNFOVEATE_MIP_CUBIC><<<grd, blk, 0, st>>>(dv, pyr, rgb, nullptr, out);
     } else {
         float2 *qtab = reinterpret_cast<float2 *>(pyramid);
         const dim3 gq((unsigned)((W + 255) / 256), (unsigned)H);
-        k_q_table<<<gq, 256, 0, st>>>(W, H, dv.fov, fx, fy, alpha, p_lut, p_n, qtab);
+        k_q_table<<<gq, 256, 0, st>>>(dv, 1.f / (float)W, 1.f / (float)H, qtab);
         k_unfoveate<PR_UNFOVEATE_PROJECTED><<<grd, blk, 0, st>>>(dv, pyr, rgb, qtab, out);
     }
     return cudaGetLastError();
@@ -408,12 +505,12 @@ size_t display_batch_scratch_floats(int method, const DisplayEntry *e, int n)
     return f;
 }
 
-// Table layout (MIP): n DisplayBatchView, then kMaxMipLevels arrays of n + 1
-// block offsets: the display pixels' at index 0, pyramid level k's at k.
+// Table layout (MIP): n DisplayBatchView, then two arrays of n + 1 block
+// offsets: the display pixels', then the pyramid tiles'.
 size_t display_batch_table_bytes(int n)
 {
     const size_t views = ((sizeof(DisplayBatchView) * (size_t)n) + 15) & ~(size_t)15;
-    return views + sizeof(long long) * (size_t)kMaxMipLevels * (size_t)(n + 1);
+    return views + sizeof(long long) * 2 * (size_t)(n + 1);
 }
 
 cudaError_t launch_unfoveate_batch(int method, float sigma, const DisplayEntry *e, int n, float *scratch,
@@ -437,7 +534,7 @@ cudaError_t launch_unfoveate_batch(int method, float sigma, const DisplayEntry *
     const size_t views_bytes = ((sizeof(DisplayBatchView) * (size_t)n) + 15) & ~(size_t)15;
     DisplayBatchView *tab = static_cast<DisplayBatchView *>(h_table);
     long long *blk = reinterpret_cast<long long *>(static_cast<char *>(h_table) + views_bytes);
-    int Lmax = 1;
+    bool any_tiles = false, any_top = false;
     float *p = scratch;
     for (int q = 0; q < n; ++q) {
         DisplayBatchView &t = tab[q];
@@ -447,6 +544,8 @@ cudaError_t launch_unfoveate_batch(int method, float sigma, const DisplayEntry *
         dv.H = e[q].H;
         dv.Wd = e[q].Wd;
         dv.Hd = e[q].Hd;
+        dv.rWd = 1.f / (float)dv.Wd;
+        dv.rHd = 1.f / (float)dv.Hd;
         dv.fov = e[q].mode == PR_FOVEATED || e[q].mode == PR_BOTH;
         dv.fx = e[q].fx;
         dv.fy = e[q].fy;
@@ -461,42 +560,31 @@ cudaError_t launch_unfoveate_batch(int method, float sigma, const DisplayEntry *
         // the view's scratch: its pyramid levels 1..
         float *lp = p;
         p += view_scratch_floats(dv.W, dv.H);
-        const int L = mip_level_count(dv.W, dv.H);
-        if (L > kMaxMipLevels)
+        if (!fill_pyramid(t.pyr, dv.W, dv.H, e[q].rgb, lp))
             return cudaErrorInvalidValue;
-        t.pyr.L = L;
-        t.pyr.lev[0] = e[q].rgb;
-        t.pyr.w[0] = dv.W;
-        t.pyr.h[0] = dv.H;
-        for (int k = 1; k < L; ++k) {
-            t.pyr.w[k] = (t.pyr.w[k - 1] + 1) / 2;
-            t.pyr.h[k] = (t.pyr.h[k - 1] + 1) / 2;
-            t.pyr.lev[k] = lp;
-            lp += (size_t)3 * t.pyr.w[k] * t.pyr.h[k];
-        }
-        Lmax = std::max(Lmax, L);
-    }
-    for (int k = 0; k < kMaxMipLevels; ++k) {
-        long long *o = blk + (size_t)k * (n + 1);
-        o[0] = 0;
-        for (int q = 0; q < n; ++q) {
-            const long long items = k == 0 ? (long long)tab[q].dv.Wd * tab[q].dv.Hd
-                                           : (k < tab[q].pyr.L ? (long long)tab[q].pyr.w[k] * tab[q].pyr.h[k] : 0ll);
-            o[q + 1] = o[q] + (items + 255) / 256;
-        }
+        any_tiles |= t.pyr.L > 1;
+        any_top |= t.pyr.L > kTileLevels + 1;
+        auto row_mul = [](long long per_row) { return ((1ull << 40) + per_row - 1) / (unsigned long long)per_row; };
+        const long long dw = (dv.Wd + kDispW - 1) / kDispW, dh = (dv.Hd + kDispH - 1) / kDispH;
+        const long long tw = (dv.W + kTileSide - 1) / kTileSide, th = (dv.H + kTileSide - 1) / kTileSide;
+        t.mul_disp = row_mul(dw);
+        t.mul_tile = row_mul(tw);
+        if (q == 0)
+            blk[0] = blk[n + 1] = 0;
+        blk[q + 1] = blk[q] + dw * dh;
+        blk[n + 1 + q + 1] = blk[n + 1 + q] + tw * th;
     }
     cudaError_t err = cudaMemcpyAsync(d_table, h_table, display_batch_table_bytes(n), cudaMemcpyHostToDevice, st);
     if (err != cudaSuccess)
         return err;
     const DisplayBatchView *dtab = static_cast<const DisplayBatchView *>(d_table);
     const long long *dblk = reinterpret_cast<const long long *>(static_cast<const char *>(d_table) + views_bytes);
-    for (int k = 1; k < Lmax; ++k) {
-        const long long nb = blk[(size_t)k * (n + 1) + n];
-        if (nb > 0)
-            k_mip_down_batch<<<(unsigned)nb, 256, 0, st>>>(dtab, dblk + (size_t)k * (n + 1), n, k);
-    }
+    if (any_tiles)
+        k_mip_tile_batch<<<(unsigned)blk[2 * n + 1], kTileThreads, 0, st>>>(dtab, dblk + n + 1, n);
+    if (any_top)
+        k_mip_top_batch<<<(unsigned)n, 512, 0, st>>>(dtab);
     if (blk[n] > 0)
-        k_unfoveate_mip_batch<<<(unsigned)blk[n], 256, 0, st>>>(dtab, dblk, n);
+        k_unfoveate_mip_batch<<<(unsigned)blk[n], kDispW * kDispH, 0, st>>>(dtab, dblk, n);
     return cudaGetLastError();
 }
 

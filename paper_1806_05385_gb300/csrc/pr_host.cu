@@ -358,6 +358,8 @@ pr_status derive_view(const pr_view &in, int tile, int bound, int fp64, ViewDev 
     v.shininess = in.shininess;
     v.W = in.W;
     v.H = in.H;
+    v.rW = 1.f / (float)in.W;
+    v.rH = 1.f / (float)in.H;
     v.mode = in.mode;
     v.S = tile;
     v.tiles_x = (in.W + tile - 1) / tile;

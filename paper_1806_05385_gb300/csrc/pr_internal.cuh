@@ -77,6 +77,7 @@ struct ViewDev {
     const unsigned *scene_status;      // the scene's status word (ST_NONFINITE after an update), or null
     float *dcol, *dpos, *dvel;         // adjoint outputs [V][3]
     const float4 *rec;                 // this frame's stage (a) records (batch-wide index), or null
+    float rW, rH;                      // 1 / W, 1 / H, correctly rounded (pixel_centre)
     unsigned long long bw_mul;         // ceil(2^40 / bw), bw = strips per row: lb / bw = (lb * bw_mul) >> 40 (set_strips)
 };
 
@@ -219,6 +220,19 @@ __device__ __forceinline__ float fov_scale(float r, float alpha)
     return r > 0.f ? __powf(r * (1.0f / kSqrt2), alpha - 1.0f) : 0.f;
 }
 
+// (i + 1/2) / n, correctly rounded, for a pixel or tile index 0 <= i < n <=
+// 16384 and rn = 1 / n correctly rounded: division by a divisor known in
+// advance (Markstein 1990; Brisebarre and Muller 2004), a product and two
+// fused multiply-adds where an IEEE division takes about ten instructions
+// and a branch.  Equal to the division for every such i and n (checked
+// exhaustively), so locations keep their bits.
+__host__ __device__ __forceinline__ float pixel_centre(int i, int n, float rn)
+{
+    const float a = (float)i + 0.5f, b = (float)n;
+    const float q = a * rn;
+    return fmaf(fmaf(-q, b, a), rn, q);
+}
+
 // Pixel (i, j) -> its display location x, its time t and its ray direction
 // (dx, dy, 1) (conventions of pr.h).  FP32; the same code in every stage.
 // kLut = false: the caller knows no view uses a sampled p, and the sampled
@@ -227,8 +241,8 @@ template <bool kLut = true>
 __device__ __forceinline__ void pixel_ray(const ViewDev &v, int i, int j, float &x0, float &x1, float &t, float &dx,
                                           float &dy)
 {
-    float u0 = __fdiv_rn((float)i + 0.5f, (float)v.W);
-    float u1 = __fdiv_rn((float)j + 0.5f, (float)v.H);
+    float u0 = pixel_centre(i, v.W, v.rW);
+    float u1 = pixel_centre(j, v.H, v.rH);
     if (is_foveated(v.mode)) {
         float e0 = u0 - v.fx, e1 = u1 - v.fy;
         float r = sqrtf(fmaf(e0, e0, e1 * e1));

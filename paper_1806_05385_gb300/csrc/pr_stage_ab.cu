@@ -181,10 +181,10 @@ __device__ __forceinline__ void tile_pixel_box(const ViewDev &v, long long lt, f
     const int ty = (int)lt / v.tiles_x, tx = (int)lt - ty * v.tiles_x;
     const int i0 = tx * v.S, i1 = min(v.W, i0 + v.S) - 1;
     const int j0 = ty * v.S, j1 = min(v.H, j0 + v.S) - 1;
-    u0 = __fdiv_rn((float)i0 + 0.5f, (float)v.W);
-    u1 = __fdiv_rn((float)i1 + 0.5f, (float)v.W);
-    w0 = __fdiv_rn((float)j0 + 0.5f, (float)v.H);
-    w1 = __fdiv_rn((float)j1 + 0.5f, (float)v.H);
+    u0 = pixel_centre(i0, v.W, v.rW);
+    u1 = pixel_centre(i1, v.W, v.rW);
+    w0 = pixel_centre(j0, v.H, v.rH);
+    w1 = pixel_centre(j1, v.H, v.rH);
 }
 
 // Display box of every framebuffer tile: the box of its pixel centres, or
@@ -1113,10 +1113,8 @@ __global__ void __launch_bounds__(256, 4) k_bin(const ViewDev *__restrict__ view
                     // the tile's pixel-centre box in framebuffer coordinates
                     const int i0 = tx << sh, i1 = min(v.W, (tx + 1) << sh) - 1;
                     const int j0 = ty << sh, j1 = min(v.H, (ty + 1) << sh) - 1;
-                    const float4 fbt = make_float4(__fdiv_rn((float)i0 + 0.5f, (float)v.W),
-                                                   __fdiv_rn((float)i1 + 0.5f, (float)v.W),
-                                                   __fdiv_rn((float)j0 + 0.5f, (float)v.H),
-                                                   __fdiv_rn((float)j1 + 0.5f, (float)v.H));
+                    const float4 fbt = make_float4(pixel_centre(i0, v.W, v.rW), pixel_centre(i1, v.W, v.rW),
+                                                   pixel_centre(j0, v.H, v.rH), pixel_centre(j1, v.H, v.rH));
                     const float4 big = make_float4(-INFINITY, INFINITY, -INFINITY, INFINITY);
                     hit = tile_meets(tile_box[tile], bb, hp, 0) && tile_meets(fbt, big, hp + g * kMaxHp, nh);
                 }
