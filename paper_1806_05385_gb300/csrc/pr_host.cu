@@ -739,9 +739,15 @@ pr_status enqueue_batch(pr_workspace *ws, BatchPlan &P, int seg, bool shade, cud
     if (!shade)
         PR_TRY(launch_resolve(dv, n, pix_offs, P.npix, ws->keys.as<unsigned long long>(), reader_resets, st));
     PR_TRY(mark(5));
+    // pixels that need FP64 shading go to the flag list, which the re-test is done with
+    Deferred64 def;
+    if (P.any_fp64 && P.npix < (1ll << 32)) {
+        def.list = ws->flag_list.as<unsigned long long>();
+        def.count = &cnt->shade64;
+    }
     if (shade)  // resolves the keys too, and in a training frame runs the adjoint
         PR_TRY(launch_shade(dv, n, blk_offs, P.nblk, P.nsub, ws->keys.as<unsigned long long>(), reader_resets,
-                            !P.grads.empty(), cnt, shade_features(P.vd.data(), n), st, P.vd.data()));
+                            !P.grads.empty(), cnt, shade_features(P.vd.data(), n), st, P.vd.data(), pix_offs, def));
     if (shade && P.any_loss)  // the views' loss partial sums into the callers' losses
         PR_TRY(launch_loss_finalize(dv, n, cnt, st));
     // the reader has set every key of the frame back to ~0

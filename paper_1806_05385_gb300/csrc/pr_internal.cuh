@@ -101,9 +101,17 @@ struct Counters {
     unsigned long long hits_listed;               // (triangle, tile) hits appended by the binning count pass
     unsigned long long binned;                    // triangles with candidate tiles, listed by the bound pass
     unsigned long long binned_cand;               // or (CandList::shift > 0): that count and their candidate tiles, packed
+    unsigned long long shade64;                   // pixels the shading left to FP64
     unsigned int status;
     unsigned int depth_err_bits;  // bits of the largest FP32-vs-FP64 relative depth error (re-test)
     __host__ __device__ unsigned long long items_total() const { return items_n[0] + items_n[1] + items_n[2]; }
+};
+
+// The list of pixels that the shading kernels leave to FP64: (batch-wide
+// pixel << 32) | triangle, and their number.
+struct Deferred64 {
+    unsigned long long *list = nullptr;
+    unsigned long long *count = nullptr;
 };
 
 // The list of triangles with candidate tiles and the running sum of their

@@ -103,10 +103,14 @@ int shade_features(const ViewDev *vd, int n);
 // host_views: the host copy of the device table `views` (same contents), or
 // null; with one, a launch of up to kParamViews views passes them as a
 // kernel parameter
+// def.list: pixels that need FP64 are listed there and shaded by a launch of
+// their own (frames of fewer than 2^32 pixels; pix_offs needed), or null:
+// shaded in place
 // blk_offs, nblocks: the views' strips of nsub pixel blocks (strip_blocks)
 cudaError_t launch_shade(const ViewDev *views, int nviews, const long long *blk_offs, long long nblocks, int nsub,
                          unsigned long long *keys, bool reset_keys, bool adjoint, const Counters *frame_cnt, int feat,
-                         cudaStream_t st, const ViewDev *host_views = nullptr);
+                         cudaStream_t st, const ViewDev *host_views = nullptr, const long long *pix_offs = nullptr,
+                         const Deferred64 &def = Deferred64{});
 // a training frame's losses: each view's partial sums (loss_part) added into
 // its loss, once (skipped when the frame's forward overflowed)
 cudaError_t launch_loss_finalize(const ViewDev *views, int nviews, const Counters *frame_cnt, cudaStream_t st);

@@ -466,9 +466,13 @@ __device__ bool hit64(const ViewDev &v, const Shear64 &sh, int tri, double &num,
 // The FP32 sweeps of one pixel run across the warp's lanes (one bin entry
 // each), the pixels one after the other; their FP64 candidates go to a
 // per-warp list in shared memory, grouped by pixel.  FP64 runs at a small
-// fraction of the FP32 rate on this part, so the FP64 tests then run with
-// one lane per pixel, in step across the warp: each FP64 instruction serves
-// up to 32 pixels instead of one candidate.  Candidates that do not fit the
+// fraction of the FP32 rate on this part (an FP64 instruction holds the SM's
+// unit as long for one active lane as for 32), so the FP64 tests then run
+// with one thread per pixel of the CTA, its first threads: each FP64
+// instruction serves up to 32 pixels.  With one lane per pixel in every
+// warp, each warp's few pixels paid for a warp's instructions (1M-triangle
+// stereo frame, 27,800 flagged pixels, six per warp: 0.196 against 0.157
+// ms).  Candidates that do not fit the
 // list are tested at once and kept as the pixel's running best.
 //
 // A bin entry carries a lower bound of the nearest depth its triangle
@@ -519,7 +523,10 @@ __device__ __forceinline__ RetestPixel retest_pixel(const ViewDev *views, int nv
     return px;
 }
 
-__global__ void __launch_bounds__(kRetestWarps * 32) k_retest(const ViewDev *__restrict__ views, int nviews,
+// Bound: the sweeps' chains of dependent loads (the FP64 tests are 0.035 of
+// 0.157 ms at 126 registers, four CTAs per SM), so one wave of eight CTAs per
+// SM at 64 registers: 0.131 ms (two waves of them: 0.146).
+__global__ void __launch_bounds__(kRetestWarps * 32, 8) k_retest(const ViewDev *__restrict__ views, int nviews,
                                                               const long long *__restrict__ pix_offs,
                                                               const unsigned long long *__restrict__ scan,
                                                               const unsigned long long *__restrict__ tile_cnt,
@@ -542,8 +549,9 @@ __global__ void __launch_bounds__(kRetestWarps * 32) k_retest(const ViewDev *__r
     // pixels per warp and round: spread over every warp of the grid (the
     // pixels of a warp run one after the other), at most 32
     const long long per = max(1ll, min(32ll, (nflag + nw - 1) / nw));
-    for (long long f0 = ((long long)blockIdx.x * kRetestWarps + w) * per; f0 < nflag; f0 += nw * per) {
-        const int npx = (int)min(per, nflag - f0);
+    for (long long c0 = (long long)blockIdx.x * kRetestWarps * per; c0 < nflag; c0 += nw * per) {
+        const long long f0 = c0 + w * per;
+        const int npx = (int)max(0ll, min(per, nflag - f0));
         int used = 0;  // list entries in use (the same in every lane)
         for (int q = 0; q < npx; ++q) {
             const RetestPixel px = retest_pixel(views, nviews, pix_offs, scan, tile_cnt, flag_list, f0 + q, cap_pairs);
@@ -620,18 +628,20 @@ __global__ void __launch_bounds__(kRetestWarps * 32) k_retest(const ViewDev *__r
                 s_best[w][q] = ib;
             }
         }
-        __syncwarp();
-        // the listed candidates in FP64, one lane per pixel
-        if (lane < npx) {
-            const RetestPixel px = retest_pixel(views, nviews, pix_offs, scan, tile_cnt, flag_list, f0 + lane,
+        __syncthreads();
+        // the listed candidates in FP64, one thread per pixel of the CTA
+        const int ncta = (int)min(per * kRetestWarps, nflag - c0);
+        if ((int)threadIdx.x < ncta) {
+            const int pw = threadIdx.x / (int)per, pq = threadIdx.x - pw * (int)per;  // its sweep's warp and place
+            const RetestPixel px = retest_pixel(views, nviews, pix_offs, scan, tile_cnt, flag_list, c0 + threadIdx.x,
                                                 cap_pairs);
             const ViewDev &v = *px.v;
-            Hit64 b = s_best[w][lane];
-            const int c0 = s_start[w][lane], c1 = c0 + s_count[w][lane];
-            if (c1 > c0) {
+            Hit64 b = s_best[pw][pq];
+            const int l0 = s_start[pw][pq], l1 = l0 + s_count[pw][pq];
+            if (l1 > l0) {
                 const Shear64 sh = shear64(v, pixel_ray64(v, px.i, px.j));
-                for (int c = c0; c < c1; ++c) {
-                    const unsigned id = s_list[w][c];
+                for (int c = l0; c < l1; ++c) {
+                    const unsigned id = s_list[pw][c];
                     double num, den;
                     if (hit64(v, sh, (int)id, num, den) && better(num, den, id, b))
                         b = Hit64{num, den, id};
@@ -652,7 +662,7 @@ __global__ void __launch_bounds__(kRetestWarps * 32) k_retest(const ViewDev *__r
                 atomicAdd(&cnt->changed, 1ull);
             }
         }
-        __syncwarp();  // the list is reused by the next round
+        __syncthreads();  // the lists are reused by the next round
     }
 }
 

@@ -83,8 +83,11 @@ struct Hit64Out {
 };
 __device__ __noinline__ void pixel_hit64(const ViewDev &v, int i, int j, int ia, int ib, int ic, Hit64Out &o);
 
+// Returns false, with h unfinished, for a pixel that needs FP64 when
+// `defer64` (the caller leaves it to k_shade64).
 template <int kFeat>
-__device__ __forceinline__ void pixel_hit(const ViewDev &v, int i, int j, unsigned id, PixelHit &h)
+__device__ __forceinline__ bool pixel_hit(const ViewDev &v, int i, int j, unsigned id, PixelHit &h,
+                                          bool defer64 = false)
 {
     float x0, x1, dx, dy;
     pixel_ray<(kFeat & kFeatLut) != 0>(v, i, j, x0, x1, h.t, dx, dy);
@@ -134,8 +137,9 @@ __device__ __forceinline__ void pixel_hit(const ViewDev &v, int i, int j, unsign
         const float sm = fmaxf(fabsf(ax) + fabsf(ay), fmaxf(fabsf(bx) + fabsf(by), fabsf(cx) + fabsf(cy)));
         const float zm = fmaxf(fabsf(h.A.z), fmaxf(fabsf(h.B.z), fabsf(h.C.z)));
         const float mag = zm * (1.f + fabsf(dx) + fabsf(dy)) + sm;
-        if (2.f * kRelCoordShade * mag * sm > kBaryRel * fabsf(h.det))
-        {
+        if (2.f * kRelCoordShade * mag * sm > kBaryRel * fabsf(h.det)) {
+            if (defer64)
+                return false;
             Hit64Out o;
             pixel_hit64(v, i, j, h.ia, h.ib, h.ic, o);
             if (o.has_b) {
@@ -169,6 +173,7 @@ __device__ __forceinline__ void pixel_hit(const ViewDev &v, int i, int j, unsign
         h.ndh = dot3(h.n, h.hv);
         h.spec = h.ndh > 0.f ? v.k_s * powf(h.ndh, v.shininess) : 0.f;
     }
+    return true;
 }
 
 __device__ __noinline__ void pixel_hit64(const ViewDev &v, int i, int j, int ia, int ib, int ic, Hit64Out &h)
@@ -179,7 +184,8 @@ __device__ __noinline__ void pixel_hit64(const ViewDev &v, int i, int j, int ia,
     double P[3][3];
     for (int k = 0; k < 3; ++k) {
         const float4 va = v.vtx[2 * vid[k]], vb = v.vtx[2 * vid[k] + 1];
-        const double p[3] = {va.x, va.y, va.z}, e[3] = {p[0] + (double)va.w, p[1] + (double)vb.x, p[2] + (double)vb.y};
+        const double p[3] = {va.x, va.y, va.z},
+                     e[3] = {p[0] + (double)va.w, p[1] + (double)vb.x, p[2] + (double)vb.y};
         for (int r = 0; r < 3; ++r) {
             const double S = (double)v.R0[3 * r] * p[0] + (double)v.R0[3 * r + 1] * p[1] + (double)v.R0[3 * r + 2] * p[2] +
                              (double)v.T0[r];
@@ -438,13 +444,13 @@ struct TriangleSum {
 };
 
 // Adds the block's pixels (valid lanes, triangle id; their numbers in the
-// warp's rows, columns of the other lanes zero) to the running sum,
-// triangle by triangle.  Called by the whole warp.
+// warp's rows) to the running sum, triangle by triangle.  others: lanes that
+// are not valid but whose columns are not zero.  Called by the whole warp.
 __device__ __forceinline__ void sum_block(const ViewDev &v, const float *rows, const ValueLane &vl, bool valid,
-                                          unsigned id, TriangleSum &ts)
+                                          unsigned id, TriangleSum &ts, unsigned others = 0u)
 {
-    const unsigned all = __ballot_sync(0xffffffffu, valid);
-    unsigned rem = all;
+    unsigned rem = __ballot_sync(0xffffffffu, valid);
+    const unsigned all = rem | others;
     const float4 *x4 = reinterpret_cast<const float4 *>(rows + vl.x);
     const float4 *y4 = reinterpret_cast<const float4 *>(rows + vl.y);
     unsigned m = __ballot_sync(0xffffffffu, valid && id == ts.id);  // the running triangle first
@@ -506,11 +512,18 @@ __device__ __forceinline__ bool frame_overflowed(const Counters *frame_cnt)
 // Bound: instruction issue (73 % of peak on 64 views, DRAM 27 %, about 850
 // warp instructions per block that shows a triangle) and, on the background,
 // DRAM writes.
+//
+// def.list (the precision form): pixels whose barycentrics need FP64 are not
+// shaded here but listed for k_shade64.  An FP64 instruction holds the SM's
+// unit as long for one lane as for 32, and the pixels that need it are few
+// and scattered (1M-triangle stereo frame: 290,000 of 9.3 M pixels, most
+// warps with one to three): run in place they took 0.18 of 0.47 ms, listed
+// 0.155.
 template <bool kAdjoint, int kFeat>
 __device__ __forceinline__ void shade_body(const ViewDev *__restrict__ views, int nviews,
                                            const long long *__restrict__ blk_offs, long long nblocks, int nsub,
                                            unsigned long long *__restrict__ keys, int reset_keys,
-                                           const Counters *__restrict__ frame_cnt)
+                                           const Counters *__restrict__ frame_cnt, const Deferred64 def)
 {
     __shared__ unsigned s_id[kShadeWarps][kBlkH * kIdPitch];
     __shared__ __align__(16) float s_rows[kAdjoint ? kShadeWarps : 1][kAdjoint ? kRows * kRowPitch : 4];
@@ -602,31 +615,47 @@ __device__ __forceinline__ void shade_body(const ViewDev *__restrict__ views, in
         const int x = (__ffs(live) - 1) * kBlkW + lane % kBlkW, y = lane / kBlkW;
         const unsigned id = s_id[warp][y * kIdPitch + x];
         const int pi = sp.i0 + x, pj = sp.j0 + y, lin = pj * W + pi;
-        const bool hit = id != 0xFFFFFFFFu;
+        bool hit = id != 0xFFFFFFFFu;
+        // the upstream gradient (or L2 target) does not depend on the hit:
+        // its loads go out first
+        float gin[3] = {0.f, 0.f, 0.f};
+        if (kAdjoint && grad && hit) {
+            if (v.target_u8) {
+                gin[0] = u8_unit(v.target_u8[lin]);
+                gin[1] = u8_unit(v.target_u8[plane + lin]);
+                gin[2] = u8_unit(v.target_u8[2 * plane + lin]);
+            } else {
+                const float *gsrc = v.grad_in ? v.grad_in : v.target;
+                gin[0] = gsrc[lin];
+                gin[1] = gsrc[plane + lin];
+                gin[2] = gsrc[2 * plane + lin];
+            }
+        }
+        PixelHit h;
+        bool later = false;
+        if (hit) {
+            hit = pixel_hit<kFeat>(v, pi, pj, id, h, (kFeat & kFeatF64) && def.list);
+            later = !hit;
+        }
+        if (kFeat & kFeatF64) {
+            const unsigned m = __ballot_sync(0xffffffffu, later);
+            if (m) {
+                unsigned long long base = 0;
+                if (lane == __ffs(m) - 1)
+                    base = atomicAdd(def.count, (unsigned long long)__popc(m));
+                base = __shfl_sync(0xffffffffu, base, __ffs(m) - 1);
+                if (later)
+                    def.list[base + __popc(m & ((1u << lane) - 1u))] =
+                        ((unsigned long long)(v.pix_off + lin) << 32) | id;
+            }
+        }
         if (kAdjoint && grad && !hit) {
 #pragma unroll
             for (int r = 0; r < kRows; ++r)
                 rows[r * kRowPitch + lane] = 0.f;
         }
         if (hit) {
-            // the upstream gradient (or L2 target) does not depend on the
-            // hit: its loads go out first
-            float gin[3] = {0.f, 0.f, 0.f};
-            if (kAdjoint && grad) {
-                if (v.target_u8) {
-                    gin[0] = u8_unit(v.target_u8[lin]);
-                    gin[1] = u8_unit(v.target_u8[plane + lin]);
-                    gin[2] = u8_unit(v.target_u8[2 * plane + lin]);
-                } else {
-                    const float *gsrc = v.grad_in ? v.grad_in : v.target;
-                    gin[0] = gsrc[lin];
-                    gin[1] = gsrc[plane + lin];
-                    gin[2] = gsrc[2 * plane + lin];
-                }
-            }
-            PixelHit h;
             PixelAlbedo pa;
-            pixel_hit<kFeat>(v, pi, pj, id, h);
             pixel_albedo(v, h, pa);
             const float rgb[3] = {fmaf(pa.a[0], h.sigma, h.spec), fmaf(pa.a[1], h.sigma, h.spec),
                                   fmaf(pa.a[2], h.sigma, h.spec)};
@@ -670,18 +699,102 @@ __device__ __forceinline__ void shade_body(const ViewDev *__restrict__ views, in
 template <bool kAdjoint, int kFeat>
 __global__ void __launch_bounds__(kShadeThreads, shade_ctas(kFeat))
     k_shade(const ViewDev *__restrict__ views, int nviews, const long long *__restrict__ blk_offs, long long nblocks, int nsub,
-            unsigned long long *__restrict__ keys, int reset_keys, const Counters *__restrict__ frame_cnt)
+            unsigned long long *__restrict__ keys, int reset_keys, const Counters *__restrict__ frame_cnt,
+            const Deferred64 def)
 {
-    shade_body<kAdjoint, kFeat>(views, nviews, blk_offs, nblocks, nsub, keys, reset_keys, frame_cnt);
+    shade_body<kAdjoint, kFeat>(views, nviews, blk_offs, nblocks, nsub, keys, reset_keys, frame_cnt, def);
 }
 
 template <bool kAdjoint, int kFeat>
 __global__ void __launch_bounds__(kShadeThreads, shade_ctas(kFeat))
     k_shade_pv(const __grid_constant__ ParamViews pv, int nviews, const long long *__restrict__ blk_offs,
                long long nblocks, int nsub, unsigned long long *__restrict__ keys, int reset_keys,
-               const Counters *__restrict__ frame_cnt)
+               const Counters *__restrict__ frame_cnt, const Deferred64 def)
 {
-    shade_body<kAdjoint, kFeat>(pv.v, nviews, blk_offs, nblocks, nsub, keys, reset_keys, frame_cnt);
+    shade_body<kAdjoint, kFeat>(pv.v, nviews, blk_offs, nblocks, nsub, keys, reset_keys, frame_cnt, def);
+}
+
+// The pixels that the shading kernels left to FP64, one lane each, so that
+// every FP64 instruction serves 32 of them: the same pixel hit with its FP64
+// path, colour, loss and adjoint.  Bound: the FP64 unit (225 FP64
+// instructions per pixel at about 18 cycles of the SM per warp instruction:
+// 0.120 of 0.155 ms for 290,000 pixels).  A warp's pixels are neighbours in the
+// list, so most share a few triangles, summed as in the shading kernels
+// (27 atomics per pixel instead: 0.287 against 0.155 ms for 290,000 pixels).
+constexpr int kShade64Threads = 128, kShade64Ctas = 4;
+template <bool kAdjoint, int kFeat>
+__global__ void __launch_bounds__(kShade64Threads, kShade64Ctas)
+    k_shade64(const ViewDev *__restrict__ views, int nviews, const long long *__restrict__ pix_offs,
+              const Counters *__restrict__ frame_cnt, const Deferred64 def)
+{
+    __shared__ __align__(16) float s_rows[kAdjoint ? kShade64Threads / 32 : 1][kAdjoint ? kRows * kRowPitch : 4];
+    const long long n = (long long)*def.count;
+    const bool adjoint = kAdjoint && !frame_overflowed(frame_cnt);
+    const int lane = threadIdx.x & 31;
+    float *rows = s_rows[kAdjoint ? threadIdx.x >> 5 : 0];
+    const ValueLane vl = value_lane();
+    for (long long k0 = (long long)blockIdx.x * kShade64Threads + (threadIdx.x & ~31); k0 < n;
+         k0 += (long long)gridDim.x * kShade64Threads) {
+        int q = -1;  // the view of the lane's pixel, if it takes part in the adjoint
+        unsigned id = 0xFFFFFFFFu;
+        if (k0 + lane < n) {
+            const unsigned long long e = def.list[k0 + lane];
+            const long long g = (long long)(e >> 32);
+            id = (unsigned)e;
+            const int vq = find_view(pix_offs, nviews, g);
+            const ViewDev &v = views[vq];
+            const int lin = (int)(g - v.pix_off), plane = v.W * v.H, pj = lin / v.W, pi = lin - pj * v.W;
+            PixelHit h;
+            PixelAlbedo pa;
+            pixel_hit<kFeat>(v, pi, pj, id, h);
+            pixel_albedo(v, h, pa);
+            const float rgb[3] = {fmaf(pa.a[0], h.sigma, h.spec), fmaf(pa.a[1], h.sigma, h.spec),
+                                  fmaf(pa.a[2], h.sigma, h.spec)};
+            if (v.rgb_out) {
+                v.rgb_out[lin] = rgb[0];
+                v.rgb_out[plane + lin] = rgb[1];
+                v.rgb_out[2 * plane + lin] = rgb[2];
+            }
+            if (kAdjoint && adjoint && (v.grad_in || v.target || v.target_u8)) {
+                q = vq;
+                float gin[3];
+#pragma unroll
+                for (int c = 0; c < 3; ++c) {
+                    if (v.grad_in) {
+                        gin[c] = v.grad_in[c * plane + lin];
+                    } else {
+                        const float t = v.target_u8 ? u8_unit(v.target_u8[c * plane + lin]) : v.target[c * plane + lin];
+                        gin[c] = 2.f * (rgb[c] - t);
+                    }
+                }
+                if (v.loss)  // sum (rgb - target)^2
+                    atomicAdd(&v.loss_part[(unsigned)(k0 + lane) & (kLossSlots - 1)],
+                              0.25f * fmaf(gin[0], gin[0], fmaf(gin[1], gin[1], gin[2] * gin[2])));
+                adjoint_rows<kFeat>(v, h, pa, gin[0], gin[1], gin[2], rows + lane);
+            }
+        }
+        if (kAdjoint && adjoint) {
+            if (q < 0) {
+#pragma unroll
+                for (int r = 0; r < kRows; ++r)
+                    rows[r * kRowPitch + lane] = 0.f;
+            }
+            __syncwarp();
+            unsigned rem = __ballot_sync(0xffffffffu, q >= 0);
+            const unsigned all = rem;
+            while (rem) {  // view by view
+                const int vq = __shfl_sync(0xffffffffu, q, __ffs(rem) - 1);
+                const unsigned m = __ballot_sync(0xffffffffu, q == vq);
+                TriangleSum ts;
+                ts.s = 0.f;
+                ts.id = 0xFFFFFFFFu;
+                sum_block(views[vq], rows, vl, q == vq, id, ts, all & ~m);
+                add_triangle(views[vq], ts.id, ts.s);
+                rem &= ~m;
+            }
+            __syncwarp();  // the rows are written again by the next round
+        }
+    }
 }
 
 // A training frame's losses: one block per view sums the view's partial
@@ -735,43 +848,47 @@ static const ParamViews *param_views(const ViewDev *host_views, int nviews)
 template <bool kAdjoint, int kFeat>
 static void launch_shade_one(unsigned g, const ViewDev *views, const ParamViews *pv, int nviews,
                              const long long *blk_offs, long long nblocks, int nsub, unsigned long long *keys,
-                             int reset_keys, const Counters *frame_cnt, cudaStream_t st)
+                             int reset_keys, const Counters *frame_cnt, const Deferred64 &def, cudaStream_t st)
 {
     if (pv)
         k_shade_pv<kAdjoint, kFeat><<<g, kShadeThreads, 0, st>>>(*pv, nviews, blk_offs, nblocks, nsub, keys, reset_keys,
-                                                                 frame_cnt);
+                                                                 frame_cnt, def);
     else
         k_shade<kAdjoint, kFeat><<<g, kShadeThreads, 0, st>>>(views, nviews, blk_offs, nblocks, nsub, keys, reset_keys,
-                                                              frame_cnt);
+                                                              frame_cnt, def);
 }
 
 template <bool kAdjoint>
 static void launch_shade_t(int feat, unsigned g, const ViewDev *views, const ParamViews *pv, int nviews,
                            const long long *blk_offs, long long nblocks, int nsub, unsigned long long *keys, int reset_keys,
-                           const Counters *frame_cnt, cudaStream_t st)
+                           const Counters *frame_cnt, const Deferred64 &def, cudaStream_t st)
 {
     if (feat == kFeatF64) {  // the precision form without the specular and sampled-foveation paths
-        launch_shade_one<kAdjoint, kFeatF64>(g, views, pv, nviews, blk_offs, nblocks, nsub, keys, reset_keys, frame_cnt, st);
+        launch_shade_one<kAdjoint, kFeatF64>(g, views, pv, nviews, blk_offs, nblocks, nsub, keys, reset_keys, frame_cnt,
+                                             def, st);
         return;
     }
     if (feat & kFeatF64) {  // the precision form with either: one variant with every path (same bits)
         launch_shade_one<kAdjoint, kFeatSpec | kFeatLut | kFeatF64>(g, views, pv, nviews, blk_offs, nblocks, nsub, keys,
-                                                                    reset_keys, frame_cnt, st);
+                                                                    reset_keys, frame_cnt, def, st);
         return;
     }
     switch (feat) {
     case 0:
-        launch_shade_one<kAdjoint, 0>(g, views, pv, nviews, blk_offs, nblocks, nsub, keys, reset_keys, frame_cnt, st);
+        launch_shade_one<kAdjoint, 0>(g, views, pv, nviews, blk_offs, nblocks, nsub, keys, reset_keys, frame_cnt,
+                                             def, st);
         break;
     case kFeatSpec:
-        launch_shade_one<kAdjoint, kFeatSpec>(g, views, pv, nviews, blk_offs, nblocks, nsub, keys, reset_keys, frame_cnt, st);
+        launch_shade_one<kAdjoint, kFeatSpec>(g, views, pv, nviews, blk_offs, nblocks, nsub, keys, reset_keys, frame_cnt,
+                                             def, st);
         break;
     case kFeatLut:
-        launch_shade_one<kAdjoint, kFeatLut>(g, views, pv, nviews, blk_offs, nblocks, nsub, keys, reset_keys, frame_cnt, st);
+        launch_shade_one<kAdjoint, kFeatLut>(g, views, pv, nviews, blk_offs, nblocks, nsub, keys, reset_keys, frame_cnt,
+                                             def, st);
         break;
     default:
         launch_shade_one<kAdjoint, kFeatSpec | kFeatLut>(g, views, pv, nviews, blk_offs, nblocks, nsub, keys, reset_keys,
-                                                         frame_cnt, st);
+                                                         frame_cnt, def, st);
     }
 }
 
@@ -789,17 +906,44 @@ int shade_features(const ViewDev *vd, int n)
     return f;
 }
 
+template <bool kAdjoint>
+static void launch_shade64(int feat, const ViewDev *views, int nviews, const long long *pix_offs,
+                           const Counters *frame_cnt, const Deferred64 &def, cudaStream_t st)
+{
+    static int grid = 0;
+    if (grid == 0) {
+        int dev = 0, sms = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        grid = sms * kShade64Ctas;
+    }
+    if (feat == kFeatF64)
+        k_shade64<kAdjoint, kFeatF64><<<grid, kShade64Threads, 0, st>>>(views, nviews, pix_offs, frame_cnt, def);
+    else
+        k_shade64<kAdjoint, kFeatSpec | kFeatLut | kFeatF64>
+            <<<grid, kShade64Threads, 0, st>>>(views, nviews, pix_offs, frame_cnt, def);
+}
+
 cudaError_t launch_shade(const ViewDev *views, int nviews, const long long *blk_offs, long long nblocks, int nsub,
                          unsigned long long *keys, bool reset_keys, bool adjoint, const Counters *frame_cnt, int feat,
-                         cudaStream_t st, const ViewDev *host_views)
+                         cudaStream_t st, const ViewDev *host_views, const long long *pix_offs,
+                         const Deferred64 &def)
 {
     if (nblocks > 0) {
         const unsigned g = shade_grid(nblocks);
         const ParamViews *pv = param_views(host_views, nviews);
         if (adjoint)
-            launch_shade_t<true>(feat, g, views, pv, nviews, blk_offs, nblocks, nsub, keys, reset_keys, frame_cnt, st);
+            launch_shade_t<true>(feat, g, views, pv, nviews, blk_offs, nblocks, nsub, keys, reset_keys, frame_cnt, def,
+                                 st);
         else
-            launch_shade_t<false>(feat, g, views, pv, nviews, blk_offs, nblocks, nsub, keys, reset_keys, frame_cnt, st);
+            launch_shade_t<false>(feat, g, views, pv, nviews, blk_offs, nblocks, nsub, keys, reset_keys, frame_cnt, def,
+                                  st);
+        if ((feat & kFeatF64) && def.list) {
+            if (adjoint)
+                launch_shade64<true>(feat, views, nviews, pix_offs, frame_cnt, def, st);
+            else
+                launch_shade64<false>(feat, views, nviews, pix_offs, frame_cnt, def, st);
+        }
     }
     return cudaGetLastError();
 }
