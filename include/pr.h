@@ -123,7 +123,8 @@ typedef struct {
     int32_t bound;        /* pr_bound */
     int32_t tile;         /* bin tile side in pixels: 8, 16 or 32; 0 = library default (16) */
     int32_t fp64_retest;  /* 1: re-test fragments flagged by the FP32 error bound in FP64 */
-    int32_t seg;          /* triangles per fragment work item; 0 = default (256), at most 1024 */
+    int32_t seg;          /* triangles per fragment work item, at most 1024; 0 = default (256, or fewer in
+                             a frame with too few bin entries to fill the GPU so) */
     int32_t fov_bound;    /* pr_fov_bound.  SIMPLE and RECURSIVE rest on the paper's assumption that
                              an edge's displacement is unimodal (ternary search); the library seeds
                              the search with a coarse scan and adds half a pixel, but they are not

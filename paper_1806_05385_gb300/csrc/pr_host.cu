@@ -441,6 +441,7 @@ struct BatchPlan {
     bool any_fp64 = false;
     bool any_paper_fov = false;  // some foveated view asks for the paper's edge bound
     bool any_loss = false;       // some view of a training frame accumulates its loss
+    bool any_seg = false;        // the caller left the run length to the library
     double max_cand = 0;         // no frame has more candidate (triangle, tile) pairs: sum of T x tiles
     std::vector<Cls> classes;
     // output staging: per view (in order) device pointers used by kernels
@@ -717,10 +718,12 @@ pr_status enqueue_batch(pr_workspace *ws, BatchPlan &P, int seg, bool shade, cud
     io.ncls = (int)P.classes.size();
     for (int c = 0; c < io.ncls; ++c)
         io.cls_end[c] = P.classes[c].tile_hi;
-    PR_TRY(launch_tile_alloc(tile_cnt, scan, ws->fill.as<unsigned>(), P.ntiles, seg, cnt, io, st));
+    // (the precision form keeps long runs: shorter ones see fewer nearer
+    // triangles, and so flag more pixels)
+    PR_TRY(launch_tile_alloc(tile_cnt, scan, ws->fill.as<unsigned>(), P.ntiles, seg, P.any_seg && !P.any_fp64, cnt, io,
+                             st));
     PR_TRY(launch_bin_scatter(ws->hit_entry.as<unsigned long long>(), ws->hit_tile.as<unsigned>(),
-                              ws->fill.as<unsigned>(), ws->pairs.as<unsigned long long>(), ws->cap_pairs, P.ntiles, cnt,
-                              st));
+                              ws->fill.as<unsigned>(), ws->pairs.as<unsigned long long>(), io, P.ntiles, cnt, st));
     PR_TRY(launch_sort_items(io, P.ntiles, seg, ws->pairs.as<unsigned long long>(), cnt, st));
     PR_TRY(mark(2));
     int *heads = ws->heads.as<int>();
@@ -808,6 +811,7 @@ pr_status run_batch(pr_workspace *ws, const pr_batch_view *views, int n, const p
 {
     pr_params prm = default_params(params);
     BatchPlan P;
+    P.any_seg = !params || params->seg <= 0;
     pr_status s = plan_batch(views, n, prm, P, grads);
     if (s != PR_OK)
         return s;
@@ -830,7 +834,7 @@ pr_status run_batch(pr_workspace *ws, const pr_batch_view *views, int n, const p
         ws->cap_pairs = std::max<long long>(ws->cap_pairs, (long long)c.pairs_total + 1024);
         ws->cap_pairs = std::min(ws->cap_pairs + ws->cap_pairs / 4, kMaxPairs);  // size_workspace grows both to these
         const long long items =
-            (long long)std::max(c.items_n[0], std::max(c.items_n[1], c.items_n[2])) + 1024;
+            (long long)std::max(c.items_n(0), std::max(c.items_n(1), c.items_n(2))) + 1024;
         if (items > ws->cap_items)
             ws->want_items = std::min(items + items / 4, kMaxPairs);
     }
@@ -1323,6 +1327,7 @@ pr_status pr_graph_capture_frame(pr_workspace *ws, const pr_batch_view *views, i
         return s;
     pr_params prm = default_params(params);
     BatchPlan P;
+    P.any_seg = !params || params->seg <= 0;
     s = plan_batch(views, n, prm, P, grads);
     if (s != PR_OK)
         return s;

@@ -97,14 +97,16 @@ constexpr int kMaxClasses = 3;  // tile sizes (8, 16, 32): a frame's fragment la
 struct Counters {
     unsigned long long tests, hits, culled, flagged, changed;
     unsigned long long pairs_total;               // bin entries handed out to the tiles
-    unsigned long long items_n[kMaxClasses];      // work items per tile-size class
+    unsigned long long items_long[kMaxClasses];   // work items per tile-size class: long runs, the rest
+    unsigned long long items_rest[kMaxClasses];
     unsigned long long hits_listed;               // (triangle, tile) hits appended by the binning count pass
     unsigned long long binned;                    // triangles with candidate tiles, listed by the bound pass
     unsigned long long binned_cand;               // or (CandList::shift > 0): that count and their candidate tiles, packed
     unsigned long long shade64;                   // pixels the shading left to FP64
     unsigned int status;
     unsigned int depth_err_bits;  // bits of the largest FP32-vs-FP64 relative depth error (re-test)
-    __host__ __device__ unsigned long long items_total() const { return items_n[0] + items_n[1] + items_n[2]; }
+    __host__ __device__ unsigned long long items_n(int c) const { return items_long[c] + items_rest[c]; }
+    __host__ __device__ unsigned long long items_total() const { return items_n(0) + items_n(1) + items_n(2); }
 };
 
 // The list of pixels that the shading kernels leave to FP64: (batch-wide
@@ -113,6 +115,14 @@ struct Deferred64 {
     unsigned long long *list = nullptr;
     unsigned long long *count = nullptr;
 };
+
+// Place of item k of a class in its array of cap items: the long runs first,
+// from the front, the others from the back, so that both are written without
+// knowing the other's number.
+__host__ __device__ __forceinline__ long long item_place(long long k, long long nlong, long long cap)
+{
+    return k < nlong ? k : cap - 1 - (k - nlong);
+}
 
 // The list of triangles with candidate tiles and the running sum of their
 // candidate counts (the index space of the binning pass).  shift > 0: the

@@ -45,7 +45,8 @@ cudaError_t launch_bin_count(const ViewDev *views, int nviews, const long long *
                              const float4 *tile_box, unsigned long long *tile_cnt, unsigned long long *hit_entry,
                              unsigned *hit_tile, long long cap_pairs, Counters *cnt, cudaStream_t st);
 // Where the fragment stage's work items go: class c (the tiles before
-// cls_end[c], after the previous class's) to items[c cap_items ..].
+// cls_end[c], after the previous class's) to items[c cap_items ..]
+// (item_place).
 struct ItemsOut {
     const ViewDev *views = nullptr;
     int nviews = 0;
@@ -55,11 +56,14 @@ struct ItemsOut {
     int ncls = 0;
     long long cls_end[kMaxClasses] = {};
 };
-// every tile's place in the bins (off, and cursor for the scatter) and its work items
+// every tile's place in the bins (off, and cursor for the scatter) and its
+// work items: runs of at most seg entries (any_seg: or fewer, where the frame
+// has too few entries to give every resident CTA some)
 cudaError_t launch_tile_alloc(const unsigned long long *tile_cnt, unsigned long long *off, unsigned *cursor,
-                              long long ntiles, int seg, Counters *cnt, const ItemsOut &io, cudaStream_t st);
+                              long long ntiles, int seg, bool any_seg, Counters *cnt, const ItemsOut &io,
+                              cudaStream_t st);
 cudaError_t launch_bin_scatter(const unsigned long long *hit_entry, const unsigned *hit_tile, unsigned *cursor,
-                               unsigned long long *pairs, long long cap_pairs, long long ntiles, Counters *cnt,
+                               unsigned long long *pairs, const ItemsOut &io, long long ntiles, Counters *cnt,
                                cudaStream_t st);
 // the list's offsets from the counts (list.shift = 0); the caller cleared
 // the state's ticket and flags (state[0, scan_state_words))

@@ -1163,8 +1163,12 @@ __global__ void __launch_bounds__(256) k_bin_scatter(const unsigned long long *_
                                                      const unsigned *__restrict__ hit_tile,
                                                      unsigned int *__restrict__ cursor,
                                                      unsigned long long *__restrict__ pairs, long long cap_pairs,
-                                                     long long ntiles, Counters *cnt)
+                                                     long long cap_items, long long ntiles, Counters *cnt)
 {
+    // a class's items are written from both ends of its array: too many of
+    // them together have overwritten each other
+    if (blockIdx.x == 0 && threadIdx.x < kMaxClasses && cnt->items_n(threadIdx.x) > (unsigned long long)cap_items)
+        atomicOr(&cnt->status, ST_OVERFLOW_ITEMS);
     const long long n = min((long long)cnt->hits_listed, cap_pairs);
     const int lane = threadIdx.x & 31;
     const long long stride = (long long)gridDim.x * blockDim.x;
@@ -1195,109 +1199,6 @@ __global__ void __launch_bounds__(256) k_bin_scatter(const unsigned long long *_
     }
 }
 
-// Places in the bins.  Bins need no order among the tiles, so a CTA of 256
-// tiles takes its stretch of the bin buffer and of each class's work items
-// with one atomic each, instead of a scan over all tiles (stereo HMD frame,
-// 18,000 tiles: the scan's five CTAs with eight tiles per thread and a chain
-// of look-backs took 12-13 us).  Each tile's bin is cut into runs of at most
-// seg triangles, item = (view, tile in view, first entry, end entry).  Runs
-// past the bin buffer (its scatter overflowed) are clamped to it, so the
-// frame stays in bounds; the overflow status reruns it.
-constexpr int kAllocThreads = 256;
-__global__ void __launch_bounds__(kAllocThreads) k_tile_alloc(const unsigned long long *__restrict__ tile_cnt,
-                                                              unsigned long long *__restrict__ off_out,
-                                                              unsigned *__restrict__ cursor, long long ntiles,
-                                                              int seg, Counters *cnt, const ItemsOut io)
-{
-    __shared__ unsigned long long s_n[kAllocThreads / 32];
-    __shared__ unsigned s_it[kMaxClasses][kAllocThreads / 32];
-    __shared__ unsigned long long s_pairs;              // the CTA's first bin entry
-    __shared__ unsigned long long s_items[kMaxClasses];  // its first item of each class
-    const long long g = (long long)blockIdx.x * kAllocThreads + threadIdx.x;
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const unsigned long long n = g < ntiles ? tile_cnt[g] : 0ull;
-    // a 32-bit division where the count allows it
-    const unsigned nit = n <= 0x7FFFFFFFull ? ((unsigned)n + (unsigned)seg - 1u) / (unsigned)seg
-                                            : (unsigned)((n + seg - 1) / seg);
-    const int cls = (io.ncls > 1 && g >= io.cls_end[0]) + (io.ncls > 2 && g >= io.cls_end[1]);
-    unsigned long long inc = n;  // entries and items (of its class) up to this lane
-    unsigned iit[kMaxClasses];
-#pragma unroll
-    for (int c = 0; c < kMaxClasses; ++c)
-        iit[c] = cls == c ? nit : 0u;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const unsigned long long y = __shfl_up_sync(0xffffffffu, inc, o);
-        if (lane >= o)
-            inc += y;
-#pragma unroll
-        for (int c = 0; c < kMaxClasses; ++c) {
-            if (c >= io.ncls)
-                break;
-            const unsigned z = __shfl_up_sync(0xffffffffu, iit[c], o);
-            if (lane >= o)
-                iit[c] += z;
-        }
-    }
-    if (lane == 31) {
-        s_n[w] = inc;
-#pragma unroll
-        for (int c = 0; c < kMaxClasses; ++c)
-            s_it[c][w] = iit[c];
-    }
-    __syncthreads();
-    if (threadIdx.x <= kMaxClasses) {  // thread 0: the entries, thread 1 + c: the items of class c
-        unsigned long long sum = 0;
-#pragma unroll
-        for (int k = 0; k < kAllocThreads / 32; ++k)
-            sum += threadIdx.x == 0 ? s_n[k] : (unsigned long long)s_it[threadIdx.x - 1][k];
-        unsigned long long base = 0;
-        if (sum)
-            base = atomicAdd(threadIdx.x == 0 ? &cnt->pairs_total : &cnt->items_n[threadIdx.x - 1], sum);
-        if (threadIdx.x == 0)
-            s_pairs = base;
-        else
-            s_items[threadIdx.x - 1] = base;
-    }
-    __syncthreads();
-    if (g >= ntiles)
-        return;
-    long long off = (long long)(s_pairs + inc - n);
-    long long ioff = (long long)s_items[cls] - nit;
-#pragma unroll
-    for (int c = 0; c < kMaxClasses; ++c)
-        if (cls == c)
-            ioff += iit[c];
-    for (int k = 0; k < w; ++k) {
-        off += (long long)s_n[k];
-        ioff += s_it[cls][k];
-    }
-    off_out[g] = (unsigned long long)off;
-    cursor[g] = (unsigned)off;
-    if (n == 0)
-        return;
-    const int vi = find_view(io.tile_offs, io.nviews, g);
-    const int lt = (int)(g - io.views[vi].tile_off);
-    int4 *items = io.items + (long long)cls * io.cap_items;
-    for (unsigned q = 0; q < nit; ++q) {
-        const long long b0 = min(off + (long long)q * seg, io.cap_pairs),
-                        b1 = min(off + min((long long)n, ((long long)q + 1) * seg), io.cap_pairs);
-        if (ioff + q < io.cap_items)
-            items[ioff + q] = make_int4(vi, lt, (int)b0, (int)b1);
-        else
-            atomicOr(&cnt->status, ST_OVERFLOW_ITEMS);
-    }
-}
-
-cudaError_t launch_tile_alloc(const unsigned long long *tile_cnt, unsigned long long *off, unsigned *cursor,
-                              long long ntiles, int seg, Counters *cnt, const ItemsOut &io, cudaStream_t st)
-{
-    if (ntiles > 0)
-        k_tile_alloc<<<(unsigned)((ntiles + kAllocThreads - 1) / kAllocThreads), kAllocThreads, 0, st>>>(
-            tile_cnt, off, cursor, ntiles, seg, cnt, io);
-    return cudaGetLastError();
-}
-
 static int sm_count()
 {
     static int n = 0;
@@ -1308,6 +1209,156 @@ static int sm_count()
         n = sms > 0 ? sms : 1;
     }
     return n;
+}
+
+// Places in the bins.  Bins need no order among the tiles, so a CTA of 256
+// tiles takes its stretch of the bin buffer and of each class's work items
+// with one atomic each, instead of a scan over all tiles (stereo HMD frame,
+// 18,000 tiles: the scan's five CTAs with eight tiles per thread and a chain
+// of look-backs took 12-13 us).  Each tile's bin is cut into runs of at most
+// seg triangles, item = (view, tile column | row << 16, first entry, end
+// entry).  Runs past the bin buffer (its scatter overflowed) are clamped to
+// it, so the frame stays in bounds; the overflow status reruns it.
+//
+// Length of the runs.  A warp of the fragment stage tests a run's triangles
+// one after the other, some 0.2-0.3 us each, so a frame's longest run bounds
+// the stage from below (256 triangles: about 60 us) and a long run that
+// starts last is waited for.  Two measures.  Runs of kLongRun triangles or
+// more come first in the queue (32 and 128: the same).  And with any_seg runs
+// are cut to a power of two, at least 32, near the larger of entries / (2
+// spread), two runs for every resident CTA (spread of them), and twice the
+// mean bin (of spread tiles at least): shorter ones cost tests, since every
+// run starts without the nearer triangles of the others (HMD frame, 256 /
+// 128 / 64 / 32: 12.1 / 12.9 / 18.0 / 29.3 M tests), so only frames with idle
+// CTAs and bins far above the mean are cut.  Fragment stage, runs of 256 in
+// tile order / long runs first / cut too: 256^2 frame 26.7 / 26.5 / 13.2 us,
+// odd-sized eye 35 / 33 / 25, lens eye 52 / 50 / 37, 8 views 85 / 77 / 64, HMD
+// frame 91 / 75 / 73, 1M triangles 252 / 211 / 211; 512^2 frame of even bins 18
+// to 20 either way, 25 if cut to 64.
+constexpr int kAllocThreads = 256;
+constexpr int kMinSeg = 32, kLongRun = 64;
+__global__ void __launch_bounds__(kAllocThreads) k_tile_alloc(const unsigned long long *__restrict__ tile_cnt,
+                                                              unsigned long long *__restrict__ off_out,
+                                                              unsigned *__restrict__ cursor, long long ntiles,
+                                                              int seg, int spread, Counters *cnt, const ItemsOut io)
+{
+    __shared__ unsigned long long s_n[kAllocThreads / 32];
+    __shared__ unsigned s_it[2 * kMaxClasses][kAllocThreads / 32];  // long runs, the others, per class
+    __shared__ unsigned long long s_pairs;                           // the CTA's first bin entry
+    __shared__ unsigned long long s_items[2 * kMaxClasses];          // its first items
+    if (spread) {
+        const unsigned long long per = max(cnt->hits_listed / (2u * (unsigned)spread),
+                                           2ull * cnt->hits_listed / (unsigned long long)max(ntiles, (long long)spread));
+        int s = kMinSeg;
+        while (s < seg && 2ull * s <= per)
+            s *= 2;
+        // as long as the items fit: ntiles + entries / s of them at most
+        while (s < seg && (unsigned long long)ntiles + cnt->hits_listed / s > (unsigned long long)io.cap_items)
+            s *= 2;
+        seg = min(s, seg);
+    }
+    const int long_run = min(kLongRun, seg);
+    const long long g = (long long)blockIdx.x * kAllocThreads + threadIdx.x;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const unsigned long long n = g < ntiles ? tile_cnt[g] : 0ull;
+    // whole runs are long; the last, shorter one may be
+    unsigned whole, tail;  // a 32-bit division where the count allows it
+    if (n <= 0xFFFFFFFFull) {
+        whole = (unsigned)n / (unsigned)seg;
+        tail = (unsigned)n - whole * (unsigned)seg;
+    } else {
+        whole = (unsigned)(n / (unsigned)seg);
+        tail = (unsigned)(n - (unsigned long long)whole * (unsigned)seg);
+    }
+    const unsigned nit = whole + (tail != 0u);
+    const unsigned nlong = whole + (tail >= (unsigned)long_run);
+    const int cls = (io.ncls > 1 && g >= io.cls_end[0]) + (io.ncls > 2 && g >= io.cls_end[1]);
+    unsigned long long inc = n;  // entries, and runs of each kind and class, up to this lane
+    unsigned iit[2 * kMaxClasses];
+#pragma unroll
+    for (int c = 0; c < kMaxClasses; ++c) {
+        iit[2 * c] = cls == c ? nlong : 0u;
+        iit[2 * c + 1] = cls == c ? nit - nlong : 0u;
+    }
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned long long y = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o)
+            inc += y;
+#pragma unroll
+        for (int c = 0; c < 2 * kMaxClasses; ++c) {
+            if (c >= 2 * io.ncls)
+                break;
+            const unsigned z = __shfl_up_sync(0xffffffffu, iit[c], o);
+            if (lane >= o)
+                iit[c] += z;
+        }
+    }
+    if (lane == 31) {
+        s_n[w] = inc;
+#pragma unroll
+        for (int c = 0; c < 2 * kMaxClasses; ++c)
+            s_it[c][w] = iit[c];
+    }
+    __syncthreads();
+    if (threadIdx.x <= 2 * kMaxClasses) {  // thread 0: the entries, thread 1 + c: the runs of one kind and class
+        const int c = threadIdx.x - 1;
+        unsigned long long sum = 0;
+#pragma unroll
+        for (int k = 0; k < kAllocThreads / 32; ++k)
+            sum += c < 0 ? s_n[k] : (unsigned long long)s_it[c][k];
+        unsigned long long base = 0;
+        if (sum)
+            base = atomicAdd(c < 0 ? &cnt->pairs_total : (c & 1 ? &cnt->items_rest[c >> 1] : &cnt->items_long[c >> 1]),
+                             sum);
+        if (c < 0)
+            s_pairs = base;
+        else
+            s_items[c] = base;
+    }
+    __syncthreads();
+    if (g >= ntiles)
+        return;
+    long long off = (long long)(s_pairs + inc - n);
+    long long olong = (long long)s_items[2 * cls] - nlong, orest = (long long)s_items[2 * cls + 1] - (nit - nlong);
+#pragma unroll
+    for (int c = 0; c < kMaxClasses; ++c)
+        if (cls == c) {
+            olong += iit[2 * c];
+            orest += iit[2 * c + 1];
+        }
+    for (int k = 0; k < w; ++k) {
+        off += (long long)s_n[k];
+        olong += s_it[2 * cls][k];
+        orest += s_it[2 * cls + 1][k];
+    }
+    off_out[g] = (unsigned long long)off;
+    cursor[g] = (unsigned)off;
+    if (n == 0)
+        return;
+    const int vi = find_view(io.tile_offs, io.nviews, g);
+    const ViewDev &v = io.views[vi];
+    const int lt = (int)(g - v.tile_off), ty = lt / v.tiles_x, tx = lt - ty * v.tiles_x;
+    int4 *items = io.items + (long long)cls * io.cap_items;
+    for (unsigned q = 0; q < nit; ++q) {
+        const long long b0 = min(off + (long long)q * seg, io.cap_pairs),
+                        b1 = min(off + min((long long)n, ((long long)q + 1) * seg), io.cap_pairs);
+        const long long at = q < nlong ? olong + q : io.cap_items - 1 - orest;  // one run at most is not long
+        if (at >= 0 && at < io.cap_items)
+            items[at] = make_int4(vi, tx | (ty << 16), (int)b0, (int)b1);
+        else
+            atomicOr(&cnt->status, ST_OVERFLOW_ITEMS);
+    }
+}
+
+cudaError_t launch_tile_alloc(const unsigned long long *tile_cnt, unsigned long long *off, unsigned *cursor,
+                              long long ntiles, int seg, bool any_seg, Counters *cnt, const ItemsOut &io,
+                              cudaStream_t st)
+{
+    if (ntiles > 0)
+        k_tile_alloc<<<(unsigned)((ntiles + kAllocThreads - 1) / kAllocThreads), kAllocThreads, 0, st>>>(
+            tile_cnt, off, cursor, ntiles, seg, any_seg ? sm_count() * 7 : 0, cnt, io);
+    return cudaGetLastError();
 }
 
 // k_bin_scatter: one wave of 256-thread CTAs (8 per SM)
@@ -1334,11 +1385,11 @@ cudaError_t launch_bin_count(const ViewDev *views, int nviews, const long long *
 }
 
 cudaError_t launch_bin_scatter(const unsigned long long *hit_entry, const unsigned *hit_tile, unsigned *cursor,
-                               unsigned long long *pairs, long long cap_pairs, long long ntiles, Counters *cnt,
+                               unsigned long long *pairs, const ItemsOut &io, long long ntiles, Counters *cnt,
                                cudaStream_t st)
 {
-    const int grid = (int)std::min<long long>(bin_grid(), (cap_pairs + 255) / 256);
-    k_bin_scatter<<<grid, 256, 0, st>>>(hit_entry, hit_tile, cursor, pairs, cap_pairs, ntiles, cnt);
+    const int grid = (int)std::min<long long>(bin_grid(), (io.cap_pairs + 255) / 256);
+    k_bin_scatter<<<grid, 256, 0, st>>>(hit_entry, hit_tile, cursor, pairs, io.cap_pairs, io.cap_items, ntiles, cnt);
     return cudaGetLastError();
 }
 
@@ -1706,14 +1757,15 @@ __global__ void __launch_bounds__(kSortWarps * 32) k_sort_items(const int4 *__re
     __shared__ unsigned s_gid[kSortWarps][kSortRegMax];
     __shared__ unsigned long long s_run[kSortWarps][kLong ? kMaxSeg : 1];
     // the classes' items one after the other
-    const long long n0 = min((long long)cnt->items_n[0], cap_items), n1 = min((long long)cnt->items_n[1], cap_items),
-                    n2 = min((long long)cnt->items_n[2], cap_items);
+    const long long n0 = (long long)cnt->items_n(0), n1 = (long long)cnt->items_n(1), n2 = (long long)cnt->items_n(2);
     const long long nitems = n0 + n1 + n2;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     unsigned long long *run = s_run[w];
     const long long nwarps = (long long)gridDim.x * kSortWarps;
     for (long long it = (long long)blockIdx.x * kSortWarps + w; it < nitems; it += nwarps) {
-        const int4 item = items[it < n0 ? it : (it < n0 + n1 ? it - n0 + cap_items : it - n0 - n1 + 2 * cap_items)];
+        const int c = (it >= n0) + (it >= n0 + n1);
+        const long long k = it - (c > 0 ? n0 : 0) - (c > 1 ? n1 : 0);
+        const int4 item = items[c * cap_items + item_place(k, (long long)cnt->items_long[c], cap_items)];
         const int n = item.w - item.z;
         unsigned long long *e = pairs + item.z;
         if (n <= 1)

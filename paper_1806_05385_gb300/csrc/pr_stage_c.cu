@@ -176,7 +176,7 @@ constexpr int kStageF4 = 5;
 template <int S, bool kFlag>
 __global__ void __launch_bounds__(S *S / 2, PR_FRAG_MINB(S *S / 2))
     k_fragment(const ViewDev *__restrict__ views, const int4 *__restrict__ items,
-               const unsigned long long *__restrict__ nitems, long long cap_items, int *__restrict__ head,
+               int cls, long long cap_items, int *__restrict__ head,
                const unsigned long long *__restrict__ pairs, const float4 *__restrict__ rec,
                unsigned long long *__restrict__ keys, unsigned *__restrict__ flag_bits,
                long long *__restrict__ flag_list, Counters *cnt)
@@ -195,7 +195,7 @@ __global__ void __launch_bounds__(S *S / 2, PR_FRAG_MINB(S *S / 2))
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int ci = (warp % WPR) * 8 + (lane & 7);
     const int cj0 = (warp / WPR) * 8 + (lane >> 3), cj1 = cj0 + 4;
-    const long long it_hi = min((long long)*nitems, cap_items);
+    const long long nlong = (long long)cnt->items_long[cls], it_hi = (long long)cnt->items_n(cls);
     float4 *wrec = s_rec[warp];
     unsigned long long n_tests = 0, n_hits = 0;
 
@@ -208,9 +208,11 @@ __global__ void __launch_bounds__(S *S / 2, PR_FRAG_MINB(S *S / 2))
             break;
         if (threadIdx.x == 0)  // the next item, fetched while this one runs
             s_item[par ^ 1] = atomicAdd(head, 1);
-        const int4 item = items[it];
+        const int4 item = items[item_place(it, nlong, cap_items)];
+        // the first chunk's bin entries load while the pixels' rays are formed
+        unsigned long long e = item.z + lane < item.w ? pairs[item.z + lane] : ~0ull;
         const ViewDev &v = views[item.x];
-        const int tx = item.y % v.tiles_x, ty = item.y / v.tiles_x;
+        const int tx = item.y & 0xffff, ty = item.y >> 16;
         const int i = tx * S + ci, j0 = ty * S + cj0, j1 = ty * S + cj1;
         const bool ok0 = i < v.W && j0 < v.H, ok1 = i < v.W && j1 < v.H;
         float x00, x01, t0, dx0, dy0, x10, x11, t1, dx1, dy1;
@@ -245,7 +247,8 @@ __global__ void __launch_bounds__(S *S / 2, PR_FRAG_MINB(S *S / 2))
         for (int k0 = item.z; k0 < item.w; k0 += 32) {
             float wmax = warp_maxf(fmaxf(ok0 ? bd0 : 0.f, ok1 ? bd1 : 0.f)) * cull;
             const int kk = k0 + lane;
-            const unsigned long long e = kk < item.w ? pairs[kk] : ~0ull;
+            if (k0 != item.z)
+                e = kk < item.w ? pairs[kk] : ~0ull;
             const float key = depth_from_order_key((unsigned)(e >> 32));
             const unsigned stopm = __ballot_sync(0xffffffffu, kk >= item.w || key * 0.99999f > wmax);
             // entries ascend, so every lane from the first stop on stops too
@@ -273,8 +276,9 @@ __global__ void __launch_bounds__(S *S / 2, PR_FRAG_MINB(S *S / 2))
                 // the bests move with every test: re-check the cut before each
                 // (every 8 tests instead: 0.098 ms against 0.089 on the HMD
                 // frame, 0.385 against 0.276 ms on the 1M-triangle frame)
-                wmax = warp_maxf(fmaxf(ok0 ? bd0 : 0.f, ok1 ? bd1 : 0.f)) * cull;
-                if (__shfl_sync(0xffffffffu, key, k) * 0.99999f > wmax) {
+                // (a vote: no lane's farther pixel could still see it)
+                const float near = __shfl_sync(0xffffffffu, key, k) * 0.99999f;
+                if (!__any_sync(0xffffffffu, near <= fmaxf(ok0 ? bd0 : 0.f, ok1 ? bd1 : 0.f) * cull)) {
                     stop = true;
                     break;
                 }
@@ -345,8 +349,9 @@ int fragment_grid(int S, bool flag, long long ntiles, long long ttot, int seg)
     const int g = flag ? (S == 8 ? grid_for<8, true>() : (S == 16 ? grid_for<16, true>() : grid_for<32, true>()))
                        : (S == 8 ? grid_for<8, false>() : (S == 16 ? grid_for<16, false>() : grid_for<32, false>()));
     // a guess at the items of a small frame: one per tile, and the runs of bins
-    // that hold every triangle eight times
-    return (int)std::min<long long>(g, std::max<long long>(ntiles + 8 * ttot / seg, 1));
+    // that hold every triangle eight times (runs of 32 at least, unless the
+    // caller asks for shorter ones)
+    return (int)std::min<long long>(g, std::max<long long>(ntiles + 8 * ttot / std::min(seg, 32), 1));
 }
 
 template <bool kFlag>
@@ -356,18 +361,17 @@ static cudaError_t launch_fragment_t(int S, const ViewDev *views, const ItemsOut
                                      cudaStream_t st)
 {
     const int4 *items = io.items + (long long)cls * io.cap_items;
-    const unsigned long long *n = &cnt->items_n[cls];
     switch (S) {
     case 8:
-        k_fragment<8, kFlag><<<grid, 32, 0, st>>>(views, items, n, io.cap_items, head, pairs, rec, keys, flag_bits,
+        k_fragment<8, kFlag><<<grid, 32, 0, st>>>(views, items, cls, io.cap_items, head, pairs, rec, keys, flag_bits,
                                                   flag_list, cnt);
         break;
     case 16:
-        k_fragment<16, kFlag><<<grid, 128, 0, st>>>(views, items, n, io.cap_items, head, pairs, rec, keys, flag_bits,
+        k_fragment<16, kFlag><<<grid, 128, 0, st>>>(views, items, cls, io.cap_items, head, pairs, rec, keys, flag_bits,
                                                     flag_list, cnt);
         break;
     case 32:
-        k_fragment<32, kFlag><<<grid, 512, 0, st>>>(views, items, n, io.cap_items, head, pairs, rec, keys, flag_bits,
+        k_fragment<32, kFlag><<<grid, 512, 0, st>>>(views, items, cls, io.cap_items, head, pairs, rec, keys, flag_bits,
                                                     flag_list, cnt);
         break;
     default:

@@ -45,7 +45,8 @@ def test_mixed_tile_classes_equal_single_views(pr, seg, fov_bound):
         batch = [entry(v, t) for v, t in views]
         pr.pr_rasterize_batch(ws, batch, prm)
         got = pr.pr_workspace_stats(ws)
-        want = dict(pairs=0, items=0, culled=0)
+        # left to the library (0), the run length follows the frame's entries
+        want = dict(pairs=0, culled=0, **({"items": 0} if seg else {}))
         for e in batch:
             one = entry(e[1], e[5])
             pr.pr_rasterize_batch(ws1, [one], prm)
@@ -53,7 +54,8 @@ def test_mixed_tile_classes_equal_single_views(pr, seg, fov_bound):
             for k in want:
                 want[k] += pr.pr_workspace_stats(ws1)[k]
         assert {k: got[k] for k in want} == want
-        assert want["items"] >= want["pairs"] if seg == 1 else want["items"] > 0
+        assert want["pairs"] > 1000 and got["items"] > 0
+        assert seg != 1 or got["items"] == want["pairs"]
     finally:
         pr.pr_workspace_free(ws)
         pr.pr_workspace_free(ws1)
