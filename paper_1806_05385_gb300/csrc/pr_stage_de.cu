@@ -615,27 +615,49 @@ __device__ __forceinline__ void shade_body(const ViewDev *__restrict__ views, in
         const int x = (__ffs(live) - 1) * kBlkW + lane % kBlkW, y = lane / kBlkW;
         const unsigned id = s_id[warp][y * kIdPitch + x];
         const int pi = sp.i0 + x, pj = sp.j0 + y, lin = pj * W + pi;
-        bool hit = id != 0xFFFFFFFFu;
-        // the upstream gradient (or L2 target) does not depend on the hit:
-        // its loads go out first
-        float gin[3] = {0.f, 0.f, 0.f};
-        if (kAdjoint && grad && hit) {
-            if (v.target_u8) {
-                gin[0] = u8_unit(v.target_u8[lin]);
-                gin[1] = u8_unit(v.target_u8[plane + lin]);
-                gin[2] = u8_unit(v.target_u8[2 * plane + lin]);
-            } else {
-                const float *gsrc = v.grad_in ? v.grad_in : v.target;
-                gin[0] = gsrc[lin];
-                gin[1] = gsrc[plane + lin];
-                gin[2] = gsrc[2 * plane + lin];
+        bool done = false, later = false;
+        if (id != 0xFFFFFFFFu) {
+            // the upstream gradient (or L2 target) does not depend on the
+            // hit: its loads go out first
+            float gin[3] = {0.f, 0.f, 0.f};
+            if (kAdjoint && grad) {
+                if (v.target_u8) {
+                    gin[0] = u8_unit(v.target_u8[lin]);
+                    gin[1] = u8_unit(v.target_u8[plane + lin]);
+                    gin[2] = u8_unit(v.target_u8[2 * plane + lin]);
+                } else {
+                    const float *gsrc = v.grad_in ? v.grad_in : v.target;
+                    gin[0] = gsrc[lin];
+                    gin[1] = gsrc[plane + lin];
+                    gin[2] = gsrc[2 * plane + lin];
+                }
             }
-        }
-        PixelHit h;
-        bool later = false;
-        if (hit) {
-            hit = pixel_hit<kFeat>(v, pi, pj, id, h, (kFeat & kFeatF64) && def.list);
-            later = !hit;
+            PixelHit h;
+            if (pixel_hit<kFeat>(v, pi, pj, id, h, (kFeat & kFeatF64) && def.list)) {
+                PixelAlbedo pa;
+                pixel_albedo(v, h, pa);
+                const float rgb[3] = {fmaf(pa.a[0], h.sigma, h.spec), fmaf(pa.a[1], h.sigma, h.spec),
+                                      fmaf(pa.a[2], h.sigma, h.spec)};
+                if (v.rgb_out) {
+                    v.rgb_out[lin] = rgb[0];
+                    v.rgb_out[plane + lin] = rgb[1];
+                    v.rgb_out[2 * plane + lin] = rgb[2];
+                }
+                if (kAdjoint && grad) {
+                    if (!v.grad_in) {
+                        // L2 loss sum (rgb - target)^2: its gradient from this frame's image
+                        const float e0 = rgb[0] - gin[0], e1 = rgb[1] - gin[1], e2 = rgb[2] - gin[2];
+                        lsum += fmaf(e0, e0, fmaf(e1, e1, e2 * e2));
+                        gin[0] = 2.f * e0;
+                        gin[1] = 2.f * e1;
+                        gin[2] = 2.f * e2;
+                    }
+                    adjoint_rows<kFeat>(v, h, pa, gin[0], gin[1], gin[2], rows + lane);
+                }
+                done = true;
+            } else {
+                later = true;
+            }
         }
         if (kFeat & kFeatF64) {
             const unsigned m = __ballot_sync(0xffffffffu, later);
@@ -649,36 +671,14 @@ __device__ __forceinline__ void shade_body(const ViewDev *__restrict__ views, in
                         ((unsigned long long)(v.pix_off + lin) << 32) | id;
             }
         }
-        if (kAdjoint && grad && !hit) {
-#pragma unroll
-            for (int r = 0; r < kRows; ++r)
-                rows[r * kRowPitch + lane] = 0.f;
-        }
-        if (hit) {
-            PixelAlbedo pa;
-            pixel_albedo(v, h, pa);
-            const float rgb[3] = {fmaf(pa.a[0], h.sigma, h.spec), fmaf(pa.a[1], h.sigma, h.spec),
-                                  fmaf(pa.a[2], h.sigma, h.spec)};
-            if (v.rgb_out) {
-                v.rgb_out[lin] = rgb[0];
-                v.rgb_out[plane + lin] = rgb[1];
-                v.rgb_out[2 * plane + lin] = rgb[2];
-            }
-            if (kAdjoint && grad) {
-                if (!v.grad_in) {
-                    // L2 loss sum (rgb - target)^2: its gradient from this frame's image
-                    const float e0 = rgb[0] - gin[0], e1 = rgb[1] - gin[1], e2 = rgb[2] - gin[2];
-                    lsum += fmaf(e0, e0, fmaf(e1, e1, e2 * e2));
-                    gin[0] = 2.f * e0;
-                    gin[1] = 2.f * e1;
-                    gin[2] = 2.f * e2;
-                }
-                adjoint_rows<kFeat>(v, h, pa, gin[0], gin[1], gin[2], rows + lane);
-            }
-        }
         if (kAdjoint && grad) {
+            if (!done) {
+#pragma unroll
+                for (int r = 0; r < kRows; ++r)
+                    rows[r * kRowPitch + lane] = 0.f;
+            }
             __syncwarp();
-            sum_block(v, rows, vl, hit, id, ts);
+            sum_block(v, rows, vl, done, id, ts);
             __syncwarp();  // the rows are written again by the next block
         }
     }
