@@ -30,15 +30,14 @@ __host__ __device__ inline float cross2(float2 a, float2 b) { return a.x * b.y -
 // neither one catch per vertex nor a fixed root branch.
 //
 // S: camera-space vertices at t = 0, D: their motion over the frame (all
-// points must have z > 0 over [t_lo, t_hi]).  Returns false when no point of
+// points must have z > 0 over [t_lo, t_hi]); kx, ky, ks as above.  Returns false when no point of
 // the triangle is ever met by the scan.  FP32 with explicit tolerances: every
 // root gets a margin of kEpsT, near-double roots contribute their vertex,
 // and the end conditions are tested with an evaluation-error allowance.
 // ---------------------------------------------------------------------------
-__host__ __device__ inline bool catch_interval(const float3 S[3], const float3 D[3], float tan_x, float tan_y,
-                                               float d0, float d1, float t_lo, float t_hi, float &tmin, float &tmax)
+__host__ __device__ inline bool catch_interval(const float3 S[3], const float3 D[3], float kx, float ky, float ks,
+                                               float t_lo, float t_hi, float &tmin, float &tmax)
 {
-    const float kx = d0 / tan_x, ky = d1 / tan_y, ks = d0 + d1;
     float lo = INFINITY, hi = -INFINITY;
     bool lo_le = false, lo_ge = false, hi_le = false, hi_ge = false;
     bool finite = true;

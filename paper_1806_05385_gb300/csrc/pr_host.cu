@@ -337,6 +337,13 @@ pr_status derive_view(const pr_view &in, int tile, int bound, int fp64, ViewDev 
     }
     v.d0 = in.d[0];
     v.d1 = in.d[1];
+    const float dn = v.d1 == 0.f ? v.d0 : (v.d0 == 0.f ? v.d1 : std::sqrt(v.d0 * v.d0 + v.d1 * v.d1));
+    v.idn = dn > 0.f ? 1.f / dn : 0.f;
+    v.kx = in.d[0] / in.tan_x;
+    v.ky = in.d[1] / in.tan_y;
+    v.itan_x = 1.f / in.tan_x;
+    v.itan_y = 1.f / in.tan_y;
+    v.kD1 = std::pow(kSqrt2, 1.f - v.inv_alpha);
     v.t_lo = 0.f;
     v.t_hi = std::min(1.f, in.d[0] + in.d[1]);
     double lw[3] = {in.light_w[0], in.light_w[1], in.light_w[2]};
@@ -380,7 +387,6 @@ pr_status make_viewdev(const pr_view &in, const pr_scene *sc, int tile, int boun
     if (ds != PR_OK)
         return ds;
     v.T = (int)sc->T;
-    v.V = (int)sc->V;
     v.vtx = sc->vtx.as<float4>();
     v.col4 = sc->col.as<float4>();
     v.tri4 = sc->tri.as<int4>();
@@ -1544,7 +1550,8 @@ int32_t pr_debug_catch_interval(const pr_view *view, const float *S, const float
     }
     const float t_hi = std::min(1.f, view->d[0] + view->d[1]);
     float lo = 0.f, hi = 0.f;
-    const bool ok = catch_interval(s3, d3, view->tan_x, view->tan_y, view->d[0], view->d[1], 0.f, t_hi, lo, hi);
+    const bool ok = catch_interval(s3, d3, view->d[0] / view->tan_x, view->d[1] / view->tan_y, view->d[0] + view->d[1], 0.f,
+                                   t_hi, lo, hi);
     t_out[0] = lo;
     t_out[1] = hi;
     return ok ? 1 : 0;

@@ -61,7 +61,7 @@ struct ViewDev {
     int fov_bound;                     // pr_fov_bound
     long long tri_off, tile_off, pix_off;  // offsets of this view in the batch-wide arrays
     long long blk_off;                 // offset of its strips of pixel blocks (stages d, e)
-    int T, V;
+    int T;
     const float4 *vtx;                 // scene vertices, two float4 each: (px, py, pz, vx), (vy, vz, 0, 0)
     const float4 *col4;                // per-vertex colour (r, g, b, 0)
     const int4 *tri4;                  // per-triangle vertex indices (i0, i1, i2, 0)
@@ -78,19 +78,22 @@ struct ViewDev {
     float *dcol, *dpos, *dvel;         // adjoint outputs [V][3]
     const float4 *rec;                 // this frame's stage (a) records (batch-wide index), or null
     float rW, rH;                      // 1 / W, 1 / H, correctly rounded (pixel_centre)
+    float kx, ky, itan_x, itan_y;      // d0 / tan_x, d1 / tan_y, 1 / tan_x, 1 / tan_y
+    float idn;                         // 1 / |d| (0 without a scan direction)
+    float kD1;                         // D^(1 - 1/alpha): q^-1 maps distance r to kD1 r^(1/alpha)
     unsigned long long bw_mul;         // ceil(2^40 / bw), bw = strips per row: lb / bw = (lb * bw_mul) >> 40 (set_strips)
 };
 
 // The views of a launch passed by value in the kernel's parameter space, for
-// batches of up to kParamViews views (72 x 416 bytes, within the 32 KB a
-// launch may pass).  A kernel then reads their fields through the constant
+// batches of up to kParamViews views (within the 32,764 bytes a launch may
+// pass).  A kernel then reads their fields through the constant
 // cache (warp-uniform, off the L1 path) and can re-read one instead of
 // holding it in a register.  Larger batches read the device table.
 constexpr int kParamViews = 72;
 struct ParamViews {
     ViewDev v[kParamViews];
 };
-static_assert(sizeof(ParamViews) <= 30 * 1024, "the view table must fit the kernel parameter space");
+static_assert(sizeof(ParamViews) <= 32764 - 128, "the view table must fit the kernel parameter space");
 
 constexpr int kMaxClasses = 3;  // tile sizes (8, 16, 32): a frame's fragment launches
 
@@ -325,10 +328,13 @@ __device__ inline Ray64 pixel_ray64(const ViewDev &v, int i, int j)
 }
 
 // Display location (unit coordinates) of a camera-space point with z > 0.
+// kQuick: to a few ulps, for a bound that is grown by far more (an IEEE
+// division is about ten instructions and a branch).
+template <bool kQuick = false>
 __device__ __forceinline__ float2 project(const ViewDev &v, float3 p)
 {
-    float iz = 1.0f / p.z;
-    return make_float2(fmaf(0.5f * p.x * iz, 1.0f / v.tan_x, 0.5f), fmaf(0.5f * p.y * iz, 1.0f / v.tan_y, 0.5f));
+    const float iz = kQuick ? __fdividef(1.0f, p.z) : 1.0f / p.z;
+    return make_float2(fmaf(0.5f * p.x * iz, v.itan_x, 0.5f), fmaf(0.5f * p.y * iz, v.itan_y, 0.5f));
 }
 
 // A float as an unsigned integer of the same order (negative values

@@ -114,7 +114,6 @@ pr_status view_constants(const pr_view &in, int tile, int bound, const float4 *v
     if (s != PR_OK)
         return s;
     v.T = (int)T;
-    v.V = (int)V;
     v.vtx = vtx;
     v.col4 = col4;
     v.tri4 = tri4;

@@ -244,26 +244,37 @@ __device__ __forceinline__ float4 support_halfplane(float2 n, const float2 (&q)[
 // from f; rlo is a lower bound of the distance from f to R, used when f is
 // outside R.  The preimage then lies in the annular sector of those angles
 // and of the radii p^-1 of the nearest and farthest distance.
-template <int N>
-__device__ __forceinline__ float4 fov_sector_preimage(const float2 (&pts)[N], int n, float2 f, float inv_alpha,
-                                                      float eps, bool f_inside, float rlo, const float *lut = nullptr,
-                                                      int lut_n = 0)
+//
+// The power map's radii come from the quick power: its relative error, about
+// 1e-6 for the distances and exponents a view can have, is a tenth of the
+// margins below.
+__device__ __forceinline__ float pinv_quick(const ViewDev &v, float r)
 {
-    const SampledP sp{lut, lut_n};
-    float rmax = 0.f;
+    if (v.p_lut) {
+        const SampledP sp{v.p_lut, v.p_n};
+        return sp.pinv(r);
+    }
+    return v.kD1 * __powf(r, v.inv_alpha);
+}
+
+template <int N>
+__device__ __forceinline__ float4 fov_sector_preimage(const ViewDev &v, const float2 (&pts)[N], int n, float eps,
+                                                      bool f_inside, float rlo)
+{
+    const float2 f = make_float2(v.fx, v.fy);
+    float r2 = 0.f;
 #pragma unroll
     for (int k = 0; k < N; ++k)
         if (k < n) {
             const float2 w = f2sub(pts[k], f);
-            rmax = fmaxf(rmax, sqrtf(w.x * w.x + w.y * w.y));
+            r2 = fmaxf(r2, w.x * w.x + w.y * w.y);
         }
-    rmax += eps;
-    const float kD1 = powf(kSqrt2, 1.f - inv_alpha);
-    const float rho1 = (lut ? sp.pinv(rmax) : kD1 * powf(rmax, inv_alpha)) * (1.f + 1e-5f) + 1e-6f;
+    const float rmax = sqrtf(r2) + eps;
+    const float rho1 = pinv_quick(v, rmax) * (1.f + 1e-5f) + 1e-6f;
     const float rmin = f_inside ? 0.f : fmaxf(0.f, rlo - eps);
     if (rmin <= 0.f)
         return sector_box(f, make_float2(1.f, 0.f), make_float2(1.f, 0.f), 0.f, rho1, true);
-    const float rho0 = (lut ? sp.pinv(rmin) : kD1 * powf(rmin, inv_alpha)) * (1.f - 1e-5f);
+    const float rho0 = pinv_quick(v, rmin) * (1.f - 1e-5f);
     // f lies outside the convex hull of the points: their directions from
     // f span less than half a turn, and one sweep finds the two extremes
     float2 a = f2sub(pts[0], f), b = a;
@@ -276,12 +287,12 @@ __device__ __forceinline__ float4 fov_sector_preimage(const float2 (&pts)[N], in
             if (cross2(b, w) > 0.f)
                 b = w;
         }
-    const float la = sqrtf(a.x * a.x + a.y * a.y), lb = sqrtf(b.x * b.x + b.y * b.y);
-    a = make_float2(a.x / la, a.y / la);
-    b = make_float2(b.x / lb, b.y / lb);
+    const float ia = rsqrtf(a.x * a.x + a.y * a.y), ib = rsqrtf(b.x * b.x + b.y * b.y);
+    a = make_float2(a.x * ia, a.y * ia);
+    b = make_float2(b.x * ib, b.y * ib);
     // the region grown by eps spans a little more angle: asin(eps / r)
-    a = rot_small(a, -(eps / fmaxf(la, eps) + 1e-6f));
-    b = rot_small(b, eps / fmaxf(lb, eps) + 1e-6f);
+    a = rot_small(a, -(fminf(eps * ia, 1.f) + 1e-6f));
+    b = rot_small(b, fminf(eps * ib, 1.f) + 1e-6f);
     if (cross2(a, b) <= 0.f)  // span reached half a turn: give up on angles
         return sector_box(f, a, b, 0.f, rho1, true);
     return sector_box(f, a, b, rho0, rho1, false);
@@ -551,7 +562,7 @@ __device__ __forceinline__ void compute_bound(const ViewDev &v, const float3 S[3
         for (int k = 0; k < 6; ++k) {
             if (k >= np)
                 break;
-            const float2 x = project(v, P[k]);
+            const float2 x = project<true>(v, P[k]);
             bx0 = fminf(bx0, x.x);
             bx1 = fmaxf(bx1, x.x);
             by0 = fminf(by0, x.y);
@@ -562,13 +573,11 @@ __device__ __forceinline__ void compute_bound(const ViewDev &v, const float3 S[3
         bx1 += m;
         by0 -= m;
         by1 += m;
-        const float2 f = make_float2(v.fx, v.fy);
-        const float dbx = fmaxf(fmaxf(bx0 - f.x, f.x - bx1), 0.f), dby = fmaxf(fmaxf(by0 - f.y, f.y - by1), 0.f);
+        const float dbx = fmaxf(fmaxf(bx0 - v.fx, v.fx - bx1), 0.f), dby = fmaxf(fmaxf(by0 - v.fy, v.fy - by1), 0.f);
         const float rlo = sqrtf(dbx * dbx + dby * dby);
         const float2 corners[4] = {make_float2(bx0, by0), make_float2(bx1, by0), make_float2(bx1, by1),
                                    make_float2(bx0, by1)};
-        const float4 fb = fov_sector_preimage(corners, 4, f, v.inv_alpha, 2.f * eps, rlo <= 2.f * eps, rlo, v.p_lut,
-                                              v.p_n);
+        const float4 fb = fov_sector_preimage(v, corners, 4, 2.f * eps, rlo <= 2.f * eps, rlo);
         // pixel centres inside the preimage box, 1/100 pixel of slack (as below)
         const float fi0 = ceilf(fb.x * v.W - 0.51f), fi1 = floorf(fb.y * v.W - 0.49f);
         const float fj0 = ceilf(fb.z * v.H - 0.51f), fj1 = floorf(fb.w * v.H - 0.49f);
@@ -590,7 +599,7 @@ __device__ __forceinline__ void compute_bound(const ViewDev &v, const float3 S[3
         float tmin = B.tmin, tmax = B.tmax;
         if (rolling) {
             if (v.bound == PR_BOUND_ZENON) {
-                if (!catch_interval(S, D, v.tan_x, v.tan_y, v.d0, v.d1, v.t_lo, v.t_hi, tmin, tmax)) {
+                if (!catch_interval(S, D, v.kx, v.ky, v.d0 + v.d1, v.t_lo, v.t_hi, tmin, tmax)) {
                     B.culled = true;
                     return;
                 }
@@ -648,16 +657,21 @@ __device__ __forceinline__ void compute_bound(const ViewDev &v, const float3 S[3
     }
     if (strip) {
         // the time strip t_min <= d . x <= t_max (covered pixels satisfy t = r(x))
-        const float dn = sqrtf(v.d0 * v.d0 + v.d1 * v.d1);
+        // (an axis-aligned scan exactly: its strip and the box sides cut to it
+        // are the same lines)
+        const float slo = (B.tmin - kEpsT) * v.idn, shi = (B.tmax + kEpsT) * v.idn;
+        float2 sn = make_float2(v.d0 * v.idn, v.d1 * v.idn);
         if (v.d1 == 0.f) {
-            xmin = fmaxf(xmin, (B.tmin - kEpsT) / v.d0);
-            xmax = fminf(xmax, (B.tmax + kEpsT) / v.d0);
+            xmin = fmaxf(xmin, slo);
+            xmax = fminf(xmax, shi);
+            sn.x = 1.f;
         } else if (v.d0 == 0.f) {
-            ymin = fmaxf(ymin, (B.tmin - kEpsT) / v.d1);
-            ymax = fminf(ymax, (B.tmax + kEpsT) / v.d1);
+            ymin = fmaxf(ymin, slo);
+            ymax = fminf(ymax, shi);
+            sn.y = 1.f;
         }
-        B.hp[kHpStrip] = make_float4(-v.d0 / dn, -v.d1 / dn, (B.tmin - kEpsT) / dn, 0.f);
-        B.hp[kHpStrip + 1] = make_float4(v.d0 / dn, v.d1 / dn, -(B.tmax + kEpsT) / dn, 0.f);
+        B.hp[kHpStrip] = make_float4(-sn.x, -sn.y, slo, 0.f);
+        B.hp[kHpStrip + 1] = make_float4(sn.x, sn.y, -shi, 0.f);
         B.hmask |= 3u << kHpStrip;
     }
     // clip to the viewport (every ray's display location lies in [0,1]^2)
@@ -727,14 +741,14 @@ __device__ __forceinline__ void compute_bound(const ViewDev &v, const float3 S[3
             if (B.hmask & (1u << h))
                 rlo = fmaxf(rlo, fmaf(B.hp[h].x, f.x, fmaf(B.hp[h].y, f.y, B.hp[h].z)));
         const bool inside = rlo <= 2.f * eps;
-        float4 fb;
-        if (use_hull) {
-            fb = fov_sector_preimage(Q, nq, f, v.inv_alpha, 2.f * eps, inside, rlo, v.p_lut, v.p_n);
-        } else {
-            const float2 corners[4] = {make_float2(xmin, ymin), make_float2(xmax, ymin), make_float2(xmax, ymax),
-                                       make_float2(xmin, ymax)};
-            fb = fov_sector_preimage(corners, 4, f, v.inv_alpha, 2.f * eps, inside, rlo, v.p_lut, v.p_n);
+        if (!use_hull) {  // the box's corners stand for the points
+            Q[0] = make_float2(xmin, ymin);
+            Q[1] = make_float2(xmax, ymin);
+            Q[2] = make_float2(xmax, ymax);
+            Q[3] = make_float2(xmin, ymax);
+            nq = 4;
         }
+        const float4 fb = fov_sector_preimage(v, Q, nq, 2.f * eps, inside, rlo);
         u0 = fb.x;
         u1 = fb.y;
         w0 = fb.z;
@@ -766,7 +780,15 @@ __device__ __forceinline__ void compute_bound(const ViewDev &v, const float3 S[3
 // tiles (tiles of its framebuffer box) is also appended to the list.  A
 // culled triangle leaves only its empty tbox: nothing downstream reads the
 // rest (its record alone would be 96 of the pass's 204 bytes).
-__global__ void __launch_bounds__(128, 6) k_bound(const ViewDev *__restrict__ views, int nviews,
+//
+// Bound: instruction fetch and issue (the code of every kind of view is
+// long), then the gathers' latency.  64 views (5.1 M triangles) / 1M-triangle
+// stereo / HMD stereo frame: 0.331 / 0.163 / 0.046 ms with general powers in
+// the foveation preimages, a square root per point and the preimage's code
+// three times; 0.268 / 0.107 / 0.032 ms with the quick power, one square
+// root and two copies; 0.245 / 0.103 / 0.032 ms at 64 registers (eight CTAs of
+// 128 per SM instead of six).
+__global__ void __launch_bounds__(128, 8) k_bound(const ViewDev *__restrict__ views, int nviews,
                                                const long long *__restrict__ tri_offs, long long ttot,
                                                float4 *__restrict__ rec, float4 *__restrict__ hp,
                                                int4 *__restrict__ tbox, const CandList list, Counters *cnt)
