@@ -139,7 +139,8 @@ constexpr long long kMaxPairs = 0x7FFFFFFFll;  // bin entries per frame: work it
 
 // Scratch of one batched frame.
 struct pr_workspace {
-    DevBuf views, offs, rec, hp, tbox, tile_box, tile_cnt, scan, fill, sums, pairs, items, keys, counters, heads;
+    DevBuf views;  // a call's view table, then its offsets (triangles, tiles, pixels, strips: n + 1 each)
+    DevBuf rec, hp, tbox, tile_box, tile_cnt, scan, fill, sums, pairs, items, keys, counters, heads;
     DevBuf hit_entry, hit_tile;  // (triangle, tile) hits of the binning count pass, before the scatter
     DevBuf mip;                  // display step: MIP pyramid of the framebuffer image
     DevBuf disp;                 // batched display step: its view and block tables
@@ -157,8 +158,11 @@ struct pr_workspace {
     // shading) sets the keys it reads back to ~0, so a frame clears only
     // beyond this count (and after a new allocation)
     long long keys_clean_n = 0;
-    PinnedBuf<ViewDev> h_views;
-    PinnedBuf<long long> h_offs;
+    PinnedBuf<char> h_tab;          // the host copy of the table and offsets
+    ViewDev *h_views() const { return reinterpret_cast<ViewDev *>(h_tab.p); }
+    long long *h_offs(int n) const { return reinterpret_cast<long long *>(h_tab.p + sizeof(ViewDev) * (size_t)n); }
+    const long long *offs(int n) const { return reinterpret_cast<const long long *>(views.as<ViewDev>() + n); }
+    static size_t table_bytes(int n) { return sizeof(ViewDev) * (size_t)n + sizeof(long long) * 4 * (size_t)(n + 1); }
     PinnedBuf<Counters> h_cnt;
     pr_stats stats{};
     long long last_T = 0;          // triangles of the last frame (debug bounds)
@@ -279,7 +283,7 @@ struct pr_graph {
     long long npix = 0;
     bool reader_resets = false;         // the replay's reader sets the keys back to ~0 (and its start clears none)
     bool stage_times = false;           // stage events captured as graph nodes
-    DevBuf views, offs;                 // the graph's own view and offset tables
+    DevBuf views;                       // the graph's own view and offset tables
     PinnedBuf<Counters> h_cnt;          // the graph's own copy of its last replay's counters
     std::vector<const void *> buffers;  // the workspace's buffers at capture
 };
@@ -563,8 +567,7 @@ pr_status plan_batch(const pr_batch_view *views, int n, const pr_params &prm, Ba
 pr_status size_workspace(pr_workspace *ws, const BatchPlan &P, int seg)
 {
     const int n = (int)P.vd.size();
-    PR_TRY(ensure(ws->views, sizeof(ViewDev) * n));
-    PR_TRY(ensure(ws->offs, sizeof(long long) * 4 * (n + 1)));
+    PR_TRY(ensure(ws->views, pr_workspace::table_bytes(n)));
     PR_TRY(ensure(ws->rec, sizeof(float4) * kRecF4 * std::max(P.ttot, 1ll)));
     PR_TRY(ensure(ws->hp, sizeof(float4) * kMaxHp * std::max(P.ttot, 1ll)));
     PR_TRY(ensure(ws->tbox, sizeof(int4) * std::max(P.ttot, 1ll)));
@@ -604,14 +607,13 @@ pr_status size_workspace(pr_workspace *ws, const BatchPlan &P, int seg)
         PR_TRY(ensure(ws->items, sizeof(int4) * want_items));
     }
     ws->cap_items = std::min((long long)(ws->items.cap / sizeof(int4)) / kMaxClasses, kMaxPairs);
-    PR_TRY(ws->h_views.ensure(n));
-    PR_TRY(ws->h_offs.ensure(4 * (n + 1)));
+    PR_TRY(ws->h_tab.ensure(pr_workspace::table_bytes(n)));
     PR_TRY(ws->h_cnt.ensure(1));
     return PR_OK;
 }
 
 // Writes the frame's view and offset tables into the workspace's pinned
-// host copies (h_views: n views; h_offs: triangle, tile, pixel and warp
+// host copy (h_views: n views; h_offs: triangle, tile, pixel and warp
 // block offsets, n + 1 each).  shade: views with an rgb output get one.
 void fill_tables(pr_workspace *ws, BatchPlan &P, bool shade)
 {
@@ -636,9 +638,9 @@ void fill_tables(pr_workspace *ws, BatchPlan &P, bool shade)
             v.dpos = g.dpos;
             v.dvel = g.dvel;
         }
-        ws->h_views.p[q] = v;
+        ws->h_views()[q] = v;
     }
-    long long *ho = ws->h_offs.p;
+    long long *ho = ws->h_offs(n);
     for (int q = 0; q <= n; ++q) {
         ho[q] = P.tri_off[q];
         ho[n + 1 + q] = P.tile_off[q];
@@ -660,10 +662,9 @@ pr_status enqueue_batch(pr_workspace *ws, BatchPlan &P, int seg, bool shade, cud
     char *stage = ws->stage.as<char>();
     if (!tab_views) {
         fill_tables(ws, P, shade);
-        PR_TRY(cudaMemcpyAsync(ws->views.p, ws->h_views.p, sizeof(ViewDev) * n, cudaMemcpyHostToDevice, st));
-        PR_TRY(cudaMemcpyAsync(ws->offs.p, ws->h_offs.p, sizeof(long long) * 4 * (n + 1), cudaMemcpyHostToDevice, st));
+        PR_TRY(cudaMemcpyAsync(ws->views.p, ws->h_tab.p, pr_workspace::table_bytes(n), cudaMemcpyHostToDevice, st));
         tab_views = ws->views.as<ViewDev>();
-        tab_offs = ws->offs.as<long long>();
+        tab_offs = ws->offs(n);
     }
     const ViewDev *dv = tab_views;
     const long long *tri_offs = tab_offs, *tile_offs = tri_offs + n + 1, *pix_offs = tile_offs + n + 1;
@@ -776,8 +777,7 @@ pr_status enqueue_batch(pr_workspace *ws, BatchPlan &P, int seg, bool shade, cud
     }
     // the frame's counters to the host: the workspace's copy, or the graph's
     // own (so a replay's status can be read while the next replay runs)
-    PR_TRY(cudaMemcpyAsync(h_cnt ? h_cnt : ws->h_cnt.p, ws->counters.p, sizeof(Counters), cudaMemcpyDeviceToHost,
-                           st));
+    PR_TRY(launch_publish(cnt, h_cnt ? h_cnt : ws->h_cnt.p, st));
     return PR_OK;
 }
 
@@ -860,24 +860,6 @@ pr_status single_view(pr_scene *sc, const pr_view *view, const pr_params *params
     bv.depth_out = depth_out;
     bv.rgb_out = rgb_out;
     return run_batch(&sc->ws, &bv, 1, params, rgb_out != nullptr, st);
-}
-
-// One-view table for stages (d)/(e) called on their own.
-pr_status upload_single(pr_scene *sc, ViewDev &v, int &nsub, long long &nblk, cudaStream_t st)
-{
-    pr_workspace *ws = &sc->ws;
-    PR_TRY(ensure(ws->views, sizeof(ViewDev)));
-    PR_TRY(ensure(ws->offs, sizeof(long long) * 6));
-    PR_TRY(ws->h_views.ensure(1));
-    PR_TRY(ws->h_offs.ensure(6));
-    long long *o = ws->h_offs.p;
-    nsub = set_strips(&v, 1, o);
-    nblk = o[1];
-    ws->h_views.p[0] = v;
-    o[2] = o[3] = o[4] = o[5] = 0;
-    PR_TRY(cudaMemcpyAsync(ws->views.p, ws->h_views.p, sizeof(ViewDev), cudaMemcpyHostToDevice, st));
-    PR_TRY(cudaMemcpyAsync(ws->offs.p, o, sizeof(long long) * 2, cudaMemcpyHostToDevice, st));
-    return PR_OK;
 }
 
 }  // namespace
@@ -1089,12 +1071,9 @@ pr_status pr_shade(pr_scene *sc, const pr_view *view, const uint32_t *id, float 
         PR_TRY(ensure(*ob, sizeof(float) * 3 * np));
     v.id_in = did;
     v.rgb_out = host_out ? ob->as<float>() : rgb_out;
-    int nsub = 1;
-    long long nblk = 0;
-    s = upload_single(sc, v, nsub, nblk, st);
-    if (s != PR_OK)
-        return s;
-    PR_TRY(launch_shade(sc->ws.views.as<ViewDev>(), 1, sc->ws.offs.as<long long>(), nblk, nsub, nullptr, false, false,
+    long long blk[2];
+    const int nsub = set_strips(&v, 1, blk);  // one view: no table in device memory
+    PR_TRY(launch_shade(nullptr, 1, nullptr, blk[1], nsub, nullptr, false, false,
                         nullptr, shade_features(&v, 1), st, &v));
     if (host_out)
         PR_TRY(cudaMemcpyAsync(rgb_out, ob->p, sizeof(float) * 3 * np, cudaMemcpyDeviceToHost, st));
@@ -1143,12 +1122,9 @@ pr_status pr_backward(pr_scene *sc, const pr_view *view, const uint32_t *id, con
     v.dcol = douts[0];
     v.dpos = douts[1];
     v.dvel = douts[2];
-    int nsub = 1;
-    long long nblk = 0;
-    s = upload_single(sc, v, nsub, nblk, st);
-    if (s != PR_OK)
-        return s;
-    PR_TRY(launch_backward(sc->ws.views.as<ViewDev>(), 1, sc->ws.offs.as<long long>(), nblk, nsub, shade_features(&v, 1),
+    long long blk[2];
+    const int nsub = set_strips(&v, 1, blk);  // one view: no table in device memory
+    PR_TRY(launch_backward(nullptr, 1, nullptr, blk[1], nsub, shade_features(&v, 1),
                            st, &v));
     for (int a = 0; a < 3; ++a)
         if (host[a])
@@ -1162,11 +1138,9 @@ pr_status pr_backward_batch(pr_workspace *ws, const pr_backward_view *views, int
     if (!ws || !views || n < 1)
         return PR_ERR_INVALID_ARG;
     cudaStream_t st = (cudaStream_t)stream;
-    PR_TRY(ws->h_views.ensure(n));
-    PR_TRY(ws->h_offs.ensure(n + 1));
-    PR_TRY(ensure(ws->views, sizeof(ViewDev) * n));
-    PR_TRY(ensure(ws->offs, sizeof(long long) * (n + 1)));
-    long long *blk = ws->h_offs.p;
+    PR_TRY(ws->h_tab.ensure(pr_workspace::table_bytes(n)));
+    PR_TRY(ensure(ws->views, pr_workspace::table_bytes(n)));
+    long long *blk = ws->h_offs(n);
     for (int k = 0; k < n; ++k) {
         const pr_backward_view &b = views[k];
         if (!b.scene || !b.id || !b.grad_rgb || !is_device_ptr(b.id) || !is_device_ptr(b.grad_rgb) ||
@@ -1182,13 +1156,15 @@ pr_status pr_backward_batch(pr_workspace *ws, const pr_backward_view *views, int
         v.dcol = b.dcol;
         v.dpos = b.dpos;
         v.dvel = b.dvel;
-        ws->h_views.p[k] = v;
+        ws->h_views()[k] = v;
     }
-    const int nsub = set_strips(ws->h_views.p, n, blk);
-    PR_TRY(cudaMemcpyAsync(ws->views.p, ws->h_views.p, sizeof(ViewDev) * n, cudaMemcpyHostToDevice, st));
-    PR_TRY(cudaMemcpyAsync(ws->offs.p, blk, sizeof(long long) * (n + 1), cudaMemcpyHostToDevice, st));
-    PR_TRY(launch_backward(ws->views.as<ViewDev>(), n, ws->offs.as<long long>(), blk[n], nsub,
-                           shade_features(ws->h_views.p, n), st, ws->h_views.p));
+    const int nsub = set_strips(ws->h_views(), n, blk);
+    // a small batch's views travel with the launch: only the offsets go up
+    const size_t from = shade_reads_params(n) ? sizeof(ViewDev) * (size_t)n : 0;
+    PR_TRY(cudaMemcpyAsync(ws->views.as<char>() + from, ws->h_tab.p + from,
+                           sizeof(ViewDev) * (size_t)n + sizeof(long long) * (n + 1) - from, cudaMemcpyHostToDevice, st));
+    PR_TRY(launch_backward(ws->views.as<ViewDev>(), n, ws->offs(n), blk[n], nsub, shade_features(ws->h_views(), n), st,
+                           ws->h_views()));
     PR_TRY(cudaStreamSynchronize(st));
     return PR_OK;
 }
@@ -1350,17 +1326,13 @@ pr_status pr_graph_capture_frame(pr_workspace *ws, const pr_batch_view *views, i
     // replays upload nothing, and later calls on the workspace cannot change it
     const int nv = (int)P.vd.size();
     fill_tables(ws, P, true);
-    cudaError_t e = ensure(g->views, sizeof(ViewDev) * nv);
-    if (e == cudaSuccess)
-        e = ensure(g->offs, sizeof(long long) * 4 * (nv + 1));
+    cudaError_t e = ensure(g->views, pr_workspace::table_bytes(nv));
     if (e == cudaSuccess)
         e = g->h_cnt.ensure(1);
     if (e == cudaSuccess)
         std::memcpy(g->h_cnt.p, ws->h_cnt.p, sizeof(Counters));  // the eager run's, until the first replay
     if (e == cudaSuccess)
-        e = cudaMemcpy(g->views.p, ws->h_views.p, sizeof(ViewDev) * nv, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess)
-        e = cudaMemcpy(g->offs.p, ws->h_offs.p, sizeof(long long) * 4 * (nv + 1), cudaMemcpyHostToDevice);
+        e = cudaMemcpy(g->views.p, ws->h_tab.p, pr_workspace::table_bytes(nv), cudaMemcpyHostToDevice);
     if (e != cudaSuccess) {
         delete g;
         cudaGetLastError();
@@ -1375,7 +1347,8 @@ pr_status pr_graph_capture_frame(pr_workspace *ws, const pr_batch_view *views, i
     g->stage_times = prm.graph_stage_times != 0;
     // a capture runs nothing: the keys keep the state the eager run left
     const long long clean_n = ws->keys_clean_n;
-    s = enqueue_batch(ws, P, prm.seg, true, st, g->views.as<ViewDev>(), g->offs.as<long long>(), g->stage_times,
+    s = enqueue_batch(ws, P, prm.seg, true, st, g->views.as<ViewDev>(),
+                      reinterpret_cast<const long long *>(g->views.as<ViewDev>() + nv), g->stage_times,
                       g->h_cnt.p);
     ws->keys_clean_n = clean_n;
     g->reader_resets = keys_reset_by_reader(P.npix);

@@ -90,10 +90,14 @@ struct ViewDev {
 // cache (warp-uniform, off the L1 path) and can re-read one instead of
 // holding it in a register.  Larger batches read the device table.
 constexpr int kParamViews = 72;
+// A launch's parameters are copied for every launch, so batches of up to
+// kFewViews views pass a table of that size (3.6 instead of 32 KB).
+constexpr int kFewViews = 8;
+template <int N>
 struct ParamViews {
-    ViewDev v[kParamViews];
+    ViewDev v[N];
 };
-static_assert(sizeof(ParamViews) <= 32764 - 128, "the view table must fit the kernel parameter space");
+static_assert(sizeof(ParamViews<kParamViews>) <= 32764 - 128, "the view table must fit the kernel parameter space");
 
 constexpr int kMaxClasses = 3;  // tile sizes (8, 16, 32): a frame's fragment launches
 

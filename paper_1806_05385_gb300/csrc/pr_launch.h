@@ -106,7 +106,9 @@ cudaError_t launch_resolve(const ViewDev *views, int nviews, const long long *pi
 int shade_features(const ViewDev *vd, int n);
 // host_views: the host copy of the device table `views` (same contents), or
 // null; with one, a launch of up to kParamViews views passes them as a
-// kernel parameter
+// kernel parameter (shade_reads_params) and reads neither the device table
+// nor, for one view, blk_offs
+bool shade_reads_params(int nviews);
 // def.list: pixels that need FP64 are listed there and shaded by a launch of
 // their own (frames of fewer than 2^32 pixels; pix_offs needed), or null:
 // shaded in place
@@ -117,6 +119,9 @@ cudaError_t launch_shade(const ViewDev *views, int nviews, const long long *blk_
                          const Deferred64 &def = Deferred64{});
 // a training frame's losses: each view's partial sums (loss_part) added into
 // its loss, once (skipped when the frame's forward overflowed)
+// copies the frame's counters to pinned host memory (a kernel of a few
+// stores: a copy node takes about 6 us longer)
+cudaError_t launch_publish(const Counters *cnt, Counters *host, cudaStream_t st);
 cudaError_t launch_loss_finalize(const ViewDev *views, int nviews, const Counters *frame_cnt, cudaStream_t st);
 cudaError_t launch_backward(const ViewDev *views, int nviews, const long long *blk_offs, long long nblocks, int nsub,
                             int feat, cudaStream_t st, const ViewDev *host_views = nullptr);

@@ -1467,6 +1467,21 @@ cudaError_t launch_frame_init(const ViewDev *views, int nviews, const long long 
     return cudaGetLastError();
 }
 
+// The end of a frame: its counters to the host's pinned copy.
+__global__ void k_publish(const Counters *__restrict__ cnt, Counters *__restrict__ host)
+{
+    static_assert(sizeof(Counters) % 8 == 0 && sizeof(Counters) / 8 <= 32, "one word per lane");
+    const int k = threadIdx.x;
+    if (k < (int)(sizeof(Counters) / 8))
+        reinterpret_cast<unsigned long long *>(host)[k] = reinterpret_cast<const unsigned long long *>(cnt)[k];
+}
+
+cudaError_t launch_publish(const Counters *cnt, Counters *host, cudaStream_t st)
+{
+    k_publish<<<1, 32, 0, st>>>(cnt, host);
+    return cudaGetLastError();
+}
+
 // ---------------------------------------------------------------- scan
 
 // Exclusive prefix sum of u64 words in one pass (decoupled look-back,

@@ -705,9 +705,9 @@ __global__ void __launch_bounds__(kShadeThreads, shade_ctas(kFeat))
     shade_body<kAdjoint, kFeat>(views, nviews, blk_offs, nblocks, nsub, keys, reset_keys, frame_cnt, def);
 }
 
-template <bool kAdjoint, int kFeat>
+template <int kN, bool kAdjoint, int kFeat>
 __global__ void __launch_bounds__(kShadeThreads, shade_ctas(kFeat))
-    k_shade_pv(const __grid_constant__ ParamViews pv, int nviews, const long long *__restrict__ blk_offs,
+    k_shade_pv(const __grid_constant__ ParamViews<kN> pv, int nviews, const long long *__restrict__ blk_offs,
                long long nblocks, int nsub, unsigned long long *__restrict__ keys, int reset_keys,
                const Counters *__restrict__ frame_cnt, const Deferred64 def)
 {
@@ -834,32 +834,37 @@ static unsigned shade_grid(long long nblocks)
     return (unsigned)((nblocks * 32 + kShadeThreads - 1) / kShadeThreads);
 }
 
-// The parameter table of a launch's views (null: the batch is too large, or
-// the caller has no host copy; the kernels then read the device table).
-static const ParamViews *param_views(const ViewDev *host_views, int nviews)
+// The parameter table of a launch's views, from their host copy.
+template <int kN>
+static const ParamViews<kN> &param_views(const ViewDev *host_views, int nviews)
 {
-    static thread_local ParamViews pv;
-    if (!host_views || nviews < 1 || nviews > kParamViews)
-        return nullptr;
+    static thread_local ParamViews<kN> pv;
     std::memcpy(pv.v, host_views, sizeof(ViewDev) * (size_t)nviews);
-    return &pv;
+    return pv;
 }
 
+bool shade_reads_params(int nviews) { return nviews >= 1 && nviews <= kParamViews; }
+
 template <bool kAdjoint, int kFeat>
-static void launch_shade_one(unsigned g, const ViewDev *views, const ParamViews *pv, int nviews,
+static void launch_shade_one(unsigned g, const ViewDev *views, const ViewDev *host_views, int nviews,
                              const long long *blk_offs, long long nblocks, int nsub, unsigned long long *keys,
                              int reset_keys, const Counters *frame_cnt, const Deferred64 &def, cudaStream_t st)
 {
-    if (pv)
-        k_shade_pv<kAdjoint, kFeat><<<g, kShadeThreads, 0, st>>>(*pv, nviews, blk_offs, nblocks, nsub, keys, reset_keys,
-                                                                 frame_cnt, def);
-    else
+    if (!host_views || !shade_reads_params(nviews))
         k_shade<kAdjoint, kFeat><<<g, kShadeThreads, 0, st>>>(views, nviews, blk_offs, nblocks, nsub, keys, reset_keys,
                                                               frame_cnt, def);
+    else if (nviews <= kFewViews)
+        k_shade_pv<kFewViews, kAdjoint, kFeat><<<g, kShadeThreads, 0, st>>>(
+            param_views<kFewViews>(host_views, nviews), nviews, blk_offs, nblocks, nsub, keys, reset_keys, frame_cnt,
+            def);
+    else
+        k_shade_pv<kParamViews, kAdjoint, kFeat><<<g, kShadeThreads, 0, st>>>(
+            param_views<kParamViews>(host_views, nviews), nviews, blk_offs, nblocks, nsub, keys, reset_keys, frame_cnt,
+            def);
 }
 
 template <bool kAdjoint>
-static void launch_shade_t(int feat, unsigned g, const ViewDev *views, const ParamViews *pv, int nviews,
+static void launch_shade_t(int feat, unsigned g, const ViewDev *views, const ViewDev *pv, int nviews,
                            const long long *blk_offs, long long nblocks, int nsub, unsigned long long *keys, int reset_keys,
                            const Counters *frame_cnt, const Deferred64 &def, cudaStream_t st)
 {
@@ -931,7 +936,7 @@ cudaError_t launch_shade(const ViewDev *views, int nviews, const long long *blk_
 {
     if (nblocks > 0) {
         const unsigned g = shade_grid(nblocks);
-        const ParamViews *pv = param_views(host_views, nviews);
+        const ViewDev *pv = host_views;
         if (adjoint)
             launch_shade_t<true>(feat, g, views, pv, nviews, blk_offs, nblocks, nsub, keys, reset_keys, frame_cnt, def,
                                  st);
@@ -1024,22 +1029,26 @@ __global__ void __launch_bounds__(kShadeThreads, kBackwardCtas)
     backward_body<kFeat>(views, nviews, blk_offs, nblocks, nsub);
 }
 
-template <int kFeat>
+template <int kN, int kFeat>
 __global__ void __launch_bounds__(kShadeThreads, kBackwardCtas)
-    k_backward_pv(const __grid_constant__ ParamViews pv, int nviews, const long long *__restrict__ blk_offs,
+    k_backward_pv(const __grid_constant__ ParamViews<kN> pv, int nviews, const long long *__restrict__ blk_offs,
                   long long nblocks, int nsub)
 {
     backward_body<kFeat>(pv.v, nviews, blk_offs, nblocks, nsub);
 }
 
 template <int kFeat>
-static void launch_backward_one(unsigned g, const ViewDev *views, const ParamViews *pv, int nviews,
+static void launch_backward_one(unsigned g, const ViewDev *views, const ViewDev *host_views, int nviews,
                                 const long long *blk_offs, long long nblocks, int nsub, cudaStream_t st)
 {
-    if (pv)
-        k_backward_pv<kFeat><<<g, kShadeThreads, 0, st>>>(*pv, nviews, blk_offs, nblocks, nsub);
-    else
+    if (!host_views || !shade_reads_params(nviews))
         k_backward<kFeat><<<g, kShadeThreads, 0, st>>>(views, nviews, blk_offs, nblocks, nsub);
+    else if (nviews <= kFewViews)
+        k_backward_pv<kFewViews, kFeat><<<g, kShadeThreads, 0, st>>>(param_views<kFewViews>(host_views, nviews), nviews,
+                                                                     blk_offs, nblocks, nsub);
+    else
+        k_backward_pv<kParamViews, kFeat><<<g, kShadeThreads, 0, st>>>(param_views<kParamViews>(host_views, nviews),
+                                                                       nviews, blk_offs, nblocks, nsub);
 }
 
 cudaError_t launch_backward(const ViewDev *views, int nviews, const long long *blk_offs, long long nblocks, int nsub,
@@ -1047,7 +1056,7 @@ cudaError_t launch_backward(const ViewDev *views, int nviews, const long long *b
 {
     if (nblocks > 0) {
         const unsigned g = shade_grid(nblocks);
-        const ParamViews *pv = param_views(host_views, nviews);
+        const ViewDev *pv = host_views;
         if (feat & kFeatF64) {
             launch_backward_one<kFeatSpec | kFeatLut | kFeatF64>(g, views, pv, nviews, blk_offs, nblocks, nsub, st);
             return cudaGetLastError();
