@@ -78,25 +78,40 @@ __global__ void k_scene_check(const float4 *__restrict__ vtx, const float4 *__re
 }
 
 // Batched scene update: the statuses are cleared, then every vertex of every
-// scene of the chunk takes its new arrays and is checked (blockIdx.y: scene).
+// scene of the chunk takes its new arrays and is checked.  The grid holds the
+// scenes' blocks one after the other (first: each scene's first block), and
+// an array that is replaced is not read (64 scenes, 2.6 M vertices, all
+// three arrays: 36 us against 59 with a block row per scene as long as the
+// largest and every record read first).
 struct SceneUpdateChunk {
     SceneUpdate u[kSceneUpdateChunk];
+    int first[kSceneUpdateChunk + 1];
     int n;
 };
 
-__global__ void k_scene_status_clear(const SceneUpdateChunk c)
+__global__ void k_scene_status_clear(const __grid_constant__ SceneUpdateChunk c)
 {
     if ((int)threadIdx.x < c.n)
         *c.u[threadIdx.x].status = 0u;
 }
 
-__global__ void k_scene_update_batch(const SceneUpdateChunk c)
+__global__ void __launch_bounds__(256) k_scene_update_batch(const __grid_constant__ SceneUpdateChunk c)
 {
-    const SceneUpdate &u = c.u[blockIdx.y];
-    const long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    int lo = 0, hi = c.n - 1;  // the block's scene
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (c.first[mid] <= (int)blockIdx.x)
+            lo = mid;
+        else
+            hi = mid - 1;
+    }
+    const SceneUpdate &u = c.u[lo];
+    const long long k = (long long)((int)blockIdx.x - c.first[lo]) * blockDim.x + threadIdx.x;
     if (k >= u.V)
         return;
-    float4 a = u.vtx[2 * k], b = u.vtx[2 * k + 1], cl = u.col4[k];
+    float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = a, cl = a;
+    if (!u.pos || !u.vel)
+        a = u.vtx[2 * k];
     if (u.pos) {
         a.x = u.pos[3 * k];
         a.y = u.pos[3 * k + 1];
@@ -105,12 +120,16 @@ __global__ void k_scene_update_batch(const SceneUpdateChunk c)
     if (u.vel) {
         a.w = u.vel[3 * k];
         b = make_float4(u.vel[3 * k + 1], u.vel[3 * k + 2], 0.f, 0.f);
+    } else {
+        b = u.vtx[2 * k + 1];
     }
+    cl = u.col ? make_float4(u.col[3 * k], u.col[3 * k + 1], u.col[3 * k + 2], 0.f) : u.col4[k];
+    if (u.pos || u.vel)
+        u.vtx[2 * k] = a;
+    if (u.vel)
+        u.vtx[2 * k + 1] = b;
     if (u.col)
-        cl = make_float4(u.col[3 * k], u.col[3 * k + 1], u.col[3 * k + 2], 0.f);
-    u.vtx[2 * k] = a;
-    u.vtx[2 * k + 1] = b;
-    u.col4[k] = cl;
+        u.col4[k] = cl;
     const bool ok = isfinite(a.x) && isfinite(a.y) && isfinite(a.z) && isfinite(a.w) && isfinite(b.x) &&
                     isfinite(b.y) && isfinite(cl.x) && isfinite(cl.y) && isfinite(cl.z);
     if (!ok)
@@ -122,14 +141,14 @@ cudaError_t launch_scene_update_batch(const SceneUpdate *u, int n, cudaStream_t 
     for (int c0 = 0; c0 < n; c0 += kSceneUpdateChunk) {
         SceneUpdateChunk c;
         c.n = std::min(kSceneUpdateChunk, n - c0);
-        long long vmax = 0;
+        c.first[0] = 0;
         for (int k = 0; k < c.n; ++k) {
             c.u[k] = u[c0 + k];
-            vmax = std::max(vmax, c.u[k].V);
+            c.first[k + 1] = c.first[k] + (int)((c.u[k].V + 255) / 256);  // V <= 2^30: 2^22 blocks, 2^28 in all
         }
         k_scene_status_clear<<<1, kSceneUpdateChunk, 0, st>>>(c);
-        if (vmax > 0)
-            k_scene_update_batch<<<dim3((unsigned)((vmax + 255) / 256), (unsigned)c.n), 256, 0, st>>>(c);
+        if (c.first[c.n] > 0)
+            k_scene_update_batch<<<(unsigned)c.first[c.n], 256, 0, st>>>(c);
     }
     return cudaGetLastError();
 }
