@@ -346,10 +346,10 @@ typedef struct {
 } pr_unfoveate_entry;
 
 /* The display step of n views (Sec. 3.1.1, "Display") in one sequence.
- * MIP: one launch per pyramid level over every view that has the level and
- * one over the display pixels of all views, the pyramids side by side in the
- * workspace.  Projected filter: the single-view kernels view after view,
- * each view's q table in the same scratch.  Entry k's out equals that of
+ * MIP: two launches for the pyramids of all views, side by side in the
+ * workspace (16 bytes per texel above the image), and one over the display
+ * pixels of all views.  Projected filter: the single-view kernels view after
+ * view, each view's table of taps (16 bytes per pixel) in the same scratch.  Entry k's out equals that of
  * pr_unfoveate with the same view, rgb, out, Wd, Hd and params->method and
  * sigma, bit for bit; params->Wd and Hd are ignored.  Scratch grows on
  * demand.  The view

@@ -15,8 +15,10 @@
 //    filter into the foveated domain); weights are taken relative to the
 //    nearest sample, whose factor cancels, so they cannot all underflow.
 //
-// One thread per display pixel, CTAs of 32 x 8 pixels (neighbouring rows
-// share their texels in L1); planar rgb in and out, coalesced along x.
+// One thread per display pixel; planar rgb in and out.  What a tap reads
+// lies together: the pyramid's texels above level 0 are (r, g, b, 0), and the
+// projected filter first makes a table of (scale of q, r, g, b) per
+// framebuffer pixel.
 #include <algorithm>
 #include <cstring>
 
@@ -27,7 +29,10 @@ namespace pr {
 constexpr int kMaxMipLevels = 16;  // 16384 x 16384 needs 15
 
 struct MipPyramid {
-    const float *lev[kMaxMipLevels];  // level 0 = the framebuffer image, the others in the call's scratch
+    // level 0 = the framebuffer image (planar); the others in the call's
+    // scratch, a texel's (r, g, b, 0) side by side
+    const float *rgb;
+    float4 *lev[kMaxMipLevels];
     int w0, h0;                       // size of level 0; level k has ceil(w0 / 2^k) x ceil(h0 / 2^k) texels
     int L;
 };
@@ -43,7 +48,8 @@ struct DisplayView {
     float alpha, inv_alpha;
     const float *p_lut;  // or: the sampled p (then alpha is unused)
     int p_n;
-    float rWd, rHd;      // 1 / Wd, 1 / Hd, correctly rounded (pixel_centre)
+    float rW, rH;        // 1 / W, 1 / H, correctly rounded (pixel_centre)
+    float rWd, rHd;      // 1 / Wd, 1 / Hd, the same
     float scale;         // max(W / Wd, H / Hd)
     float sigma;         // projected filter width, display pixels
 };
@@ -75,48 +81,50 @@ __device__ __forceinline__ void mip_tile(const MipPyramid &pyr, int tx, int ty)
     __shared__ float s_a[3][kTileSide / 2 * (kTileSide / 2)], s_b[3][kTileSide / 4 * (kTileSide / 4)];
     const int W = pyr.w0, H = pyr.h0;
     const int top = min(kTileLevels, pyr.L - 1);
-    if (top >= 1) {  // level 1 from the image: sixteen loads of a thread in flight
+    if (top >= 1) {  // level 1 from the image
         constexpr int side = kTileSide / 2, per = side * side / kTileThreads;
         const int w = mip_size(W, 1), h = mip_size(H, 1);
-        const float *src = pyr.lev[0];
-        float *dst = const_cast<float *>(pyr.lev[1]);
-        for (int c = 0; c < 3; ++c, src += (size_t)W * H, dst += (size_t)w * h) {
+        const unsigned plane = (unsigned)W * (unsigned)H;  // <= 2^28
 #pragma unroll
-            for (int i = 0; i < per; ++i) {
-                const int t = threadIdx.x + i * kTileThreads;
-                const int x = tx * side + t % side, y = ty * side + t / side;
-                if (x >= w || y >= h)
-                    continue;
-                const bool xr = 2 * x + 1 < W, yr = 2 * y + 1 < H;
-                const float *p = src + (unsigned)(2 * y * W + 2 * x);
+        for (int i = 0; i < per; ++i) {
+            const int t = threadIdx.x + i * kTileThreads;
+            const int x = tx * side + t % side, y = ty * side + t / side;
+            if (x >= w || y >= h)
+                continue;
+            const bool xr = 2 * x + 1 < W, yr = 2 * y + 1 < H;
+            const float *p = pyr.rgb + (unsigned)(2 * y * W + 2 * x);
+            float v[3];
+#pragma unroll
+            for (int c = 0; c < 3; ++c, p += plane) {
                 const float *p1 = p + W;
-                const float v = mip_mean(__ldg(p), xr ? __ldg(p + 1) : 0.f, yr ? __ldg(p1) : 0.f,
-                                         xr && yr ? __ldg(p1 + 1) : 0.f, xr, yr);
-                dst[(unsigned)(y * w + x)] = v;
-                s_a[c][t] = v;
+                v[c] = mip_mean(__ldg(p), xr ? __ldg(p + 1) : 0.f, yr ? __ldg(p1) : 0.f, xr && yr ? __ldg(p1 + 1) : 0.f,
+                                xr, yr);
+                s_a[c][t] = v[c];
             }
+            pyr.lev[1][(unsigned)(y * w + x)] = make_float4(v[0], v[1], v[2], 0.f);
         }
         __syncthreads();
     }
     for (int k = 2; k <= top; ++k) {
         const int side = kTileSide >> k, lg = kTileLevels - k;  // the tile's texels of this level
         const int w = mip_size(W, k), h = mip_size(H, k), wb = mip_size(W, k - 1), hb = mip_size(H, k - 1);
-        float *dst = const_cast<float *>(pyr.lev[k]);
-        const unsigned plane = (unsigned)w * (unsigned)h;
-        for (int u = threadIdx.x; u < 3 * side * side; u += kTileThreads) {
-            const int c = u >> (2 * lg), t = u & (side * side - 1);
+        for (int t = threadIdx.x; t < side * side; t += kTileThreads) {
             const int ly = t >> lg, lx = t & (side - 1);
             const int x = (tx << lg) + lx, y = (ty << lg) + ly;
             if (x >= w || y >= h)
                 continue;
             const bool xr = 2 * x + 1 < wb, yr = 2 * y + 1 < hb;
-            const float *p = (k & 1 ? s_b[c] : s_a[c]) + 4 * side * ly + 2 * lx;  // odd levels sit in s_a, even in s_b
-            const float v = mip_mean(p[0], p[1], p[2 * side], p[2 * side + 1], xr, yr);
-            dst[plane * c + (unsigned)(y * w + x)] = v;
-            if (k & 1)
-                s_a[c][t] = v;
-            else
-                s_b[c][t] = v;
+            float v[3];
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                const float *p = (k & 1 ? s_b[c] : s_a[c]) + 4 * side * ly + 2 * lx;  // odd levels sit in s_a, even in s_b
+                v[c] = mip_mean(p[0], p[1], p[2 * side], p[2 * side + 1], xr, yr);
+                if (k & 1)
+                    s_a[c][t] = v[c];
+                else
+                    s_b[c][t] = v[c];
+            }
+            pyr.lev[k][(unsigned)(y * w + x)] = make_float4(v[0], v[1], v[2], 0.f);
         }
         __syncthreads();
     }
@@ -129,13 +137,14 @@ __device__ __forceinline__ void mip_top(const MipPyramid &pyr)
     for (int k = kTileLevels + 1; k < pyr.L; ++k) {
         const int w = mip_size(pyr.w0, k), h = mip_size(pyr.h0, k);
         const int wb = mip_size(pyr.w0, k - 1), hb = mip_size(pyr.h0, k - 1);
-        const float *src = pyr.lev[k - 1];
-        float *dst = const_cast<float *>(pyr.lev[k]);
-        for (int t = threadIdx.x; t < 3 * w * h; t += blockDim.x) {
-            const int c = t / (w * h), y = (t - c * w * h) / w, x = t - c * w * h - y * w;
+        const float4 *src = pyr.lev[k - 1], none = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int t = threadIdx.x; t < w * h; t += blockDim.x) {
+            const int y = t / w, x = t - y * w;
             const bool xr = 2 * x + 1 < wb, yr = 2 * y + 1 < hb;
-            const float *p = src + (size_t)c * wb * hb + (size_t)(2 * y) * wb + 2 * x;
-            dst[t] = mip_mean(p[0], xr ? p[1] : 0.f, yr ? p[wb] : 0.f, xr && yr ? p[wb + 1] : 0.f, xr, yr);
+            const float4 *p = src + (size_t)(2 * y) * wb + 2 * x;
+            const float4 a = p[0], b = xr ? p[1] : none, c = yr ? p[wb] : none, d = xr && yr ? p[wb + 1] : none;
+            pyr.lev[k][t] = make_float4(mip_mean(a.x, b.x, c.x, d.x, xr, yr), mip_mean(a.y, b.y, c.y, d.y, xr, yr),
+                                        mip_mean(a.z, b.z, c.z, d.z, xr, yr), 0.f);
         }
         __syncthreads();  // this level is the next one's source
     }
@@ -152,22 +161,35 @@ __global__ void __launch_bounds__(512) k_mip_top(const MipPyramid pyr) { mip_top
 // eighty instructions; the same bits).
 __device__ __forceinline__ float radial_pow(float x, float e) { return e == 1.f ? x : powf(x, e); }
 
-// Display location q(c) of every framebuffer pixel centre c (the offset from
-// the fovea scaled by (|e|/D)^(alpha - 1)), for the projected filter.
-__global__ void k_q_table(const DisplayView dv, float rW, float rH, float2 *__restrict__ table)
+// 2^x by the special-function unit alone: exp2f scales its argument around
+// results below 2^-126, which a weight beside the reference sample's 1 may
+// lose.
+__device__ __forceinline__ float exp2_ftz(float x)
+{
+    float y;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
+// What a tap of the projected filter reads of a framebuffer pixel c: the
+// factor (|e|/D)^(alpha - 1) that q scales its offset e from the fovea by
+// (1 without foveation, where offsets are taken from 0), and its colour.
+__global__ void k_tap_table(const DisplayView dv, const float *__restrict__ rgb,
+                            float4 *__restrict__ table)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y;
     if (i >= dv.W)
         return;
-    float q0 = pixel_centre(i, dv.W, rW), q1 = pixel_centre(j, dv.H, rH);
+    const unsigned o = (unsigned)(j * dv.W + i), plane = (unsigned)dv.W * (unsigned)dv.H;  // <= 2^28
+    const float r0 = rgb[o], g0 = rgb[plane + o], b0 = rgb[2 * plane + o];
+    float s = 1.f;
     if (dv.fov) {
-        const float e0 = q0 - dv.fx, e1 = q1 - dv.fy, r = sqrtf(fmaf(e0, e0, e1 * e1));
+        const float e0 = pixel_centre(i, dv.W, dv.rW) - dv.fx, e1 = pixel_centre(j, dv.H, dv.rH) - dv.fy,
+                    r = sqrtf(fmaf(e0, e0, e1 * e1));
         const SampledP sp{dv.p_lut, dv.p_n};
-        const float s = r > 0.f ? (dv.p_lut ? sp.p(r) / r : radial_pow(r * (1.f / kSqrt2), dv.alpha - 1.f)) : 0.f;
-        q0 = fmaf(e0, s, dv.fx);
-        q1 = fmaf(e1, s, dv.fy);
+        s = r > 0.f ? (dv.p_lut ? sp.p(r) / r : radial_pow(r * (1.f / kSqrt2), dv.alpha - 1.f)) : 0.f;
     }
-    table[(size_t)j * dv.W + i] = make_float2(q0, q1);
+    table[o] = make_float4(s, r0, g0, b0);
 }
 
 // Cubic B-spline weights of the taps at -1, 0, 1 for a sample at d in
@@ -185,8 +207,32 @@ __device__ __forceinline__ void bspline_taps(float d, float (&w)[3])
 }
 
 // 3-tap cubic sample of one level at texel coordinates (s, t): the three
-// taps of each row first, then the rows.
-__device__ __forceinline__ void sample3(const float *__restrict__ lev, int w, int h, float s, float t, float out[3])
+// taps of each row first, then the rows.  kPlanar: level 0, the image;
+// otherwise a level of interleaved texels, where one 16-byte load serves a
+// tap's three channels.
+struct Texels {
+    const float *img;
+    const float4 *lev;
+    unsigned plane;  // <= 2^28
+};
+
+template <bool kPlanar>
+__device__ __forceinline__ float3 texel(const Texels &tx, unsigned o)
+{
+    if (kPlanar)
+        return make_float3(__ldg(tx.img + o), __ldg(tx.img + tx.plane + o), __ldg(tx.img + 2 * tx.plane + o));
+    const float4 v = __ldg(tx.lev + o);
+    return make_float3(v.x, v.y, v.z);
+}
+
+__device__ __forceinline__ float3 taps3(const float (&w)[3], float3 a, float3 b, float3 c)
+{
+    return make_float3(fmaf(w[0], a.x, fmaf(w[1], b.x, w[2] * c.x)), fmaf(w[0], a.y, fmaf(w[1], b.y, w[2] * c.y)),
+                       fmaf(w[0], a.z, fmaf(w[1], b.z, w[2] * c.z)));
+}
+
+template <bool kPlanar>
+__device__ __forceinline__ void sample3(const Texels &tx, int w, int h, float s, float t, float out[3])
 {
     const float fs = floorf(s + 0.5f), ft = floorf(t + 0.5f);
     float wx[3], wy[3];
@@ -194,39 +240,32 @@ __device__ __forceinline__ void sample3(const float *__restrict__ lev, int w, in
     bspline_taps(t - ft, wy);
     const float inv = 1.f / ((wx[0] + wx[1] + wx[2]) * (wy[0] + wy[1] + wy[2]));  // sums of about 1
     const int is = (int)fs, it = (int)ft;
-    const unsigned plane = (unsigned)w * (unsigned)h;  // <= 2^28
-    out[0] = out[1] = out[2] = 0.f;
+    float3 row[3];
     if (is >= 1 && is < w - 1 && it >= 1 && it < h - 1) {
-        // inside: the taps are neighbours, nine row addresses serve all
-        const float *p = lev + (unsigned)((it - 1) * w + is - 1);
+        // inside: the taps are neighbours
+        const unsigned o = (unsigned)((it - 1) * w + is - 1);
 #pragma unroll
-        for (int c = 0; c < 3; ++c, p += plane) {
-            const float *r1 = p + w, *r2 = r1 + w;
-            const float a = fmaf(wx[0], __ldg(p), fmaf(wx[1], __ldg(p + 1), wx[2] * __ldg(p + 2)));
-            const float b = fmaf(wx[0], __ldg(r1), fmaf(wx[1], __ldg(r1 + 1), wx[2] * __ldg(r1 + 2)));
-            const float d = fmaf(wx[0], __ldg(r2), fmaf(wx[1], __ldg(r2 + 1), wx[2] * __ldg(r2 + 2)));
-            out[c] = fmaf(wy[2], d, fmaf(wy[1], b, wy[0] * a)) * inv;
+        for (int k = 0; k < 3; ++k) {
+            const unsigned ok = o + (unsigned)(k * w);
+            row[k] = taps3(wx, texel<kPlanar>(tx, ok), texel<kPlanar>(tx, ok + 1), texel<kPlanar>(tx, ok + 2));
         }
-        return;
-    }
-    const int x0 = min(max(is - 1, 0), w - 1), x1 = min(max(is, 0), w - 1), x2 = min(max(is + 1, 0), w - 1);
-    const unsigned r0 = (unsigned)(min(max(it - 1, 0), h - 1) * w), r1 = (unsigned)(min(max(it, 0), h - 1) * w),
-                   r2 = (unsigned)(min(max(it + 1, 0), h - 1) * w);
-    const float *p = lev;
+    } else {
+        const int x0 = min(max(is - 1, 0), w - 1), x1 = min(max(is, 0), w - 1), x2 = min(max(is + 1, 0), w - 1);
 #pragma unroll
-    for (int c = 0; c < 3; ++c, p += plane) {
-        const float a = fmaf(wx[0], __ldg(p + (r0 + x0)), fmaf(wx[1], __ldg(p + (r0 + x1)), wx[2] * __ldg(p + (r0 + x2))));
-        const float b = fmaf(wx[0], __ldg(p + (r1 + x0)), fmaf(wx[1], __ldg(p + (r1 + x1)), wx[2] * __ldg(p + (r1 + x2))));
-        const float d = fmaf(wx[0], __ldg(p + (r2 + x0)), fmaf(wx[1], __ldg(p + (r2 + x1)), wx[2] * __ldg(p + (r2 + x2))));
-        out[c] = fmaf(wy[2], d, fmaf(wy[1], b, wy[0] * a)) * inv;
+        for (int k = 0; k < 3; ++k) {
+            const unsigned r = (unsigned)(min(max(it - 1 + k, 0), h - 1) * w);
+            row[k] = taps3(wx, texel<kPlanar>(tx, r + x0), texel<kPlanar>(tx, r + x1), texel<kPlanar>(tx, r + x2));
+        }
     }
+    out[0] = fmaf(wy[2], row[2].x, fmaf(wy[1], row[1].x, wy[0] * row[0].x)) * inv;
+    out[1] = fmaf(wy[2], row[2].y, fmaf(wy[1], row[1].y, wy[0] * row[0].y)) * inv;
+    out[2] = fmaf(wy[2], row[2].z, fmaf(wy[1], row[1].z, wy[0] * row[0].z)) * inv;
 }
 
 // Display pixel (a, b) of a view.
 template <int kMethod>
 __device__ __forceinline__ void unfoveate_pixel(const DisplayView &dv, const MipPyramid &pyr,
-                                                const float *__restrict__ rgb, const float2 *__restrict__ qtab,
-                                                float *__restrict__ out, int a, int b)
+                                                const float4 *__restrict__ tab, float *__restrict__ out, int a, int b)
 {
     const float x0 = pixel_centre(a, dv.Wd, dv.rWd), x1 = pixel_centre(b, dv.Hd, dv.rHd);
     // u = q^-1(x): the offset from the fovea scaled by (|e|/D)^(1/alpha - 1)
@@ -255,10 +294,16 @@ __device__ __forceinline__ void unfoveate_pixel(const DisplayView &dv, const Mip
         const float f = lambda - (float)k0;
         float s0[3], s1[3];
         const int w0 = mip_size(dv.W, k0), h0 = mip_size(dv.H, k0);
-        sample3(pyr.lev[k0], w0, h0, fmaf(u0, (float)w0, -0.5f), fmaf(u1, (float)h0, -0.5f), s0);
+        const Texels tx0{pyr.rgb, pyr.lev[k0], (unsigned)dv.W * (unsigned)dv.H};
+        const float c0 = fmaf(u0, (float)w0, -0.5f), c1 = fmaf(u1, (float)h0, -0.5f);
+        if (k0 == 0)
+            sample3<true>(tx0, w0, h0, c0, c1, s0);
+        else
+            sample3<false>(tx0, w0, h0, c0, c1, s0);
         if (f > 0.f) {
             const int w1 = mip_size(dv.W, k1), h1 = mip_size(dv.H, k1);
-            sample3(pyr.lev[k1], w1, h1, fmaf(u0, (float)w1, -0.5f), fmaf(u1, (float)h1, -0.5f), s1);
+            const Texels tx1{nullptr, pyr.lev[k1], 0u};  // f > 0: k1 = k0 + 1
+            sample3<false>(tx1, w1, h1, fmaf(u0, (float)w1, -0.5f), fmaf(u1, (float)h1, -0.5f), s1);
             for (int c = 0; c < 3; ++c)
                 res[c] = fmaf(f, s1[c] - s0[c], s0[c]);
         } else {
@@ -282,42 +327,63 @@ __device__ __forceinline__ void unfoveate_pixel(const DisplayView &dv, const Mip
         const float k2 = -0.5f / (dv.sigma * dv.sigma);
         const float fWd = (float)dv.Wd, fHd = (float)dv.Hd;
         const unsigned plane = (unsigned)dv.W * (unsigned)dv.H;  // <= 2^28
-        const float2 qm = __ldg(qtab + (unsigned)(j * dv.W + i));
-        float qm0 = qm.x, qm1 = qm.y;
+        // offsets from the fovea (from 0 without foveation, so that q = c)
+        const float fx = dv.fov ? dv.fx : 0.f, fy = dv.fov ? dv.fy : 0.f;
+        const float sm = __ldg(&tab[(unsigned)(j * dv.W + i)].x);
+        float qm0 = fmaf(pixel_centre(i, dv.W, dv.rW) - fx, sm, fx), qm1 = fmaf(pixel_centre(j, dv.H, dv.rH) - fy, sm, fy);
         {
             const float d0 = (x0 - qm0) * fWd, d1 = (x1 - qm1) * fHd;
             if (k2 * fmaf(d0, d0, d1 * d1) < -60.f) {
                 float d2min = INFINITY;
                 for (int dy = dy0; dy <= dy1; ++dy) {
-                    const float2 *qr = qtab + (unsigned)((j + dy) * dv.W + i + dx0);
-                    for (int dx = dx0; dx <= dx1; ++dx, ++qr) {
-                        const float2 q = __ldg(qr);
-                        const float e0 = (x0 - q.x) * fWd, e1 = (x1 - q.y) * fHd;
-                        const float q2 = fmaf(e0, e0, e1 * e1);
+                    const float4 *tr = tab + (unsigned)((j + dy) * dv.W + i);
+                    const float e1 = pixel_centre(j + dy, dv.H, dv.rH) - fy;
+                    for (int dx = dx0; dx <= dx1; ++dx) {
+                        const float s = __ldg(&tr[dx].x);
+                        const float q0 = fmaf(pixel_centre(i + dx, dv.W, dv.rW) - fx, s, fx), q1 = fmaf(e1, s, fy);
+                        const float f0 = (x0 - q0) * fWd, f1 = (x1 - q1) * fHd;
+                        const float q2 = fmaf(f0, f0, f1 * f1);
                         if (q2 < d2min) {
                             d2min = q2;
-                            qm0 = q.x;
-                            qm1 = q.y;
+                            qm0 = q0;
+                            qm1 = q1;
                         }
                     }
                 }
             }
         }
-        const float s0 = 2.f * x0, s1 = 2.f * x1;
+        // weight of a sample at q: 2^((qm - q)(2 x - qm - q) . (kw, kh))
+        const float2 qm2 = make_float2(qm0, qm1), far = make_float2(2.f * x0 - qm0, 2.f * x1 - qm1);
         const float kw = k2 * 1.44269504f * fWd * fWd, kh = k2 * 1.44269504f * fHd * fHd;  // exp as a power of two
         float acc[3] = {0.f, 0.f, 0.f}, wsum = 0.f;
-        for (int dy = dy0; dy <= dy1; ++dy) {
-            const unsigned o = (unsigned)((j + dy) * dv.W + i + dx0);
-            const float2 *qr = qtab + o;
-            const float *p0 = rgb + o, *p1 = p0 + plane, *p2 = p1 + plane;
-            for (int dx = 0; dx <= dx1 - dx0; ++dx) {
-                const float2 q = __ldg(qr + dx);
-                const float t0 = (qm0 - q.x) * (s0 - q.x - qm0), t1 = (qm1 - q.y) * (s1 - q.y - qm1);
-                const float w = exp2f(fmaf(t0, kw, t1 * kh));
-                wsum += w;
-                acc[0] = fmaf(w, __ldg(p0 + dx), acc[0]);
-                acc[1] = fmaf(w, __ldg(p1 + dx), acc[1]);
-                acc[2] = fmaf(w, __ldg(p2 + dx), acc[2]);
+        const float2 fov = make_float2(fx, fy);
+        auto tap = [&](float e0, float e1, float4 c) {
+            const float2 minus = make_float2(-1.f, -1.f), q = __ffma2_rn(make_float2(e0, e1), make_float2(c.x, c.x), fov);
+            const float2 t = __fmul2_rn(__ffma2_rn(q, minus, qm2), __ffma2_rn(q, minus, far));
+            const float w = exp2_ftz(fmaf(t.x, kw, t.y * kh));
+            wsum += w;
+            acc[0] = fmaf(w, c.y, acc[0]);
+            acc[1] = fmaf(w, c.z, acc[1]);
+            acc[2] = fmaf(w, c.w, acc[2]);
+        };
+        const float4 *tr = tab + (unsigned)((j + dy0) * dv.W + i + dx0);
+        if (dx1 - dx0 == 4) {  // five taps a row (all but two columns at either side), their loads in flight together
+            float e0[5];
+#pragma unroll
+            for (int dx = 0; dx < 5; ++dx)
+                e0[dx] = pixel_centre(i - 2 + dx, dv.W, dv.rW) - fx;
+#pragma unroll 1
+            for (int dy = dy0; dy <= dy1; ++dy, tr += dv.W) {
+                const float e1 = pixel_centre(j + dy, dv.H, dv.rH) - fy;
+#pragma unroll
+                for (int dx = 0; dx < 5; ++dx)
+                    tap(e0[dx], e1, __ldg(tr + dx));
+            }
+        } else {
+            for (int dy = dy0; dy <= dy1; ++dy, tr += dv.W) {
+                const float e1 = pixel_centre(j + dy, dv.H, dv.rH) - fy;
+                for (int dx = dx0; dx <= dx1; ++dx)
+                    tap(pixel_centre(i + dx, dv.W, dv.rW) - fx, e1, __ldg(tr + (dx - dx0)));
             }
         }
         const float inv = 1.f / wsum;
@@ -330,18 +396,35 @@ __device__ __forceinline__ void unfoveate_pixel(const DisplayView &dv, const Mip
     out[2 * dplane + o] = res[2];
 }
 
-// CTAs of the display kernels: 32 x 8 display pixels.
+// CTAs of the display kernels: 32 x 8 display pixels, six per SM, a warp's
+// pixels 16 x 2.  Bound: the L1 data pipe (71 to 77 % busy) and issue.  q^-1
+// is curved, so a row of 32 display pixels reads up to fifteen rows of
+// texels, and every texel row of a tap is a cache line of its own: squarer
+// warps meet fewer (32 x 1 / 16 x 2 / 8 x 4 with planar texels: projected
+// filter, 1440 x 1600 to 1800 x 2000, 171 / 152 / 156 us a pass; MIP, 16
+// views, 414 / 408 / 426), and so does one 16-byte load per tap instead of
+// one per channel (and for q): 152 -> 132 and 408 -> 391 us.  Six CTAs per
+// SM (40 registers) against four and five: 126 / 132 / 130 and 383 / 394 /
+// 391 us.
 constexpr int kDispW = 32, kDispH = 8;
+constexpr int kWarpW = 16, kWarpH = 32 / kWarpW;
+constexpr int kDispCtas = 6;
+
+__device__ __forceinline__ int2 disp_pixel(int bx, int by)
+{
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, per = kDispW / kWarpW;
+    return make_int2(bx * kDispW + (w % per) * kWarpW + lane % kWarpW, by * kDispH + (w / per) * kWarpH + lane / kWarpW);
+}
 
 template <int kMethod>
-__global__ void __launch_bounds__(kDispW *kDispH) k_unfoveate(const DisplayView dv, const MipPyramid pyr,
-                                                             const float *__restrict__ rgb,
-                                                             const float2 *__restrict__ qtab, float *__restrict__ out)
+__global__ void __launch_bounds__(kDispW *kDispH, kDispCtas) k_unfoveate(const DisplayView dv, const MipPyramid pyr,
+                                                             const float4 *__restrict__ tab, float *__restrict__ out)
 {
-    const int a = blockIdx.x * kDispW + threadIdx.x % kDispW, b = blockIdx.y * kDispH + threadIdx.x / kDispW;
+    const int2 at = disp_pixel(blockIdx.x, blockIdx.y);
+    const int a = at.x, b = at.y;
     if (a >= dv.Wd || b >= dv.Hd)
         return;
-    unfoveate_pixel<kMethod>(dv, pyr, rgb, qtab, out, a, b);
+    unfoveate_pixel<kMethod>(dv, pyr, tab, out, a, b);
 }
 
 // ---- the batched display step (MIP): many views, two launches for their
@@ -352,8 +435,7 @@ __global__ void __launch_bounds__(kDispW *kDispH) k_unfoveate(const DisplayView 
 // are the same.
 struct DisplayBatchView {
     DisplayView dv;
-    MipPyramid pyr;  // level 0 = rgb
-    const float *rgb;
+    MipPyramid pyr;
     float *out;
     // block / blocks per row as (block * mul) >> 40: the round-up reciprocals
     // of Granlund and Montgomery (1994), exact for blocks < 2^23 and rows of
@@ -386,7 +468,7 @@ __global__ void __launch_bounds__(512) k_mip_top_batch(const DisplayBatchView *_
 }
 
 // The display pixels of every view.
-__global__ void __launch_bounds__(kDispW *kDispH, 5) k_unfoveate_mip_batch(const DisplayBatchView *__restrict__ tab,
+__global__ void __launch_bounds__(kDispW *kDispH, kDispCtas) k_unfoveate_mip_batch(const DisplayBatchView *__restrict__ tab,
                                                                           const long long *__restrict__ blk, int n)
 {
     const int q = block_view(blk, n, blockIdx.x);
@@ -394,10 +476,11 @@ __global__ void __launch_bounds__(kDispW *kDispH, 5) k_unfoveate_mip_batch(const
     const DisplayView dv = e.dv;
     const unsigned t = (unsigned)(blockIdx.x - blk[q]);
     const int by = (int)((t * e.mul_disp) >> 40), bx = (int)t - by * ((dv.Wd + kDispW - 1) / kDispW);
-    const int a = bx * kDispW + threadIdx.x % kDispW, b = by * kDispH + threadIdx.x / kDispW;
+    const int2 at = disp_pixel(bx, by);
+    const int a = at.x, b = at.y;
     if (a >= dv.Wd || b >= dv.Hd)
         return;
-    unfoveate_pixel<PR_UNFOVEATE_MIP_CUBIC>(dv, e.pyr, e.rgb, nullptr, e.out, a, b);
+    unfoveate_pixel<PR_UNFOVEATE_MIP_CUBIC>(dv, e.pyr, nullptr, e.out, a, b);
 }
 
 int mip_level_count(int W, int H)
@@ -411,18 +494,19 @@ int mip_level_count(int W, int H)
     return L;
 }
 
-// Scratch floats of the display step: the MIP pyramid, or the q table of
-// the projected filter (2 per framebuffer pixel).
-size_t mip_pyramid_floats(int W, int H)
+// Scratch floats of a view's display step, four per texel: the levels above
+// the image (MIP), or the tap table of the projected filter.
+size_t display_scratch_floats(int method, int W, int H)
 {
+    if (method == PR_UNFOVEATE_PROJECTED)
+        return (size_t)4 * W * H;
     size_t n = 0;
-    for (;;) {
-        n += (size_t)3 * W * H;
-        if (W == 1 && H == 1)
-            return n;
+    while (W > 1 || H > 1) {
         W = (W + 1) / 2;
         H = (H + 1) / 2;
+        n += (size_t)4 * W * H;
     }
+    return n;
 }
 
 // Level pointers of a pyramid with its levels 1 .. L - 1 at `p` one after the
@@ -434,16 +518,17 @@ static bool fill_pyramid(MipPyramid &pyr, int W, int H, const float *rgb, float 
         return false;
     pyr.w0 = W;
     pyr.h0 = H;
-    pyr.lev[0] = rgb;
+    pyr.rgb = rgb;
+    pyr.lev[0] = nullptr;
     for (int k = 1; k < pyr.L; ++k) {
-        pyr.lev[k] = p;
-        p += (size_t)3 * mip_size(W, k) * mip_size(H, k);
+        pyr.lev[k] = reinterpret_cast<float4 *>(p);
+        p += (size_t)4 * mip_size(W, k) * mip_size(H, k);
     }
     return true;
 }
 
 cudaError_t launch_unfoveate(int method, int W, int H, int mode, float fx, float fy, float alpha, const float *p_lut,
-                             int p_n, int Wd, int Hd, float sigma, const float *rgb, float *pyramid, float *out,
+                             int p_n, int Wd, int Hd, float sigma, const float *rgb, float *scratch, float *out,
                              cudaStream_t st)
 {
     DisplayView dv;
@@ -451,6 +536,8 @@ cudaError_t launch_unfoveate(int method, int W, int H, int mode, float fx, float
     dv.H = H;
     dv.Wd = Wd;
     dv.Hd = Hd;
+    dv.rW = 1.f / (float)W;
+    dv.rH = 1.f / (float)H;
     dv.rWd = 1.f / (float)Wd;
     dv.rHd = 1.f / (float)Hd;
     dv.fov = mode == PR_FOVEATED || mode == PR_BOTH;
@@ -466,41 +553,30 @@ cudaError_t launch_unfoveate(int method, int W, int H, int mode, float fx, float
     std::memset(&pyr, 0, sizeof pyr);
     const dim3 blk(kDispW * kDispH), grd((unsigned)((Wd + kDispW - 1) / kDispW), (unsigned)((Hd + kDispH - 1) / kDispH));
     if (method == PR_UNFOVEATE_MIP_CUBIC) {
-        if (!fill_pyramid(pyr, W, H, rgb, pyramid))
+        if (!fill_pyramid(pyr, W, H, rgb, scratch))
             return cudaErrorInvalidValue;
         if (pyr.L > 1)
             k_mip_tile<<<dim3((unsigned)((W + kTileSide - 1) / kTileSide), (unsigned)((H + kTileSide - 1) / kTileSide)),
                          kTileThreads, 0, st>>>(pyr);
         if (pyr.L > kTileLevels + 1)
             k_mip_top<<<1, 512, 0, st>>>(pyr);
-        k_unfoveate<PR_UNFOVEATE_MIP_CUBIC><<<grd, blk, 0, st>>>(dv, pyr, rgb, nullptr, out);
+        k_unfoveate<PR_UNFOVEATE_MIP_CUBIC><<<grd, blk, 0, st>>>(dv, pyr, nullptr, out);
     } else {
-        float2 *qtab = reinterpret_cast<float2 *>(pyramid);
+        float4 *tab = reinterpret_cast<float4 *>(scratch);
         const dim3 gq((unsigned)((W + 255) / 256), (unsigned)H);
-        k_q_table<<<gq, 256, 0, st>>>(dv, 1.f / (float)W, 1.f / (float)H, qtab);
-        k_unfoveate<PR_UNFOVEATE_PROJECTED><<<grd, blk, 0, st>>>(dv, pyr, rgb, qtab, out);
+        k_tap_table<<<gq, 256, 0, st>>>(dv, rgb, tab);
+        k_unfoveate<PR_UNFOVEATE_PROJECTED><<<grd, blk, 0, st>>>(dv, pyr, tab, out);
     }
     return cudaGetLastError();
-}
-
-static size_t view_scratch_floats(int W, int H)
-{
-    return (mip_pyramid_floats(W, H) + 3) & ~(size_t)3;  // 16-byte aligned carve
-}
-
-static size_t qtab_floats(int W, int H)
-{
-    return ((size_t)2 * W * H + 3) & ~(size_t)3;
 }
 
 size_t display_batch_scratch_floats(int method, const DisplayEntry *e, int n)
 {
     size_t f = 0;
     for (int q = 0; q < n; ++q) {
-        if (method == PR_UNFOVEATE_MIP_CUBIC)
-            f += view_scratch_floats(e[q].W, e[q].H);  // every view's pyramid, side by side
-        else
-            f = std::max(f, qtab_floats(e[q].W, e[q].H));  // one view's q table at a time
+        const size_t v = display_scratch_floats(method, e[q].W, e[q].H);
+        // every view's pyramid, side by side; one view's tap table at a time
+        f = method == PR_UNFOVEATE_MIP_CUBIC ? f + v : std::max(f, v);
     }
     return f;
 }
@@ -544,6 +620,8 @@ cudaError_t launch_unfoveate_batch(int method, float sigma, const DisplayEntry *
         dv.H = e[q].H;
         dv.Wd = e[q].Wd;
         dv.Hd = e[q].Hd;
+        dv.rW = 1.f / (float)dv.W;
+        dv.rH = 1.f / (float)dv.H;
         dv.rWd = 1.f / (float)dv.Wd;
         dv.rHd = 1.f / (float)dv.Hd;
         dv.fov = e[q].mode == PR_FOVEATED || e[q].mode == PR_BOTH;
@@ -555,11 +633,10 @@ cudaError_t launch_unfoveate_batch(int method, float sigma, const DisplayEntry *
         dv.p_n = e[q].p_n;
         dv.scale = fmaxf((float)dv.W / (float)dv.Wd, (float)dv.H / (float)dv.Hd);
         dv.sigma = sigma;
-        t.rgb = e[q].rgb;
         t.out = e[q].out;
         // the view's scratch: its pyramid levels 1..
         float *lp = p;
-        p += view_scratch_floats(dv.W, dv.H);
+        p += display_scratch_floats(method, dv.W, dv.H);
         if (!fill_pyramid(t.pyr, dv.W, dv.H, e[q].rgb, lp))
             return cudaErrorInvalidValue;
         any_tiles |= t.pyr.L > 1;

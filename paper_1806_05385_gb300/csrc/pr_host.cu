@@ -1203,8 +1203,8 @@ pr_status pr_unfoveate(pr_workspace *ws, const pr_view *view, const float *rgb, 
         return PR_ERR_INVALID_ARG;
     const pr_view &v = *view;
     cudaStream_t st = (cudaStream_t)stream;
-    // scratch: the MIP pyramid, or the projected filter's table of q (2 floats per pixel)
-    PR_TRY(ensure(ws->mip, sizeof(float) * mip_pyramid_floats(v.W, v.H)));
+    // scratch: the MIP pyramid, or the projected filter's tap table
+    PR_TRY(ensure(ws->mip, sizeof(float) * std::max<size_t>(display_scratch_floats(p.method, v.W, v.H), 1)));
     float *pyr = ws->mip.as<float>();
     PR_TRY(launch_unfoveate(p.method, v.W, v.H, v.mode, v.fovea[0], v.fovea[1], v.alpha,
                             v.foveation ? v.foveation->lut : nullptr, v.foveation ? v.foveation->n : 0, p.Wd, p.Hd,

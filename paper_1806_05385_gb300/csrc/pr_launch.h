@@ -126,11 +126,11 @@ cudaError_t launch_loss_finalize(const ViewDev *views, int nviews, const Counter
 cudaError_t launch_backward(const ViewDev *views, int nviews, const long long *blk_offs, long long nblocks, int nsub,
                             int feat, cudaStream_t st, const ViewDev *host_views = nullptr);
 
-// display step: unfoveation of a framebuffer image (pyramid: scratch of
-// mip_pyramid_floats(W, H) floats for the MIP method)
-size_t mip_pyramid_floats(int W, int H);
+// display step: unfoveation of a framebuffer image, with scratch of
+// display_scratch_floats (a multiple of 4; 16-byte aligned)
+size_t display_scratch_floats(int method, int W, int H);
 cudaError_t launch_unfoveate(int method, int W, int H, int mode, float fx, float fy, float alpha, const float *p_lut,
-                             int p_n, int Wd, int Hd, float sigma, const float *rgb, float *pyramid, float *out,
+                             int p_n, int Wd, int Hd, float sigma, const float *rgb, float *scratch, float *out,
                              cudaStream_t st);
 // the batched display step: n views, each with its own size, mode and
 // display size, one method and filter width for all
@@ -143,8 +143,7 @@ struct DisplayEntry {
     const float *rgb;  // device [3][H][W]
     float *out;        // device [3][Hd][Wd]
 };
-// scratch floats of the batch (MIP: each view's pyramid, 16-byte aligned;
-// the projected filter needs none)
+// scratch floats of the batch (16-byte aligned)
 size_t display_batch_scratch_floats(int method, const DisplayEntry *e, int n);
 // bytes of the host and device tables of a batch of n views
 size_t display_batch_table_bytes(int n);
