@@ -1038,38 +1038,40 @@ __device__ __forceinline__ long long warp_owner(const unsigned long long *cand_o
     return lo;
 }
 
-// The same for one lane's p (a plain binary search): only for pairs that a
-// warp's window of 32 list entries does not reach, which needs entries
-// without candidates (the paper's foveation bounds can empty a box).
-__device__ __forceinline__ long long owner_of(const unsigned long long *cand_off, long long m, long long p)
-{
-    long long lo = 0, hi = m - 1;
-    while (lo < hi) {
-        const long long mid = (lo + hi + 1) >> 1;
-        if ((long long)cand_off[mid] <= p)
-            lo = mid;
-        else
-            hi = mid - 1;
-    }
-    return lo;
-}
+constexpr int kBinChunks = 8, kBinWarps = 8, kBinGroup = 4;
 
-constexpr int kBinChunks = 8;
-
+// Each warp takes tasks of nch x 32 consecutive candidate pairs, up to
+// kBinChunks x 32 where there are enough of them: a frame with few pairs
+// spreads them over more of the resident warps.  The list entry of a task's
+// first pair comes from a warp-wide 32-ary search; every later entry marks
+// the pair it starts at in shared memory (of several that start at one pair
+// the last: entries may have no candidates, the paper's foveation bounds can
+// empty a box), and a pair belongs to the last mark at or before it, found
+// by a ballot.  The pairs' chains of dependent loads (list entry, pixel box,
+// tile and region boxes, half-planes) then run four chunks at a time, so
+// four loads of a lane are in flight at each link, and the hits are gathered
+// in shared memory for one atomic on the hit list per task and stores
+// without gaps.
+//
+// Bound: the latency of those chains and issue.  Against one chunk at a time
+// with a window of entries searched by shuffles: 64 views 0.169 -> 0.133 ms,
+// 1M-triangle stereo frame 0.107 -> 0.090, stereo HMD frame 0.028 -> 0.027.
+//
 // 256 threads, at most 64 registers: four CTAs (32 warps) per SM.  The
 // grid is four waves of them (bin_count_grid): the task loop is
 // grid-stride, so CTAs that start late take the place of those whose tasks
 // ran short, which evens out the end of the pass.
-__global__ void __launch_bounds__(256, 4) k_bin(const ViewDev *__restrict__ views, int nviews,
-                                             const long long *__restrict__ tri_offs, long long ttot,
-                                             const CandList list, const float4 *__restrict__ rec,
-                                             const float4 *__restrict__ hp, const int4 *__restrict__ tbox,
-                                             const float4 *__restrict__ tile_box,
-                                             unsigned long long *__restrict__ tile_cnt,
-                                             unsigned long long *__restrict__ hit_entry,
-                                             unsigned *__restrict__ hit_tile, long long cap_pairs, int resident,
-                                             Counters *cnt)
+__global__ void __launch_bounds__(kBinWarps * 32, 4) k_bin(
+    const ViewDev *__restrict__ views, int nviews, const long long *__restrict__ tri_offs, long long ttot,
+    const CandList list, const float4 *__restrict__ rec, const float4 *__restrict__ hp, const int4 *__restrict__ tbox,
+    const float4 *__restrict__ tile_box, unsigned long long *__restrict__ tile_cnt,
+    unsigned long long *__restrict__ hit_entry, unsigned *__restrict__ hit_tile, long long cap_pairs, int resident,
+    Counters *cnt)
 {
+    __shared__ int s_own[kBinWarps][kBinChunks * 32];       // entry (less the task's first) that starts at a pair
+    __shared__ unsigned s_key[kBinWarps][kBinChunks * 32];  // the task's hits
+    __shared__ unsigned s_tri[kBinWarps][kBinChunks * 32];
+    __shared__ unsigned s_tile[kBinWarps][kBinChunks * 32];
     const long long m = (long long)list.length(cnt);
     const unsigned long long *__restrict__ cand_off = list.off;
     const int *__restrict__ binned = list.binned;
@@ -1078,123 +1080,137 @@ __global__ void __launch_bounds__(256, 4) k_bin(const ViewDev *__restrict__ view
     if (m == 0)
         return;
     const long long total = (long long)(list.shift ? cnt->binned_cand >> list.shift : cand_off[m]);
-    const int lane = threadIdx.x & 31;
-    const long long nwarps = (long long)gridDim.x * (blockDim.x >> 5);
-    // Each warp takes tasks of nch x 32 consecutive candidate pairs, up to
-    // kBinChunks x 32 where there are enough of them: a task's chunks run one
-    // after the other, each a chain of dependent loads, so a frame with few
-    // pairs spreads them over more of the resident warps (512^2, 10k
-    // triangles: 7 us, 20.7 us with eight chunks always).  The list entry of the task's first pair comes
-    // from a warp-wide 32-ary search; the entries of each chunk's pairs then
-    // follow from the offsets of the next 32 entries, loaded with one
-    // coalesced read and searched with shuffles (every entry owns at least
-    // one pair, so 32 pairs never reach past them).  All lanes run the same
-    // iterations (for the shuffles).
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const unsigned upto = 0xffffffffu >> (31 - lane);  // lanes up to this one
+    int *own = s_own[warp];
+    const long long nwarps = (long long)gridDim.x * kBinWarps;
     const int nch = (int)min((long long)kBinChunks, (total + 32ll * resident - 1) / (32ll * resident));
-    for (long long pt = ((long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * (32 * nch); pt < total;
+    int vq = 0;  // the view of the lane's last triangle, and its triangles
+    long long v_lo = 0, v_hi = 0;
+    for (long long pt = ((long long)blockIdx.x * kBinWarps + warp) * (32 * nch); pt < total;
          pt += nwarps * (32 * nch)) {
-        long long e0 = warp_owner(cand_off, m, pt);
-        // the task's hits: per chunk the ballot, the lane's entry and tile
-        unsigned want_c[kBinChunks];
-        unsigned long long ent_c[kBinChunks];
-        unsigned tile_c[kBinChunks];
+        const int np = (int)min(32ll * nch, total - pt);  // the task's pairs
+        const long long e0 = warp_owner(cand_off, m, pt);
+        for (int c = 0; c < nch; ++c)
+            own[32 * c + lane] = 0;
+        // entry e0 starts at or before the task's first pair (at most 2^22 before it)
+        int start = (int)((long long)cand_off[e0] - pt), rel = 0;
+        __syncwarp();
+        for (int r = 1 + lane;; r += 128) {
+            unsigned long long o[4];
 #pragma unroll
-        for (int c = 0; c < kBinChunks; ++c) {
-            want_c[c] = 0u;
-            ent_c[c] = 0ull;
-            tile_c[c] = 0u;
-            const long long pw = pt + 32 * c;
-            if (c >= nch || pw >= total)
-                continue;  // warp-uniform
-            const long long p = pw + lane;
-            const long long el = e0 + 1 + lane;
-            const unsigned long long o = el < m ? cand_off[el] : (el == m ? (unsigned long long)total : ~0ull);
-            // every lane takes part in every shuffle; the fallback search
-            // (no warp operations) runs after them
-            int k = 0;  // offsets of the window at or below p
-            for (int sstep = 16; sstep > 0; sstep >>= 1) {
-                const unsigned long long probe = __shfl_sync(0xffffffffu, o, k + sstep - 1);
-                if (probe <= (unsigned long long)p)
-                    k += sstep;
-            }
-            const bool beyond = __shfl_sync(0xffffffffu, o, 31) <= (unsigned long long)p;
-            const long long e = beyond ? owner_of(cand_off, m, p) : e0 + k;
-            e0 = __shfl_sync(0xffffffffu, e, 31);  // owners ascend with p
-            bool hit = false, ok_tile = true;
-            long long tile = -1;
-            unsigned key = 0u;
-            long long g = 0;
-            if (p < total) {
-                g = binned[e];
-                const int4 tb = tbox[g];
-                key = (unsigned)tb.w;
-                const ViewDev &v = views[find_view(tri_offs, nviews, g)];
-                const int sh = __ffs(v.S) - 1;  // S is a power of two
-                const int tx0 = (tb.x & 0xffff) >> sh, tx1 = (tb.x >> 16) >> sh;
-                const int ty0 = (tb.y & 0xffff) >> sh;
-                const int w = tx1 - tx0 + 1;
-                const unsigned long long off = cand_off[e];
-                const int q = (int)(p - (long long)off);  // < tiles of one view
-                const int qy = q / w;
-                const int tx = tx0 + (q - qy * w), ty = ty0 + qy;
-                tile = v.tile_off + (long long)ty * v.tiles_x + tx;
-                if (tx < 0 || ty < 0 || tx >= v.tiles_x || ty >= v.tiles_y) {  // never for a consistent bound
-                    atomicOr(&cnt->status, ST_BAD_INDEX);
-                    tile = v.tile_off;
-                    ok_tile = false;
-                }
-                const float4 bb = rec[g * kRecF4 + 4];
-                const bool fbspace = (tb.z & 0x100) != 0;
-                const int nh = w > 1 || (tb.y >> 16) >> sh != ty0 ? (tb.z & 0xff) : 0;  // more than one candidate
-                if (!ok_tile) {
-                    hit = false;
-                } else if (!fbspace) {
-                    hit = tile_meets(tile_box[tile], bb, hp + g * kMaxHp, nh);
-                } else {
-                    // the tile's pixel-centre box in framebuffer coordinates
-                    const int i0 = tx << sh, i1 = min(v.W, (tx + 1) << sh) - 1;
-                    const int j0 = ty << sh, j1 = min(v.H, (ty + 1) << sh) - 1;
-                    const float4 fbt = make_float4(pixel_centre(i0, v.W, v.rW), pixel_centre(i1, v.W, v.rW),
-                                                   pixel_centre(j0, v.H, v.rH), pixel_centre(j1, v.H, v.rH));
-                    const float4 big = make_float4(-INFINITY, INFINITY, -INFINITY, INFINITY);
-                    hit = tile_meets(tile_box[tile], bb, hp, 0) && tile_meets(fbt, big, hp + g * kMaxHp, nh);
-                }
-            }
-            want_c[c] = __ballot_sync(0xffffffffu, hit);
-            ent_c[c] = ((unsigned long long)key << 32) | (unsigned long long)g;
-            tile_c[c] = (unsigned)tile;
+            for (int k = 0; k < 4; ++k)
+                o[k] = e0 + r + 32 * k < m ? cand_off[e0 + r + 32 * k] : ~0ull;
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                if (o[k] < (unsigned long long)(pt + np))  // and beyond pt: e0 is the last entry at or before it
+                    atomicMax(&own[(int)((long long)o[k] - pt)], r + 32 * k);
+            if (__any_sync(0xffffffffu, o[3] >= (unsigned long long)(pt + np)))
+                break;  // offsets ascend
         }
-        // the task's hits go to the hit list with one atomic ...
-        unsigned ntask = 0;
+        __syncwarp();
+        int nhit = 0;
+#pragma unroll 1
+        for (int c0 = 0; c0 < nch; c0 += kBinGroup) {
+            long long g[kBinGroup];
+            int q[kBinGroup];  // the pair's number among its entry's candidates, < 2^22 (-1: no pair)
 #pragma unroll
-        for (int c = 0; c < kBinChunks; ++c)
-            ntask += __popc(want_c[c]);
-        if (ntask == 0)
+            for (int k = 0; k < kBinGroup; ++k) {
+                const int i = 32 * (c0 + k) + lane;
+                q[k] = -1;
+                g[k] = 0;
+                if (32 * (c0 + k) >= np)
+                    continue;  // warp-uniform
+                const int mark = own[i];
+                const unsigned marks = __ballot_sync(0xffffffffu, mark != 0), mine = marks & upto;
+                const int src = mine ? 31 - __clz(mine) : 0;
+                const int from = __shfl_sync(0xffffffffu, mark, src);
+                const int e = mine ? from : rel, st = mine ? 32 * (c0 + k) + src : start;
+                rel = __shfl_sync(0xffffffffu, e, 31);
+                start = __shfl_sync(0xffffffffu, st, 31);
+                if (i < np) {
+                    q[k] = i - st;
+                    g[k] = binned[e0 + e];
+                }
+            }
+            int4 tb[kBinGroup];
+#pragma unroll
+            for (int k = 0; k < kBinGroup; ++k)
+                if (q[k] >= 0)
+                    tb[k] = tbox[g[k]];
+#pragma unroll
+            for (int k = 0; k < kBinGroup; ++k) {
+                if (32 * (c0 + k) >= np)
+                    break;  // warp-uniform
+                bool hit = false;
+                long long tile = 0;
+                if (q[k] >= 0) {
+                    if (g[k] < v_lo || g[k] >= v_hi) {
+                        vq = find_view(tri_offs, nviews, g[k]);
+                        v_lo = tri_offs[vq];
+                        v_hi = tri_offs[vq + 1];
+                    }
+                    const ViewDev &v = views[vq];
+                    const int sh = __ffs(v.S) - 1;  // S is a power of two
+                    const int tx0 = (tb[k].x & 0xffff) >> sh, tx1 = (tb[k].x >> 16) >> sh;
+                    const int ty0 = (tb[k].y & 0xffff) >> sh;
+                    const int w = tx1 - tx0 + 1;
+                    const int qy = q[k] / w;
+                    const int tx = tx0 + (q[k] - qy * w), ty = ty0 + qy;
+                    tile = v.tile_off + (long long)ty * v.tiles_x + tx;
+                    if (tx < 0 || ty < 0 || tx >= v.tiles_x || ty >= v.tiles_y) {  // never for a consistent bound
+                        atomicOr(&cnt->status, ST_BAD_INDEX);
+                    } else {
+                        const float4 bb = rec[g[k] * kRecF4 + 4];
+                        const float4 *h = hp + g[k] * kMaxHp;
+                        // half-planes: for triangles with more than one candidate
+                        const int nh = w > 1 || (tb[k].y >> 16) >> sh != ty0 ? (tb[k].z & 0xff) : 0;
+                        if (!(tb[k].z & 0x100)) {
+                            hit = tile_meets(tile_box[tile], bb, h, nh);
+                        } else {
+                            // the tile's pixel-centre box in framebuffer coordinates
+                            const int i0 = tx << sh, i1 = min(v.W, (tx + 1) << sh) - 1;
+                            const int j0 = ty << sh, j1 = min(v.H, (ty + 1) << sh) - 1;
+                            const float4 fbt = make_float4(pixel_centre(i0, v.W, v.rW), pixel_centre(i1, v.W, v.rW),
+                                                           pixel_centre(j0, v.H, v.rH), pixel_centre(j1, v.H, v.rH));
+                            const float4 big = make_float4(-INFINITY, INFINITY, -INFINITY, INFINITY);
+                            hit = tile_meets(tile_box[tile], bb, hp, 0) && tile_meets(fbt, big, h, nh);
+                        }
+                    }
+                }
+                const unsigned hits = __ballot_sync(0xffffffffu, hit);
+                if (hit) {
+                    const int at = nhit + __popc(hits & (upto >> 1));
+                    s_key[warp][at] = (unsigned)tb[k].w;
+                    s_tri[warp][at] = (unsigned)g[k];
+                    s_tile[warp][at] = (unsigned)tile;
+                }
+                nhit += __popc(hits);
+            }
+        }
+        __syncwarp();  // the hits are the whole warp's to read, the marks are read
+        if (nhit == 0)
             continue;
         unsigned long long wbase = 0;
         if (lane == 0)
-            wbase = atomicAdd(&cnt->hits_listed, (unsigned long long)ntask);
+            wbase = atomicAdd(&cnt->hits_listed, (unsigned long long)nhit);
         wbase = __shfl_sync(0xffffffffu, wbase, 0);
-#pragma unroll
-        for (int c = 0; c < kBinChunks; ++c) {
-            const unsigned want = want_c[c];
-            if (!want)
-                continue;  // warp-uniform
-            if ((want >> lane) & 1u) {
-                const long long slot = (long long)wbase + __popc(want & ((1u << lane) - 1u));
-                if (slot < cap_pairs) {
-                    hit_entry[slot] = ent_c[c];
-                    hit_tile[slot] = tile_c[c];
-                } else {
-                    atomicOr(&cnt->status, ST_OVERFLOW_PAIRS);
-                }
-                // ... and every tile's count with one atomic per tile met
-                const unsigned peers = __match_any_sync(want, tile_c[c]);
-                if (lane == __ffs(peers) - 1)
-                    atomicAdd(&tile_cnt[tile_c[c]], (unsigned long long)__popc(peers));
+        for (int k = lane; k < nhit; k += 32) {
+            const long long slot = (long long)wbase + k;
+            const unsigned tile = s_tile[warp][k];
+            if (slot < cap_pairs) {
+                hit_entry[slot] = ((unsigned long long)s_key[warp][k] << 32) | s_tri[warp][k];
+                hit_tile[slot] = tile;
+            } else {
+                atomicOr(&cnt->status, ST_OVERFLOW_PAIRS);
             }
-            wbase += __popc(want);
+            // every tile's count with one atomic per tile met
+            const unsigned on = nhit - (k - lane) >= 32 ? 0xffffffffu : (1u << (nhit - (k - lane))) - 1u;
+            const unsigned peers = __match_any_sync(on, tile);
+            if (lane == __ffs(peers) - 1)
+                atomicAdd(&tile_cnt[tile], (unsigned long long)__popc(peers));
         }
+        __syncwarp();  // the hits are written again by the next task
     }
 }
 
@@ -1420,7 +1436,7 @@ cudaError_t launch_bin_count(const ViewDev *views, int nviews, const long long *
                              unsigned *hit_tile, long long cap_pairs, Counters *cnt, cudaStream_t st)
 {
     if (ttot > 0)
-        k_bin<<<bin_count_grid(ttot), 256, 0, st>>>(views, nviews, tri_offs, ttot, list, rec, hp, tbox, tile_box,
+        k_bin<<<bin_count_grid(ttot), kBinWarps * 32, 0, st>>>(views, nviews, tri_offs, ttot, list, rec, hp, tbox, tile_box,
                                                     tile_cnt, hit_entry, hit_tile, cap_pairs, sm_count() * 32, cnt);
     return cudaGetLastError();
 }
