@@ -173,6 +173,12 @@ __device__ __forceinline__ void copy_async_wait_all()
 // (float4 0-3 of the record) and the time interval / D2yz float4 (5).
 constexpr int kStageF4 = 5;
 
+// Runs per claim of the work queue (64 views, 1 / 2 / 4 / 8: 0.622 / 0.511 /
+// 0.472 / 0.479 ms; the stereo HMD frame 0.083 with 1 or 4, and 0.102 to 0.111
+// with long runs claimed in batches too), and the claims that every CTA must
+// get for it.
+constexpr int kBatch = 4, kBatchClaims = 8;
+
 template <int S, bool kFlag>
 __global__ void __launch_bounds__(S *S / 2, PR_FRAG_MINB(S *S / 2))
     k_fragment(const ViewDev *__restrict__ views, const int4 *__restrict__ items,
@@ -199,113 +205,125 @@ __global__ void __launch_bounds__(S *S / 2, PR_FRAG_MINB(S *S / 2))
     float4 *wrec = s_rec[warp];
     unsigned long long n_tests = 0, n_hits = 0;
 
+    // A CTA claims long runs one by one and the others, later in the queue,
+    // by up to kBatch at a time: its warps see unlike parts of a tile and
+    // wait for each other after a claim, so a wait per claim of several runs
+    // costs less than one per run.  Only where every CTA gets kBatchClaims
+    // such claims, so that the last ones even out.
+    const int batch = (int)max(1ll, min((long long)kBatch, (it_hi - nlong) / ((long long)kBatchClaims * gridDim.x)));
+    const long long nclaims = nlong + (it_hi - nlong + batch - 1) / batch;
     if (threadIdx.x == 0)
         s_item[0] = atomicAdd(head, 1);
     __syncthreads();
     for (int par = 0;; par ^= 1) {
-        const long long it = s_item[par];
-        if (it >= it_hi)
+        const long long claim = s_item[par];
+        if (claim >= nclaims)
             break;
-        if (threadIdx.x == 0)  // the next item, fetched while this one runs
+        if (threadIdx.x == 0)  // the next claim, fetched while this one runs
             s_item[par ^ 1] = atomicAdd(head, 1);
-        const int4 item = items[item_place(it, nlong, cap_items)];
-        // the first chunk's bin entries load while the pixels' rays are formed
-        unsigned long long e = item.z + lane < item.w ? pairs[item.z + lane] : ~0ull;
-        const ViewDev &v = views[item.x];
-        const int tx = item.y & 0xffff, ty = item.y >> 16;
-        const int i = tx * S + ci, j0 = ty * S + cj0, j1 = ty * S + cj1;
-        const bool ok0 = i < v.W && j0 < v.H, ok1 = i < v.W && j1 < v.H;
-        float x00, x01, t0, dx0, dy0, x10, x11, t1, dx1, dy1;
-        pixel_ray(v, min(i, v.W - 1), min(j0, v.H - 1), x00, x01, t0, dx0, dy0);
-        pixel_ray(v, min(i, v.W - 1), min(j1, v.H - 1), x10, x11, t1, dx1, dy1);
-        // the warp's block in display space and time (valid pixels only)
-        const float wx0 = warp_minf(fminf(ok0 ? x00 : INFINITY, ok1 ? x10 : INFINITY));
-        const float wx1 = warp_maxf(fmaxf(ok0 ? x00 : -INFINITY, ok1 ? x10 : -INFINITY));
-        const float wy0 = warp_minf(fminf(ok0 ? x01 : INFINITY, ok1 ? x11 : INFINITY));
-        const float wy1 = warp_maxf(fmaxf(ok0 ? x01 : -INFINITY, ok1 ? x11 : -INFINITY));
-        // with a horizontal scan (d1 = 0) the time strip is already part of
-        // every triangle's display box; otherwise test the interval too
-        float wt0 = -INFINITY, wt1 = INFINITY;
-        if (is_rolling(v.mode) && v.d1 != 0.f) {
-            wt0 = warp_minf(fminf(ok0 ? t0 : INFINITY, ok1 ? t1 : INFINITY));
-            wt1 = warp_maxf(fmaxf(ok0 ? t0 : -INFINITY, ok1 ? t1 : -INFINITY));
-        }
-        const float zn = v.z_near;
-        const unsigned id_base = (unsigned)v.tri_off;
-        unsigned long long best0 = ~0ull, best1 = ~0ull;
-        float bd0 = INFINITY, bd1 = INFINITY;
-        unsigned hits = 0, tested = 0;
-        bool fl0 = false, fl1 = false;
-        // The run is sorted nearest first (stage b).  Once a triangle cannot
-        // come nearer than every pixel's current best (with a margin for the
-        // FP32 depth; for the precision form also the tie band), no later
-        // one can change a pixel of this warp.  The lanes screen 32 entries
-        // at a time (depth cut, display box, time interval) while their
-        // records stream into the warp's shared memory; the warp then runs
-        // the ray tests for the survivors, in order.
-        const float cull = kFlag ? (1.f + 3.f * kTieRel) : 1.f;
-        for (int k0 = item.z; k0 < item.w; k0 += 32) {
-            float wmax = warp_maxf(fmaxf(ok0 ? bd0 : 0.f, ok1 ? bd1 : 0.f)) * cull;
-            const int kk = k0 + lane;
-            if (k0 != item.z)
-                e = kk < item.w ? pairs[kk] : ~0ull;
-            const float key = depth_from_order_key((unsigned)(e >> 32));
-            const unsigned stopm = __ballot_sync(0xffffffffu, kk >= item.w || key * 0.99999f > wmax);
-            // entries ascend, so every lane from the first stop on stops too
-            const int ncand = stopm ? __ffs(stopm) - 1 : 32;
-            const unsigned gid = (unsigned)e;
-            float d2y = 0.f, d2z = 0.f;
-            bool take = false;
-            if (lane < ncand) {
-                const float4 *r = rec + (size_t)gid * kRecF4;
-#pragma unroll
-                for (int f = 0; f < 4; ++f)
-                    copy16_async(wrec + lane * kStageF4 + f, r + f);
-                const float4 bb = __ldg(r + 4), tb = __ldg(r + 5);
-                d2y = tb.z;
-                d2z = tb.w;
-                take = !(bb.x > wx1 || bb.y < wx0 || bb.z > wy1 || bb.w < wy0 || tb.x > wt1 || tb.y < wt0);
+        const long long it0 = claim < nlong ? claim : nlong + (claim - nlong) * batch;
+        const long long it1 = claim < nlong ? it0 + 1 : min(it0 + batch, it_hi);
+        for (long long it = it0; it < it1; ++it) {
+            const int4 item = items[item_place(it, nlong, cap_items)];
+            // the first chunk's bin entries load while the pixels' rays are formed
+            unsigned long long e = item.z + lane < item.w ? pairs[item.z + lane] : ~0ull;
+            const ViewDev &v = views[item.x];
+            const int tx = item.y & 0xffff, ty = item.y >> 16;
+            const int i = tx * S + ci, j0 = ty * S + cj0, j1 = ty * S + cj1;
+            const bool ok0 = i < v.W && j0 < v.H, ok1 = i < v.W && j1 < v.H;
+            float x00, x01, t0, dx0, dy0, x10, x11, t1, dx1, dy1;
+            pixel_ray(v, min(i, v.W - 1), min(j0, v.H - 1), x00, x01, t0, dx0, dy0);
+            pixel_ray(v, min(i, v.W - 1), min(j1, v.H - 1), x10, x11, t1, dx1, dy1);
+            // the warp's block in display space and time (valid pixels only)
+            const float wx0 = warp_minf(fminf(ok0 ? x00 : INFINITY, ok1 ? x10 : INFINITY));
+            const float wx1 = warp_maxf(fmaxf(ok0 ? x00 : -INFINITY, ok1 ? x10 : -INFINITY));
+            const float wy0 = warp_minf(fminf(ok0 ? x01 : INFINITY, ok1 ? x11 : INFINITY));
+            const float wy1 = warp_maxf(fmaxf(ok0 ? x01 : -INFINITY, ok1 ? x11 : -INFINITY));
+            // with a horizontal scan (d1 = 0) the time strip is already part of
+            // every triangle's display box; otherwise test the interval too
+            float wt0 = -INFINITY, wt1 = INFINITY;
+            if (is_rolling(v.mode) && v.d1 != 0.f) {
+                wt0 = warp_minf(fminf(ok0 ? t0 : INFINITY, ok1 ? t1 : INFINITY));
+                wt1 = warp_maxf(fmaxf(ok0 ? t0 : -INFINITY, ok1 ? t1 : -INFINITY));
             }
-            copy_async_wait_all();
-            __syncwarp();
-            unsigned live = __ballot_sync(0xffffffffu, take);
-            bool stop = stopm != 0u;
-            while (live) {
-                const int k = __ffs(live) - 1;
-                live &= live - 1u;
-                // the bests move with every test: re-check the cut before each
-                // (every 8 tests instead: 0.098 ms against 0.089 on the HMD
-                // frame, 0.385 against 0.276 ms on the 1M-triangle frame)
-                // (a vote: no lane's farther pixel could still see it)
-                const float near = __shfl_sync(0xffffffffu, key, k) * 0.99999f;
-                if (!__any_sync(0xffffffffu, near <= fmaxf(ok0 ? bd0 : 0.f, ok1 ? bd1 : 0.f) * cull)) {
-                    stop = true;
-                    break;
+            const float zn = v.z_near;
+            const unsigned id_base = (unsigned)v.tri_off;
+            unsigned long long best0 = ~0ull, best1 = ~0ull;
+            float bd0 = INFINITY, bd1 = INFINITY;
+            unsigned hits = 0, tested = 0;
+            bool fl0 = false, fl1 = false;
+            // The run is sorted nearest first (stage b).  Once a triangle cannot
+            // come nearer than every pixel's current best (with a margin for the
+            // FP32 depth; for the precision form also the tie band), no later
+            // one can change a pixel of this warp.  The lanes screen 32 entries
+            // at a time (depth cut, display box, time interval) while their
+            // records stream into the warp's shared memory; the warp then runs
+            // the ray tests for the survivors, in order.
+            const float cull = kFlag ? (1.f + 3.f * kTieRel) : 1.f;
+            for (int k0 = item.z; k0 < item.w; k0 += 32) {
+                float wmax = warp_maxf(fmaxf(ok0 ? bd0 : 0.f, ok1 ? bd1 : 0.f)) * cull;
+                const int kk = k0 + lane;
+                if (k0 != item.z)
+                    e = kk < item.w ? pairs[kk] : ~0ull;
+                const float key = depth_from_order_key((unsigned)(e >> 32));
+                const unsigned stopm = __ballot_sync(0xffffffffu, kk >= item.w || key * 0.99999f > wmax);
+                // entries ascend, so every lane from the first stop on stops too
+                const int ncand = stopm ? __ffs(stopm) - 1 : 32;
+                const unsigned gid = (unsigned)e;
+                float d2y = 0.f, d2z = 0.f;
+                bool take = false;
+                if (lane < ncand) {
+                    const float4 *r = rec + (size_t)gid * kRecF4;
+    #pragma unroll
+                    for (int f = 0; f < 4; ++f)
+                        copy16_async(wrec + lane * kStageF4 + f, r + f);
+                    const float4 bb = __ldg(r + 4), tb = __ldg(r + 5);
+                    d2y = tb.z;
+                    d2z = tb.w;
+                    take = !(bb.x > wx1 || bb.y < wx0 || bb.z > wy1 || bb.w < wy0 || tb.x > wt1 || tb.y < wt0);
                 }
-                const float4 r0 = wrec[k * kStageF4 + 0], r1 = wrec[k * kStageF4 + 1];
-                const float4 r2 = wrec[k * kStageF4 + 2], r3 = wrec[k * kStageF4 + 3];
-                const float ky = __shfl_sync(0xffffffffu, d2y, k), kz = __shfl_sync(0xffffffffu, d2z, k);
-                const unsigned id = __shfl_sync(0xffffffffu, gid, k) - id_base;
-                ++tested;
-                ray_test<kFlag, kFlag>(r0, r1, r2, r3, ky, kz, t0, dx0, dy0, zn, id, best0, bd0, hits, fl0);
-                ray_test<kFlag, kFlag>(r0, r1, r2, r3, ky, kz, t1, dx1, dy1, zn, id, best1, bd1, hits, fl1);
+                copy_async_wait_all();
+                __syncwarp();
+                unsigned live = __ballot_sync(0xffffffffu, take);
+                bool stop = stopm != 0u;
+                while (live) {
+                    const int k = __ffs(live) - 1;
+                    live &= live - 1u;
+                    // the bests move with every test: re-check the cut before each
+                    // (every 8 tests instead: 0.098 ms against 0.089 on the HMD
+                    // frame, 0.385 against 0.276 ms on the 1M-triangle frame)
+                    // (a vote: no lane's farther pixel could still see it)
+                    const float near = __shfl_sync(0xffffffffu, key, k) * 0.99999f;
+                    if (!__any_sync(0xffffffffu, near <= fmaxf(ok0 ? bd0 : 0.f, ok1 ? bd1 : 0.f) * cull)) {
+                        stop = true;
+                        break;
+                    }
+                    const float4 r0 = wrec[k * kStageF4 + 0], r1 = wrec[k * kStageF4 + 1];
+                    const float4 r2 = wrec[k * kStageF4 + 2], r3 = wrec[k * kStageF4 + 3];
+                    const float ky = __shfl_sync(0xffffffffu, d2y, k), kz = __shfl_sync(0xffffffffu, d2z, k);
+                    const unsigned id = __shfl_sync(0xffffffffu, gid, k) - id_base;
+                    ++tested;
+                    ray_test<kFlag, kFlag>(r0, r1, r2, r3, ky, kz, t0, dx0, dy0, zn, id, best0, bd0, hits, fl0);
+                    ray_test<kFlag, kFlag>(r0, r1, r2, r3, ky, kz, t1, dx1, dy1, zn, id, best1, bd1, hits, fl1);
+                }
+                if (stop)
+                    break;
+                __syncwarp();  // the staged records are no longer read
             }
-            if (stop)
-                break;
+            n_tests += (unsigned long long)tested * (unsigned)(ok0 + ok1);
+            n_hits += hits;
+            const long long g0 = v.pix_off + (long long)j0 * v.W + i, g1 = v.pix_off + (long long)j1 * v.W + i;
+            if (ok0 && best0 != ~0ull)
+                atomicMin(&keys[g0], best0);
+            if (ok1 && best1 != ~0ull)
+                atomicMin(&keys[g1], best1);
+            if (kFlag) {
+                if (ok0 && fl0)
+                    flag_pixel(g0, flag_bits, flag_list, cnt);
+                if (ok1 && fl1)
+                    flag_pixel(g1, flag_bits, flag_list, cnt);
+            }
             __syncwarp();  // the staged records are no longer read
-        }
-        n_tests += (unsigned long long)tested * (unsigned)(ok0 + ok1);
-        n_hits += hits;
-        const long long g0 = v.pix_off + (long long)j0 * v.W + i, g1 = v.pix_off + (long long)j1 * v.W + i;
-        if (ok0 && best0 != ~0ull)
-            atomicMin(&keys[g0], best0);
-        if (ok1 && best1 != ~0ull)
-            atomicMin(&keys[g1], best1);
-        if (kFlag) {
-            if (ok0 && fl0)
-                flag_pixel(g0, flag_bits, flag_list, cnt);
-            if (ok1 && fl1)
-                flag_pixel(g1, flag_bits, flag_list, cnt);
         }
         __syncthreads();  // s_item[par ^ 1] is written; s_item[par] may be reused
     }

@@ -1,7 +1,8 @@
 """The binning count pass at the edges of its tasks (32 to 256 consecutive
 candidate pairs of a warp): triangles that span many tasks beside ones with a
 single candidate, list lengths around a warp and a task, entries that lose all
-candidates (the paper's foveation bounds).  Images are the exact nearest hits whatever the tiles,
+candidates (the paper's foveation bounds); and the fragment stage's claims of
+several runs at once.  Images are the exact nearest hits whatever the tiles,
 bounds and runs, so every setting gives the same bits."""
 import numpy as np
 import pytest
@@ -55,6 +56,28 @@ def test_large_and_small_triangles_in_one_list(pr, mode, n):
             for bound, fov in (("zenon", "sector"), ("zenon", "recursive"), ("quad", "simple"), ("trivial", "sector")):
                 got = _frame(pr, ws, h, view, tile, pr.make_params(bound, 0, 0, 0, fov))
                 assert all(torch.equal(a, b) for a, b in zip(got, want)), (tile, bound, fov)
+    finally:
+        pr.pr_scene_free(h)
+        pr.pr_workspace_free(ws)
+
+
+@pytest.mark.parametrize("tile,side", [(16, 2240), (32, 2400)])
+def test_claims_of_several_runs(pr, tile, side):
+    """seg = 1 makes every run count as long, claimed one by one; with runs
+    left to the library this frame's are short and many."""
+    import torch
+    rng = np.random.default_rng(tile)
+    z = rng.uniform(2, 10, (40_000, 1, 1))
+    xy = rng.uniform(-0.6, 0.6, (40_000, 1, 2)) + rng.uniform(-0.01, 0.01, (40_000, 3, 2))
+    pos = (np.concatenate([xy, np.ones_like(xy[..., :1])], 2) * z).reshape(-1, 3)
+    h = _scene(pr, pos, np.arange(len(pos)).reshape(-1, 3))
+    view = _view(side, side - 37, S.MODE_ROLLING)
+    ws = pr.pr_workspace_create()
+    try:
+        got = _frame(pr, ws, h, view, tile, pr.make_params("zenon", 0, 0, 0, "sector"))
+        assert pr.pr_workspace_stats(ws)["items"] > 16 * 152 * (7 if tile == 16 else 1)
+        want = _frame(pr, ws, h, view, tile, pr.make_params("zenon", 0, 0, 1, "sector"))
+        assert all(torch.equal(a, b) for a, b in zip(got, want))
     finally:
         pr.pr_scene_free(h)
         pr.pr_workspace_free(ws)
