@@ -128,12 +128,9 @@ __device__ __forceinline__ void ray_test(const float4 r0, const float4 r1, const
     }
 }
 
-// Build-time knob of the fragment kernel: the occupancy it is compiled for
-// (resident warps per SM, which caps registers).
-#ifndef PR_FRAG_WARPS
-#define PR_FRAG_WARPS 24
-#endif
-#define PR_FRAG_MINB(nt) (PR_FRAG_WARPS > 0 ? (PR_FRAG_WARPS * 32) / (nt) : 1)
+// Occupancy the fragment kernel is compiled for, in resident warps per SM
+// (which caps registers): 28 at 72, in the precision form 24 at 80.
+__host__ __device__ constexpr int frag_ctas(int threads, bool flag) { return ((flag ? 24 : 28) * 32) / threads; }
 
 // Marks pixel g for the FP64 re-test (once: a bitmap de-duplicates the
 // pixels that several items flag) and appends it to the flag list.
@@ -174,13 +171,14 @@ __device__ __forceinline__ void copy_async_wait_all()
 constexpr int kStageF4 = 5;
 
 // Runs per claim of the work queue (64 views, 1 / 2 / 4 / 8: 0.622 / 0.511 /
-// 0.472 / 0.479 ms; the stereo HMD frame 0.083 with 1 or 4, and 0.102 to 0.111
-// with long runs claimed in batches too), and the claims that every CTA must
-// get for it.
-constexpr int kBatch = 4, kBatchClaims = 8;
+// 0.472 / 0.479 ms; with long runs claimed in batches too, the stereo HMD
+// frame takes 0.102 to 0.111 instead of 0.083 ms), and the claims that every
+// CTA must get for it (with 8 instead of 32 the HMD and 1M-triangle steps,
+// whose CTAs get 10 to 20 runs each, were about 1 % slower).
+constexpr int kBatch = 4, kBatchClaims = 32;
 
 template <int S, bool kFlag>
-__global__ void __launch_bounds__(S *S / 2, PR_FRAG_MINB(S *S / 2))
+__global__ void __launch_bounds__(S *S / 2, frag_ctas(S *S / 2, kFlag))
     k_fragment(const ViewDev *__restrict__ views, const int4 *__restrict__ items,
                int cls, long long cap_items, int *__restrict__ head,
                const unsigned long long *__restrict__ pairs, const float4 *__restrict__ rec,
@@ -191,7 +189,7 @@ __global__ void __launch_bounds__(S *S / 2, PR_FRAG_MINB(S *S / 2))
     constexpr int NW = NT / 32;    // warps
     constexpr int WPR = S / 8;     // 8x8 warp blocks per tile row
     __shared__ float4 s_rec[NW][32 * kStageF4];  // per warp: the records of its current 32 candidates
-    __shared__ long long s_item[2];
+    __shared__ int s_claim[2];
 
     // an attempt whose bins overflowed is rerun by the host: entries of the
     // dropped hits were never written, so nothing here may read the bins;
@@ -201,7 +199,7 @@ __global__ void __launch_bounds__(S *S / 2, PR_FRAG_MINB(S *S / 2))
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int ci = (warp % WPR) * 8 + (lane & 7);
     const int cj0 = (warp / WPR) * 8 + (lane >> 3), cj1 = cj0 + 4;
-    const long long nlong = (long long)cnt->items_long[cls], it_hi = (long long)cnt->items_n(cls);
+    const int nlong = (int)cnt->items_long[cls], it_hi = (int)cnt->items_n(cls);  // the queue's head is an int too
     float4 *wrec = s_rec[warp];
     unsigned long long n_tests = 0, n_hits = 0;
 
@@ -210,20 +208,20 @@ __global__ void __launch_bounds__(S *S / 2, PR_FRAG_MINB(S *S / 2))
     // wait for each other after a claim, so a wait per claim of several runs
     // costs less than one per run.  Only where every CTA gets kBatchClaims
     // such claims, so that the last ones even out.
-    const int batch = (int)max(1ll, min((long long)kBatch, (it_hi - nlong) / ((long long)kBatchClaims * gridDim.x)));
-    const long long nclaims = nlong + (it_hi - nlong + batch - 1) / batch;
+    const int batch = max(1, min(kBatch, (it_hi - nlong) / (kBatchClaims * (int)gridDim.x)));
+    const int nclaims = nlong + (it_hi - nlong + batch - 1) / batch;
     if (threadIdx.x == 0)
-        s_item[0] = atomicAdd(head, 1);
+        s_claim[0] = atomicAdd(head, 1);
     __syncthreads();
     for (int par = 0;; par ^= 1) {
-        const long long claim = s_item[par];
+        const int claim = s_claim[par];
         if (claim >= nclaims)
             break;
         if (threadIdx.x == 0)  // the next claim, fetched while this one runs
-            s_item[par ^ 1] = atomicAdd(head, 1);
-        const long long it0 = claim < nlong ? claim : nlong + (claim - nlong) * batch;
-        const long long it1 = claim < nlong ? it0 + 1 : min(it0 + batch, it_hi);
-        for (long long it = it0; it < it1; ++it) {
+            s_claim[par ^ 1] = atomicAdd(head, 1);
+        int it = claim < nlong ? claim : nlong + (claim - nlong) * batch;
+        const int it1 = claim < nlong ? it + 1 : min(it + batch, it_hi);
+        for (; it < it1; ++it) {
             const int4 item = items[item_place(it, nlong, cap_items)];
             // the first chunk's bin entries load while the pixels' rays are formed
             unsigned long long e = item.z + lane < item.w ? pairs[item.z + lane] : ~0ull;
@@ -325,7 +323,7 @@ __global__ void __launch_bounds__(S *S / 2, PR_FRAG_MINB(S *S / 2))
             }
             __syncwarp();  // the staged records are no longer read
         }
-        __syncthreads();  // s_item[par ^ 1] is written; s_item[par] may be reused
+        __syncthreads();  // s_claim[par ^ 1] is written; s_claim[par] may be reused
     }
     for (int o = 16; o > 0; o >>= 1) {
         n_tests += __shfl_xor_sync(0xffffffffu, n_tests, o);

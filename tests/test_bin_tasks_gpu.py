@@ -61,10 +61,11 @@ def test_large_and_small_triangles_in_one_list(pr, mode, n):
         pr.pr_workspace_free(ws)
 
 
-@pytest.mark.parametrize("tile,side", [(16, 2240), (32, 2400)])
-def test_claims_of_several_runs(pr, tile, side):
+@pytest.mark.parametrize("tile,side,views", [(16, 2240, 4), (32, 2400, 2)])
+def test_claims_of_several_runs(pr, tile, side, views):
     """seg = 1 makes every run count as long, claimed one by one; with runs
-    left to the library this frame's are short and many."""
+    left to the library these frames' are short and many (enough for claims of
+    several with a fragment CTA of every resident warp)."""
     import torch
     rng = np.random.default_rng(tile)
     z = rng.uniform(2, 10, (40_000, 1, 1))
@@ -72,12 +73,20 @@ def test_claims_of_several_runs(pr, tile, side):
     pos = (np.concatenate([xy, np.ones_like(xy[..., :1])], 2) * z).reshape(-1, 3)
     h = _scene(pr, pos, np.arange(len(pos)).reshape(-1, 3))
     view = _view(side, side - 37, S.MODE_ROLLING)
+    n = view.W * view.H
     ws = pr.pr_workspace_create()
     try:
-        got = _frame(pr, ws, h, view, tile, pr.make_params("zenon", 0, 0, 0, "sector"))
-        assert pr.pr_workspace_stats(ws)["items"] > 16 * 152 * (7 if tile == 16 else 1)
-        want = _frame(pr, ws, h, view, tile, pr.make_params("zenon", 0, 0, 1, "sector"))
-        assert all(torch.equal(a, b) for a, b in zip(got, want))
+        out = {}
+        for seg in (0, 1):
+            out[seg] = [(torch.empty(n, dtype=torch.int32, device="cuda"), torch.empty(n, device="cuda"))
+                        for _ in range(views)]
+            pr.pr_rasterize_batch(ws, [(h, view, *o, None, tile) for o in out[seg]],
+                                  pr.make_params("zenon", 0, 0, seg, "sector"))
+            if seg == 0:
+                ctas = 7 if tile == 16 else 1
+                assert pr.pr_workspace_stats(ws)["items"] > 2 * 32 * 152 * ctas
+        for got, want in zip(out[0], out[1]):
+            assert all(torch.equal(a, b) for a, b in zip(got, want))
     finally:
         pr.pr_scene_free(h)
         pr.pr_workspace_free(ws)
