@@ -296,9 +296,19 @@ struct Ray64 {
     double t, dx, dy;
 };
 
+// a / b in FP64 given 1 / b to FP32: each residual step squares the quotient's
+// relative error (2^-24, 2^-48, below rounding).  Five FP64 operations for an
+// IEEE division's eight to ten; that unit is what the FP64 paths wait for.
+__device__ __forceinline__ double quotient64(double a, double b, double r)
+{
+    const double q = a * r, p = fma(fma(-q, b, a), r, q);
+    return fma(fma(-p, b, a), r, p);
+}
+
 __device__ inline Ray64 pixel_ray64(const ViewDev &v, int i, int j)
 {
-    double x0 = ((double)i + 0.5) / (double)v.W, x1 = ((double)j + 0.5) / (double)v.H;
+    double x0 = quotient64((double)((float)i + 0.5f), (double)v.W, (double)v.rW),
+           x1 = quotient64((double)((float)j + 0.5f), (double)v.H, (double)v.rH);
     if (is_foveated(v.mode)) {
         const double f0 = v.fx, f1 = v.fy;
         const double e0 = x0 - f0, e1 = x1 - f1;
@@ -314,7 +324,8 @@ __device__ inline Ray64 pixel_ray64(const ViewDev &v, int i, int j)
             } else {
                 // (r / D)^(alpha - 1); the integer exponents of the usual
                 // power maps exactly or by one rounded product
-                const double xr = r / 1.4142135623730950488;
+                const double D = 1.4142135623730950488, rD = 0.70710678118654752440, q = r * rD;
+                const double xr = fma(fma(-q, D, r), rD, q);  // r / D
                 s = v.alpha == 2.f ? xr : (v.alpha == 3.f ? xr * xr : pow(xr, (double)v.alpha - 1.0));
             }
             x0 = f0 + e0 * s;

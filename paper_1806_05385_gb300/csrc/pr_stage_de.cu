@@ -194,10 +194,15 @@ __device__ __noinline__ void pixel_hit64(const ViewDev &v, int i, int j, int ia,
             P[k][r] = (1.0 - ry.t) * S + ry.t * E;
         }
     }
-    double w[3];
+    // w_0 = dir.(B x C) of the vertices sheared along the ray (x - dx z, y - dy z)
+    double e[3][2], w[3];
     for (int k = 0; k < 3; ++k) {
-        const double *b = P[(k + 1) % 3], *c = P[(k + 2) % 3];
-        w[k] = d[0] * (b[1] * c[2] - b[2] * c[1]) + d[1] * (b[2] * c[0] - b[0] * c[2]) + d[2] * (b[0] * c[1] - b[1] * c[0]);
+        e[k][0] = P[k][0] - d[0] * P[k][2];
+        e[k][1] = P[k][1] - d[1] * P[k][2];
+    }
+    for (int k = 0; k < 3; ++k) {
+        const double *b = e[(k + 1) % 3], *c = e[(k + 2) % 3];
+        w[k] = b[0] * c[1] - b[1] * c[0];
     }
     const double sw = w[0] + w[1] + w[2];
     h.has_b = sw != 0.0;
