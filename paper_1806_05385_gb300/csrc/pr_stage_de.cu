@@ -592,12 +592,7 @@ __device__ __forceinline__ void shade_body(const ViewDev *__restrict__ views, in
                         v.depth_out[lin] = bg ? INFINITY : __uint_as_float((unsigned)(key[k] >> 32));
                 }
                 if (!hit) {
-                    if (v.rgb_out) {
-                        v.rgb_out[lin] = 0.f;
-                        v.rgb_out[plane + lin] = 0.f;
-                        v.rgb_out[2 * plane + lin] = 0.f;
-                    }
-                    if (kAdjoint && grad && v.loss) {
+                    if (kAdjoint && grad && v.loss) {  // before the colour: rgb_out may be the target's own buffer
                         float e0, e1, e2;
                         if (v.target_u8) {
                             e0 = u8_unit(v.target_u8[lin]);
@@ -609,6 +604,11 @@ __device__ __forceinline__ void shade_body(const ViewDev *__restrict__ views, in
                             e2 = v.target[2 * plane + lin];
                         }
                         lsum += fmaf(e0, e0, fmaf(e1, e1, e2 * e2));
+                    }
+                    if (v.rgb_out) {
+                        v.rgb_out[lin] = 0.f;
+                        v.rgb_out[plane + lin] = 0.f;
+                        v.rgb_out[2 * plane + lin] = 0.f;
                     }
                 }
             }
@@ -758,6 +758,14 @@ __global__ void __launch_bounds__(kShade64Threads, kShade64Ctas)
             const int vq = find_view(pix_offs, nviews, g);
             const ViewDev &v = views[vq];
             const int lin = (int)(g - v.pix_off), plane = v.W * v.H, pj = lin / v.W, pi = lin - pj * v.W;
+            const bool grad = kAdjoint && adjoint && (v.grad_in || v.target || v.target_u8);
+            float gin[3] = {0.f, 0.f, 0.f};  // the gradient or target, before the colour: rgb_out may be its buffer
+            if (grad) {
+#pragma unroll
+                for (int c = 0; c < 3; ++c)
+                    gin[c] = v.target_u8 ? u8_unit(v.target_u8[c * plane + lin])
+                                         : (v.grad_in ? v.grad_in : v.target)[c * plane + lin];
+            }
             PixelHit h;
             PixelAlbedo pa;
             pixel_hit<kFeat>(v, pi, pj, id, h);
@@ -769,17 +777,12 @@ __global__ void __launch_bounds__(kShade64Threads, kShade64Ctas)
                 v.rgb_out[plane + lin] = rgb[1];
                 v.rgb_out[2 * plane + lin] = rgb[2];
             }
-            if (kAdjoint && adjoint && (v.grad_in || v.target || v.target_u8)) {
+            if (grad) {
                 q = vq;
-                float gin[3];
+                if (!v.grad_in) {
 #pragma unroll
-                for (int c = 0; c < 3; ++c) {
-                    if (v.grad_in) {
-                        gin[c] = v.grad_in[c * plane + lin];
-                    } else {
-                        const float t = v.target_u8 ? u8_unit(v.target_u8[c * plane + lin]) : v.target[c * plane + lin];
-                        gin[c] = 2.f * (rgb[c] - t);
-                    }
+                    for (int c = 0; c < 3; ++c)
+                        gin[c] = 2.f * (rgb[c] - gin[c]);
                 }
                 if (v.loss)  // sum (rgb - target)^2
                     atomicAdd(&v.loss_part[(unsigned)(k0 + lane) & (kLossSlots - 1)],
