@@ -1,0 +1,44 @@
+"""The projected filter at the ends of what it accepts: colours near the
+largest float, and display pixels on both sides of the distance at which the
+window's centre no longer serves as the reference of the weights."""
+import numpy as np
+import pytest
+
+from paper_1806_05385_gb300 import scenes as S
+from tests.test_parity_gpu import small_case
+from tests.test_unfoveate_gpu import _covered, _unfoveate_gpu
+
+pytestmark = pytest.mark.gpu
+
+
+def _case(W=131, H=97):
+    _, view = small_case(S.MODE_FOVEATED, W=W, H=H)
+    return view, np.random.default_rng(5).uniform(size=(3, H, W)).astype(np.float32)
+
+
+def test_colours_near_the_largest_float(pr):
+    """Colours of 2^110, display pixels up to 16 in the exponent nearer to
+    another sample than to the window's centre: the image is 2^110 times the image of colours in [0, 1].  Both pass through
+    exponents (qm - q)(2x - qm - q) k with k = Wd^2 log2(e) / (2 sigma^2) =
+    4.5e5, whose second factor is rounded at 2^-24: an error of 2^-23 k |qm - q|
+    in an exponent, 3e-4 for samples within 4 sigma, twice (the two images)."""
+    view, img = _case()
+    Wd, Hd = 3 * view.W, 3 * view.H
+    one = _unfoveate_gpu(pr, view, img, Wd, Hd, "projected", 0.5)
+    big = _unfoveate_gpu(pr, view, img * np.float32(2.0 ** 110), Wd, Hd, "projected", 0.5)
+    assert np.isfinite(big).all()
+    cov = _covered(view, Wd, Hd).reshape(Hd, Wd)
+    assert np.abs(big * np.float32(2.0 ** -110) - one)[:, cov].max() < 1e-3
+
+
+def test_both_references_match_the_oracle(pr, oracle):
+    """Six display pixels per framebuffer pixel and a narrow filter: centres on
+    both sides of exp(-16).  The exponents' error as above with k =
+    5e6 and samples of one framebuffer pixel apart (0.015 at the most
+    stretched): 1e-2."""
+    view, img = _case()
+    Wd, Hd = 6 * view.W, 6 * view.H
+    g = _unfoveate_gpu(pr, view, img, Wd, Hd, "projected", 0.3)
+    o, margin = oracle.unfoveate(view, img, Wd, Hd, "projected", 0.3)
+    bad = (np.abs(g - o).max(axis=0).reshape(-1) > 1e-2) & _covered(view, Wd, Hd) & (margin >= 1e-3)
+    assert np.isfinite(g).all() and not bad.any()
