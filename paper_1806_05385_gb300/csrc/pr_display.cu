@@ -327,11 +327,14 @@ __device__ __forceinline__ void unfoveate_pixel(const DisplayView &dv, const Mip
         // largest float over 50 stay in range, and the sum is at least
         // 2^-24.  Display pixels farther from their centre sample (beyond the
         // framebuffer's disc, or a display of far more pixels) look for the
-        // nearest sample first, whose weight is 1.  (Up to -60 and unscaled
-        // the same time to 1 %, but weights of e^60 overflowed colours above
-        // 1e11; all pixels from the nearest sample: 180 against 171 us.)
+        // nearest sample first, whose weight is 1.  (Up to -60 and unscaled: the
+        // same time, 128 us, but weights of e^60 overflowed colours above 1e11.)
+        // k2 is bounded so that its products with Wd^2, Hd^2 <= 2^28 and
+        // locations stay finite (the reference's own offset 0 times an
+        // infinite factor is not a number): a filter of sigma 2e-15 display
+        // pixels is as narrow as any below it.
         const int dx0 = max(-2, -i), dx1 = min(2, dv.W - 1 - i), dy0 = max(-2, -j), dy1 = min(2, dv.H - 1 - j);
-        const float k2 = -0.5f / (dv.sigma * dv.sigma);
+        const float k2 = fmaxf(-0.5f / (dv.sigma * dv.sigma), -1e29f);
         const float fWd = (float)dv.Wd, fHd = (float)dv.Hd;
         const unsigned plane = (unsigned)dv.W * (unsigned)dv.H;  // <= 2^28
         // offsets from the fovea (from 0 without foveation, so that q = c)

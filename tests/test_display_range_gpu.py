@@ -1,6 +1,7 @@
-"""The projected filter at the ends of what it accepts: colours near the
-largest float, and display pixels on both sides of the distance at which the
-window's centre no longer serves as the reference of the weights."""
+"""The projected filter at the ends of what it accepts: filter widths far below
+a display pixel, colours near the largest float, and display pixels on both
+sides of the distance at which the window's centre no longer serves as the
+reference of the weights."""
 import numpy as np
 import pytest
 
@@ -14,6 +15,21 @@ pytestmark = pytest.mark.gpu
 def _case(W=131, H=97):
     _, view = small_case(S.MODE_FOVEATED, W=W, H=H)
     return view, np.random.default_rng(5).uniform(size=(3, H, W)).astype(np.float32)
+
+
+@pytest.mark.parametrize("sigma", [1e-6, 1e-16, 1e-18, 1e-19, 1e-38])
+def test_tiny_sigma_takes_the_nearest_sample(pr, oracle, sigma):
+    """Any width far below the sample distances gives the nearest sample.  FP32
+    and FP64 may take different ones where two are equally near to about
+    1e-4 display pixels: one pixel in a thousand at most."""
+    view, img = _case()
+    Wd, Hd = 172, 127
+    g = _unfoveate_gpu(pr, view, img, Wd, Hd, "projected", sigma)
+    assert np.isfinite(g).all()
+    o, margin = oracle.unfoveate(view, img, Wd, Hd, "projected", sigma)
+    bad = (np.abs(g - o.astype(np.float32)).max(axis=0).reshape(-1) > 0) & _covered(view, Wd, Hd) & (margin >= 1e-3)
+    assert bad.mean() < 1e-3
+    assert np.array_equal(g, _unfoveate_gpu(pr, view, img, Wd, Hd, "projected", 1e-12))
 
 
 def test_colours_near_the_largest_float(pr):
