@@ -55,13 +55,13 @@ struct ItemsOut {
     long long cap_items = 0, cap_pairs = 0;
     int ncls = 0;
     long long cls_end[kMaxClasses] = {};
+    int spread[kMaxClasses] = {};  // fragment_spread of the class, 0: its runs are not cut
 };
 // every tile's place in the bins (off, and cursor for the scatter) and its
-// work items: runs of at most seg entries (any_seg: or fewer, where the frame
-// has too few entries to give every resident CTA some)
+// work items: runs of at most seg entries (classes with a spread: or fewer,
+// where the frame has too few entries to give every resident CTA some)
 cudaError_t launch_tile_alloc(const unsigned long long *tile_cnt, unsigned long long *off, unsigned *cursor,
-                              long long ntiles, int seg, bool any_seg, Counters *cnt, const ItemsOut &io,
-                              cudaStream_t st);
+                              long long ntiles, int seg, Counters *cnt, const ItemsOut &io, cudaStream_t st);
 cudaError_t launch_bin_scatter(const unsigned long long *hit_entry, const unsigned *hit_tile, unsigned *cursor,
                                unsigned long long *pairs, const ItemsOut &io, long long ntiles, Counters *cnt,
                                cudaStream_t st);
@@ -89,6 +89,9 @@ cudaError_t launch_sort_items(const ItemsOut &io, long long ntiles, int seg, uns
 cudaError_t launch_fragment(int S, bool flag, const ViewDev *views, const ItemsOut &io, int cls, int *head,
                             const unsigned long long *pairs, const float4 *rec, unsigned long long *keys,
                             unsigned *flag_bits, long long *flag_list, Counters *cnt, int grid, cudaStream_t st);
+// CTAs that a frame's runs should reach (launch_tile_alloc): the fragment
+// kernel's resident ones, for tiles of 8 as many as for tiles of 16
+int fragment_spread(int S);
 // resident CTAs of the fragment kernel, or fewer for a frame of few items
 int fragment_grid(int S, bool flag, long long ntiles, long long ttot, int seg);
 cudaError_t launch_retest(const ViewDev *views, int nviews, const long long *pix_offs, const unsigned long long *scan,

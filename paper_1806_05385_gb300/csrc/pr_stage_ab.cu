@@ -1281,28 +1281,37 @@ static int sm_count()
 // one after the other, some 0.2-0.3 us each, so a frame's longest run bounds
 // the stage from below (256 triangles: about 60 us) and a long run that
 // starts last is waited for.  Two measures.  Runs of kLongRun triangles or
-// more come first in the queue (32 and 128: the same).  And with any_seg runs
-// are cut to a power of two, at least 32, near the larger of entries / (2
-// spread), two runs for every resident CTA (spread of them), and twice the
-// mean bin (of spread tiles at least): shorter ones cost tests, since every
-// run starts without the nearer triangles of the others (HMD frame, 256 /
-// 128 / 64 / 32: 12.1 / 12.9 / 18.0 / 29.3 M tests), so only frames with idle
-// CTAs and bins far above the mean are cut.  Fragment stage, runs of 256 in
-// tile order / long runs first / cut too: 256^2 frame 26.7 / 26.5 / 13.2 us,
-// odd-sized eye 35 / 33 / 25, lens eye 52 / 50 / 37, 8 views 85 / 77 / 64, HMD
-// frame 91 / 75 / 73, 1M triangles 252 / 211 / 211; 512^2 frame of even bins 18
-// to 20 either way, 25 if cut to 64.
+// more come first in the queue (32 and 128: the same).  And where the caller
+// leaves the length open, runs are cut to a power of two, at least 32, near the
+// larger of entries / (2 spread), two runs for every resident CTA of the class's
+// fragment kernel (spread of them: 7 per SM for tiles of 16, 1 for 32; for 8 as
+// for 16), and twice the mean bin (of spread tiles at least): shorter ones cost
+// tests, since every run starts without the nearer triangles of the others (HMD
+// frame, 256 / 128 / 64 / 32: 12.1 / 12.9 / 18.0 / 29.3 M tests), so only frames
+// with idle CTAs and bins far above the mean are cut.  Fragment stage, tiles of
+// 16, runs of 256 in tile order / long runs first / cut too: 256^2 frame 26.7 /
+// 26.5 / 13.2 us, odd-sized eye 35 / 33 / 25, lens eye 52 / 50 / 37, 8 views 85
+// / 77 / 64, HMD frame 91 / 75 / 73, 1M triangles 252 / 211 / 211; 512^2 frame
+// of even bins 18 to 20 either way, 25 if cut to 64.  The whole frame with tiles
+// of 32, spread of 7 / 1 per SM: HMD frame 355 / 322 us, 8 views 433 / 351, eye
+// 174 / 162, 256^2 112 / 111; with tiles of 8, spread of 28 (what is resident) /
+// 7 per SM: 8 views 376 / 369, HMD frame 478 / 479, eye 176 / 176, 256^2 117 /
+// 119.  A batch of several tile sizes, whose classes share the entries counted
+// here, keeps 7 for all: 8 views 373 us, 392 with 1 for its tiles of 32.
 constexpr int kAllocThreads = 256;
 constexpr int kMinSeg = 32, kLongRun = 64;
 __global__ void __launch_bounds__(kAllocThreads) k_tile_alloc(const unsigned long long *__restrict__ tile_cnt,
                                                               unsigned long long *__restrict__ off_out,
                                                               unsigned *__restrict__ cursor, long long ntiles,
-                                                              int seg, int spread, Counters *cnt, const ItemsOut io)
+                                                              int seg, Counters *cnt, const ItemsOut io)
 {
     __shared__ unsigned long long s_n[kAllocThreads / 32];
     __shared__ unsigned s_it[2 * kMaxClasses][kAllocThreads / 32];  // long runs, the others, per class
     __shared__ unsigned long long s_pairs;                           // the CTA's first bin entry
     __shared__ unsigned long long s_items[2 * kMaxClasses];          // its first items
+    const long long g = (long long)blockIdx.x * kAllocThreads + threadIdx.x;
+    const int cls = (io.ncls > 1 && g >= io.cls_end[0]) + (io.ncls > 2 && g >= io.cls_end[1]);
+    const int spread = cls == 0 ? io.spread[0] : (cls == 1 ? io.spread[1] : io.spread[2]);
     if (spread) {
         const unsigned long long per = max(cnt->hits_listed / (2u * (unsigned)spread),
                                            2ull * cnt->hits_listed / (unsigned long long)max(ntiles, (long long)spread));
@@ -1315,7 +1324,6 @@ __global__ void __launch_bounds__(kAllocThreads) k_tile_alloc(const unsigned lon
         seg = min(s, seg);
     }
     const int long_run = min(kLongRun, seg);
-    const long long g = (long long)blockIdx.x * kAllocThreads + threadIdx.x;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const unsigned long long n = g < ntiles ? tile_cnt[g] : 0ull;
     // whole runs are long; the last, shorter one may be
@@ -1329,7 +1337,6 @@ __global__ void __launch_bounds__(kAllocThreads) k_tile_alloc(const unsigned lon
     }
     const unsigned nit = whole + (tail != 0u);
     const unsigned nlong = whole + (tail >= (unsigned)long_run);
-    const int cls = (io.ncls > 1 && g >= io.cls_end[0]) + (io.ncls > 2 && g >= io.cls_end[1]);
     unsigned long long inc = n;  // entries, and runs of each kind and class, up to this lane
     unsigned iit[2 * kMaxClasses];
 #pragma unroll
@@ -1409,12 +1416,11 @@ __global__ void __launch_bounds__(kAllocThreads) k_tile_alloc(const unsigned lon
 }
 
 cudaError_t launch_tile_alloc(const unsigned long long *tile_cnt, unsigned long long *off, unsigned *cursor,
-                              long long ntiles, int seg, bool any_seg, Counters *cnt, const ItemsOut &io,
-                              cudaStream_t st)
+                              long long ntiles, int seg, Counters *cnt, const ItemsOut &io, cudaStream_t st)
 {
     if (ntiles > 0)
         k_tile_alloc<<<(unsigned)((ntiles + kAllocThreads - 1) / kAllocThreads), kAllocThreads, 0, st>>>(
-            tile_cnt, off, cursor, ntiles, seg, any_seg ? sm_count() * 7 : 0, cnt, io);
+            tile_cnt, off, cursor, ntiles, seg, cnt, io);
     return cudaGetLastError();
 }
 

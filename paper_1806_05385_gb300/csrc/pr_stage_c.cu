@@ -360,10 +360,17 @@ static int grid_for()
     return g;
 }
 
+static int fragment_resident(int S, bool flag)
+{
+    return flag ? (S == 8 ? grid_for<8, true>() : (S == 16 ? grid_for<16, true>() : grid_for<32, true>()))
+                : (S == 8 ? grid_for<8, false>() : (S == 16 ? grid_for<16, false>() : grid_for<32, false>()));
+}
+
+int fragment_spread(int S) { return fragment_resident(std::max(S, 16), false); }
+
 int fragment_grid(int S, bool flag, long long ntiles, long long ttot, int seg)
 {
-    const int g = flag ? (S == 8 ? grid_for<8, true>() : (S == 16 ? grid_for<16, true>() : grid_for<32, true>()))
-                       : (S == 8 ? grid_for<8, false>() : (S == 16 ? grid_for<16, false>() : grid_for<32, false>()));
+    const int g = fragment_resident(S, flag);
     // a guess at the items of a small frame: one per tile, and the runs of bins
     // that hold every triangle eight times (runs of 32 at least, unless the
     // caller asks for shorter ones)
