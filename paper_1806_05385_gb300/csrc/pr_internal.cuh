@@ -296,13 +296,26 @@ struct Ray64 {
     double t, dx, dy;
 };
 
-// a / b in FP64 given 1 / b to FP32: each residual step squares the quotient's
-// relative error (2^-24, 2^-48, below rounding).  Five FP64 operations for an
-// IEEE division's eight to ten; that unit is what the FP64 paths wait for.
-__device__ __forceinline__ double quotient64(double a, double b, double r)
+// a / b in FP64 for a = i + 1/2 and a size b = n (0 <= i < n <= 16384) given
+// r = 1 / n to FP32: each residual step squares the quotient's relative error
+// (2^-24, 2^-48, 2^-72), and no such quotient lies within 2^-68 of the middle
+// between two FP64 numbers, so it is the division's result (checked for every i
+// and n).  Five FP64 operations for an IEEE division's eight to ten; that unit
+// is what the FP64 paths wait for.
+__host__ __device__ __forceinline__ double quotient64(double a, double b, double r)
 {
     const double q = a * r, p = fma(fma(-q, b, a), r, q);
     return fma(fma(-p, b, a), r, p);
+}
+
+// r / sqrt(2) in FP64 by the correctly rounded reciprocal of that (rounded)
+// divisor: a product and two fused multiply-adds give the division's result
+// (Markstein 1990).
+__host__ __device__ __forceinline__ double over_sqrt2(double r)
+{
+    const double D = 1.4142135623730950488, rD = 1.0 / 1.4142135623730950488;  // folded, rounded to nearest
+    const double q = r * rD;
+    return fma(fma(-q, D, r), rD, q);
 }
 
 __device__ inline Ray64 pixel_ray64(const ViewDev &v, int i, int j)
@@ -324,8 +337,7 @@ __device__ inline Ray64 pixel_ray64(const ViewDev &v, int i, int j)
             } else {
                 // (r / D)^(alpha - 1); the integer exponents of the usual
                 // power maps exactly or by one rounded product
-                const double D = 1.4142135623730950488, rD = 0.70710678118654752440, q = r * rD;
-                const double xr = fma(fma(-q, D, r), rD, q);  // r / D
+                const double xr = over_sqrt2(r);
                 s = v.alpha == 2.f ? xr : (v.alpha == 3.f ? xr * xr : pow(xr, (double)v.alpha - 1.0));
             }
             x0 = f0 + e0 * s;
