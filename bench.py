@@ -269,6 +269,17 @@ def aggregate(local_ms: float, local_pixels: int, dist=None, device="cpu"):
     return float(p.item()) / (ms * 1e-3) / 1e6, ms
 
 
+def stage_a_bytes(triangles, culled, vertices, tiles, cleared_pixels):
+    """Bytes the bound pass and the frame init cannot do without: per
+    triangle-view its indices (16 B) and pixel box (16 B); per vertex its
+    record (32 B: position and velocity), read once; per triangle-view that is
+    not culled its record (96 B) and its place (4 B) and offset (8 B) in the
+    list; per tile a display box (16 B) and a cleared count (8 B); 8 B per key
+    cleared.  Half-planes (16 B each, up to seven per kept triangle) are not
+    counted."""
+    return 32 * triangles + 32 * vertices + 108 * (triangles - culled) + 24 * tiles + 8 * cleared_pixels
+
+
 def our_arm(args, rank, world):
     import torch
     from paper_1806_05385_gb300 import binding as B
@@ -699,22 +710,21 @@ def our_arm(args, rank, world):
                                     "(CUDA events on the launching stream, inside replays of the frame graph captured "
                                     "with stage events, ten replays)"}
     roof, roof2 = (roof_shade, roof_frag) if shade_ms > frag_ms else (roof_frag, roof_shade)
-    # stage (a) with the frame init, HBM: per triangle-view at least 84 B in
-    # (three vertices' positions and velocities, indices) and 120 B out
-    # (record, pixel box, candidate count); per pixel the 8 B key set to
-    # ~0; per tile 16 B display box + 20 B counts and cursors
+    # stage (a) with the frame init, HBM.  (The key clear, 8 B per pixel, only
+    # where the frame's keys fit in L2: a larger frame's keys are set back by
+    # the previous frame's shading.)
     ttot = sum(wl.scenes[wl.scene_of[k]].T for k in range(len(views)))
+    verts = sum(wl.scenes[wl.scene_of[k]].V for k in range(len(views)))
     ntiles = sum(((v.W + tiles[k] - 1) // tiles[k]) * ((v.H + tiles[k] - 1) // tiles[k]) for k, v in enumerate(views))
-    # (the key clear, 8 B per pixel, only where the frame's keys fit in L2:
-    # a larger frame's keys are set back by the previous frame's shading)
-    a_bytes = 204 * ttot + (8 * pix if 8 * pix <= (96 << 20) else 0) + 36 * ntiles
+    a_bytes = stage_a_bytes(ttot, st["culled"], verts, ntiles, pix if 8 * pix <= (96 << 20) else 0)
     a_gbs = a_bytes / (stage_ms[0] * 1e-3) / 1e9 if stage_ms[0] > 0 else 0.0
     roof_a = {"bound": "hbm", "achieved": a_gbs, "peak": hbm_peak, "unit": "GB/s",
               "frac": a_gbs / hbm_peak if hbm_peak else None, "traffic": None,
               "kernel": "k_frame_init + k_bound (stage a)", "time_ms": stage_ms[0], "algorithmic_bytes": a_bytes,
-              "achieved_basis": "204 B per triangle-view + 8 B per pixel (frames with keys within 96 MB) + "
-                                "36 B per tile (lower bound: the "
-                                "half-planes of kept triangles not counted) / stage (a) event time"}
+              "achieved_basis": "16 B of indices and a 16 B pixel box per triangle-view, 32 B per vertex of each "
+                                "view's scene, 108 B (record, list place and offset) per triangle-view that is not "
+                                "culled, 24 B per tile, 8 B per pixel in frames with keys within 96 MB (lower bound: "
+                                "the half-planes of kept triangles not counted) / stage (a) event time"}
     roof = dict(roof, secondary=roof2, stage_a=roof_a)
 
     cpu = None
