@@ -736,10 +736,10 @@ def our_arm(args, rank, world):
                "tests_per_s": r["tests"] / r["seconds"]}
 
     n_classes = len({(t, wl.fp64) for t in tiles})
-    # frame init (with the tile boxes), bound, candidate scan, bin count, tile scan (with the work
-    # items), bin scatter, run sort, one fragment launch per (tile, precision) class, [FP64 re-test],
-    # resolve + shade + loss + adjoint, the losses' partial sums
-    kernels_step = 9 + n_classes + (1 if wl.fp64 else 0)
+    # frame init (with the tile boxes), bound, bin count, bin places (with the work items), bin scatter,
+    # run sort, one fragment launch per (tile, precision) class, [FP64 re-test], resolve + shade + loss +
+    # adjoint, [FP64 shading], the losses' partial sums, the counters' copy to the host
+    kernels_step = 9 + n_classes + (2 if wl.fp64 else 0)
     line = {
         "metric": METRIC, "value": value, "unit": "Mpix/s", "n_gpus": world, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": mean_ms, "higher_is_better": True, "scaling": "weak",
@@ -750,7 +750,7 @@ def our_arm(args, rank, world):
                            "run sort, fragment, [FP64 re-test], resolve + shade + L2 loss against each view's 8-bit "
                            "target image + adjoint (one kernel); the status of the step's last replay is read after it",
                    "l2": f"flushed before every timed step (256 MB write); between the frames of a step, inputs larger "
-                         f"than L2: each frame reads {96 * ttot / 1e6:.0f} MB of stage (a) records and writes "
+                         f"than L2: each frame reads {96 * (ttot - st['culled']) / 1e6:.0f} MB of stage (a) records and writes "
                          f"{20 * pix / 1e6:.0f} MB of images", "parallelism": f"replicas x{world}"},
         "roofline": roof,
         "cpu_baseline": cpu,
