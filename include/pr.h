@@ -452,6 +452,10 @@ pr_status pr_debug_bounds(const pr_scene *scene, int32_t *pix_box, float *t_rang
  * Culled triangles have no half-planes.  Synchronises the device. */
 pr_status pr_debug_halfplanes(const pr_scene *scene, float *hp, int32_t *info);
 
+/* Pixels of the workspace's last eager frame that the precision form's
+ * shading left to its FP64 launch (0 without fp64_retest).  For tests. */
+pr_status pr_debug_deferred(const pr_workspace *ws, int64_t *pixels);
+
 /* Host evaluation of the stage (a) catch-up interval for one triangle (the
  * Zenon bound of Sec. 4.2.4): S, E float [3][3] camera-space vertices at
  * t = 0 and t = 1; writes [t_min, t_max] and returns 1, or returns 0 when

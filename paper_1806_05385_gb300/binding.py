@@ -32,7 +32,8 @@ EXPORTS = ("pr_scene_upload", "pr_scene_update", "pr_scene_free", "pr_rasterize"
            "pr_debug_catch_interval", "pr_status_string", "pr_version", "pr_rasterize_noalloc",
            "pr_backward_batch", "pr_frame_batch", "pr_graph_capture_frame", "pr_unfoveate", "pr_foveation_create",
            "pr_foveation_free", "pr_graph_enqueue", "pr_graph_status", "pr_measure_fp32_peak",
-           "pr_debug_scan_timeout", "pr_debug_halfplanes", "pr_scene_update_batch", "pr_unfoveate_batch")
+           "pr_debug_scan_timeout", "pr_debug_halfplanes", "pr_debug_deferred", "pr_scene_update_batch",
+           "pr_unfoveate_batch")
 
 
 class PrError(RuntimeError):
@@ -131,6 +132,7 @@ def load(build_if_missing: bool = True):
             "pr_workspace_stats": ([P, C.POINTER(PrStats)], I32),
             "pr_debug_bounds": ([P, P, P], I32),
             "pr_debug_halfplanes": ([P, P, P], I32),
+            "pr_debug_deferred": ([P, C.POINTER(C.c_int64)], I32),
             "pr_debug_catch_interval": ([C.POINTER(PrView), P, P, P], I32),
             "pr_status_string": ([I32], C.c_char_p),
             "pr_version": ([], I32),
@@ -485,6 +487,14 @@ def pr_debug_halfplanes(scene, T: int):
     info = np.empty(T, np.int32)
     _check(load().pr_debug_halfplanes(C.c_void_p(scene), _ptr(hp), _ptr(info)), "pr_debug_halfplanes")
     return hp, info
+
+
+def pr_debug_deferred(ws) -> int:
+    """Pixels of the workspace's last eager frame shaded by the precision
+    form's FP64 launch."""
+    n = C.c_int64()
+    _check(load().pr_debug_deferred(C.c_void_p(ws), C.byref(n)), "pr_debug_deferred")
+    return n.value
 
 
 def pr_debug_catch_interval(view, S, E):

@@ -1470,6 +1470,14 @@ pr_status pr_workspace_stats(const pr_workspace *ws, pr_stats *out)
     return PR_OK;
 }
 
+pr_status pr_debug_deferred(const pr_workspace *ws, int64_t *pixels)
+{
+    if (!ws || !pixels || !ws->h_cnt.p)
+        return PR_ERR_INVALID_ARG;
+    *pixels = (int64_t)ws->h_cnt.p->shade64;
+    return PR_OK;
+}
+
 pr_status pr_debug_bounds(const pr_scene *sc, int32_t *pix_box, float *t_range)
 {
     if (!sc || !pix_box || !t_range)
