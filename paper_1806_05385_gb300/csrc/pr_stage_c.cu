@@ -173,9 +173,12 @@ constexpr int kStageF4 = 5;
 // Runs per claim of the work queue (64 views, 1 / 2 / 4 / 8: 0.622 / 0.511 /
 // 0.472 / 0.479 ms; with long runs claimed in batches too, the stereo HMD
 // frame takes 0.102 to 0.111 instead of 0.083 ms), and the claims that every
-// CTA must get for it (with 8 instead of 32 the HMD and 1M-triangle steps,
-// whose CTAs get 10 to 20 runs each, were about 1 % slower).
-constexpr int kBatch = 4, kBatchClaims = 32;
+// CTA must get for it (fragment stage with 64 / 32 / 16 / 8 / 4 / 1: 64 views
+// 636 / 479 / 476 / 476 / 476 / 478 us; 1M-triangle stereo frame and 20 views,
+// whose CTAs get 16 to 32 short runs each, 176 / 176 / 176 / 149 / 149 / 149 and
+// 200 / 200 / 200 / 175 / 177 / 176; with 1 the HMD frame, of fewer, 90 against
+// 84).
+constexpr int kBatch = 4, kBatchClaims = 8;
 
 template <int S, bool kFlag>
 __global__ void __launch_bounds__(S *S / 2, frag_ctas(S *S / 2, kFlag))
