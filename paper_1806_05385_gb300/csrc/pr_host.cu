@@ -723,13 +723,12 @@ pr_status enqueue_batch(pr_workspace *ws, BatchPlan &P, int seg, bool shade, cud
     io.cap_items = ws->cap_items;
     io.cap_pairs = ws->cap_pairs;
     io.ncls = (int)P.classes.size();
-    for (int c = 0; c < io.ncls; ++c) {
+    for (int c = 0; c < io.ncls; ++c)
         io.cls_end[c] = P.classes[c].tile_hi;
-        // (the precision form keeps long runs: shorter ones see fewer nearer
-        // triangles, and so flag more pixels)
-        io.spread[c] = P.any_seg && !P.any_fp64 ? fragment_spread(io.ncls == 1 ? P.classes[c].S : 16) : 0;
-    }
-    PR_TRY(launch_tile_alloc(tile_cnt, scan, ws->fill.as<unsigned>(), P.ntiles, seg, cnt, io, st));
+    // (the precision form keeps long runs: shorter ones see fewer nearer
+    // triangles, and so flag more pixels)
+    const int spread = P.any_seg && !P.any_fp64 ? fragment_spread(io.ncls == 1 ? P.classes[0].S : 16) : 0;
+    PR_TRY(launch_tile_alloc(tile_cnt, scan, ws->fill.as<unsigned>(), P.ntiles, seg, spread, cnt, io, st));
     PR_TRY(launch_bin_scatter(ws->hit_entry.as<unsigned long long>(), ws->hit_tile.as<unsigned>(),
                               ws->fill.as<unsigned>(), ws->pairs.as<unsigned long long>(), io, P.ntiles, cnt, st));
     PR_TRY(launch_sort_items(io, P.ntiles, seg, ws->pairs.as<unsigned long long>(), cnt, st));

@@ -55,13 +55,13 @@ struct ItemsOut {
     long long cap_items = 0, cap_pairs = 0;
     int ncls = 0;
     long long cls_end[kMaxClasses] = {};
-    int spread[kMaxClasses] = {};  // fragment_spread of the class, 0: its runs are not cut
 };
 // every tile's place in the bins (off, and cursor for the scatter) and its
-// work items: runs of at most seg entries (classes with a spread: or fewer,
-// where the frame has too few entries to give every resident CTA some)
+// work items: runs of at most seg entries (spread > 0: or fewer, where the
+// frame has too few entries to give so many CTAs some)
 cudaError_t launch_tile_alloc(const unsigned long long *tile_cnt, unsigned long long *off, unsigned *cursor,
-                              long long ntiles, int seg, Counters *cnt, const ItemsOut &io, cudaStream_t st);
+                              long long ntiles, int seg, int spread, Counters *cnt, const ItemsOut &io,
+                              cudaStream_t st);
 cudaError_t launch_bin_scatter(const unsigned long long *hit_entry, const unsigned *hit_tile, unsigned *cursor,
                                unsigned long long *pairs, const ItemsOut &io, long long ntiles, Counters *cnt,
                                cudaStream_t st);

@@ -238,8 +238,8 @@ extern "C" pr_status pr_rasterize_noalloc(const float *pos, const float *vel, co
     io.cap_pairs = cap_pairs;
     io.ncls = 1;
     io.cls_end[0] = nt;
-    io.spread[0] = !params || params->seg <= 0 ? fragment_spread(tile) : 0;
-    NA_TRY(launch_tile_alloc(tile_cnt, scan, fill, nt, seg, cnt, io, st));
+    const int spread = !params || params->seg <= 0 ? fragment_spread(tile) : 0;
+    NA_TRY(launch_tile_alloc(tile_cnt, scan, fill, nt, seg, spread, cnt, io, st));
     NA_TRY(launch_bin_scatter(hit_entry, hit_tile, fill, pairs, io, nt, cnt, st));
     NA_TRY(launch_sort_items(io, nt, seg, pairs, cnt, st));
     NA_TRY(launch_fragment(tile, false, dv, io, 0, heads, pairs, rec, keys, nullptr, nullptr, cnt,

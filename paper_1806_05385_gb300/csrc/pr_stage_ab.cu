@@ -1283,7 +1283,7 @@ static int sm_count()
 // starts last is waited for.  Two measures.  Runs of kLongRun triangles or
 // more come first in the queue (32 and 128: the same).  And where the caller
 // leaves the length open, runs are cut to a power of two, at least 32, near the
-// larger of entries / (2 spread), two runs for every resident CTA of the class's
+// larger of entries / (2 spread), two runs for every resident CTA of the
 // fragment kernel (spread of them: 7 per SM for tiles of 16, 1 for 32; for 8 as
 // for 16), and twice the mean bin (of spread tiles at least): shorter ones cost
 // tests, since every run starts without the nearer triangles of the others (HMD
@@ -1303,15 +1303,12 @@ constexpr int kMinSeg = 32, kLongRun = 64;
 __global__ void __launch_bounds__(kAllocThreads) k_tile_alloc(const unsigned long long *__restrict__ tile_cnt,
                                                               unsigned long long *__restrict__ off_out,
                                                               unsigned *__restrict__ cursor, long long ntiles,
-                                                              int seg, Counters *cnt, const ItemsOut io)
+                                                              int seg, int spread, Counters *cnt, const ItemsOut io)
 {
     __shared__ unsigned long long s_n[kAllocThreads / 32];
     __shared__ unsigned s_it[2 * kMaxClasses][kAllocThreads / 32];  // long runs, the others, per class
     __shared__ unsigned long long s_pairs;                           // the CTA's first bin entry
     __shared__ unsigned long long s_items[2 * kMaxClasses];          // its first items
-    const long long g = (long long)blockIdx.x * kAllocThreads + threadIdx.x;
-    const int cls = (io.ncls > 1 && g >= io.cls_end[0]) + (io.ncls > 2 && g >= io.cls_end[1]);
-    const int spread = cls == 0 ? io.spread[0] : (cls == 1 ? io.spread[1] : io.spread[2]);
     if (spread) {
         const unsigned long long per = max(cnt->hits_listed / (2u * (unsigned)spread),
                                            2ull * cnt->hits_listed / (unsigned long long)max(ntiles, (long long)spread));
@@ -1324,6 +1321,7 @@ __global__ void __launch_bounds__(kAllocThreads) k_tile_alloc(const unsigned lon
         seg = min(s, seg);
     }
     const int long_run = min(kLongRun, seg);
+    const long long g = (long long)blockIdx.x * kAllocThreads + threadIdx.x;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const unsigned long long n = g < ntiles ? tile_cnt[g] : 0ull;
     // whole runs are long; the last, shorter one may be
@@ -1337,6 +1335,7 @@ __global__ void __launch_bounds__(kAllocThreads) k_tile_alloc(const unsigned lon
     }
     const unsigned nit = whole + (tail != 0u);
     const unsigned nlong = whole + (tail >= (unsigned)long_run);
+    const int cls = (io.ncls > 1 && g >= io.cls_end[0]) + (io.ncls > 2 && g >= io.cls_end[1]);
     unsigned long long inc = n;  // entries, and runs of each kind and class, up to this lane
     unsigned iit[2 * kMaxClasses];
 #pragma unroll
@@ -1416,11 +1415,12 @@ __global__ void __launch_bounds__(kAllocThreads) k_tile_alloc(const unsigned lon
 }
 
 cudaError_t launch_tile_alloc(const unsigned long long *tile_cnt, unsigned long long *off, unsigned *cursor,
-                              long long ntiles, int seg, Counters *cnt, const ItemsOut &io, cudaStream_t st)
+                              long long ntiles, int seg, int spread, Counters *cnt, const ItemsOut &io,
+                              cudaStream_t st)
 {
     if (ntiles > 0)
         k_tile_alloc<<<(unsigned)((ntiles + kAllocThreads - 1) / kAllocThreads), kAllocThreads, 0, st>>>(
-            tile_cnt, off, cursor, ntiles, seg, cnt, io);
+            tile_cnt, off, cursor, ntiles, seg, spread, cnt, io);
     return cudaGetLastError();
 }
 
