@@ -319,7 +319,7 @@ typedef enum {
     PR_UNFOVEATE_PROJECTED = 1  /* the framebuffer pixel holding q^-1(x) and its 5x5 neighbourhood, weighted
                                    by exp(-d^2 / (2 sigma^2)), d = display-pixel distance between x and q of
                                    each pixel centre, normalised by the weights' sum (computed relative
-                                   to the nearest sample, so far from the framebuffer they do not all
+                                   to a near sample, so far from the framebuffer they do not all
                                    underflow) */
 } pr_unfoveate_method;
 

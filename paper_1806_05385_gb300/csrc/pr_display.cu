@@ -608,9 +608,10 @@ cudaError_t launch_unfoveate_batch(int method, float sigma, const DisplayEntry *
     if (n <= 0)
         return cudaSuccess;
     if (method == PR_UNFOVEATE_PROJECTED) {
-        // view after view with the single-view kernels (q table, then the
-        // filter), each view's q table in the same scratch: the table of all
-        // views at once, or of L2-sized groups, was measured slower
+        // view after view with the single-view kernels (tap table, then the
+        // filter), each view's table in the same scratch (with a table of 8
+        // bytes per pixel, that of all views at once, or of L2-sized groups,
+        // was measured slower)
         for (int q = 0; q < n; ++q) {
             const cudaError_t err = launch_unfoveate(method, e[q].W, e[q].H, e[q].mode, e[q].fx, e[q].fy, e[q].alpha,
                                                      e[q].p_lut, e[q].p_n, e[q].Wd, e[q].Hd, sigma, e[q].rgb, scratch,

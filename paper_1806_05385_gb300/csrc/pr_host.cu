@@ -142,7 +142,7 @@ struct pr_workspace {
     DevBuf views;  // a call's view table, then its offsets (triangles, tiles, pixels, strips: n + 1 each)
     DevBuf rec, hp, tbox, tile_box, tile_cnt, scan, fill, sums, pairs, items, keys, counters, heads;
     DevBuf hit_entry, hit_tile;  // (triangle, tile) hits of the binning count pass, before the scatter
-    DevBuf mip;                  // display step: MIP pyramid of the framebuffer image
+    DevBuf mip;                  // display step: MIP pyramids (levels 1 up), or the projected filter's tap table (16 B per pixel)
     DevBuf disp;                 // batched display step: its view and block tables
     PinnedBuf<char> h_disp;      // ... and their host copy
     cudaEvent_t disp_ev = nullptr;  // recorded after the table copy of the last batched display call

@@ -26,9 +26,13 @@ __host__ __device__ inline long long pixel_blocks(int W, int H, int nsub = 1)
 // Blocks per strip for a launch over this many blocks: strips of four keep
 // four blocks' loads in flight per warp and share the warp's set-up (64
 // views, 2.74 M blocks: 1.33 against 2.04 ms for the training frame's
-// shading; stereo HMD frame, 144,000 blocks: 0.126 against 0.162 ms), but a
-// launch with fewer blocks than about twice the 152 x 40 resident warps
-// times four leaves SMs idle with them.
+// shading; stereo HMD frame, 144,000 blocks: 0.126 against 0.162 ms), but in a
+// launch of few blocks they leave SMs idle, the longer the more triangles a
+// block shows.  Shading of a training frame, strips of one / four: one view of
+// 20,000 blocks 36 / 41 us, 30,000 45 / 45, 40,000 55 / 51, 50,000 65 / 59,
+// 60,000 75 / 67; eight small views of 20,000 to 60,000 triangles each 58 / 69
+// at 40,000 blocks, 74 / 92 at 60,000, 88 / 88 at 80,000, 118 / 110 at 120,000.
+// The line lies between the two kinds.
 constexpr long long kStripMinBlocks = 40000;
 inline int strip_blocks(long long nblocks) { return nblocks >= kStripMinBlocks ? 4 : 1; }
 constexpr int kMaxSeg = 1024;                      // longest bin run of one work item (pr_params.seg)

@@ -120,11 +120,11 @@ cudaError_t launch_shade(const ViewDev *views, int nviews, const long long *blk_
                          unsigned long long *keys, bool reset_keys, bool adjoint, const Counters *frame_cnt, int feat,
                          cudaStream_t st, const ViewDev *host_views = nullptr, const long long *pix_offs = nullptr,
                          const Deferred64 &def = Deferred64{});
-// a training frame's losses: each view's partial sums (loss_part) added into
-// its loss, once (skipped when the frame's forward overflowed)
 // copies the frame's counters to pinned host memory (a kernel of a few
 // stores: a copy node takes about 6 us longer)
 cudaError_t launch_publish(const Counters *cnt, Counters *host, cudaStream_t st);
+// a training frame's losses: each view's partial sums (loss_part) added into
+// its loss, once (skipped when the frame's forward overflowed)
 cudaError_t launch_loss_finalize(const ViewDev *views, int nviews, const Counters *frame_cnt, cudaStream_t st);
 cudaError_t launch_backward(const ViewDev *views, int nviews, const long long *blk_offs, long long nblocks, int nsub,
                             int feat, cudaStream_t st, const ViewDev *host_views = nullptr);

@@ -264,9 +264,11 @@ __device__ __forceinline__ float4 support_halfplane(float2 n, const float2 (&q)[
 // outside R.  The preimage then lies in the annular sector of those angles
 // and of the radii p^-1 of the nearest and farthest distance.
 //
-// The power map's radii come from the quick power: its relative error, about
-// 1e-6 for the distances and exponents a view can have, is a tenth of the
-// margins below.
+// The power map's radii come from the quick power kD1 2^(log2(r) / alpha).  By
+// the documented errors (log2: 2^-22 for r in [1/2, 2], 2 ulp beyond; 2^x: 2 ulp)
+// its relative error is at most 5e-6, half of the margins below, for r from 1e-8
+// to 2^16.  Smaller radii are far below a pixel, and the preimages of farther
+// regions lie ten viewports and more away, where no margin decides.
 __device__ __forceinline__ float pinv_quick(const ViewDev &v, float r)
 {
     if (v.p_lut) {
@@ -806,7 +808,7 @@ __device__ __forceinline__ void compute_bound(const ViewDev &v, const float3 S[3
 // the foveation preimages, a square root per point and the preimage's code
 // three times; 0.268 / 0.107 / 0.032 ms with the quick power, one square
 // root and two copies; 0.245 / 0.103 / 0.032 ms at 64 registers (eight CTAs of
-// 128 per SM instead of six).
+// 128 per SM instead of six; 48 bytes per thread spilled).
 __global__ void __launch_bounds__(128, 8) k_bound(const ViewDev *__restrict__ views, int nviews,
                                                const long long *__restrict__ tri_offs, long long ttot,
                                                float4 *__restrict__ rec, float4 *__restrict__ hp,

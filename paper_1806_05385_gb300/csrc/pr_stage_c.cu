@@ -128,8 +128,9 @@ __device__ __forceinline__ void ray_test(const float4 r0, const float4 r1, const
     }
 }
 
-// Occupancy the fragment kernel is compiled for, in resident warps per SM
-// (which caps registers): 28 at 72, in the precision form 24 at 80.
+// CTAs per SM the fragment kernel is compiled for (which caps registers): 28
+// warps for tiles of 8 and 16, in the precision form 24 (72 and 80 registers);
+// a tile of 32 is one CTA of 16 warps (93 and 113 registers).
 __host__ __device__ constexpr int frag_ctas(int threads, bool flag) { return ((flag ? 24 : 28) * 32) / threads; }
 
 // Marks pixel g for the FP64 re-test (once: a bitmap de-duplicates the

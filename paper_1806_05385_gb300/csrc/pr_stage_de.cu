@@ -243,9 +243,11 @@ __device__ __noinline__ void pixel_hit64(const ViewDev &v, int i, int j, int ia,
 // (48 registers; the precision form and the stand-alone adjoint 18, 56
 // registers).  A CTA's slot frees only when its slowest warp finishes, and
 // the warps of a CTA see different strips (background, one triangle,
-// several), so small CTAs keep the SM fuller.  Training frame's shading,
-// 64 views / HMD frame / 1M-triangle precision form: 1.29 / 0.126 / 0.493 ms
-// with 20, 1.34 / 0.128 / 0.475 with 18, 1.37 / 0.127 / 0.464 with 16; the
+// several), so small CTAs keep the SM fuller.  Training frame's shading, 64
+// views / HMD frame: 1.29 / 0.126 ms with 20, 1.34 / 0.128 with 18, 1.37 /
+// 0.127 with 16.  Precision form (with the FP64 launch), 1M-triangle stereo /
+// HMD / 8 views: 424 / 204 / 206 us with 20, 415 / 200 / 209 with 18, 409 / 196
+// / 212 with 16: 18 is within 2 % of the better on either kind.  The
 // stand-alone adjoint of four views 0.0466 ms with 20, 0.0459 with 18.
 constexpr int kShadeThreads = 64;
 constexpr int kShadeWarps = kShadeThreads / 32;
@@ -456,8 +458,8 @@ struct TriangleSum {
 // the next ones' loads go out during the sums (1 / 2 / 4 / 8 groups: HMD
 // training frame 132 / 131 / 130 / 128 us, 64 views 1.307 / 1.290 / 1.281 /
 // 1.280 ms, the adjoint of four views 49.4 / 49.3 / 46.6 / 47.2 us; the
-// precision form's step, with more registers in use, 1016 us with 2 and 1020
-// with 8).
+// precision form's shading, with more registers in use, 415 us with 2 and 423
+// with 8 on the 1M-triangle stereo frame, 200 / 201 on the HMD frame).
 constexpr int sum_unroll(int feat) { return feat & kFeatF64 ? 2 : 8; }
 template <int kUnroll>
 __device__ __forceinline__ void sum_block(const ViewDev &v, const float *rows, const ValueLane &vl, bool valid,
@@ -523,9 +525,10 @@ __device__ __forceinline__ bool frame_overflowed(const Counters *frame_cnt)
 // separate adjoint pass.  Whole warps run (the adjoint's sums).
 // views: the device table, or the kernel's parameter table (k_shade_pv).
 //
-// Bound: instruction issue (73 % of peak on 64 views, DRAM 27 %, about 850
-// warp instructions per block that shows a triangle) and, on the background,
-// DRAM writes.
+// Bound: the L1 data pipe (82 % busy on the HMD frame: the adjoint's rows and
+// the spills), instruction issue (73 % of peak, DRAM 27 % on 64 views; 740 to
+// 810 warp instructions per block that shows a triangle) and, on the
+// background, DRAM writes.
 //
 // def.list (the precision form): pixels whose barycentrics need FP64 are not
 // shaded here but listed for k_shade64.  An FP64 instruction holds the SM's
