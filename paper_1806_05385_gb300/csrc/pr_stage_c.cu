@@ -128,10 +128,12 @@ __device__ __forceinline__ void ray_test(const float4 r0, const float4 r1, const
     }
 }
 
-// CTAs per SM the fragment kernel is compiled for (which caps registers): 28
-// warps for tiles of 8 and 16, in the precision form 24 (72 and 80 registers);
-// a tile of 32 is one CTA of 16 warps (93 and 113 registers).
-__host__ __device__ constexpr int frag_ctas(int threads, bool flag) { return ((flag ? 24 : 28) * 32) / threads; }
+// CTAs per SM the fragment kernel is compiled for, in warps (which caps
+// registers): 24, at 72 registers for tiles of 16 (seven CTAs fit) and 80 in the
+// precision form; a tile of 32 is one CTA of 16 warps (95 and 114 registers).
+// Compiled for 28 (also 72 registers): loose bounds 2 % slower (Trivial, 74,000
+// triangles at 720 x 800, 57.7 against 56.6 ms), 64 views 469 / 466 us.
+__host__ __device__ constexpr int frag_ctas(int threads) { return 24 * 32 / threads; }
 
 // Marks pixel g for the FP64 re-test (once: a bitmap de-duplicates the
 // pixels that several items flag) and appends it to the flag list.
@@ -182,7 +184,7 @@ constexpr int kStageF4 = 5;
 constexpr int kBatch = 4, kBatchClaims = 8;
 
 template <int S, bool kFlag>
-__global__ void __launch_bounds__(S *S / 2, frag_ctas(S *S / 2, kFlag))
+__global__ void __launch_bounds__(S *S / 2, frag_ctas(S *S / 2))
     k_fragment(const ViewDev *__restrict__ views, const int4 *__restrict__ items,
                int cls, long long cap_items, int *__restrict__ head,
                const unsigned long long *__restrict__ pairs, const float4 *__restrict__ rec,
@@ -211,123 +213,128 @@ __global__ void __launch_bounds__(S *S / 2, frag_ctas(S *S / 2, kFlag))
     // by up to kBatch at a time: its warps see unlike parts of a tile and
     // wait for each other after a claim, so a wait per claim of several runs
     // costs less than one per run.  Only where every CTA gets kBatchClaims
-    // such claims, so that the last ones even out.
+    // such claims, so that the last ones even out.  One loop over the items with
+    // the claim inside it, and a survivor's record loaded before the vote on it:
+    // with a loop per claim and the record after the vote, frames of many tests
+    // per item (loose bounds) took 3 to 5 % longer (Quad bound, HMD frame 453
+    // against 433 us, 1M triangles 1770 / 1700; Trivial 59.6 / 56.6 ms).
     const int batch = max(1, min(kBatch, (it_hi - nlong) / (kBatchClaims * (int)gridDim.x)));
     const int nclaims = nlong + (it_hi - nlong + batch - 1) / batch;
     if (threadIdx.x == 0)
         s_claim[0] = atomicAdd(head, 1);
-    __syncthreads();
-    for (int par = 0;; par ^= 1) {
-        const int claim = s_claim[par];
-        if (claim >= nclaims)
-            break;
-        if (threadIdx.x == 0)  // the next claim, fetched while this one runs
-            s_claim[par ^ 1] = atomicAdd(head, 1);
-        int it = claim < nlong ? claim : nlong + (claim - nlong) * batch;
-        const int it1 = claim < nlong ? it + 1 : min(it + batch, it_hi);
-        for (; it < it1; ++it) {
-            const int4 item = items[item_place(it, nlong, cap_items)];
-            // the first chunk's bin entries load while the pixels' rays are formed
-            unsigned long long e = item.z + lane < item.w ? pairs[item.z + lane] : ~0ull;
-            const ViewDev &v = views[item.x];
-            const int tx = item.y & 0xffff, ty = item.y >> 16;
-            const int i = tx * S + ci, j0 = ty * S + cj0, j1 = ty * S + cj1;
-            const bool ok0 = i < v.W && j0 < v.H, ok1 = i < v.W && j1 < v.H;
-            float x00, x01, t0, dx0, dy0, x10, x11, t1, dx1, dy1;
-            pixel_ray(v, min(i, v.W - 1), min(j0, v.H - 1), x00, x01, t0, dx0, dy0);
-            pixel_ray(v, min(i, v.W - 1), min(j1, v.H - 1), x10, x11, t1, dx1, dy1);
-            // the warp's block in display space and time (valid pixels only)
-            const float wx0 = warp_minf(fminf(ok0 ? x00 : INFINITY, ok1 ? x10 : INFINITY));
-            const float wx1 = warp_maxf(fmaxf(ok0 ? x00 : -INFINITY, ok1 ? x10 : -INFINITY));
-            const float wy0 = warp_minf(fminf(ok0 ? x01 : INFINITY, ok1 ? x11 : INFINITY));
-            const float wy1 = warp_maxf(fmaxf(ok0 ? x01 : -INFINITY, ok1 ? x11 : -INFINITY));
-            // with a horizontal scan (d1 = 0) the time strip is already part of
-            // every triangle's display box; otherwise test the interval too
-            float wt0 = -INFINITY, wt1 = INFINITY;
-            if (is_rolling(v.mode) && v.d1 != 0.f) {
-                wt0 = warp_minf(fminf(ok0 ? t0 : INFINITY, ok1 ? t1 : INFINITY));
-                wt1 = warp_maxf(fmaxf(ok0 ? t0 : -INFINITY, ok1 ? t1 : -INFINITY));
+    int par = 1, it = 0, it1 = 0;
+    for (;; ++it) {
+        if (it >= it1) {
+            __syncthreads();  // s_claim[par ^ 1] is written; s_claim[par] may be reused
+            par ^= 1;
+            const int claim = s_claim[par];
+            if (claim >= nclaims)
+                break;
+            if (threadIdx.x == 0)  // the next claim, fetched while this one runs
+                s_claim[par ^ 1] = atomicAdd(head, 1);
+            it = claim < nlong ? claim : nlong + (claim - nlong) * batch;
+            it1 = claim < nlong ? it + 1 : min(it + batch, it_hi);
+        }
+        const int4 item = items[item_place(it, nlong, cap_items)];
+        // the first chunk's bin entries load while the pixels' rays are formed
+        unsigned long long e = item.z + lane < item.w ? pairs[item.z + lane] : ~0ull;
+        const ViewDev &v = views[item.x];
+        const int tx = item.y & 0xffff, ty = item.y >> 16;
+        const int i = tx * S + ci, j0 = ty * S + cj0, j1 = ty * S + cj1;
+        const bool ok0 = i < v.W && j0 < v.H, ok1 = i < v.W && j1 < v.H;
+        float x00, x01, t0, dx0, dy0, x10, x11, t1, dx1, dy1;
+        pixel_ray(v, min(i, v.W - 1), min(j0, v.H - 1), x00, x01, t0, dx0, dy0);
+        pixel_ray(v, min(i, v.W - 1), min(j1, v.H - 1), x10, x11, t1, dx1, dy1);
+        // the warp's block in display space and time (valid pixels only)
+        const float wx0 = warp_minf(fminf(ok0 ? x00 : INFINITY, ok1 ? x10 : INFINITY));
+        const float wx1 = warp_maxf(fmaxf(ok0 ? x00 : -INFINITY, ok1 ? x10 : -INFINITY));
+        const float wy0 = warp_minf(fminf(ok0 ? x01 : INFINITY, ok1 ? x11 : INFINITY));
+        const float wy1 = warp_maxf(fmaxf(ok0 ? x01 : -INFINITY, ok1 ? x11 : -INFINITY));
+        // with a horizontal scan (d1 = 0) the time strip is already part of
+        // every triangle's display box; otherwise test the interval too
+        float wt0 = -INFINITY, wt1 = INFINITY;
+        if (is_rolling(v.mode) && v.d1 != 0.f) {
+            wt0 = warp_minf(fminf(ok0 ? t0 : INFINITY, ok1 ? t1 : INFINITY));
+            wt1 = warp_maxf(fmaxf(ok0 ? t0 : -INFINITY, ok1 ? t1 : -INFINITY));
+        }
+        const float zn = v.z_near;
+        const unsigned id_base = (unsigned)v.tri_off;
+        unsigned long long best0 = ~0ull, best1 = ~0ull;
+        float bd0 = ok0 ? INFINITY : 0.f, bd1 = ok1 ? INFINITY : 0.f;  // 0: no pixel, nothing can win
+        unsigned hits = 0, tested = 0;
+        bool fl0 = false, fl1 = false;
+        // The run is sorted nearest first (stage b).  Once a triangle cannot
+        // come nearer than every pixel's current best (with a margin for the
+        // FP32 depth; for the precision form also the tie band), no later
+        // one can change a pixel of this warp.  The lanes screen 32 entries
+        // at a time (depth cut, display box, time interval) while their
+        // records stream into the warp's shared memory; the warp then runs
+        // the ray tests for the survivors, in order.
+        const float cull = kFlag ? (1.f + 3.f * kTieRel) : 1.f;
+        for (int k0 = item.z; k0 < item.w; k0 += 32) {
+            const float wmax = warp_maxf(fmaxf(bd0, bd1)) * cull;
+            const int kk = k0 + lane;
+            if (k0 != item.z)
+                e = kk < item.w ? pairs[kk] : ~0ull;
+            const float key = depth_from_order_key((unsigned)(e >> 32)) * 0.99999f;
+            const unsigned stopm = __ballot_sync(0xffffffffu, kk >= item.w || key > wmax);
+            // entries ascend, so every lane from the first stop on stops too
+            const int ncand = stopm ? __ffs(stopm) - 1 : 32;
+            const unsigned gid = (unsigned)e;
+            float d2y = 0.f, d2z = 0.f;
+            bool take = false;
+            if (lane < ncand) {
+                const float4 *r = rec + (size_t)gid * kRecF4;
+#pragma unroll
+                for (int f = 0; f < 4; ++f)
+                    copy16_async(wrec + lane * kStageF4 + f, r + f);
+                const float4 bb = __ldg(r + 4), tb = __ldg(r + 5);
+                d2y = tb.z;
+                d2z = tb.w;
+                take = !(bb.x > wx1 || bb.y < wx0 || bb.z > wy1 || bb.w < wy0 || tb.x > wt1 || tb.y < wt0);
             }
-            const float zn = v.z_near;
-            const unsigned id_base = (unsigned)v.tri_off;
-            unsigned long long best0 = ~0ull, best1 = ~0ull;
-            float bd0 = INFINITY, bd1 = INFINITY;
-            unsigned hits = 0, tested = 0;
-            bool fl0 = false, fl1 = false;
-            // The run is sorted nearest first (stage b).  Once a triangle cannot
-            // come nearer than every pixel's current best (with a margin for the
-            // FP32 depth; for the precision form also the tie band), no later
-            // one can change a pixel of this warp.  The lanes screen 32 entries
-            // at a time (depth cut, display box, time interval) while their
-            // records stream into the warp's shared memory; the warp then runs
-            // the ray tests for the survivors, in order.
-            const float cull = kFlag ? (1.f + 3.f * kTieRel) : 1.f;
-            for (int k0 = item.z; k0 < item.w; k0 += 32) {
-                float wmax = warp_maxf(fmaxf(ok0 ? bd0 : 0.f, ok1 ? bd1 : 0.f)) * cull;
-                const int kk = k0 + lane;
-                if (k0 != item.z)
-                    e = kk < item.w ? pairs[kk] : ~0ull;
-                const float key = depth_from_order_key((unsigned)(e >> 32));
-                const unsigned stopm = __ballot_sync(0xffffffffu, kk >= item.w || key * 0.99999f > wmax);
-                // entries ascend, so every lane from the first stop on stops too
-                const int ncand = stopm ? __ffs(stopm) - 1 : 32;
-                const unsigned gid = (unsigned)e;
-                float d2y = 0.f, d2z = 0.f;
-                bool take = false;
-                if (lane < ncand) {
-                    const float4 *r = rec + (size_t)gid * kRecF4;
-    #pragma unroll
-                    for (int f = 0; f < 4; ++f)
-                        copy16_async(wrec + lane * kStageF4 + f, r + f);
-                    const float4 bb = __ldg(r + 4), tb = __ldg(r + 5);
-                    d2y = tb.z;
-                    d2z = tb.w;
-                    take = !(bb.x > wx1 || bb.y < wx0 || bb.z > wy1 || bb.w < wy0 || tb.x > wt1 || tb.y < wt0);
-                }
-                copy_async_wait_all();
-                __syncwarp();
-                unsigned live = __ballot_sync(0xffffffffu, take);
-                bool stop = stopm != 0u;
-                while (live) {
-                    const int k = __ffs(live) - 1;
-                    live &= live - 1u;
-                    // the bests move with every test: re-check the cut before each
-                    // (every 8 tests instead: 0.098 ms against 0.089 on the HMD
-                    // frame, 0.385 against 0.276 ms on the 1M-triangle frame)
-                    // (a vote: no lane's farther pixel could still see it)
-                    const float near = __shfl_sync(0xffffffffu, key, k) * 0.99999f;
-                    if (!__any_sync(0xffffffffu, near <= fmaxf(ok0 ? bd0 : 0.f, ok1 ? bd1 : 0.f) * cull)) {
-                        stop = true;
-                        break;
-                    }
-                    const float4 r0 = wrec[k * kStageF4 + 0], r1 = wrec[k * kStageF4 + 1];
-                    const float4 r2 = wrec[k * kStageF4 + 2], r3 = wrec[k * kStageF4 + 3];
-                    const float ky = __shfl_sync(0xffffffffu, d2y, k), kz = __shfl_sync(0xffffffffu, d2z, k);
-                    const unsigned id = __shfl_sync(0xffffffffu, gid, k) - id_base;
-                    ++tested;
-                    ray_test<kFlag, kFlag>(r0, r1, r2, r3, ky, kz, t0, dx0, dy0, zn, id, best0, bd0, hits, fl0);
-                    ray_test<kFlag, kFlag>(r0, r1, r2, r3, ky, kz, t1, dx1, dy1, zn, id, best1, bd1, hits, fl1);
-                }
-                if (stop)
+            copy_async_wait_all();
+            __syncwarp();
+            unsigned live = __ballot_sync(0xffffffffu, take);
+            bool stop = stopm != 0u;
+            while (live) {
+                const int k = __ffs(live) - 1;
+                live &= live - 1u;
+                // the bests move with every test: re-check the cut before each
+                // (every 8 tests instead: 0.098 ms against 0.089 on the HMD
+                // frame, 0.385 against 0.276 ms on the 1M-triangle frame)
+                // (a vote: no lane's farther pixel could still see it)
+                const float4 r0 = wrec[k * kStageF4 + 0], r1 = wrec[k * kStageF4 + 1];
+                const float4 r2 = wrec[k * kStageF4 + 2], r3 = wrec[k * kStageF4 + 3];
+                const float near = __shfl_sync(0xffffffffu, key, k);
+                if (!__any_sync(0xffffffffu, near <= fmaxf(bd0, bd1) * cull)) {
+                    stop = true;
                     break;
-                __syncwarp();  // the staged records are no longer read
+                }
+                const float ky = __shfl_sync(0xffffffffu, d2y, k), kz = __shfl_sync(0xffffffffu, d2z, k);
+                const unsigned id = __shfl_sync(0xffffffffu, gid, k) - id_base;
+                ++tested;
+                ray_test<kFlag, kFlag>(r0, r1, r2, r3, ky, kz, t0, dx0, dy0, zn, id, best0, bd0, hits, fl0);
+                ray_test<kFlag, kFlag>(r0, r1, r2, r3, ky, kz, t1, dx1, dy1, zn, id, best1, bd1, hits, fl1);
             }
-            n_tests += (unsigned long long)tested * (unsigned)(ok0 + ok1);
-            n_hits += hits;
-            const long long g0 = v.pix_off + (long long)j0 * v.W + i, g1 = v.pix_off + (long long)j1 * v.W + i;
-            if (ok0 && best0 != ~0ull)
-                atomicMin(&keys[g0], best0);
-            if (ok1 && best1 != ~0ull)
-                atomicMin(&keys[g1], best1);
-            if (kFlag) {
-                if (ok0 && fl0)
-                    flag_pixel(g0, flag_bits, flag_list, cnt);
-                if (ok1 && fl1)
-                    flag_pixel(g1, flag_bits, flag_list, cnt);
-            }
+            if (stop)
+                break;
             __syncwarp();  // the staged records are no longer read
         }
-        __syncthreads();  // s_claim[par ^ 1] is written; s_claim[par] may be reused
+        n_tests += (unsigned long long)tested * (unsigned)(ok0 + ok1);
+        n_hits += hits;
+        const long long g0 = v.pix_off + (long long)j0 * v.W + i, g1 = v.pix_off + (long long)j1 * v.W + i;
+        if (ok0 && best0 != ~0ull)
+            atomicMin(&keys[g0], best0);
+        if (ok1 && best1 != ~0ull)
+            atomicMin(&keys[g1], best1);
+        if (kFlag) {
+            if (ok0 && fl0)
+                flag_pixel(g0, flag_bits, flag_list, cnt);
+            if (ok1 && fl1)
+                flag_pixel(g1, flag_bits, flag_list, cnt);
+        }
+        __syncwarp();  // the staged records are no longer read
     }
     for (int o = 16; o > 0; o >>= 1) {
         n_tests += __shfl_xor_sync(0xffffffffu, n_tests, o);
