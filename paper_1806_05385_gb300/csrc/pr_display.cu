@@ -18,7 +18,7 @@
 // One thread per display pixel; planar rgb in and out.  What a tap reads
 // lies together: the pyramid's texels above level 0 are (r, g, b, 0), and the
 // projected filter first makes a table of (scale of q, r, g, b) per
-// framebuffer pixel.
+// framebuffer pixel (direct_taps: not for small displays without foveation).
 #include <algorithm>
 #include <cstring>
 
@@ -266,8 +266,27 @@ __device__ __forceinline__ void sample3(const Texels &tx, int w, int h, float s,
     out[2] = fmaf(wy[2], row[2].z, fmaf(wy[1], row[1].z, wy[0] * row[0].z)) * inv;
 }
 
-// Display pixel (a, b) of a view.
-template <int kMethod>
+// Where the projected filter's taps come from: the table, or (kDirect) the
+// image itself, where q scales by 1.
+template <bool kDirect>
+struct TapSource {
+    using Texel = float4;
+    static __device__ __forceinline__ const float4 *base(const float4 *tab, const float *) { return tab; }
+    static __device__ __forceinline__ float4 tap(const float4 *t, unsigned) { return __ldg(t); }
+};
+template <>
+struct TapSource<true> {
+    using Texel = float;
+    static __device__ __forceinline__ const float *base(const float4 *, const float *rgb) { return rgb; }
+    static __device__ __forceinline__ float4 tap(const float *t, unsigned plane)
+    {
+        return make_float4(1.f, __ldg(t), __ldg(t + plane), __ldg(t + 2 * plane));
+    }
+};
+
+// Display pixel (a, b) of a view.  kDirect (the projected filter without
+// foveation): the taps come from the image, there is no table.
+template <int kMethod, bool kDirect = false>
 __device__ __forceinline__ void unfoveate_pixel(const DisplayView &dv, const MipPyramid &pyr,
                                                 const float4 *__restrict__ tab, float *__restrict__ out, int a, int b)
 {
@@ -339,7 +358,8 @@ __device__ __forceinline__ void unfoveate_pixel(const DisplayView &dv, const Mip
         const unsigned plane = (unsigned)dv.W * (unsigned)dv.H;  // <= 2^28
         // offsets from the fovea (from 0 without foveation, so that q = c)
         const float fx = dv.fov ? dv.fx : 0.f, fy = dv.fov ? dv.fy : 0.f;
-        const float sm = __ldg(&tab[(unsigned)(j * dv.W + i)].x);
+        using Src = TapSource<kDirect>;
+        const float sm = kDirect ? 1.f : __ldg(&tab[(unsigned)(j * dv.W + i)].x);
         float qm0 = fmaf(pixel_centre(i, dv.W, dv.rW) - fx, sm, fx), qm1 = fmaf(pixel_centre(j, dv.H, dv.rH) - fy, sm, fy);
         float shift;
         {
@@ -352,7 +372,7 @@ __device__ __forceinline__ void unfoveate_pixel(const DisplayView &dv, const Mip
                     const float4 *tr = tab + (unsigned)((j + dy) * dv.W + i);
                     const float e1 = pixel_centre(j + dy, dv.H, dv.rH) - fy;
                     for (int dx = dx0; dx <= dx1; ++dx) {
-                        const float s = __ldg(&tr[dx].x);
+                        const float s = kDirect ? 1.f : __ldg(&tr[dx].x);
                         const float q0 = fmaf(pixel_centre(i + dx, dv.W, dv.rW) - fx, s, fx), q1 = fmaf(e1, s, fy);
                         const float f0 = (x0 - q0) * fWd, f1 = (x1 - q1) * fHd;
                         const float q2 = fmaf(f0, f0, f1 * f1);
@@ -379,7 +399,7 @@ __device__ __forceinline__ void unfoveate_pixel(const DisplayView &dv, const Mip
             acc[1] = fmaf(w, c.z, acc[1]);
             acc[2] = fmaf(w, c.w, acc[2]);
         };
-        const float4 *tr = tab + (unsigned)((j + dy0) * dv.W + i + dx0);
+        const typename Src::Texel *tr = Src::base(tab, pyr.rgb) + (unsigned)((j + dy0) * dv.W + i + dx0);
         if (dx1 - dx0 == 4) {  // five taps a row (all but two columns at either side), their loads in flight together
             float e0[5];
 #pragma unroll
@@ -390,13 +410,13 @@ __device__ __forceinline__ void unfoveate_pixel(const DisplayView &dv, const Mip
                 const float e1 = pixel_centre(j + dy, dv.H, dv.rH) - fy;
 #pragma unroll
                 for (int dx = 0; dx < 5; ++dx)
-                    tap(e0[dx], e1, __ldg(tr + dx));
+                    tap(e0[dx], e1, Src::tap(tr + dx, plane));
             }
         } else {
             for (int dy = dy0; dy <= dy1; ++dy, tr += dv.W) {
                 const float e1 = pixel_centre(j + dy, dv.H, dv.rH) - fy;
                 for (int dx = dx0; dx <= dx1; ++dx)
-                    tap(pixel_centre(i + dx, dv.W, dv.rW) - fx, e1, __ldg(tr + (dx - dx0)));
+                    tap(pixel_centre(i + dx, dv.W, dv.rW) - fx, e1, Src::tap(tr + (dx - dx0), plane));
             }
         }
         const float inv = 1.f / wsum;
@@ -429,7 +449,7 @@ __device__ __forceinline__ int2 disp_pixel(int bx, int by)
     return make_int2(bx * kDispW + (w % per) * kWarpW + lane % kWarpW, by * kDispH + (w / per) * kWarpH + lane / kWarpW);
 }
 
-template <int kMethod>
+template <int kMethod, bool kDirect = false>
 __global__ void __launch_bounds__(kDispW *kDispH, kDispCtas) k_unfoveate(const DisplayView dv, const MipPyramid pyr,
                                                              const float4 *__restrict__ tab, float *__restrict__ out)
 {
@@ -437,7 +457,7 @@ __global__ void __launch_bounds__(kDispW *kDispH, kDispCtas) k_unfoveate(const D
     const int a = at.x, b = at.y;
     if (a >= dv.Wd || b >= dv.Hd)
         return;
-    unfoveate_pixel<kMethod>(dv, pyr, tab, out, a, b);
+    unfoveate_pixel<kMethod, kDirect>(dv, pyr, tab, out, a, b);
 }
 
 // ---- the batched display step (MIP): many views, two launches for their
@@ -540,6 +560,18 @@ static bool fill_pyramid(MipPyramid &pyr, int W, int H, const float *rgb, float 
     return true;
 }
 
+// Whether the projected filter takes its taps from the image: without
+// foveation q is the identity, and the table (28 bytes moved per framebuffer
+// pixel, to save two of a tap's three loads) pays only for about as many display
+// pixels as the framebuffer has.  2160 x 2160 and 4096 x 4096, table / image, at
+// 1/16 of its side 40 / 12 and 99 / 16 us, 1/4 51 / 20 and 145 / 54, 1/2 65 / 38
+// and 196 / 111, 0.6 77 / 49 and 240 / 152; at the full side the image loses (125
+// / 142 and 411 / 477 in a slower form of it, 108 / 96 at 0.8 of the side).
+static bool direct_taps(const DisplayView &dv)
+{
+    return !dv.fov && 3ll * dv.Wd * dv.Hd <= 2ll * dv.W * dv.H;
+}
+
 cudaError_t launch_unfoveate(int method, int W, int H, int mode, float fx, float fy, float alpha, const float *p_lut,
                              int p_n, int Wd, int Hd, float sigma, const float *rgb, float *scratch, float *out,
                              cudaStream_t st)
@@ -575,6 +607,11 @@ cudaError_t launch_unfoveate(int method, int W, int H, int mode, float fx, float
             k_mip_top<<<1, 512, 0, st>>>(pyr);
         k_unfoveate<PR_UNFOVEATE_MIP_CUBIC><<<grd, blk, 0, st>>>(dv, pyr, nullptr, out);
     } else {
+        pyr.rgb = rgb;
+        if (direct_taps(dv)) {
+            k_unfoveate<PR_UNFOVEATE_PROJECTED, true><<<grd, blk, 0, st>>>(dv, pyr, nullptr, out);
+            return cudaGetLastError();
+        }
         float4 *tab = reinterpret_cast<float4 *>(scratch);
         const dim3 gq((unsigned)((W + 255) / 256), (unsigned)H);
         k_tap_table<<<gq, 256, 0, st>>>(dv, rgb, tab);

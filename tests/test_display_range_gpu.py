@@ -1,13 +1,14 @@
 """The projected filter at the ends of what it accepts: filter widths far below
-a display pixel, colours near the largest float, and display pixels on both
-sides of the distance at which the window's centre no longer serves as the
-reference of the weights."""
+a display pixel, colours near the largest float, display pixels on both sides of
+the distance at which the window's centre no longer serves as the reference of
+the weights, and displays without foveation on both sides of two thirds of the
+framebuffer's pixels, up to which the taps come from the image."""
 import numpy as np
 import pytest
 
 from paper_1806_05385_gb300 import scenes as S
 from tests.test_parity_gpu import small_case
-from tests.test_unfoveate_gpu import _covered, _unfoveate_gpu
+from tests.test_unfoveate_gpu import TOL, _covered, _unfoveate_gpu
 
 pytestmark = pytest.mark.gpu
 
@@ -58,3 +59,20 @@ def test_both_references_match_the_oracle(pr, oracle):
     o, margin = oracle.unfoveate(view, img, Wd, Hd, "projected", 0.3)
     bad = (np.abs(g - o).max(axis=0).reshape(-1) > 1e-2) & _covered(view, Wd, Hd) & (margin >= 1e-3)
     assert np.isfinite(g).all() and not bad.any()
+
+
+@pytest.mark.parametrize("mode", [S.MODE_CLASSIC, S.MODE_ROLLING])
+@pytest.mark.parametrize("size", [(1, 1, 1, 1), (2, 3, 2, 2), (2, 3, 5, 1), (5, 4, 3, 4), (5, 4, 7, 2), (131, 97, 92, 92),
+                                  (131, 97, 92, 93), (257, 33, 16, 8), (64, 300, 200, 64), (300, 64, 64, 201)])
+def test_taps_from_image_and_table(pr, oracle, mode, size):
+    """Both forms against the oracle with the tolerance of the other display
+    tests; a constant image stays constant."""
+    W, H, Wd, Hd = size
+    _, view = small_case(mode, W=W, H=H)
+    img = np.random.default_rng(W + 7 * Hd).uniform(size=(3, H, W)).astype(np.float32)
+    for sigma in (0.5, 2.0):
+        g = _unfoveate_gpu(pr, view, img, Wd, Hd, "projected", sigma)
+        o, margin = oracle.unfoveate(view, img, Wd, Hd, "projected", sigma)
+        assert not np.any((np.abs(g - o).max(axis=0).reshape(-1) > TOL) & (margin >= 1e-3))
+        flat = _unfoveate_gpu(pr, view, np.full_like(img, 0.375), Wd, Hd, "projected", sigma)
+        assert np.abs(flat - 0.375).max() < 1e-6
