@@ -430,7 +430,8 @@ __device__ __forceinline__ void unfoveate_pixel(const DisplayView &dv, const Mip
 }
 
 // CTAs of the display kernels: 32 x 8 display pixels, six per SM, a warp's
-// pixels 16 x 2.  Bound: the L1 data pipe (71 to 77 % busy) and issue.  q^-1
+// pixels 16 x 2.  Bound: the L1 data pipe for the MIP form (79 % busy, issue 66
+// %), issue for the projected filter (84 %, L1 64 %).  q^-1
 // is curved, so a row of 32 display pixels reads up to fifteen rows of
 // texels, and every texel row of a tap is a cache line of its own: squarer
 // warps meet fewer (32 x 1 / 16 x 2 / 8 x 4 with planar texels: projected
