@@ -285,8 +285,10 @@ struct TapSource<true> {
 };
 
 // Display pixel (a, b) of a view.  kDirect (the projected filter without
-// foveation): the taps come from the image, there is no table.
-template <int kMethod, bool kDirect = false>
+// foveation): the taps come from the image, there is no table.  kNarrow: a
+// filter so narrow (narrow_filter) that the rounding of two equally near samples'
+// locations could make an exponent large and positive; it is cut at 1.
+template <int kMethod, bool kDirect = false, bool kNarrow = false>
 __device__ __forceinline__ void unfoveate_pixel(const DisplayView &dv, const MipPyramid &pyr,
                                                 const float4 *__restrict__ tab, float *__restrict__ out, int a, int b)
 {
@@ -393,7 +395,8 @@ __device__ __forceinline__ void unfoveate_pixel(const DisplayView &dv, const Mip
         auto tap = [&](float e0, float e1, float4 c) {
             const float2 minus = make_float2(-1.f, -1.f), q = __ffma2_rn(make_float2(e0, e1), make_float2(c.x, c.x), fov);
             const float2 t = __fmul2_rn(__ffma2_rn(q, minus, qm2), __ffma2_rn(q, minus, far));
-            const float w = exp2_ftz(fmaf(t.x, kw, fmaf(t.y, kh, shift)));
+            const float x = fmaf(t.x, kw, fmaf(t.y, kh, shift));
+            const float w = exp2_ftz(kNarrow ? fminf(x, 1.f) : x);
             wsum += w;
             acc[0] = fmaf(w, c.y, acc[0]);
             acc[1] = fmaf(w, c.z, acc[1]);
@@ -450,7 +453,7 @@ __device__ __forceinline__ int2 disp_pixel(int bx, int by)
     return make_int2(bx * kDispW + (w % per) * kWarpW + lane % kWarpW, by * kDispH + (w / per) * kWarpH + lane / kWarpW);
 }
 
-template <int kMethod, bool kDirect = false>
+template <int kMethod, bool kDirect = false, bool kNarrow = false>
 __global__ void __launch_bounds__(kDispW *kDispH, kDispCtas) k_unfoveate(const DisplayView dv, const MipPyramid pyr,
                                                              const float4 *__restrict__ tab, float *__restrict__ out)
 {
@@ -458,7 +461,7 @@ __global__ void __launch_bounds__(kDispW *kDispH, kDispCtas) k_unfoveate(const D
     const int a = at.x, b = at.y;
     if (a >= dv.Wd || b >= dv.Hd)
         return;
-    unfoveate_pixel<kMethod, kDirect>(dv, pyr, tab, out, a, b);
+    unfoveate_pixel<kMethod, kDirect, kNarrow>(dv, pyr, tab, out, a, b);
 }
 
 // ---- the batched display step (MIP): many views, two launches for their
@@ -573,6 +576,16 @@ static bool direct_taps(const DisplayView &dv)
     return !dv.fov && 3ll * dv.Wd * dv.Hd <= 2ll * dv.W * dv.H;
 }
 
+// Whether a weight's exponent (qm - q)(2x - qm - q) k, k = Wd^2 / (2 sigma^2
+// ln 2), of two samples equally near to x may come out as large as 10: |qm - q|
+// is at most ten framebuffer pixels, and the second factor, 0 but for rounding,
+// 2^-22.  The weights of wider filters need no cut, an instruction per tap.
+static bool narrow_filter(const DisplayView &dv)
+{
+    const double k = 0.7214 * std::max((double)dv.Wd * dv.Wd, (double)dv.Hd * dv.Hd) / ((double)dv.sigma * dv.sigma);
+    return 10.0 / std::min(dv.W, dv.H) * 2.4e-7 * k > 10.0;
+}
+
 cudaError_t launch_unfoveate(int method, int W, int H, int mode, float fx, float fy, float alpha, const float *p_lut,
                              int p_n, int Wd, int Hd, float sigma, const float *rgb, float *scratch, float *out,
                              cudaStream_t st)
@@ -609,14 +622,21 @@ cudaError_t launch_unfoveate(int method, int W, int H, int mode, float fx, float
         k_unfoveate<PR_UNFOVEATE_MIP_CUBIC><<<grd, blk, 0, st>>>(dv, pyr, nullptr, out);
     } else {
         pyr.rgb = rgb;
+        const bool narrow = narrow_filter(dv);
         if (direct_taps(dv)) {
-            k_unfoveate<PR_UNFOVEATE_PROJECTED, true><<<grd, blk, 0, st>>>(dv, pyr, nullptr, out);
+            if (narrow)
+                k_unfoveate<PR_UNFOVEATE_PROJECTED, true, true><<<grd, blk, 0, st>>>(dv, pyr, nullptr, out);
+            else
+                k_unfoveate<PR_UNFOVEATE_PROJECTED, true><<<grd, blk, 0, st>>>(dv, pyr, nullptr, out);
             return cudaGetLastError();
         }
         float4 *tab = reinterpret_cast<float4 *>(scratch);
         const dim3 gq((unsigned)((W + 255) / 256), (unsigned)H);
         k_tap_table<<<gq, 256, 0, st>>>(dv, rgb, tab);
-        k_unfoveate<PR_UNFOVEATE_PROJECTED><<<grd, blk, 0, st>>>(dv, pyr, tab, out);
+        if (narrow)
+            k_unfoveate<PR_UNFOVEATE_PROJECTED, false, true><<<grd, blk, 0, st>>>(dv, pyr, tab, out);
+        else
+            k_unfoveate<PR_UNFOVEATE_PROJECTED><<<grd, blk, 0, st>>>(dv, pyr, tab, out);
     }
     return cudaGetLastError();
 }

@@ -33,6 +33,20 @@ def test_tiny_sigma_takes_the_nearest_sample(pr, oracle, sigma):
     assert np.array_equal(g, _unfoveate_gpu(pr, view, img, Wd, Hd, "projected", 1e-12))
 
 
+@pytest.mark.parametrize("sigma", [1e-3, 1e-6, 1e-9, 1e-16])
+@pytest.mark.parametrize("case", [(S.MODE_CLASSIC, 640, 480, 320, 240), (S.MODE_CLASSIC, 1000, 600, 500, 900),
+                                  (S.MODE_FOVEATED, 64, 64, 32, 32), (S.MODE_FOVEATED, 100, 60, 25, 15)])
+def test_equally_near_samples_under_a_narrow_filter(pr, case, sigma):
+    """Displays whose pixel centres lie midway between samples: whichever of
+    them FP32 calls nearest, the pixel is a mean of colours of its window."""
+    mode, W, H, Wd, Hd = case
+    p0, p1 = S.head_poses(1.0, 0.0)
+    view = S.View(W=W, H=H, tan_x=0.5, tan_y=0.5, pose0=p0, pose1=p1, mode=mode, fovea=(0.5, 0.5))
+    img = np.random.default_rng(3).uniform(0.25, 0.75, size=(3, H, W)).astype(np.float32)
+    g = _unfoveate_gpu(pr, view, img, Wd, Hd, "projected", sigma)
+    assert np.isfinite(g).all() and g.min() >= 0.25 * (1 - 1e-6) and g.max() <= 0.75 * (1 + 1e-6)
+
+
 def test_colours_near_the_largest_float(pr):
     """Colours of 2^110, display pixels up to 16 in the exponent nearer to
     another sample than to the window's centre: the image is 2^110 times the image of colours in [0, 1].  Both pass through
